@@ -1,4 +1,5 @@
-"""ctypes binding of ``libheterospec.so``: argument marshalling only.
+"""Python binding of ``libheterospec.so``: argument marshalling only, by ctypes and, for the calls of a step, by the
+``_native`` module (csrc/py_native.cpp), which reads the tensor bundles below without ctypes structures.
 
 Every function has the name and the meaning of the C entry point in ``include/heterospec.h``;
 torch tensors provide device memory and the current CUDA stream, nothing is computed here.
@@ -138,6 +139,21 @@ def _stream():
     return C.c_void_p(torch.cuda.current_stream().cuda_stream)
 
 
+def native():
+    """The module that makes the step calls (once loaded, it shares the library of lib())."""
+    global _native
+    if _native is None:
+        lib()
+        from . import _native as mod
+        mod.setup(torch.float32, torch.bfloat16)
+        _native = mod
+    return _native
+
+
+_native = None
+_raw_stream = torch._C._cuda_getCurrentRawStream
+
+
 def hs_device_error(ctx: "Context") -> int:
     v = C.c_int32(0)
     _check(lib().hs_device_error(ctx.handle, C.byref(v)), "hs_device_error")
@@ -269,10 +285,8 @@ def hs_entropy_quantify(ctx: Context, tree: TreeBatch, draft_logits: torch.Tenso
                         out: Optional[QuantOut] = None) -> QuantOut:
     if out is None:
         out = QuantOut(tree.n_nodes_total, tree.batch, policy["top_k"], draft_logits.device)
-    t, p, o = tree.c(), make_policy(policy), out.c()
-    _check(lib().hs_entropy_quantify(ctx.handle, C.byref(t), _ptr(draft_logits), _dtype_code(draft_logits),
-                                     draft_logits.stride(0), draft_logits.shape[1], C.byref(p), C.byref(o), _stream()),
-           "hs_entropy_quantify")
+    _check((_native or native()).entropy_quantify(ctx.handle.value or 0, tree, draft_logits, policy, out,
+                                                  _raw_stream(ctx.device)), "hs_entropy_quantify")
     return out
 
 
@@ -300,10 +314,8 @@ def hs_entropy_quantify_prune(ctx: Context, tree: TreeBatch, draft_logits: torch
         out = QuantOut(tree.n_nodes_total, tree.batch, policy["top_k"], draft_logits.device)
     if pruned_out is None:
         pruned_out = PrunedTree(tree.n_nodes_total, tree.batch, tree.parent.device)
-    t, p, o, q = tree.c(), make_policy(policy), out.c(), pruned_out.c()
-    _check(lib().hs_entropy_quantify_prune(ctx.handle, C.byref(t), _ptr(draft_logits), _dtype_code(draft_logits),
-                                           draft_logits.stride(0), draft_logits.shape[1], C.byref(p), C.byref(o),
-                                           C.byref(q), _stream()), "hs_entropy_quantify_prune")
+    _check((_native or native()).entropy_quantify_prune(ctx.handle.value or 0, tree, draft_logits, policy, out, pruned_out,
+                                                        _raw_stream(ctx.device)), "hs_entropy_quantify_prune")
     return out, pruned_out
 
 
@@ -311,8 +323,7 @@ def hs_stratify_prune(ctx: Context, tree: TreeBatch, quant: QuantOut, policy: di
                       out: Optional[PrunedTree] = None) -> PrunedTree:
     if out is None:
         out = PrunedTree(tree.n_nodes_total, tree.batch, tree.parent.device)
-    t, q, p, o = tree.c(), quant.c(), make_policy(policy), out.c()
-    _check(lib().hs_stratify_prune(ctx.handle, C.byref(t), C.byref(q), C.byref(p), C.byref(o), _stream()),
+    _check((_native or native()).stratify_prune(ctx.handle.value or 0, tree, quant, policy, out, _raw_stream(ctx.device)),
            "hs_stratify_prune")
     return out
 
@@ -321,9 +332,8 @@ def hs_stratify_prune_budget(ctx: Context, tree: TreeBatch, quant: QuantOut, pol
                              budget: int, out: Optional[PrunedTree] = None) -> PrunedTree:
     if out is None:
         out = PrunedTree(tree.n_nodes_total, tree.batch, tree.parent.device)
-    t, q, p, o = tree.c(), quant.c(), make_policy(policy), out.c()
-    _check(lib().hs_stratify_prune_budget(ctx.handle, C.byref(t), C.byref(q), C.byref(p), _ptr(slo_class), budget,
-                                          C.byref(o), _stream()), "hs_stratify_prune_budget")
+    _check((_native or native()).stratify_prune_budget(ctx.handle.value or 0, tree, quant, policy, slo_class, budget, out,
+                                                       _raw_stream(ctx.device)), "hs_stratify_prune_budget")
     return out
 
 
@@ -335,17 +345,11 @@ def hs_tree_verify_attention(ctx: Context, pruned: PrunedTree, q: torch.Tensor, 
                              lse_out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """q/out [rows, hq, 128] bf16; k_tree/v_tree [rows, hkv, 128]; k_cache/v_cache [tokens, hkv, 128] (any
     token/head strides that are multiples of 8 elements, innermost dimension contiguous)."""
-    rows, hq, hd = q.shape
-    hkv = k_tree.shape[1]
     if out is None:
         out = torch.empty_like(q)
-    d = _AttnDesc(batch, rows, max_nodes, k_cache.shape[0], max_kv_len, hq, hkv, hd, layout, _ptr(node_off),
-                  _ptr(kv_off), k_cache.stride(0) if k_cache.shape[0] else hkv * hd,
-                  k_cache.stride(1) if k_cache.shape[0] else hd,
-                  float(sm_scale if sm_scale is not None else hd ** -0.5))
-    p = pruned.c()
-    _check(lib().hs_tree_verify_attention(ctx.handle, C.byref(p), C.byref(d), _ptr(q), _ptr(k_tree), _ptr(v_tree),
-                                          _ptr(k_cache), _ptr(v_cache), _ptr(out), _ptr(lse_out), _stream()),
+    _check((_native or native()).tree_verify_attention(ctx.handle.value or 0, pruned, q, k_tree, v_tree, k_cache, v_cache,
+                                                       kv_off, batch, max_nodes, max_kv_len, layout, node_off, sm_scale,
+                                                       out, lse_out, _raw_stream(ctx.device)),
            "hs_tree_verify_attention")
     return out
 
@@ -357,11 +361,8 @@ def hs_accept_path(ctx: Context, tree: TreeBatch, pruned: PrunedTree, target_log
                    out: Optional[AcceptOut] = None) -> AcceptOut:
     if out is None:
         out = AcceptOut(tree.batch, path_cap, target_logits.device)
-    t, p, o = tree.c(), pruned.c(), out.c()
-    _check(lib().hs_accept_path(ctx.handle, C.byref(t), C.byref(p), _ptr(target_logits), target_layout,
-                                _ptr(draft_logits), _dtype_code(target_logits), target_logits.stride(0),
-                                target_logits.shape[1], _ptr(mode), _ptr(temperature), seed, offset, _ptr(uniforms),
-                                C.byref(o), _stream()),
+    _check((_native or native()).accept_path(ctx.handle.value or 0, tree, pruned, target_logits, target_layout, draft_logits,
+                                             mode, temperature, seed, offset, uniforms, out, _raw_stream(ctx.device)),
            "hs_accept_path")
     return out
 
@@ -389,26 +390,24 @@ class ExpandState(_Bundle):
 
 
 def hs_expand_init(ctx: Context, st: ExpandState) -> None:
-    c = st.c()
-    _check(lib().hs_expand_init(ctx.handle, C.byref(c), _stream()), "hs_expand_init")
+    _check((_native or native()).expand_init(ctx.handle.value or 0, st, _raw_stream(ctx.device)), "hs_expand_init")
 
 
 def hs_expand_level(ctx: Context, st: ExpandState, quant: QuantOut) -> None:
     """One expansion level from the row statistics of the frontier rows (row b * top_k + j = frontier j of b)."""
-    c = st.c()
-    _check(lib().hs_expand_level(ctx.handle, C.byref(c), _ptr(quant.topk_val), _ptr(quant.topk_idx),
-                                 _ptr(quant.row_lse), quant.topk_val.shape[1], _stream()), "hs_expand_level")
+    _check((_native or native()).expand_level(ctx.handle.value or 0, st, quant.topk_val, quant.topk_idx, quant.row_lse,
+                                              _raw_stream(ctx.device)), "hs_expand_level")
 
 
 def hs_rerank(ctx: Context, st: ExpandState, n_top: Optional[torch.Tensor], n_default: int):
     """Returns (node_off, parent, token, cand_id, depth): the reranked trees as one CSR batch."""
     dev = st.parent.device
     rows = st.batch * min(st.cap, max(n_default, int(n_top.max()) if n_top is not None else 0))
-    i = lambda *s: torch.zeros(*s, dtype=torch.int32, device=dev)
-    node_off, parent, token, cand_id, depth = i(st.batch + 1), i(rows), i(rows), i(rows), i(rows)
-    c = st.c()
-    _check(lib().hs_rerank(ctx.handle, C.byref(c), _ptr(n_top), n_default, _ptr(node_off), _ptr(parent), _ptr(token),
-                           _ptr(cand_id), _ptr(depth), _stream()), "hs_rerank")
+    # one allocation and one fill for the five arrays (entries past the kept nodes are zero)
+    node_off, parent, token, cand_id, depth = torch.zeros(st.batch + 1 + 4 * rows, dtype=torch.int32, device=dev).split(
+        (st.batch + 1, rows, rows, rows, rows))
+    _check((_native or native()).rerank(ctx.handle.value or 0, st, n_top, n_default, node_off, parent, token, cand_id, depth,
+                                        _raw_stream(ctx.device)), "hs_rerank")
     return node_off, parent, token, cand_id, depth
 
 
@@ -419,7 +418,7 @@ def hs_cart_workspace_bytes(n: int) -> int:
 def hs_cart_fit(ctx: Context, x: torch.Tensor, y: torch.Tensor, depth: int = 3):
     """Trains the stratifier on (Phi(P*), Terminal Confidence Rank) pairs.  Returns (thresholds [2^depth - 1], status [1])."""
     th = torch.empty((1 << depth) - 1, dtype=torch.float32, device=x.device)
-    status = torch.zeros(1, dtype=torch.int32, device=x.device)
+    status = torch.empty(1, dtype=torch.int32, device=x.device)          # (written by the call)
     _check(lib().hs_cart_fit(ctx.handle, _ptr(x), _ptr(y), x.numel(), depth, _ptr(th), _ptr(status), _stream()),
            "hs_cart_fit")
     return th, status

@@ -1,13 +1,16 @@
-"""Builds the CUDA library in-tree: ``paper_2505_13254_b200/libheterospec.so`` (sm_100a only)."""
+"""Builds the CUDA library in-tree: ``paper_2505_13254_b200/libheterospec.so`` (sm_100a only), and ``_native``, the
+module through which the Python binding makes the step calls."""
 
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libheterospec.so")
+NATIVE = os.path.join(HERE, "_native" + sysconfig.get_config_var("EXT_SUFFIX"))
 SOURCES = ["hs_api.cu", "row_stats.cu", "stratify_prune.cu", "tree_attention.cu", "accept.cu", "expand.cu", "cart.cu"]
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
          "-Xcompiler", "-fPIC", "--use_fast_math=false"]
@@ -21,9 +24,9 @@ def _nvcc() -> str:
 
 
 def needs_build() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(NATIVE):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(NATIVE))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(HERE, "..", "include", "heterospec.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -52,6 +55,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if pr.returncode != 0:
             raise RuntimeError(f"nvcc failed on {src}")
     subprocess.check_call([nvcc, "-shared", "-o", LIB, *objs, "-cudart", "static"])
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                           os.path.join(CSRC, "py_native.cpp"), "-o", NATIVE, "-L", HERE, "-l:libheterospec.so",
+                           "-Wl,-rpath,$ORIGIN"])
     return LIB
 
 
