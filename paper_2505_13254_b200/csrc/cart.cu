@@ -1,12 +1,24 @@
 // hs_cart_fit: training of the entropy stratifier on the device (Sec. 4.2, Eq. 2).
 //
-// One feature (x = Phi(P*)) and one target (y = Terminal Confidence Rank): the samples are sorted by x once (bitonic
-// network: chunks of 1024 in shared memory, wider exchanges in global memory), running sums of y and y^2 in double
-// precision follow, and then every layer of the tree scores all split positions of all its nodes in parallel from
-// the running sums - a node is a contiguous range of the sorted samples, a split at position i costs
-//     L = nL / N * (SyyL - SyL^2 / nL) + nR / N * (SyyR - SyR^2 / nR)           (Eq. 2)
+// One feature (x = Phi(P*)) and one target (y = Terminal Confidence Rank): the samples are sorted by x once, and then
+// every layer of the tree scores all split positions of all its nodes in parallel from running sums of y and y^2 in
+// double precision - a node is a contiguous range of the sorted samples, a split at position i costs
+//     N L = nL SyyL - SyL^2 + nR SyyR - SyR^2           (Eq. 2 times the node's sample count)
 // - and takes, per node, the position with the smallest L (ties: the smallest), between distinct feature values
-// only.  The threshold is the midpoint of the two neighbouring feature values.
+// only.  The threshold is the midpoint of the two neighbouring feature values.  (The form without divisions orders the
+// positions of a node as L does, is exact for integer ranks, and costs ten fp64 operations instead of sixty.)
+//
+// Sort: least-significant-digit radix sort of 64-bit keys (order bits of x : bits of y), four passes over the 8-bit digits
+// of x; stable, so equal feature values keep their order and need no more passes.  A bitonic network took 65 launches
+// and 0.9 ms on 2^20 samples (every exchange distance beyond shared memory is a pass over all keys); a pass here reads and
+// writes the keys once, which stay in L2.
+//   up to CT_SMALL samples   cart_small_kernel: one CTA sorts in shared memory and fits all layers - one launch, no round
+//                            trips between layers (17 us at 600 samples, 49 us at 8192; were 68 and 90).
+//   more                     cart_pack_kernel (keys, digit counts of all passes), four cart_radix_kernel, cart_sums_kernel
+//                            (sums per block and their scan), one cart_level_kernel per layer: 70 us at 8193 samples (nine
+//                            launches, latency), 121 us at 2^20 and depth 3 (was 990 us): 12 us pack, 12 - 17 us a pass
+//                            (issue of the ranking ballots, and the look-back), 17 us a layer (fp64 chains and the last
+//                            CTA's reduction over the tiles).
 #include <math_constants.h>
 
 #include "hs_common.cuh"
@@ -14,165 +26,546 @@
 #include "hs_ptx.cuh"
 
 #define CT_THREADS 256
-#define CT_CHUNK 1024
+#define CT_ITEMS 16
+#define CT_TILE (CT_THREADS * CT_ITEMS)      // keys per CTA: 4096
+#define CT_WINDOW 16                         // tiles ahead that are looked at together
 #define CT_MAX_DEPTH 6
-#define CT_SPLIT_BLOCKS 64          // blocks that share the split positions of one node
-
-// key = (order-preserving bits of x) : (bits of y); padding keys are all ones and sort to the end
-__global__ void cart_pack_kernel(const float* x, const float* y, int n, int P, unsigned long long* keys) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P) return;
-    keys[i] = i < n ? (((unsigned long long)float_order_bits(x[i]) << 32) | __float_as_uint(y[i])) : ~0ull;
-}
-
-__device__ __forceinline__ void cmp_swap(unsigned long long& a, unsigned long long& b, bool up) {
-    if ((a > b) == up) { const unsigned long long t = a; a = b; b = t; }
-}
-
-// all exchange distances below CT_CHUNK of the merge step of width k (k >= 2), inside shared memory;
-// with k <= CT_CHUNK and first == true the chunk is sorted from scratch
-__global__ void __launch_bounds__(CT_CHUNK / 2) cart_sort_chunk_kernel(unsigned long long* keys, int k_lo, int k_hi) {
-    __shared__ unsigned long long s[CT_CHUNK];
-    const int tid = threadIdx.x;
-    const size_t base = (size_t)blockIdx.x * CT_CHUNK;
-    s[tid] = keys[base + tid];
-    s[tid + CT_CHUNK / 2] = keys[base + tid + CT_CHUNK / 2];
-    __syncthreads();
-    for (int k = k_lo; k <= k_hi; k <<= 1) {
-        for (int j = min(k >> 1, CT_CHUNK / 2); j > 0; j >>= 1) {
-            const int i = 2 * tid - (tid & (j - 1));           // lower index of this thread's pair
-            const bool up = (((base + i) & (size_t)k) == 0);
-            cmp_swap(s[i], s[i + j], up);
-            __syncthreads();
-        }
-    }
-    keys[base + tid] = s[tid];
-    keys[base + tid + CT_CHUNK / 2] = s[tid + CT_CHUNK / 2];
-}
-
-// one exchange distance j >= CT_CHUNK of the merge step of width k, in global memory
-__global__ void cart_sort_global_kernel(unsigned long long* keys, int P, int j, int k) {
-    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (size_t)P / 2) return;
-    const size_t i = 2 * t - (t & (size_t)(j - 1));
-    const bool up = ((i & (size_t)k) == 0);
-    unsigned long long a = keys[i], b = keys[i + j];
-    if ((a > b) == up) { keys[i] = b; keys[i + j] = a; }
-}
-
-// running sums: block-wise inclusive scans of y and y^2 (double), the blocks' totals, their scan, the offsets
-__global__ void __launch_bounds__(CT_THREADS) cart_scan_blocks_kernel(const unsigned long long* keys, int n, double* sy,
-                                                                      double* syy, double* blk) {
-    __shared__ double s_a[CT_THREADS], s_b[CT_THREADS];
-    const int tid = threadIdx.x;
-    const int i = blockIdx.x * CT_THREADS + tid;
-    double a = 0.0, b = 0.0;
-    if (i < n) { a = (double)__uint_as_float((unsigned int)keys[i]); b = a * a; }
-    s_a[tid] = a; s_b[tid] = b;
-    __syncthreads();
-    for (int o = 1; o < CT_THREADS; o <<= 1) {
-        double ua = 0.0, ub = 0.0;
-        if (tid >= o) { ua = s_a[tid - o]; ub = s_b[tid - o]; }
-        __syncthreads();
-        s_a[tid] += ua; s_b[tid] += ub;
-        __syncthreads();
-    }
-    if (i < n) { sy[i + 1] = s_a[tid]; syy[i + 1] = s_b[tid]; }          // (exclusive sums: entry i = samples before i)
-    if (tid == CT_THREADS - 1) { blk[2 * blockIdx.x] = s_a[tid]; blk[2 * blockIdx.x + 1] = s_b[tid]; }
-    if (i == 0) { sy[0] = 0.0; syy[0] = 0.0; }
-}
-__global__ void cart_scan_totals_kernel(double* blk, int nblk) {     // one thread: the blocks' totals in order
-    double a = 0.0, b = 0.0;
-    for (int i = 0; i < nblk; ++i) {
-        const double ta = blk[2 * i], tb = blk[2 * i + 1];
-        blk[2 * i] = a; blk[2 * i + 1] = b;
-        a += ta; b += tb;
-    }
-}
-__global__ void __launch_bounds__(CT_THREADS) cart_scan_add_kernel(int n, double* sy, double* syy, const double* blk) {
-    const int i = blockIdx.x * CT_THREADS + threadIdx.x;
-    if (i < n) { sy[i + 1] += blk[2 * blockIdx.x]; syy[i + 1] += blk[2 * blockIdx.x + 1]; }
-}
-
-struct CartLevel {
-    const unsigned long long* keys;
-    const double* sy;
-    const double* syy;
-    const int* bnd;        // [nodes + 1] node boundaries (positions in the sorted order) of this layer
-    int* bnd_next;         // [2 * nodes + 1]
-    double* part_l;        // [nodes][CT_SPLIT_BLOCKS] best loss of a block
-    int* part_i;           // [nodes][CT_SPLIT_BLOCKS] its position
-    float* thresholds;     // [2^depth - 1] ascending
-    int* status;
-    int nodes, level, depth;
-};
+#define CT_MAX_NODES (1 << (CT_MAX_DEPTH - 1))
+#define CT_SMALL_THREADS 1024
+#define CT_SMALL_ITEMS 8
+#define CT_SMALL (CT_SMALL_THREADS * CT_SMALL_ITEMS)
 
 __device__ __forceinline__ float key_x(unsigned long long k) { return order_bits_float((unsigned int)(k >> 32)); }
-
-__global__ void __launch_bounds__(CT_THREADS) cart_split_scan_kernel(const CartLevel c) {
-    __shared__ double s_l[CT_THREADS];
-    __shared__ int s_i[CT_THREADS];
-    const int node = blockIdx.y, tid = threadIdx.x;
-    const int lo = c.bnd[node], hi = c.bnd[node + 1];
-    const double N = (double)(hi - lo);
-    double best = CUDART_INF;
-    int best_i = 0x7fffffff;
-    const double sy_lo = c.sy[lo], syy_lo = c.syy[lo], sy_hi = c.sy[hi], syy_hi = c.syy[hi];
-    for (int i = lo + 1 + blockIdx.x * CT_THREADS + tid; i < hi; i += CT_SPLIT_BLOCKS * CT_THREADS) {
-        if (!(key_x(c.keys[i - 1]) < key_x(c.keys[i]))) continue;       // a threshold lies between distinct values
-        const double nl = (double)(i - lo), nr = (double)(hi - i);
-        const double yl = c.sy[i] - sy_lo, yyl = c.syy[i] - syy_lo;
-        const double yr = sy_hi - c.sy[i], yyr = syy_hi - c.syy[i];
-        const double l = nl / N * (yyl - yl * yl / nl) + nr / N * (yyr - yr * yr / nr);
-        if (l < best) { best = l; best_i = i; }                          // (ascending i: the first minimum stays)
+__device__ __forceinline__ double key_y(unsigned long long k) { return (double)__uint_as_float((unsigned int)k); }
+__device__ __forceinline__ unsigned long long cart_key(float x, float y) {
+    return ((unsigned long long)float_order_bits(x) << 32) | __float_as_uint(y);
+}
+__device__ __forceinline__ unsigned int key_digit(unsigned long long k, int pass) { return (unsigned int)(k >> (32 + 8 * pass)) & 255u; }
+// a double as an unsigned integer of the same order
+__device__ __forceinline__ unsigned long long order_bits_d(double v) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+    return (u >> 63) ? ~u : (u | (1ull << 63));
+}
+// The lanes of the warp whose 8-bit digit equals this lane's: eight ballots, or one match for the uppermost digit (its
+// cost grows with the number of different values: 12.5 us a pass instead of 17 there, 18.4 on mantissa digits).
+__device__ __forceinline__ unsigned int digit_peers(unsigned int d, int pass) {
+    if (pass == 3) return __match_any_sync(HS_FULL_MASK, d);
+    unsigned int m = HS_FULL_MASK;
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const unsigned int v = __ballot_sync(HS_FULL_MASK, (d >> b) & 1u);
+        m &= ((d >> b) & 1u) ? v : ~v;
     }
-    s_l[tid] = best; s_i[tid] = best_i;
+    return m;
+}
+// Rank of every key of a warp's NITEM x 32 keys (item-major) among the warp's keys of the same digit; cnt: the warp's 256
+// digit counters, zero before.
+template <int NITEM>
+__device__ __forceinline__ void warp_ranks(const unsigned long long (&k)[NITEM], int pass, int* cnt, int lane, int (&rank)[NITEM]) {
+#pragma unroll
+    for (int i = 0; i < NITEM; ++i) {
+        const unsigned int d = key_digit(k[i], pass), peers = digit_peers(d, pass);
+        const int before = cnt[d];
+        __syncwarp();
+        if ((peers >> lane) == 1u) cnt[d] = before + __popc(peers);        // (the highest lane of the group)
+        rank[i] = before + __popc(peers & ((1u << lane) - 1u));
+        __syncwarp();
+    }
+}
+// exclusive prefix over 256 values, one per thread 0..255 (all threads of the CTA call it)
+__device__ __forceinline__ int scan256(int v, int* s_warp, int tid) {
+    const int lane = tid & 31, warp = tid >> 5;
+    int incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int u = __shfl_up_sync(HS_FULL_MASK, incl, o); if (lane >= o) incl += u; }
+    if (lane == 31 && warp < 8) s_warp[warp] = incl;
     __syncthreads();
-    for (int o = CT_THREADS / 2; o > 0; o >>= 1) {
-        if (tid < o) {
-            const double l2 = s_l[tid + o];
-            const int i2 = s_i[tid + o];
-            if (l2 < s_l[tid] || (l2 == s_l[tid] && i2 < s_i[tid])) { s_l[tid] = l2; s_i[tid] = i2; }
+    int before = incl - v;
+    for (int w = 0; w < 8; ++w) if (w < warp) before += s_warp[w];
+    return before;
+}
+
+// ---- one layer: all split positions of a block of sorted keys -----------------------------------------------------
+struct LayerSmem {
+    int bnd[CT_MAX_NODES + 1];                       // node boundaries (positions in the sorted order)
+    double sy[CT_MAX_NODES + 1], syy[CT_MAX_NODES + 1];   // running sums at the boundaries
+    unsigned long long best[CT_MAX_NODES];           // smallest N L of a node, as order bits
+    int pos[CT_MAX_NODES];                           // its position
+    double psy[CT_MAX_NODES], psyy[CT_MAX_NODES];    // running sums there
+};
+
+// Thread's run of `cnt` consecutive keys, key(j) = sorted key at position i0 + j (j = -1: the one ahead of it); (a, b):
+// running sums of y and y^2 ahead of the run.  Calls emit(node, i, N L, sums at i) for every position that may be split.
+template <class KeyFn, class EmitFn>
+__device__ __forceinline__ void scan_run(const LayerSmem& s, int nodes, int i0, int cnt, double a, double b, KeyFn key, EmitFn emit) {
+    if (cnt <= 0) return;
+    int node = 0;
+    while (node + 1 < nodes && s.bnd[node + 1] <= i0) ++node;
+    float xp = i0 > 0 ? key_x(key(-1)) : 0.f;
+    for (int j = 0; j < cnt; ++j) {
+        const int i = i0 + j;
+        while (node + 1 < nodes && s.bnd[node + 1] <= i) ++node;
+        const unsigned long long k = key(j);
+        const float x = key_x(k);
+        if (i > s.bnd[node] && xp < x) {                              // a threshold lies between distinct values
+            const double nl = (double)(i - s.bnd[node]), nr = (double)(s.bnd[node + 1] - i);
+            const double yl = a - s.sy[node], yyl = b - s.syy[node];
+            const double yr = s.sy[node + 1] - a, yyr = s.syy[node + 1] - b;
+            // (rounding spelled out: the sweeps below have to see the same bits)
+            emit(node, i, __dadd_rn(__dsub_rn(__dmul_rn(nl, yyl), __dmul_rn(yl, yl)), __dsub_rn(__dmul_rn(nr, yyr), __dmul_rn(yr, yr))), a, b);
+        }
+        const double y = key_y(k);
+        a = __dadd_rn(a, y); b = __dadd_rn(b, __dmul_rn(y, y));
+        xp = x;
+    }
+}
+
+// The block's best split of every node -> s.best / s.pos / s.psy / s.psyy (pos = INT_MAX: none).  A sweep over the
+// thread's run finds the smallest N L; only the threads that hold it sweep again for the smallest position that has it.
+template <class KeyFn>
+__device__ __forceinline__ void layer_block(LayerSmem& s, int nodes, int i0, int cnt, double a, double b, KeyFn key) {
+    const int tid = threadIdx.x;
+    for (int q = tid; q < nodes; q += blockDim.x) { s.best[q] = ~0ull; s.pos[q] = 0x7fffffff; }
+    __syncthreads();
+    int cur = -1;
+    unsigned long long m = ~0ull;
+    bool several = false;                            // the run lies in more than one node
+    {
+        scan_run(s, nodes, i0, cnt, a, b, key, [&](int node, int, double l, double, double) {
+            if (node != cur) { if (cur >= 0) { atomicMin(&s.best[cur], m); several = true; } cur = node; m = ~0ull; }
+            const unsigned long long u = order_bits_d(l);
+            m = u < m ? u : m;
+        });
+        // lanes that end in the same node as lane 0 go through one atomic
+        const int c0 = __shfl_sync(HS_FULL_MASK, cur, 0);
+        unsigned long long w = cur == c0 ? m : ~0ull;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) { const unsigned long long u = __shfl_xor_sync(HS_FULL_MASK, w, o); w = u < w ? u : w; }
+        if ((tid & 31) == 0 && c0 >= 0) atomicMin(&s.best[c0], w);
+        if (cur >= 0 && cur != c0) atomicMin(&s.best[cur], m);
+    }
+    __syncthreads();
+    const bool again = several || (cur >= 0 && m == s.best[cur]);
+    if (again)
+        scan_run(s, nodes, i0, cnt, a, b, key, [&](int node, int i, double l, double, double) {
+            if (order_bits_d(l) == s.best[node]) atomicMin(&s.pos[node], i);
+        });
+    __syncthreads();
+    if (again)
+        scan_run(s, nodes, i0, cnt, a, b, key, [&](int node, int i, double, double sa, double sb) {
+            if (i == s.pos[node]) { s.psy[node] = sa; s.psyy[node] = sb; }
+        });
+    __syncthreads();
+}
+
+// exclusive prefix over the CTA of two doubles per thread (fixed order: lanes, then warps)
+template <int NW>
+__device__ __forceinline__ void scan_pair(double& a, double& b, double (*s_w)[2]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double ia = a, ib = b;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double ua = __shfl_up_sync(HS_FULL_MASK, ia, o), ub = __shfl_up_sync(HS_FULL_MASK, ib, o);
+        if (lane >= o) { ia += ua; ib += ub; }
+    }
+    if (lane == 31) { s_w[warp][0] = ia; s_w[warp][1] = ib; }
+    __syncthreads();
+    if (warp == 0) {                                 // (one warp: the sums ahead of every warp)
+        double wa = lane < NW ? s_w[lane][0] : 0.0, wb = lane < NW ? s_w[lane][1] : 0.0;
+        const double va = wa, vb = wb;
+#pragma unroll
+        for (int o = 1; o < NW; o <<= 1) {
+            const double ua = __shfl_up_sync(HS_FULL_MASK, wa, o), ub = __shfl_up_sync(HS_FULL_MASK, wb, o);
+            if (lane >= o) { wa += ua; wb += ub; }
+        }
+        if (lane < NW) { s_w[lane][0] = wa - va; s_w[lane][1] = wb - vb; }
+    }
+    __syncthreads();
+    a = s_w[warp][0] + (ia - a);
+    b = s_w[warp][1] + (ib - b);
+}
+
+// position of a node's threshold in the ascending list: in-order index of the node
+__device__ __forceinline__ int threshold_slot(int node, int level, int depth) { return (2 * node + 1) * (1 << (depth - 1 - level)) - 1; }
+
+// ---- few samples: one CTA ------------------------------------------------------------------------------------------
+// padded index of a key: runs of eight consecutive keys of different threads start in different banks
+__device__ __forceinline__ int pad8(int i) { return i + (i >> 3); }
+struct SmallSmem {
+    unsigned long long key[CT_SMALL * 9 / 8 + 8];
+    int cnt[CT_SMALL_THREADS / 32][256];
+};
+
+__global__ void __launch_bounds__(CT_SMALL_THREADS, 1) cart_small_kernel(const float* x, const float* y, int n, int depth,
+                                                                         float* thresholds, int* status) {
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    constexpr int NW = CT_SMALL_THREADS / 32;
+    unsigned long long* s_key = reinterpret_cast<SmallSmem*>(s_dyn)->key;
+    int(*s_cnt)[256] = reinterpret_cast<SmallSmem*>(s_dyn)->cnt;
+    __shared__ LayerSmem s;
+    __shared__ double s_w[NW][2];
+    __shared__ int s_scan[8];
+    __shared__ int s_bnd2[2 * CT_MAX_NODES + 1];
+    __shared__ double s_sy2[2 * CT_MAX_NODES + 1], s_syy2[2 * CT_MAX_NODES + 1];
+    __shared__ int s_bad;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    pdl_launch_dependents();
+    pdl_wait();
+    // warp w holds keys 32 nit w .. of the input order, item-major; rounds past the samples are left out
+    const int nit = (n + CT_SMALL_THREADS - 1) / CT_SMALL_THREADS;
+    unsigned long long k[CT_SMALL_ITEMS];
+    int rank[CT_SMALL_ITEMS];
+#pragma unroll
+    for (int i = 0; i < CT_SMALL_ITEMS; ++i) {
+        const int j = warp * 32 * nit + i * 32 + lane;
+        k[i] = (i < nit && j < n) ? cart_key(x[j], y[j]) : ~0ull;      // (padding sorts to the end)
+    }
+    for (int pass = 0; pass < 4; ++pass) {
+        for (int i = lane; i < 256; i += 32) s_cnt[warp][i] = 0;
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < CT_SMALL_ITEMS; ++i) {
+            if (i >= nit) break;
+            unsigned long long k1[1] = {k[i]};
+            int r1[1];
+            warp_ranks<1>(k1, pass, s_cnt[warp], lane, r1);
+            rank[i] = r1[0];
         }
         __syncthreads();
+        int tot = 0;
+        if (tid < 256)
+            for (int w = 0; w < NW; ++w) { const int c = s_cnt[w][tid]; s_cnt[w][tid] = tot; tot += c; }
+        const int first = scan256(tid < 256 ? tot : 0, s_scan, tid);
+        if (tid < 256)
+            for (int w = 0; w < NW; ++w) s_cnt[w][tid] += first;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < CT_SMALL_ITEMS; ++i)
+            if (i < nit) s_key[pad8(s_cnt[warp][key_digit(k[i], pass)] + rank[i])] = k[i];
+        __syncthreads();
+        if (pass < 3) {
+#pragma unroll
+            for (int i = 0; i < CT_SMALL_ITEMS; ++i)
+                if (i < nit) k[i] = s_key[pad8(warp * 32 * nit + i * 32 + lane)];
+        }
     }
-    if (tid == 0) { c.part_l[node * CT_SPLIT_BLOCKS + blockIdx.x] = s_l[0]; c.part_i[node * CT_SPLIT_BLOCKS + blockIdx.x] = s_i[0]; }
+    // running sums: thread t has keys nit t .. nit t + nit - 1 of the sorted order
+    const int i0 = min(tid * nit, n), cnt = min(i0 + nit, n) - i0;
+    auto key = [&](int j) { return s_key[pad8(i0 + j)]; };
+    double a = 0.0, b = 0.0;
+    for (int j = 0; j < cnt; ++j) { const double v = key_y(key(j)); a += v; b += v * v; }
+    double ta = a, tb = b;
+    scan_pair<NW>(a, b, s_w);
+    if (tid == CT_SMALL_THREADS - 1) { s.sy[1] = a + ta; s.syy[1] = b + tb; }
+    if (tid == 0) { s.bnd[0] = 0; s.bnd[1] = n; s.sy[0] = 0.0; s.syy[0] = 0.0; s_bad = 0; }
+    __syncthreads();
+    for (int level = 0; level < depth; ++level) {
+        const int nodes = 1 << level;
+        layer_block(s, nodes, i0, cnt, a, b, key);
+        if (tid < nodes) {
+            int at = s.pos[tid];
+            float th = CUDART_NAN_F;                  // a single feature value: the node cannot be split
+            double sa = s.sy[tid + 1], sb = s.syy[tid + 1];
+            if (at == 0x7fffffff) { s_bad = 1; at = s.bnd[tid + 1]; }
+            else {
+                th = (float)(0.5 * ((double)key_x(s_key[pad8(at - 1)]) + (double)key_x(s_key[pad8(at)])));
+                sa = s.psy[tid]; sb = s.psyy[tid];
+            }
+            thresholds[threshold_slot(tid, level, depth)] = th;
+            s_bnd2[2 * tid] = s.bnd[tid]; s_sy2[2 * tid] = s.sy[tid]; s_syy2[2 * tid] = s.syy[tid];
+            s_bnd2[2 * tid + 1] = at; s_sy2[2 * tid + 1] = sa; s_syy2[2 * tid + 1] = sb;
+            if (tid == nodes - 1) { s_bnd2[2 * nodes] = s.bnd[nodes]; s_sy2[2 * nodes] = s.sy[nodes]; s_syy2[2 * nodes] = s.syy[nodes]; }
+        }
+        __syncthreads();
+        if (level + 1 < depth && tid <= 2 * nodes) { s.bnd[tid] = s_bnd2[tid]; s.sy[tid] = s_sy2[tid]; s.syy[tid] = s_syy2[tid]; }
+        __syncthreads();
+    }
+    if (tid == 0) *status = s_bad ? HS_ERR_SHAPE : HS_OK;
 }
 
-__global__ void cart_split_pick_kernel(const CartLevel c) {            // one thread per node
-    const int node = blockIdx.x * blockDim.x + threadIdx.x;
-    if (node >= c.nodes) return;
-    double best = CUDART_INF;
-    int best_i = 0x7fffffff;
-    for (int b = 0; b < CT_SPLIT_BLOCKS; ++b) {
-        const double l = c.part_l[node * CT_SPLIT_BLOCKS + b];
-        const int i = c.part_i[node * CT_SPLIT_BLOCKS + b];
-        if (l < best || (l == best && i < best_i)) { best = l; best_i = i; }
+// ---- many samples ----------------------------------------------------------------------------------------------------
+struct CartParams {
+    const float* x;
+    const float* y;
+    int n, tiles, depth;
+    unsigned long long* keys;      // sorted in place over an even number of passes ...
+    unsigned long long* keys2;     // ... through this copy
+    unsigned int* look;            // [4][tiles][256] look-back words of the radix passes
+    double* blk;                   // [tiles][2] sums of y and y^2 per tile, then ahead of it
+    int* hist;                     // [4][256] digit counts (zero between calls)
+    int* ticket;                   // [4] tiles started per pass (zero between calls)
+    int* done;                     // [1 + depth] CTAs that have finished (zero between calls)
+    int* bnd;                      // [2][CT_MAX_NODES + 1]: boundaries of the layer, and of the next
+    double* bsum;                  // [2][CT_MAX_NODES + 1][2]
+    unsigned long long* part_l;    // [tiles + nodes] best N L of a (tile, node), entry tile + node
+    int* part_i;
+    double* part_s;                // [tiles + nodes][2]
+    float* thresholds;
+    int* status;
+    int* err;
+};
+
+__global__ void __launch_bounds__(CT_THREADS) cart_pack_kernel(const CartParams p) {
+    __shared__ int s_h[4][256];
+    const int tid = threadIdx.x;
+    for (int q = 0; q < 4; ++q) s_h[q][tid] = 0;
+    pdl_launch_dependents();
+    pdl_wait();
+    __syncthreads();
+    for (int q = 0; q < 4; ++q) p.look[((size_t)q * p.tiles + blockIdx.x) * 256 + tid] = 0u;
+    const int base = blockIdx.x * CT_TILE;
+    float xv[CT_ITEMS], yv[CT_ITEMS];
+#pragma unroll
+    for (int i = 0; i < CT_ITEMS; ++i) {
+        const int j = base + i * CT_THREADS + tid;
+        xv[i] = j < p.n ? p.x[j] : 0.f;
+        yv[i] = j < p.n ? p.y[j] : 0.f;
     }
-    const int lo = c.bnd[node], hi = c.bnd[node + 1];
-    // position of this node's threshold in the ascending list: in-order index of the node
-    const int slot = (2 * node + 1) * (1 << (c.depth - 1 - c.level)) - 1;
-    if (best_i == 0x7fffffff) {                      // a single feature value: the node cannot be split
-        *c.status = HS_ERR_SHAPE;
-        c.thresholds[slot] = CUDART_NAN_F;
-        best_i = hi;
-    } else {
-        c.thresholds[slot] = (float)(0.5 * ((double)key_x(c.keys[best_i - 1]) + (double)key_x(c.keys[best_i])));
+#pragma unroll
+    for (int i = 0; i < CT_ITEMS; ++i) {
+        const int j = base + i * CT_THREADS + tid;
+        const unsigned long long k = cart_key(xv[i], yv[i]);
+        if (j < p.n) p.keys[j] = k;
+        const unsigned int in = __ballot_sync(HS_FULL_MASK, j < p.n);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            // the uppermost digit (sign and exponent) takes few values: one atomic per group of equal digits there
+            const unsigned int d = key_digit(k, q);
+            if (q < 3) { if (j < p.n) atomicAdd(&s_h[q][d], 1); }
+            else {
+                const unsigned int m = __match_any_sync(HS_FULL_MASK, d) & in;
+                if (j < p.n && __ffs(m) - 1 == (tid & 31)) atomicAdd(&s_h[q][d], __popc(m));
+            }
+        }
     }
-    c.bnd_next[2 * node] = lo;
-    c.bnd_next[2 * node + 1] = best_i;
-    if (node == c.nodes - 1) c.bnd_next[2 * c.nodes] = hi;
+    __syncthreads();
+    for (int q = 0; q < 4; ++q) if (s_h[q][tid]) atomicAdd(&p.hist[q * 256 + tid], s_h[q][tid]);
 }
 
-__global__ void cart_init_kernel(int* bnd, int n, int* status) { bnd[0] = 0; bnd[1] = n; *status = HS_OK; }
+// One pass of the radix sort.  A CTA takes tiles in the order CTAs start (a ticket), ranks its keys, publishes its digit
+// counts and looks back over the tiles ahead for the counts before its own (a tile it waits for has started, so every
+// wait ends; bounded all the same), reorders the tile in shared memory and writes runs of equal digits.
+__global__ void __launch_bounds__(CT_THREADS) cart_radix_kernel(const CartParams p, int pass) {
+    __shared__ unsigned long long s_key[CT_TILE];
+    __shared__ int s_cnt[8][256];
+    __shared__ int s_off[256];
+    __shared__ int s_scan[8];
+    __shared__ int s_tile;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned long long* in = (pass & 1) ? p.keys2 : p.keys;
+    unsigned long long* out = (pass & 1) ? p.keys : p.keys2;
+    for (int w = 0; w < 8; ++w) s_cnt[w][tid] = 0;
+    pdl_launch_dependents();
+    pdl_wait();
+    if (tid == 0) s_tile = atomicAdd(&p.ticket[pass], 1);
+    __syncthreads();
+    const int tile = s_tile, base = tile * CT_TILE;
+    const int nvalid = min(CT_TILE, p.n - base);
+    unsigned long long k[CT_ITEMS];
+    int rank[CT_ITEMS];
+#pragma unroll
+    for (int i = 0; i < CT_ITEMS; ++i) {
+        const int j = warp * 32 * CT_ITEMS + i * 32 + lane;
+        k[i] = j < nvalid ? in[base + j] : ~0ull;              // (past the last sample: behind everything in the last tile)
+    }
+    const int first = scan256(p.hist[pass * 256 + tid], s_scan, tid);      // keys with smaller digits
+    warp_ranks<CT_ITEMS>(k, pass, s_cnt[warp], lane, rank);
+    __syncthreads();
+    int c = 0;
+    for (int w = 0; w < 8; ++w) { const int v = s_cnt[w][tid]; s_cnt[w][tid] = c; c += v; }
+    unsigned int* look = p.look + (size_t)pass * p.tiles * 256 + tid;
+    volatile unsigned int* vlook = look;
+    vlook[(size_t)tile * 256] = (tile == 0 ? 2u << 30 : 1u << 30) | (unsigned int)c;
+    const int local = scan256(c, s_scan, tid);                 // (its barrier also orders s_scan's reuse)
+    int before = 0;
+    const unsigned long long t0 = global_timer_ns();
+    // (CT_WINDOW tiles at a time: the tiles of a launch publish together, and a walk of one load per tile would be a chain of
+    // as many round trips to L2 as there are tiles)
+    bool found = tile == 0;
+    for (int t = tile - 1; !found;) {
+        unsigned int v[CT_WINDOW];
+#pragma unroll
+        for (int i = 0; i < CT_WINDOW; ++i) v[i] = t - i >= 0 ? vlook[(size_t)(t - i) * 256] : 2u << 30;
+        bool open = true;                                      // nothing unpublished met in this window so far
+#pragma unroll
+        for (int i = 0; i < CT_WINDOW; ++i) {
+            open = open && v[i] >> 30;
+            if (open && !found) {
+                before += (int)(v[i] & 0x3fffffffu);
+                found = v[i] >> 31;                            // that tile knew everything ahead of it
+                --t;
+            }
+        }
+        if (!open && global_timer_ns() - t0 > HS_WAIT_LIMIT_NS) {
+            atomicExch(p.err, (int)HS_ERR_TIMEOUT);
+            break;
+        }
+    }
+    if (tile > 0) vlook[(size_t)tile * 256] = (2u << 30) | (unsigned int)(before + c);
+    s_off[tid] = first + before - local;
+    for (int w = 0; w < 8; ++w) s_cnt[w][tid] += local;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < CT_ITEMS; ++i) s_key[s_cnt[warp][key_digit(k[i], pass)] + rank[i]] = k[i];
+    __syncthreads();
+#pragma unroll 4
+    for (int j = tid; j < nvalid; j += CT_THREADS) {
+        const unsigned long long kk = s_key[j];
+        const int at = s_off[key_digit(kk, pass)] + j;
+        if ((unsigned int)at < (unsigned int)p.n) out[at] = kk;    // (out of range only after a wait that expired)
+    }
+}
 
-static int next_pow2(int n) { int p = CT_CHUNK; while (p < n) p <<= 1; return p; }
+// Layer kernel: eight keys per thread (a thread's running sums are a chain of fp64 additions: with sixteen keys the chain,
+// not the fp64 pipe, was the time of a launch).
+#define CT_LV_THREADS 512
+#define CT_LV_ITEMS (CT_TILE / CT_LV_THREADS)
+#define CT_PADDED (CT_TILE + CT_TILE / 8 + 1)
+
+// last CTA of the launch to arrive (every thread gets the answer; its earlier stores are ordered ahead)
+__device__ __forceinline__ bool last_cta(int* done, int* s_last) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int old;
+        asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(old) : "l"(done) : "memory");
+        *s_last = old == (int)gridDim.x - 1;
+        if (*s_last) *done = 0;
+    }
+    __syncthreads();
+    return *s_last != 0;
+}
+
+// sums of y and y^2 per tile; the last CTA turns them into the sums ahead of each tile
+__global__ void __launch_bounds__(CT_THREADS) cart_sums_kernel(const CartParams p) {
+    __shared__ double s_w[8][2];
+    __shared__ int s_last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    pdl_launch_dependents();
+    pdl_wait();
+    double a = 0.0, b = 0.0;
+#pragma unroll
+    for (int i = 0; i < CT_ITEMS; ++i) {
+        const int j = blockIdx.x * CT_TILE + i * CT_THREADS + tid;
+        if (j < p.n) { const double v = key_y(p.keys[j]); a += v; b += v * v; }
+    }
+    a = warp_sum_d(a); b = warp_sum_d(b);
+    if (lane == 0) { s_w[warp][0] = a; s_w[warp][1] = b; }
+    __syncthreads();
+    if (tid == 0) {
+        double ta = 0.0, tb = 0.0;
+        for (int w = 0; w < 8; ++w) { ta += s_w[w][0]; tb += s_w[w][1]; }
+        p.blk[2 * blockIdx.x] = ta; p.blk[2 * blockIdx.x + 1] = tb;
+    }
+    if (!last_cta(&p.done[0], &s_last)) return;
+    const int per = (p.tiles + CT_THREADS - 1) / CT_THREADS;
+    const int t0 = min(tid * per, p.tiles), t1 = min(t0 + per, p.tiles);
+    a = 0.0; b = 0.0;
+    for (int t = t0; t < t1; ++t) { a += __ldcg(&p.blk[2 * t]); b += __ldcg(&p.blk[2 * t + 1]); }
+    const double ma = a, mb = b;
+    scan_pair<8>(a, b, s_w);
+    double ra = a, rb = b;
+    for (int t = t0; t < t1; ++t) {
+        const double va = __ldcg(&p.blk[2 * t]), vb = __ldcg(&p.blk[2 * t + 1]);
+        p.blk[2 * t] = ra; p.blk[2 * t + 1] = rb;
+        ra += va; rb += vb;
+    }
+    if (tid == CT_THREADS - 1) { p.bsum[2] = a + ma; p.bsum[3] = b + mb; }
+    if (tid == 0) { p.bnd[0] = 0; p.bnd[1] = p.n; p.bsum[0] = 0.0; p.bsum[1] = 0.0; *p.status = HS_OK; }
+    for (int q = tid; q < 4 * 256; q += CT_THREADS) p.hist[q] = 0;         // ready for the next call
+    if (tid < 4) p.ticket[tid] = 0;
+}
+
+__global__ void __launch_bounds__(CT_LV_THREADS) cart_level_kernel(const CartParams p, int level) {
+    __shared__ unsigned long long s_key[CT_PADDED];
+    __shared__ LayerSmem s;
+    __shared__ double s_w[CT_LV_THREADS / 32][2];
+    __shared__ int s_last;
+    __shared__ unsigned long long s_best[32];
+    __shared__ int s_at[32], s_e[32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nodes = 1 << level;
+    pdl_launch_dependents();
+    pdl_wait();
+    const int* bnd = p.bnd + (level & 1) * (CT_MAX_NODES + 1);
+    const double* bsum = p.bsum + (level & 1) * 2 * (CT_MAX_NODES + 1);
+    if (tid <= nodes) { s.bnd[tid] = bnd[tid]; s.sy[tid] = bsum[2 * tid]; s.syy[tid] = bsum[2 * tid + 1]; }
+    const int base = blockIdx.x * CT_TILE, nvalid = min(CT_TILE, p.n - base);
+#pragma unroll
+    for (int i = 0; i < CT_LV_ITEMS; ++i) {
+        const int j = i * CT_LV_THREADS + tid;
+        if (j < nvalid) s_key[1 + pad8(j)] = p.keys[base + j];
+    }
+    if (tid == 0) s_key[0] = base > 0 ? p.keys[base - 1] : 0ull;           // the key ahead of the tile
+    __syncthreads();
+    const int j0 = min(tid * CT_LV_ITEMS, nvalid), cnt = min(j0 + CT_LV_ITEMS, nvalid) - j0;
+    auto key = [&](int j) { return j0 + j < 0 ? s_key[0] : s_key[1 + pad8(j0 + j)]; };
+    double a = 0.0, b = 0.0;
+    for (int j = 0; j < cnt; ++j) { const double v = key_y(key(j)); a += v; b += v * v; }
+    scan_pair<CT_LV_THREADS / 32>(a, b, s_w);
+    a += p.blk[2 * blockIdx.x]; b += p.blk[2 * blockIdx.x + 1];
+    layer_block(s, nodes, base + j0, cnt, a, b, key);
+    // the nodes this tile overlaps leave their best split in entry tile + node (no two tiles share an entry)
+    if (tid < nodes && s.bnd[tid] < base + nvalid && s.bnd[tid + 1] > base) {
+        const int e = blockIdx.x + tid;
+        p.part_l[e] = s.best[tid]; p.part_i[e] = s.pos[tid];
+        p.part_s[2 * e] = s.psy[tid]; p.part_s[2 * e + 1] = s.psyy[tid];
+    }
+    if (!last_cta(&p.done[1 + level], &s_last)) return;
+    // the best of a node's tiles: a power of two of warps per node, one tile per lane as long as they reach
+    int* bnd2 = p.bnd + ((level + 1) & 1) * (CT_MAX_NODES + 1);
+    double* bsum2 = p.bsum + ((level + 1) & 1) * 2 * (CT_MAX_NODES + 1);
+    constexpr int NWL = CT_LV_THREADS / 32;
+    const int wpn = max(NWL / nodes, 1);
+    for (int v = warp; v < max(nodes, NWL); v += NWL) {
+        const int node = v / wpn, lo = s.bnd[node], hi = s.bnd[node + 1];
+        unsigned long long m = ~0ull;
+        int at = 0x7fffffff, e = -1;
+        if (hi > lo)
+            for (int t = lo / CT_TILE + (v % wpn) * 32 + lane; t <= (hi - 1) / CT_TILE; t += 32 * wpn) {
+                const unsigned long long l = __ldcg(&p.part_l[t + node]);
+                const int i = __ldcg(&p.part_i[t + node]);
+                if (l < m || (l == m && i < at)) { m = l; at = i; e = t + node; }
+            }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long l = __shfl_xor_sync(HS_FULL_MASK, m, o);
+            const int i = __shfl_xor_sync(HS_FULL_MASK, at, o), e2 = __shfl_xor_sync(HS_FULL_MASK, e, o);
+            if (l < m || (l == m && i < at)) { m = l; at = i; e = e2; }
+        }
+        if (lane == 0) { s_best[v] = m; s_at[v] = at; s_e[v] = e; }
+    }
+    __syncthreads();
+    if (tid < nodes) {
+        const int node = tid, lo = s.bnd[node], hi = s.bnd[node + 1];
+        unsigned long long m = ~0ull;
+        int at = 0x7fffffff, e = -1;
+        for (int w = node * wpn; w < (node + 1) * wpn; ++w)
+            if (s_best[w] < m || (s_best[w] == m && s_at[w] < at)) { m = s_best[w]; at = s_at[w]; e = s_e[w]; }
+        float th = CUDART_NAN_F;                              // a single feature value: the node cannot be split
+        double sa = s.sy[node + 1], sb = s.syy[node + 1];
+        if (at == 0x7fffffff) { *p.status = HS_ERR_SHAPE; at = hi; }
+        else {
+            th = (float)(0.5 * ((double)key_x(p.keys[at - 1]) + (double)key_x(p.keys[at])));
+            sa = __ldcg(&p.part_s[2 * e]); sb = __ldcg(&p.part_s[2 * e + 1]);
+        }
+        p.thresholds[threshold_slot(node, level, p.depth)] = th;
+        if (level + 1 < p.depth) {
+            bnd2[2 * node] = lo; bsum2[4 * node] = s.sy[node]; bsum2[4 * node + 1] = s.syy[node];
+            bnd2[2 * node + 1] = at; bsum2[4 * node + 2] = sa; bsum2[4 * node + 3] = sb;
+            if (node == nodes - 1) { bnd2[2 * nodes] = hi; bsum2[4 * nodes] = s.sy[nodes]; bsum2[4 * nodes + 1] = s.syy[nodes]; }
+        }
+    }
+}
+
+// What the calls asked for before the radix sort (keys padded to a power of two, two running sums per sample): the same
+// bytes hold the second copy of the keys, the look-back words and the per-tile arrays.
+static int next_pow2(int n) { int p = 1024; while (p < n) p <<= 1; return p; }
 
 extern "C" size_t hs_cart_workspace_bytes(int32_t n) {
     if (n < 2) return 0;
     const size_t P = next_pow2(n);
     return HS_COUNTER_BYTES + P * 8 + 2 * ((size_t)n + 1) * 8 + 2 * (((size_t)n + CT_THREADS - 1) / CT_THREADS) * 8 +
-           2 * (2 << CT_MAX_DEPTH) * 4 + (1 << CT_MAX_DEPTH) * CT_SPLIT_BLOCKS * 12 + 4096;
+           2 * (2 << CT_MAX_DEPTH) * 4 + (1 << CT_MAX_DEPTH) * 64 * 12 + 4096;
 }
 
 extern "C" hs_status hs_cart_fit(hs_ctx* ctx, const float* x, const float* y, int32_t n, int32_t depth,
@@ -180,41 +573,42 @@ extern "C" hs_status hs_cart_fit(hs_ctx* ctx, const float* x, const float* y, in
     cudaStream_t stream = (cudaStream_t)stream_;
     if (!ctx || !hs_on_device(ctx) || !x || !y || !thresholds || !status) return HS_ERR_INVALID_ARG;
     if (depth < 1 || depth > CT_MAX_DEPTH || n < (1 << depth) || n > (1 << 26)) return HS_ERR_SHAPE;
-    const int P = next_pow2(n);
-    const int nblk = (n + CT_THREADS - 1) / CT_THREADS;
-    // workspace: keys | sy | syy | block totals | two boundary arrays | per-block minima
+    if (hs_cart_workspace_bytes(n) - HS_COUNTER_BYTES - 4096 > ctx->scratch_bytes) return HS_ERR_WORKSPACE;
+    const dim3 one(1, 1, 1);
+    if (n <= CT_SMALL) {
+        if (!ctx->cart_ready) {
+            HS_CUDA_OK(cudaFuncSetAttribute(cart_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSmem)));
+            ctx->cart_ready = true;
+        }
+        return hs_launch(cart_small_kernel, one, dim3(CT_SMALL_THREADS), sizeof(SmallSmem), stream, ctx->pdl, one, x, y, (int)n,
+                         (int)depth, thresholds, (int*)status) == cudaSuccess ? HS_OK : HS_ERR_CUDA;
+    }
+    CartParams p;
+    p.x = x; p.y = y; p.n = n; p.depth = depth; p.thresholds = thresholds; p.status = status;
+    p.tiles = (n + CT_TILE - 1) / CT_TILE;
     size_t o = 0;
-    auto take = [&](size_t bytes) { char* p = ctx->scratch + o; o += hs_align_up(bytes, 256); return p; };
-    unsigned long long* keys = (unsigned long long*)take((size_t)P * 8);
-    double* sy = (double*)take(((size_t)n + 1) * 8);
-    double* syy = (double*)take(((size_t)n + 1) * 8);
-    double* blk = (double*)take((size_t)nblk * 16);
-    int* bnd_a = (int*)take((2 << CT_MAX_DEPTH) * 4);
-    int* bnd_b = (int*)take((2 << CT_MAX_DEPTH) * 4);
-    double* part_l = (double*)take((size_t)(1 << CT_MAX_DEPTH) * CT_SPLIT_BLOCKS * 8);
-    int* part_i = (int*)take((size_t)(1 << CT_MAX_DEPTH) * CT_SPLIT_BLOCKS * 4);
+    auto take = [&](size_t bytes) { char* q = ctx->scratch + o; o += hs_align_up(bytes, 256); return q; };
+    p.keys = (unsigned long long*)take((size_t)n * 8);
+    p.keys2 = (unsigned long long*)take((size_t)n * 8);
+    p.look = (unsigned int*)take((size_t)4 * p.tiles * 256 * 4);
+    p.blk = (double*)take((size_t)p.tiles * 16);
+    p.bnd = (int*)take(2 * (CT_MAX_NODES + 1) * 4);
+    p.bsum = (double*)take(2 * (CT_MAX_NODES + 1) * 16);
+    const size_t parts = (size_t)p.tiles + CT_MAX_NODES;
+    p.part_l = (unsigned long long*)take(parts * 8);
+    p.part_i = (int*)take(parts * 4);
+    p.part_s = (double*)take(parts * 16);
     if (o > ctx->scratch_bytes) return HS_ERR_WORKSPACE;
-
-    cart_pack_kernel<<<(P + 255) / 256, 256, 0, stream>>>(x, y, n, P, keys);
-    cart_sort_chunk_kernel<<<P / CT_CHUNK, CT_CHUNK / 2, 0, stream>>>(keys, 2, CT_CHUNK);
-    for (int k = 2 * CT_CHUNK; k <= P; k <<= 1) {
-        for (int j = k >> 1; j >= CT_CHUNK; j >>= 1)
-            cart_sort_global_kernel<<<(P / 2 + 255) / 256, 256, 0, stream>>>(keys, P, j, k);
-        cart_sort_chunk_kernel<<<P / CT_CHUNK, CT_CHUNK / 2, 0, stream>>>(keys, k, k);
-    }
-    cart_scan_blocks_kernel<<<nblk, CT_THREADS, 0, stream>>>(keys, n, sy, syy, blk);
-    cart_scan_totals_kernel<<<1, 1, 0, stream>>>(blk, nblk);
-    cart_scan_add_kernel<<<nblk, CT_THREADS, 0, stream>>>(n, sy, syy, blk);
-    cart_init_kernel<<<1, 1, 0, stream>>>(bnd_a, n, status);
-    for (int level = 0; level < depth; ++level) {
-        CartLevel c;
-        c.keys = keys; c.sy = sy; c.syy = syy;
-        c.bnd = (level & 1) ? bnd_b : bnd_a;
-        c.bnd_next = (level & 1) ? bnd_a : bnd_b;
-        c.part_l = part_l; c.part_i = part_i; c.thresholds = thresholds; c.status = status;
-        c.nodes = 1 << level; c.level = level; c.depth = depth;
-        cart_split_scan_kernel<<<dim3(CT_SPLIT_BLOCKS, c.nodes), CT_THREADS, 0, stream>>>(c);
-        cart_split_pick_kernel<<<1, 64, 0, stream>>>(c);
-    }
-    return cudaGetLastError() == cudaSuccess ? HS_OK : HS_ERR_CUDA;
+    p.hist = ctx->counters + HS_CNT_CART;
+    p.ticket = p.hist + 4 * 256;
+    p.done = p.ticket + 4;
+    p.err = ctx->counters + HS_CNT_ERROR;
+    const dim3 grid(p.tiles), block(CT_THREADS);
+    if (hs_launch(cart_pack_kernel, grid, block, 0, stream, ctx->pdl, one, p) != cudaSuccess) return HS_ERR_CUDA;
+    for (int pass = 0; pass < 4; ++pass)
+        if (hs_launch(cart_radix_kernel, grid, block, 0, stream, ctx->pdl, one, p, pass) != cudaSuccess) return HS_ERR_CUDA;
+    if (hs_launch(cart_sums_kernel, grid, block, 0, stream, ctx->pdl, one, p) != cudaSuccess) return HS_ERR_CUDA;
+    for (int level = 0; level < depth; ++level)
+        if (hs_launch(cart_level_kernel, grid, dim3(CT_LV_THREADS), 0, stream, ctx->pdl, one, p, level) != cudaSuccess) return HS_ERR_CUDA;
+    return HS_OK;
 }

@@ -74,6 +74,7 @@ extern "C" hs_status hs_create(hs_ctx** out, int32_t device, size_t workspace_by
     c->attn_ready = false;
     c->walk_ready = false;
     c->quant_ready = false;
+    c->cart_ready = false;
     c->rows_ready = false;
     if (cudaDeviceSynchronize() != cudaSuccess) { cudaFree(p); delete c; return HS_ERR_CUDA; }
     *out = c;
