@@ -33,6 +33,18 @@ namespace cg = cooperative_groups;
 #define WALK_CLUSTER 16       // (larger than the portable 8: the launcher asks for it)
 #define WALK_THREADS 512
 
+// A bonus draw of a deterministic-proposal sequence that the CTAs of the launch share (in the workspace, one per sequence).
+#define DET_SLICES 64
+#define DET_MAX_BATCH 256     // sequences the sharing keeps counters for
+struct DetJob {
+    double sum[DET_SLICES];   // mass of each slice of the vocabulary
+    int last[DET_SLICES];     // its last token of positive mass, -1
+    const char* row;          // the target row of the node the walk ended on
+    float pm, ips, invT;      // its maximum, 1 / sum, log2(e) / temperature
+    int nrej;
+    int rej[HS_MAX_NODES];    // tokens rejected there
+};
+
 struct RowOut {           // per kept node, in the workspace
     int* tgt_arg;         // arg-max token of the target row
     float2* tgt_ms;       // {max, sum e^((x-max)/T)} of the target row
@@ -57,6 +69,8 @@ struct AcceptParams {
     uint4* partials;      // [2][max_rows][chunks] {key lo, key hi, max, sum}
     int* row_cnt;
     int* seq_cnt;         // [batch] merged target rows of a sequence (zero between launches)
+    DetJob* jobs;         // [batch], or NULL: every draw is made by the CTA that walked the tree
+    int* det_cnt;         // [4][DET_MAX_BATCH] of a job: published, slices taken, slices finished, CTAs that have left (zero between launches)
     int clustered;        // chunk kernel: the chunks of a row form a thread-block cluster and merge through shared memory
     int staged;           // the walk may stage row slices in shared memory by bulk copies (16-byte aligned rows)
     int* err;             // sticky device error word (a bounded wait that expired)
@@ -135,202 +149,7 @@ __device__ void greedy_walk(const AcceptParams& p, int b) {
 
 __device__ __forceinline__ float load_logit(const void* base, int is_bf16, size_t off);
 
-// Acceptance of sequence b with deterministic proposals by one whole CTA (Sec. 2.1 with a point-mass proposal per
-// candidate): at node cur with p = softmax(target row / T) the kept children are tried in index order; child x
-// with token t is accepted iff u_x < min(1, p_t / W), W = 1 - (mass of the tokens rejected at this node so far); a
-// rejection removes t.  When no candidate is left the bonus token is drawn by inverse CDF in token order from p
-// without the rejected tokens (running sums in double, one contiguous run of tokens per thread).
-__device__ __noinline__ void deterministic_walk(const AcceptParams& p, int b) {
-    __shared__ int s_par[HS_MAX_NODES], s_tok[HS_MAX_NODES], s_rej[HS_MAX_NODES];
-    __shared__ float s_pt[HS_MAX_NODES], s_u[HS_MAX_NODES];     // p(token of node j | its parent), its accept uniform
-    __shared__ double s_scan[HS_ROW_THREADS / 32];
-    __shared__ double s_phase[64];
-    __shared__ double s_wp[64][HS_ROW_THREADS / 32];     // per (phase, warp) sums of pass 1
-    __shared__ int s_pick[2];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = HS_ROW_THREADS;
-    const int koff = p.pr.keep_off[b];
-    const int nk = min(p.pr.n_keep[b], HS_MAX_NODES);
-    const int nbase = p.node_off[b];
-    const int cap = p.out.path_cap;
-    for (int j = tid; j < cap; j += nthr) {
-        p.out.path_nodes[b * cap + j] = -1;
-        p.out.path_compact[b * cap + j] = -1;
-        p.out.path_tokens[b * cap + j] = -1;
-    }
-    for (int j = tid; j < nk; j += nthr) {
-        s_par[j] = p.pr.new_parent[koff + j];
-        s_tok[j] = p.token[nbase + p.pr.keep_idx[koff + j]];
-    }
-    walk_sync();
-    const float invT = LOG2E / p.temperature[b];
-    const size_t esz = p.is_bf16 ? 2 : 4;
-    // every candidate's probability under its parent's target row and its uniform, all nodes at once (one round
-    // trip instead of one per sibling test); the walk below then runs from shared memory
-    for (int j = 1 + tid; j < nk; j += nthr) {
-        const int par = s_par[j];
-        const int orig = p.pr.keep_idx[koff + j];
-        float pt = 0.f;
-        if (par >= 0 && par < nk) {
-            const int prow_i = p.target_layout == HS_ROWS_ORIGINAL ? nbase + p.pr.keep_idx[koff + par] : koff + par;
-            const char* row = (const char*)p.target + (size_t)prow_i * p.row_stride * esz;
-            const float2 ms = __ldcg(&p.ro.tgt_ms[koff + par]);      // written by another CTA of this launch
-            pt = exp2f((fmaxf(load_logit(row, p.is_bf16, s_tok[j]), -1e30f) - ms.x) * invT) * (1.f / ms.y);
-        }
-        s_pt[j] = pt;
-        s_u[j] = p.uniforms ? p.uniforms[nbase + orig] : philox_uniform(p.seed, p.offset, b, orig, 0);
-    }
-    walk_sync();
-    int cur = 0, len = 0, bonus = -1;
-    for (int step = 0; step < nk; ++step) {
-        if (tid == 0 && len < cap) {
-            p.out.path_compact[b * cap + len] = cur;
-            p.out.path_nodes[b * cap + len] = p.pr.keep_idx[koff + cur];
-        }
-        const int orig_cur = p.pr.keep_idx[koff + cur];
-        const int trow = p.target_layout == HS_ROWS_ORIGINAL ? nbase + orig_cur : koff + cur;
-        const char* prow = (const char*)p.target + (size_t)trow * p.row_stride * esz;
-        const float2 pms = __ldcg(&p.ro.tgt_ms[koff + cur]);      // written by another CTA of this launch
-        const float pm = pms.x, ips = 1.f / pms.y;
-        double W = 1.0;
-        int nrej = 0, accepted = -1;
-        for (int j = cur + 1; j < nk; ++j) {                     // siblings in index order (every thread the same)
-            if (s_par[j] != cur) continue;
-            const int t = s_tok[j];
-            float pt = s_pt[j];
-            for (int k = 0; k < nrej; ++k)                       // a token rejected at this node has left the residual
-                if (s_rej[k] == t) pt = 0.f;
-            const float a = fminf(1.f, pt / (float)W);
-            if (s_u[j] < a) { accepted = j; break; }
-            const double W_next = W - (double)pt;
-            if (!(W_next > 0.0)) { nrej = 0; W = 1.0; break; }  // nothing left: fall back to p
-            walk_sync();                                     // (every thread walks the same way)
-            if (tid == 0) s_rej[nrej] = t;
-            walk_sync();
-            ++nrej;
-            W = W_next;
-        }
-        if (accepted >= 0) {
-            if (tid == 0 && len < cap) p.out.path_tokens[b * cap + len] = s_tok[accepted];
-            cur = accepted;
-            ++len;
-            continue;
-        }
-        // ---- the bonus token: inverse CDF over the vocabulary without the rejected tokens -------------------
-        // The row is taken in phases of nthr * 4 vectors; in a phase thread t owns 4 consecutive 16-byte vectors (all
-        // loads in flight together), so token order is (phase, thread, token).  Pass 1 sums
-        // every phase; then the phase that holds the crossing is summed again and scanned.
-        const float ufin = p.uniforms ? p.uniforms[p.n_nodes_total + b] : philox_uniform(p.seed, p.offset, b, 0, 1);
-        if (tid == 0) { s_pick[0] = 0x7fffffff; s_pick[1] = -1; }
-        walk_sync();                                         // s_rej, s_pick
-        const int ve = p.is_bf16 ? 8 : 4;
-        const int phase_vecs = nthr * 4;
-        // (at most 64 phases: the launcher refuses vocabularies of more than 32 chunks = 64 phases)
-        const int nph = min((p.nvec + phase_vecs - 1) / phase_vecs, 64);
-        // masses of this thread's 4 vectors of phase ph (0 past the vocabulary and for rejected tokens)
-        auto phase_mass = [&](int ph, float (&m)[4][8]) {
-            uint4 d[4];
-            const int vbase = ph * phase_vecs + tid * 4;
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                d[q] = (vbase + q < p.nvec) ? __ldg((const uint4*)prow + vbase + q) : make_uint4(0, 0, 0, 0);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                float x[8];
-                if (p.is_bf16) unpack_v<true>(d[q], x); else unpack_v<false>(d[q], x);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const int tok = (vbase + q) * ve + e;
-                    const bool in = e < ve && vbase + q < p.nvec && tok < p.vocab;
-                    m[q][e] = in ? exp2f((fmaxf(x[e], -1e30f) - pm) * invT) * ips : 0.f;
-                }
-            }
-            for (int k = 0; k < nrej; ++k) {                     // few: the siblings rejected at this node
-                const int rv = s_rej[k] / ve - vbase;
-                if (rv >= 0 && rv < 4) {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-#pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            if (q == rv && e == s_rej[k] % ve) m[q][e] = 0.f;
-                }
-            }
-        };
-        int last_pos = -1;
-#pragma unroll 2
-        for (int ph = 0; ph < nph; ++ph) {
-            float m[4][8];
-            phase_mass(ph, m);
-            double mine = 0.0;
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    mine += (double)m[q][e];
-                    if (m[q][e] > 0.f) last_pos = ((ph * phase_vecs + tid * 4 + q) * ve + e);
-                }
-            const double w = warp_sum_d(mine);
-            if (lane == 0) s_wp[ph][warp] = w;           // (no barrier per phase: the loads of the next one go out)
-        }
-        walk_sync();
-        for (int ph = tid; ph < nph; ph += nthr) {
-            double t = 0.0;
-            for (int w2 = 0; w2 < nthr / 32; ++w2) t += s_wp[ph][w2];
-            s_phase[ph] = t;
-        }
-        walk_sync();
-        double total = 0.0;
-        for (int ph = 0; ph < nph; ++ph) total += s_phase[ph];
-        const double goal = (double)ufin * total;
-        int phx = -1;                                            // first phase whose running total exceeds the goal
-        double before_ph = 0.0;
-        for (int ph = 0; ph < nph; ++ph) {
-            if (before_ph + s_phase[ph] > goal) { phx = ph; break; }
-            before_ph += s_phase[ph];
-        }
-        if (phx >= 0) {
-            float m[4][8];
-            phase_mass(phx, m);
-            double mine = 0.0;
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-                for (int e = 0; e < 8; ++e) mine += (double)m[q][e];
-            double incl = mine;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const double up = __shfl_up_sync(HS_FULL_MASK, incl, o);
-                if (lane >= o) incl += up;
-            }
-            if (lane == 31) s_scan[warp] = incl;
-            walk_sync();
-            double run = before_ph + (incl - mine);
-            for (int w2 = 0; w2 < warp; ++w2) run += s_scan[w2];
-            if (run <= goal && run + mine > goal) {              // the crossing lies in this thread's tokens
-                bool found = false;
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        run += (double)m[q][e];
-                        if (!found && run > goal) {
-                            found = true;
-                            atomicMin(&s_pick[0], (phx * phase_vecs + tid * 4 + q) * ve + e);
-                        }
-                    }
-            }
-        }
-        if (last_pos >= 0) atomicMax(&s_pick[1], last_pos);
-        walk_sync();
-        bonus = s_pick[0] != 0x7fffffff ? s_pick[0] : max(s_pick[1], 0);
-        break;
-    }
-    if (tid == 0) {
-        p.out.accept_len[b] = len;
-        p.out.bonus_token[b] = bonus;
-        p.out.terminal_rank[b] = p.pr.keep_rank[koff + cur];
-        p.out.status[b] = HS_OK;
-    }
-}
+#include "accept_det.cuh"
 
 template <bool BF16>
 __global__ void __launch_bounds__(HS_ROW_THREADS, 4) accept_rows_kernel(const __grid_constant__ AcceptParams p) {
@@ -467,8 +286,10 @@ __global__ void __launch_bounds__(HS_ROW_THREADS, 4) accept_rows_kernel(const __
     } else {
         __syncthreads();
     }
-    if (!s_flag) return;
-    if (warp == 0) {
+    const bool merges = s_flag != 0;
+    // CTAs of a deterministic-proposal sequence stay to take slices of its bonus draw (where the whole grid is resident)
+    if (!merges && !(p.jobs && md == HS_ACCEPT_DETERMINISTIC && which == 0)) return;
+    if (merges && warp == 0) {
     // the CTA that merges the row (chunks <= 32, one lane per chunk)
     unsigned long long ck = 0ull;
     float cm = -CUDART_INF_F, cs = 0.f;
@@ -494,7 +315,7 @@ __global__ void __launch_bounds__(HS_ROW_THREADS, 4) accept_rows_kernel(const __
     }
     }
     // ---- greedy sequences finish here: the last target row of a sequence to be merged walks its tree ------
-    if (md == HS_ACCEPT_REJECTION && !p.have_draft && which == 0 && i == 0) {
+    if (merges && md == HS_ACCEPT_REJECTION && !p.have_draft && which == 0 && i == 0) {
         // rejection sampling needs the draft distribution: the caller passed none
         const int cap = p.out.path_cap;
         for (int j = tid; j < cap; j += HS_ROW_THREADS) {
@@ -509,16 +330,17 @@ __global__ void __launch_bounds__(HS_ROW_THREADS, 4) accept_rows_kernel(const __
     }
     if (which != 0 || md == HS_ACCEPT_REJECTION) return;
     __syncthreads();
-    if (tid == 0) {                                // (the thread that wrote the row's merged result)
+    if (tid == 0 && merges) {                      // (the thread that wrote the row's merged result)
         int old;
         asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(old) : "l"(&p.seq_cnt[b]) : "memory");
         s_flag = (old == nk - 1);
         if (s_flag) p.seq_cnt[b] = 0;
     }
     __syncthreads();
-    if (s_flag) {
-        if (md == HS_ACCEPT_GREEDY) greedy_walk(p, b);
-        else deterministic_walk(p, b);
+    if (md == HS_ACCEPT_DETERMINISTIC) {
+        if (s_flag || p.jobs) det_chunk_tail(p, b, nk, merges && s_flag);
+    } else if (s_flag) {
+        greedy_walk(p, b);
     }
 }
 
@@ -932,6 +754,16 @@ __global__ void __launch_bounds__(AS_THREADS, 1) accept_stream_kernel(const __gr
             else deterministic_walk(p, b);
             walk_sync();                       // the walks' shared arrays are free again
         }
+        if (p.jobs) {
+            // the bonus draws of deterministic-proposal sequences are shared by all CTAs that had rows to read
+            bool any = false;
+            for (int b = tid; b < p.batch; b += HS_ROW_THREADS)
+                any |= p.mode[b] == HS_ACCEPT_DETERMINISTIC && p.pr.n_keep[b] > 0 && p.pr.status[b] == 0;
+            if (named_bar_or(2, HS_ROW_THREADS, any)) {
+                if (npend == 0) det_help(p, -1, false);
+                det_leave(p, -1, (int)((total + per - 1) / per));
+            }
+        }
     }
 }
 
@@ -1330,6 +1162,10 @@ hs_status hs_launch_accept(hs_ctx* ctx, const hs_tree_batch* tree, const hs_prun
     p.err = ctx->counters + HS_CNT_ERROR;
     p.staged = 0;
     p.clustered = 0;
+    p.jobs = nullptr;
+    p.det_cnt = ctx->counters + HS_CNT_DET;
+    o = hs_align_up(o, 256);
+    DetJob* const jobs = p.batch <= DET_MAX_BATCH && o + p.batch * sizeof(DetJob) <= ctx->scratch_bytes ? (DetJob*)(ctx->scratch + o) : nullptr;
     // without draft logits every sequence must be greedy: no draft rows to scan and no sampling walk
     cudaError_t e;
     const bool streamed = ctx->row_pass == HS_ROW_PASS_STREAM ||
@@ -1342,6 +1178,7 @@ hs_status hs_launch_accept(hs_ctx* ctx, const hs_tree_batch* tree, const hs_prun
                 return HS_ERR_CUDA;
             ctx->rows_ready = true;
         }
+        p.jobs = jobs;
         e = dtype == HS_BF16
             ? hs_launch(accept_stream_kernel<true>, dim3(ctx->sm_count), dim3(AS_THREADS), AS_SMEM_BYTES, stream, ctx->pdl, dim3(1, 1, 1), p)
             : hs_launch(accept_stream_kernel<false>, dim3(ctx->sm_count), dim3(AS_THREADS), AS_SMEM_BYTES, stream, ctx->pdl, dim3(1, 1, 1), p);
@@ -1352,6 +1189,7 @@ hs_status hs_launch_accept(hs_ctx* ctx, const hs_tree_batch* tree, const hs_prun
         // slots in one GPC and the pass gets slower than with independent CTAs
         p.clustered = p.chunks > 1 && p.chunks <= 8 &&
                       (size_t)p.chunks * rows * (p.have_draft ? 2 : 1) * 2 <= (size_t)7 * ctx->sm_count;
+        if (p.clustered) p.jobs = jobs;               // (CTAs that stay to help must not keep others from starting)
         dim3 grid(p.chunks, rows, p.have_draft ? 2 : 1), cl(p.clustered ? p.chunks : 1, 1, 1);
         e = dtype == HS_BF16
             ? hs_launch(accept_rows_kernel<true>, grid, dim3(HS_ROW_THREADS), 0, stream, ctx->pdl, cl, p)

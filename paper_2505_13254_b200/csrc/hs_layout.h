@@ -16,6 +16,7 @@
 #define HS_CNT_ACC_ROW 20480      // [2*HS_MAX_ROWS] chunks of a target / draft row
 #define HS_CNT_ACC_SEQ 53248      // [HS_MAX_BATCH] merged target rows of a sequence
 #define HS_CNT_CART 58368         // [4*256 + 16] digit counts, tickets and arrivals of the stratifier training
+#define HS_CNT_DET 59456          // [4*256] shared bonus draws of the deterministic-proposal sequences
 #define HS_CNT_ERROR 61440        // [1] sticky device error word (bounded wait expired)
 #define HS_CNT_PRUNE_DONE 61504   // [1] fused tree stage + pruning: CTAs that have read the counts ahead of theirs
 

@@ -78,6 +78,14 @@ __device__ __forceinline__ int ld_acquire_gpu(const int* p) {
 __device__ __forceinline__ void named_bar_sync(int id, int nthr) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthr) : "memory");
 }
+// The same barrier, returning whether any thread passed a true predicate.
+__device__ __forceinline__ bool named_bar_or(int id, int nthr, bool pred) {
+    int r;
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.s32 p, %3, 0;\n barrier.cta.red.or.pred q, %1, %2, p;\n selp.s32 %0, 1, 0, q;\n}\n"
+        : "=r"(r) : "r"(id), "r"(nthr), "r"((int)pred) : "memory");
+    return r != 0;
+}
 __device__ __forceinline__ void tma_load_3d(unsigned int dst, const CUtensorMap* tm, int c0, int c1, int c2,
                                             unsigned int bar) {
     asm volatile(
