@@ -30,7 +30,7 @@
 namespace cg = cooperative_groups;
 
 #define LOG2E 1.4426950408889634f
-#define WALK_CLUSTER 16       // (larger than the portable 8: the launcher asks for it)
+#define WALK_CLUSTER 16       // CTAs per sequence: 16 (larger than the portable 8: the launcher asks for it), or 8 for large batches
 #define WALK_THREADS 512
 
 // A bonus draw of a deterministic-proposal sequence that the CTAs of the launch share (in the workspace, one per sequence).
@@ -781,25 +781,39 @@ struct RowSlice {
     int v0, nv;
 };
 
-// All-gather of one 64-bit value per CTA over the cluster: warp 0 of every CTA stores its value into slot `rank` of the
-// exchange buffer of all WALK_CLUSTER CTAs (posted stores through distributed shared memory, lane r to CTA r), one
+// All-gather of one 64-bit value per CTA over the cluster of WC CTAs: warp 0 of every CTA stores its value into slot `rank`
+// of the exchange buffer of all CTAs (posted stores through distributed shared memory, lane r to CTA r), one
 // cluster barrier makes them visible, every CTA then reads its own copy.  The buffers alternate from one exchange to
 // the next (s_x[xch & 1]), so one barrier per exchange is enough: a buffer is written again only two exchanges later,
 // after a barrier that every CTA reaches with its reads done.  `v` must be valid in warp 0.
+template <int WC>
 __device__ __forceinline__ void cluster_allgather(unsigned long long v, unsigned long long (*s_x)[WALK_CLUSTER],
                                                   unsigned int& xch, unsigned int rank) {
     unsigned long long* buf = s_x[xch & 1u];
     ++xch;
-    if (threadIdx.x < WALK_CLUSTER) {
+    if (threadIdx.x < WC) {
         const unsigned int remote = cluster_map_addr(smem_u32(&buf[rank]), threadIdx.x);
         asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(remote), "l"(v) : "memory");
     }
+    __syncwarp();
     cluster_arrive();
     cluster_wait();
 }
+// the first `n` of N values as a tree (see sum8 on why)
+template <int N>
+__device__ __forceinline__ double sum_first(const double* v, int n) {
+    double a[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) a[i] = i < n ? v[i] : 0.0;
+    double t = sum8(a[0], a[1], a[2], a[3], a[4], a[5], a[6], a[7]);
+    if (N > 8) t += sum8(a[N - 8], a[N - 7], a[N - 6], a[N - 5], a[N - 4], a[N - 3], a[N - 2], a[N - 1]);
+    return t;
+}
+static_assert(WALK_THREADS / 32 == 16, "sum_first<16> sums the warps");
 
 // Sum over this CTA's share of the vocabulary of max(p_v - c q_v, 0), then over the cluster.
 // Every CTA returns the same value (fixed summation order).
+template <int WC>
 __device__ double cluster_residual_sum(const AcceptParams& p, unsigned int rank, const RowSlice& rs,
                                        float pm, float ips, float qm, float iqs, float invT,
                                        float c, double* s_part, unsigned long long (*s_x)[WALK_CLUSTER], unsigned int& xch) {
@@ -824,40 +838,47 @@ __device__ double cluster_residual_sum(const AcceptParams& p, unsigned int rank,
     if (lane == 0) s_part[warp] = w;
     __syncthreads();
     double t = 0.0;
-    if (warp == 0) {                                   // the warps' sums in a fixed order, known to every lane of warp 0
-        for (int i = 0; i < WALK_THREADS / 32; ++i) t += s_part[i];
-    }
-    const unsigned long long* got = s_x[xch & 1u];
-    cluster_allgather((unsigned long long)__double_as_longlong(t), s_x, xch, rank);
-    double tot = 0.0;
-    for (unsigned int r = 0; r < WALK_CLUSTER; ++r) tot += __longlong_as_double((long long)got[r]);
-    return tot;
+    if (warp == 0) t = sum_first<16>(s_part, 16);      // the warps' sums in a fixed order, known to every lane of warp 0
+    const double* got = reinterpret_cast<const double*>(s_x[xch & 1u]);
+    cluster_allgather<WC>((unsigned long long)__double_as_longlong(t), s_x, xch, rank);
+    return sum_first<WC>(got, WC);
 }
 
 // Inverse-CDF draw from max(p - c q, 0) in token order: smallest j whose running sum exceeds
 // u * total; if rounding leaves none, the last token with positive mass.  rs.q may be NULL (c = 0).
-// A CTA covers the tokens of its slice, a thread a contiguous run of them; running sums in double.
-__device__ int cluster_inverse_cdf(const AcceptParams& p, unsigned int rank, const RowSlice& rs,
-                                   float pm, float ips, float qm, float iqs, float invT,
-                                   float c, float u, double* s_scan, unsigned long long (*s_x)[WALK_CLUSTER],
-                                   unsigned int& xch, int* s_pick) {
+// A CTA covers the tokens of its slice, a thread a contiguous run of vectors; running sums in double.  One exchange: every
+// CTA learns the masses of all slices and with them which one holds the crossing; that CTA finds the token and writes it.
+template <int WC>
+__device__ void cluster_inverse_cdf(const AcceptParams& p, unsigned int rank, const RowSlice& rs,
+                                    float pm, float ips, float qm, float iqs, float invT,
+                                    float c, float u, double* s_scan, unsigned long long (*s_x)[WALK_CLUSTER],
+                                    unsigned int& xch, int* s_pick, int* bonus) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int ve = p.is_bf16 ? 8 : 4;
-    const int c0 = rs.v0 * ve, c1 = min(c0 + rs.nv * ve, p.vocab);
-    const int seg = (max(c1 - c0, 0) + WALK_THREADS - 1) / WALK_THREADS;
-    const int t0 = min(c0 + tid * seg, c1), t1 = min(t0 + seg, c1);
-    auto mass = [&](int j) -> float {
-        float pv = exp2f((fmaxf(load_logit(rs.p, p.is_bf16, j - c0), -1e30f) - pm) * invT) * ips;
-        if (rs.q == nullptr) return pv;
-        float qv = exp2f((fmaxf(load_logit(rs.q, p.is_bf16, j - c0), -1e30f) - qm) * invT) * iqs;
-        return fmaxf(pv - c * qv, 0.f);
+    const int run_v = (rs.nv + WALK_THREADS - 1) / WALK_THREADS;           // vectors per thread
+    const int w0 = min(tid * run_v, rs.nv), w1 = min(w0 + run_v, rs.nv);
+    auto masses = [&](int v, float (&m)[8]) {                               // of vector v of the slice
+        float x[8], y[8];
+        const uint4 a = rs.p[v];
+        if (p.is_bf16) unpack_v<true>(a, x); else unpack_v<false>(a, x);
+        if (rs.q) { const uint4 bq = rs.q[v]; if (p.is_bf16) unpack_v<true>(bq, y); else unpack_v<false>(bq, y); }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            m[e] = 0.f;
+            if (e < ve && (rs.v0 + v) * ve + e < p.vocab) {
+                m[e] = exp2f((fmaxf(x[e], -1e30f) - pm) * invT) * ips;
+                if (rs.q) m[e] = fmaxf(m[e] - c * (exp2f((fmaxf(y[e], -1e30f) - qm) * invT) * iqs), 0.f);
+            }
+        }
     };
     double mine = 0.0;
     int last_pos = -1;
-    for (int j = t0; j < t1; ++j) {
-        float r = mass(j);
-        mine += (double)r;
-        if (r > 0.f) last_pos = j;
+    for (int v = w0; v < w1; ++v) {
+        float m[8];
+        masses(v, m);
+        mine += sum8(m);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) if (m[e] > 0.f) last_pos = (rs.v0 + v) * ve + e;
     }
     if (tid == 0) { s_pick[0] = 0x7fffffff; s_pick[1] = -1; }
     // exclusive scan over the CTA's threads: inclusive shuffle scan inside a warp, then the warps' totals in order
@@ -869,45 +890,37 @@ __device__ int cluster_inverse_cdf(const AcceptParams& p, unsigned int rank, con
     }
     if (lane == 31) s_scan[warp] = incl;
     __syncthreads();
-    double wbefore = 0.0, ctot = 0.0;
+    const double ctot = sum_first<16>(s_scan, 16), wbefore = sum_first<16>(s_scan, warp);
+    const double* got = reinterpret_cast<const double*>(s_x[xch & 1u]);
+    cluster_allgather<WC>((unsigned long long)__double_as_longlong(ctot), s_x, xch, rank);
+    const double before = sum_first<WC>(got, (int)rank), goal = (double)u * sum_first<WC>(got, WC);
+    // the slice with the crossing: the first whose running total exceeds the goal (rounding leaves none: the last with mass).
+    // Lane r of every warp tries slice r.
+    const unsigned int over = __ballot_sync(HS_FULL_MASK, lane < WC && sum_first<WC>(got, lane + 1) > goal);
+    const unsigned int full = __ballot_sync(HS_FULL_MASK, lane < WC && got[lane & (WC - 1)] > 0.0);
+    const int owner = over ? __ffs(over) - 1 : (full ? 31 - __clz(full) : 0);
+    if ((int)rank != owner) return;
+    double run = before + (wbefore + (incl - mine));
+    if (run <= goal && run + mine > goal) {          // the crossing lies in this thread's run
+        bool found = false;
+        for (int v = w0; v < w1 && !found; ++v) {
+            float m[8];
+            masses(v, m);
 #pragma unroll
-    for (int w = 0; w < WALK_THREADS / 32; ++w) {
-        const double t = s_scan[w];
-        if (w < warp) wbefore += t;
-        ctot += t;
-    }
-    const unsigned long long* got = s_x[xch & 1u];
-    cluster_allgather((unsigned long long)__double_as_longlong(ctot), s_x, xch, rank);
-    double before = 0.0, total = 0.0;
-    for (unsigned int r = 0; r < WALK_CLUSTER; ++r) {
-        const double v = __longlong_as_double((long long)got[r]);
-        if (r < rank) before += v;
-        total += v;
-    }
-    const double goal = (double)u * total;
-    double run = before + wbefore + (incl - mine);
-    if (run <= goal && run + mine > goal) {          // the crossing lies in this thread's segment
-        for (int j = t0; j < t1; ++j) {
-            run += (double)mass(j);
-            if (run > goal) { atomicMin(&s_pick[0], j); break; }
+            for (int e = 0; e < 8; ++e) {
+                run += (double)m[e];
+                if (!found && run > goal) { found = true; atomicMin(&s_pick[0], (rs.v0 + v) * ve + e); }
+            }
         }
+        if (!found && last_pos >= 0) atomicMin(&s_pick[0], last_pos);       // (rounding)
     }
     if (last_pos >= 0) atomicMax(&s_pick[1], last_pos);
     __syncthreads();
-    // the CTAs' (crossing, last positive token) pairs, one 64-bit word each
-    const unsigned long long mine2 = ((unsigned long long)(unsigned int)s_pick[0] << 32) | (unsigned int)s_pick[1];
-    const unsigned long long* got2 = s_x[xch & 1u];
-    cluster_allgather(mine2, s_x, xch, rank);
-    int pick = 0x7fffffff, lastp = -1;
-    for (unsigned int r = 0; r < WALK_CLUSTER; ++r) {
-        pick = min(pick, (int)(unsigned int)(got2[r] >> 32));
-        lastp = max(lastp, (int)(unsigned int)(got2[r] & 0xffffffffu));
-    }
-    return pick != 0x7fffffff ? pick : max(lastp, 0);
+    if (tid == 0) *bonus = s_pick[0] != 0x7fffffff ? s_pick[0] : max(s_pick[1], 0);
 }
 
-__global__ void __cluster_dims__(WALK_CLUSTER, 1, 1) __launch_bounds__(WALK_THREADS, 1)
-accept_walk_kernel(const AcceptParams p) {
+template <int WC>
+__global__ void __launch_bounds__(WALK_THREADS, 1) accept_walk_kernel(const __grid_constant__ AcceptParams p) {
     cg::cluster_group cluster = cg::this_cluster();
     extern __shared__ __align__(16) unsigned char s_rows[];    // staged: this CTA's slices of p and q, `per` vectors each
     __shared__ unsigned long long s_bar;
@@ -917,7 +930,7 @@ accept_walk_kernel(const AcceptParams p) {
     unsigned int xch = 0;                  // exchanges through s_cta so far
     __shared__ int s_pick[2];
     const int tid = threadIdx.x;
-    const int b = blockIdx.x / WALK_CLUSTER;
+    const int b = blockIdx.x / WC;
     const unsigned int rank = cluster.block_rank();
     pdl_launch_dependents();
     pdl_wait();                            // arg-max and normalisers come from the row pass
@@ -946,7 +959,7 @@ accept_walk_kernel(const AcceptParams p) {
     // This CTA's slice of a row: vectors [v0, v0 + nv).  The rows of the node the walk stands on are brought into
     // shared memory once (one bulk copy each, only when a residual or the final draw needs them) and serve every
     // rejection at that node and the final draw.
-    const int per = (p.nvec + WALK_CLUSTER - 1) / WALK_CLUSTER;
+    const int per = (p.nvec + WC - 1) / WC;
     RowSlice rs;
     rs.v0 = rank * per;
     rs.nv = max(min(rs.v0 + per, p.nvec) - rs.v0, 0);
@@ -1023,7 +1036,8 @@ accept_walk_kernel(const AcceptParams p) {
         if (par >= 0 && par < j) atomicMin(&s_first[par], j);
     }
     __syncthreads();
-    int cur = 0, len = 0, bonus = -1;
+    int cur = 0, len = 0;
+    bool drawn = false;
     {
         for (int step = 0; step < nkc; ++step) {
             if (rank == 0 && tid == 0 && len < cap) {
@@ -1078,7 +1092,7 @@ accept_walk_kernel(const AcceptParams p) {
                 }
                 const float c_next = c + (float)W;
                 stage(cur, prow, qrow);
-                const double W_next = cluster_residual_sum(p, rank, rs, pm, ips, qm, iqs, invT,
+                const double W_next = cluster_residual_sum<WC>(p, rank, rs, pm, ips, qm, iqs, invT,
                                                            c_next, s_part, s_x, xch);
                 if (!(W_next > 0.0)) { c = 0.f; W = 1.0; tested = false; break; }   // p == q: fall back to p
                 c = c_next; W = W_next;
@@ -1091,15 +1105,15 @@ accept_walk_kernel(const AcceptParams p) {
             }
             const float ufin = p.uniforms ? p.uniforms[p.n_nodes_total + b] : philox_uniform(p.seed, p.offset, b, 0, 1);
             stage(cur, prow, (tested && c > 0.f) ? qrow : nullptr);
-            bonus = cluster_inverse_cdf(p, rank, rs, pm, ips, qm, iqs,
-                                        invT, c, ufin, s_scan, s_x, xch, s_pick);
+            drawn = true;
+            cluster_inverse_cdf<WC>(p, rank, rs, pm, ips, qm, iqs, invT, c, ufin, s_scan, s_x, xch, s_pick, &p.out.bonus_token[b]);
             break;
         }
     }
     // (every store into a CTA's exchange buffers precedes a barrier that CTA takes part in: it may leave now)
     if (rank == 0 && tid == 0) {
         p.out.accept_len[b] = len;
-        p.out.bonus_token[b] = bonus;
+        if (!drawn) p.out.bonus_token[b] = -1;
         p.out.terminal_rank[b] = p.pr.keep_rank[koff + cur];
         p.out.status[b] = HS_OK;
     }
@@ -1197,18 +1211,36 @@ hs_status hs_launch_accept(hs_ctx* ctx, const hs_tree_batch* tree, const hs_prun
     }
     if (e != cudaSuccess) return HS_ERR_CUDA;
     if (!p.have_draft) return HS_OK;
-    // the cluster shape of the walk is fixed at compile time (__cluster_dims__); its two row slices in shared memory
-    const size_t esz = dtype == HS_BF16 ? 2 : 4;
-    const size_t walk_smem = 2 * (size_t)((p.nvec + WALK_CLUSTER - 1) / WALK_CLUSTER) * 16;
-    p.staged = ((uintptr_t)p.target % 16 == 0) && ((uintptr_t)p.draft % 16 == 0) && ((size_t)row_stride * esz % 16 == 0) &&
-               walk_smem <= 160 * 1024;
+    // Sixteen CTAs per sequence until the batch has three times as many sequences as clusters of that size run at once (sequences
+    // in other modes leave at once, so a mixed batch needs a third to a half of them): then eight.  Budgeted batch of 32, 11 of
+    // them sampling: 22.6 us with sixteen, 19 us with eight; ragged batch of 16, 8 of them sampling: 29 us and 31 us.
     if (!ctx->walk_ready) {                  // per device (= per context): more than 48 KiB of shared memory, 16-CTA clusters
-        if (cudaFuncSetAttribute(accept_walk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) != cudaSuccess ||
-            cudaFuncSetAttribute(accept_walk_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+        if (cudaFuncSetAttribute(accept_walk_kernel<WALK_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) != cudaSuccess ||
+            cudaFuncSetAttribute(accept_walk_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) != cudaSuccess ||
+            cudaFuncSetAttribute(accept_walk_kernel<WALK_CLUSTER>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
             return HS_ERR_CUDA;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(WALK_CLUSTER * ctx->sm_count);
+        cfg.blockDim = dim3(WALK_THREADS);
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = WALK_CLUSTER; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&ctx->walk_cap, accept_walk_kernel<WALK_CLUSTER>, &cfg) != cudaSuccess) {
+            ctx->walk_cap = 0;
+            (void)cudaGetLastError();
+        }
         ctx->walk_ready = true;
     }
-    e = hs_launch(accept_walk_kernel, dim3(p.batch * WALK_CLUSTER), dim3(WALK_THREADS), p.staged ? walk_smem : 0, stream,
-                  ctx->pdl, dim3(1, 1, 1), p);
+    const size_t esz = dtype == HS_BF16 ? 2 : 4;
+    const int wc = p.batch <= 3 * ctx->walk_cap ? WALK_CLUSTER : 8;
+    const size_t walk_smem = 2 * (size_t)((p.nvec + wc - 1) / wc) * 16;       // two row slices
+    p.staged = ((uintptr_t)p.target % 16 == 0) && ((uintptr_t)p.draft % 16 == 0) && ((size_t)row_stride * esz % 16 == 0) &&
+               walk_smem <= 160 * 1024;
+    const dim3 wgrid(p.batch * wc), wcl(wc, 1, 1);
+    e = wc == WALK_CLUSTER
+        ? hs_launch(accept_walk_kernel<WALK_CLUSTER>, wgrid, dim3(WALK_THREADS), p.staged ? walk_smem : 0, stream, ctx->pdl, wcl, p)
+        : hs_launch(accept_walk_kernel<8>, wgrid, dim3(WALK_THREADS), p.staged ? walk_smem : 0, stream, ctx->pdl, wcl, p);
     return e == cudaSuccess ? HS_OK : HS_ERR_CUDA;
 }
