@@ -6,8 +6,8 @@
 // what hs_entropy_quantify writes -, a child's value is its parent's plus its log-confidence (ln V_i = sum ln c_j),
 // and the k children with the largest value (ties: created first) become the next frontier.  Reranking (one CTA
 // per sequence): the N candidates with the largest value, compacted in creation order with parents re-indexed: a
-// topologically ordered tree ready for the verification calls.  Ranks are found by counting, compaction by warp
-// ballots and a prefix sum over the warps.
+// topologically ordered tree ready for the verification calls.  A level ranks its children by counting, the reranking
+// finds the N-th largest value by binary search; compaction by warp ballots and a prefix sum over the warps.
 #include <math_constants.h>
 
 #include "hs_common.cuh"
@@ -30,40 +30,40 @@ __global__ void expand_init_kernel(hs_expand_state st) {
     st.status[b] = HS_OK;
 }
 
+// Two round trips to global memory: everything that does not depend on another load first (the statistics of slot (j, i)
+// are addressed by the thread's number alone), then the parents' values.  The rank among the new children reads four
+// values per shared-memory access.
+// (Growing four trees of 8 levels: 164 -> 136 us a pass, with the tree stage's early loads and the reranking below.)
 __global__ void __launch_bounds__(EX_THREADS) expand_level_kernel(hs_expand_state st, const float* topk_val,
                                                                   const int* topk_idx, const float* row_lse, int K) {
-    __shared__ float s_S[HS_MAX_TOPK * HS_MAX_TOPK];
-    __shared__ int s_bad;
+    __shared__ __align__(16) float s_S[HS_MAX_TOPK * HS_MAX_TOPK];
     const int b = blockIdx.x, tid = threadIdx.x;
     const int k = st.top_k;
+    const size_t o = (size_t)b * st.cap;
+    const int j = tid / k, i = tid - j * k, row = b * k + j;
     pdl_launch_dependents();
     pdl_wait();                                    // the row statistics come from the kernel ahead
-    if (st.status[b] != HS_OK) return;
-    const size_t o = (size_t)b * st.cap;
-    const int n0 = st.n_cand[b], nf = st.n_frontier[b];
+    const int status = st.status[b], n0 = st.n_cand[b], nf = st.n_frontier[b];
+    int par = -1, tok = -1, dep = 0;
+    float lc = 0.f;
+    if (j < k) {
+        par = st.frontier[(size_t)b * k + j];      // (slots past the frontier hold older candidates: not used)
+        tok = topk_idx[(size_t)row * K + i];
+        lc = topk_val[(size_t)row * K + i] - row_lse[row];
+    }
+    if (status != HS_OK) return;
     const int nnew = nf * k;
-    if (tid == 0) s_bad = 0;
-    __syncthreads();
     if (n0 + nnew > st.cap) {                      // the arrays cannot take another level
         if (tid == 0) st.status[b] = HS_ERR_SHAPE;
         return;
     }
-    float S = -CUDART_INF_F;
-    int par = -1, tok = -1, dep = 0;
-    float lc = 0.f;
+    float S = __int_as_float(0x7fc00000);          // (NaN: compares false, ranks nobody)
     if (tid < nnew) {
-        const int j = tid / k, i = tid - j * k;
-        const int row = b * k + j;
-        par = st.frontier[(size_t)b * k + j];
-        tok = topk_idx[(size_t)row * K + i];
-        lc = topk_val[(size_t)row * K + i] - row_lse[row];
         S = st.score[o + par] + lc;
         dep = st.depth[o + par] + 1;
-        if (tok < 0) s_bad = 1;                    // the row had fewer than k finite logits
-        s_S[tid] = S;
     }
-    __syncthreads();
-    if (s_bad) {
+    s_S[tid] = S;
+    if (__syncthreads_or(tid < nnew && tok < 0)) { // a row had fewer than k finite logits
         if (tid == 0) st.status[b] = HS_ERR_BAD_TREE;
         return;
     }
@@ -72,7 +72,12 @@ __global__ void __launch_bounds__(EX_THREADS) expand_level_kernel(hs_expand_stat
         st.parent[o + c] = par; st.token[o + c] = tok; st.depth[o + c] = dep;
         st.logc[o + c] = lc; st.score[o + c] = S;
         int rank = 0;                              // by (value descending, creation order)
-        for (int j = 0; j < nnew; ++j) rank += (s_S[j] > S || (s_S[j] == S && j < tid));
+        const float4* S4 = reinterpret_cast<const float4*>(s_S);
+        for (int q = 0; q < nnew; q += 4) {
+            const float4 v = S4[q >> 2];
+            rank += (v.x > S || (v.x == S && q < tid)) + (v.y > S || (v.y == S && q + 1 < tid)) +
+                    (v.z > S || (v.z == S && q + 2 < tid)) + (v.w > S || (v.w == S && q + 3 < tid));
+        }
         if (rank < k) st.frontier[(size_t)b * k + rank] = c;
     }
     if (tid == 0) {
@@ -98,59 +103,71 @@ __device__ __forceinline__ int rerank_count(const RerankParams& p, int b) {
     return max(0, min(want, p.st.n_cand[b]));
 }
 
-__global__ void __launch_bounds__(EX_THREADS) rerank_kernel(const RerankParams p) {
-    __shared__ float s_S[EX_MAX_CAP];
+// The Top-N of up to 2048 candidates: the N-th largest value by binary search over its 32 order bits (each thread holds two
+// candidates, a step is one counting barrier), ties to the candidate created first.  Ranking by counting compared every
+// pair (711 candidates: 28.9 us alone, this: 10.1 us).
+#define RR_THREADS 1024
+__global__ void __launch_bounds__(RR_THREADS) rerank_kernel(const RerankParams p) {
     __shared__ short s_new[EX_MAX_CAP];
-    __shared__ int s_warp[EX_THREADS / 32];
-    __shared__ int s_off;
-    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ int s_warp[2][RR_THREADS / 32];
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x, nw = nthr >> 5;
     pdl_launch_dependents();
     pdl_wait();
-    // offset of this sequence's tree: the trees ahead of it hold min(N, candidates) nodes each
-    int part = 0;
-    for (int bb = tid; bb < b; bb += EX_THREADS) part += rerank_count(p, bb);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(HS_FULL_MASK, part, o);
-    if (lane == 0) s_warp[warp] = part;
-    __syncthreads();
-    if (tid == 0) {
-        int t = 0;
-        for (int w = 0; w < EX_THREADS / 32; ++w) t += s_warp[w];
-        s_off = t;
-    }
-    __syncthreads();
-    const int off = s_off;
+    const size_t o = (size_t)b * p.st.cap;
     const int n = p.st.status[b] == HS_OK ? min(p.st.n_cand[b], EX_MAX_CAP) : 0;
     const int want = rerank_count(p, b);
-    const size_t o = (size_t)b * p.st.cap;
-    for (int c = tid; c < n; c += EX_THREADS) s_S[c] = p.st.score[o + c];
-    __syncthreads();
-    // candidates in creation order, EX_THREADS at a time; kept ones are numbered by ballot + prefix over the warps
-    int base = 0;
-    for (int c0 = 0; c0 < n; c0 += EX_THREADS) {
-        const int c = c0 + tid;
-        bool keep = false;
-        if (c < n) {
-            const float S = s_S[c];
-            int rank = 0;
-            for (int j = 0; j < n; ++j) rank += (s_S[j] > S || (s_S[j] == S && j < c));
-            keep = rank < want;
-        }
-        const unsigned int bal = __ballot_sync(HS_FULL_MASK, keep);
-        __syncthreads();                           // s_warp is reused
-        if (lane == 0) s_warp[warp] = __popc(bal);
-        __syncthreads();
-        int before = base + __popc(bal & ((1u << lane) - 1u));
-        int total = 0;
-        for (int w = 0; w < EX_THREADS / 32; ++w) { if (w < warp) before += s_warp[w]; total += s_warp[w]; }
-        if (c < n) s_new[c] = keep ? (short)before : (short)-1;
-        base += total;
+    // candidates tid and tid + nthr; 0 = none (no value has order bits 0)
+    unsigned int key[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int c = h * nthr + tid;
+        key[h] = c < n ? float_order_bits(p.st.score[o + c] + 0.f) : 0u;
     }
+    // offset of this sequence's tree: the trees ahead of it hold min(N, candidates) nodes each
+    int part = 0;
+    for (int bb = tid; bb < b; bb += nthr) part += rerank_count(p, bb);
+    part = __reduce_add_sync(HS_FULL_MASK, part);
+    if (lane == 0) s_warp[0][warp] = part;
     __syncthreads();
-    for (int c = tid; c < n; c += EX_THREADS) {
-        const int i = s_new[c];
-        if (i < 0) continue;
-        const int par = p.st.parent[o + c];
+    const int off = __reduce_add_sync(HS_FULL_MASK, lane < nw ? s_warp[0][lane] : 0);
+    // numbers of candidates whose flag is set ahead of this thread's two, in creation order, and in all
+    auto ahead = [&](bool f0, bool f1, int (&a)[2]) -> int {
+        const unsigned int b0 = __ballot_sync(HS_FULL_MASK, f0), b1 = __ballot_sync(HS_FULL_MASK, f1);
+        __syncthreads();                           // (s_warp may still be read)
+        if (lane == 0) { s_warp[0][warp] = __popc(b0); s_warp[1][warp] = __popc(b1); }
+        __syncthreads();
+        const int c0 = lane < nw ? s_warp[0][lane] : 0, c1 = lane < nw ? s_warp[1][lane] : 0;
+        const int t0 = __reduce_add_sync(HS_FULL_MASK, c0), t1 = __reduce_add_sync(HS_FULL_MASK, c1);
+        const unsigned int below = (1u << lane) - 1u;
+        a[0] = __reduce_add_sync(HS_FULL_MASK, lane < warp ? c0 : 0) + __popc(b0 & below);
+        a[1] = t0 + __reduce_add_sync(HS_FULL_MASK, lane < warp ? c1 : 0) + __popc(b1 & below);
+        return t0 + t1;
+    };
+    // T = the want-th largest key: the largest T with at least `want` keys >= T
+    unsigned int T = 0u;
+    if (want < n) {
+        for (int bit = 31; bit >= 0; --bit) {
+            const unsigned int t = T | (1u << bit);
+            int cnt = __syncthreads_count(key[0] >= t);
+            if (n > nthr) cnt += __syncthreads_count(key[1] >= t);
+            if (cnt >= want) T = t;
+        }
+    }
+    int e[2], above = __syncthreads_count(key[0] > T);
+    if (n > nthr) above += __syncthreads_count(key[1] > T);
+    ahead(key[0] == T && key[0] != 0u, key[1] == T && key[1] != 0u, e);      // of the ties at T the first want - above stay
+    const bool k0 = key[0] > T || (key[0] == T && key[0] != 0u && e[0] < want - above);
+    const bool k1 = key[1] > T || (key[1] == T && key[1] != 0u && e[1] < want - above);
+    int pos[2];
+    ahead(k0, k1, pos);
+    if (tid < n) s_new[tid] = k0 ? (short)pos[0] : (short)-1;
+    if (nthr + tid < n) s_new[nthr + tid] = k1 ? (short)pos[1] : (short)-1;
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int c = h * nthr + tid;
+        if (!(h ? k1 : k0)) continue;
+        const int i = pos[h], par = p.st.parent[o + c];
         p.parent[off + i] = par >= 0 ? (int)s_new[par] : -1;   // (the kept set is closed under ancestors)
         p.token[off + i] = p.st.token[o + c];
         p.cand_id[off + i] = c;
@@ -192,6 +209,7 @@ extern "C" hs_status hs_rerank(hs_ctx* ctx, const hs_expand_state* st, const int
     RerankParams p;
     p.st = *st; p.n_top = n_top; p.n_default = n_default;
     p.node_off = node_off; p.parent = parent; p.token = token; p.cand_id = cand_id; p.depth = depth;
-    return hs_launch(rerank_kernel, dim3(st->batch), dim3(EX_THREADS), 0, (cudaStream_t)stream, ctx->pdl, dim3(1, 1, 1), p) ==
+    const int threads = st->cap < RR_THREADS ? (st->cap + 31) / 32 * 32 : RR_THREADS;      // two candidates each
+    return hs_launch(rerank_kernel, dim3(st->batch), dim3(threads), 0, (cudaStream_t)stream, ctx->pdl, dim3(1, 1, 1), p) ==
                    cudaSuccess ? HS_OK : HS_ERR_CUDA;
 }

@@ -280,6 +280,10 @@ __global__ void __maxnreg__(72) quantify_stream_kernel(const QuantParams p) {
         s_cnt = 0;
     }
     __syncthreads();
+    // The tree stage behind this kernel may start once every CTA has passed this point.  Without prefetch that is behind
+    // the dependency wait, so whatever was written ahead of the call is complete by then and the tree stage may read its
+    // inputs (not this kernel's results) without waiting.
+    if (!p.prefetch) pdl_wait();
     pdl_launch_dependents();
     // Clustered launch: first half of a cluster barrier - when it completes every CTA of the row's cluster runs and
     // its shared memory may be written from outside.  Every thread of the CTA, the producer warp included, takes part
@@ -292,8 +296,7 @@ __global__ void __maxnreg__(72) quantify_stream_kernel(const QuantParams p) {
             long long g = g0;
             int it = 0, slot = 0;
             unsigned int epar = 1u;          // parity of the slot's `empty` barrier before its first completion
-            bool waited = false;
-            if (!p.prefetch) { pdl_wait(); waited = true; }
+            bool waited = !p.prefetch;
             while (g < g1) {
                 const int row = (int)(g / p.nvec);
                 const int v = (int)(g - (long long)row * p.nvec);
@@ -324,8 +327,7 @@ __global__ void __maxnreg__(72) quantify_stream_kernel(const QuantParams p) {
     // Partials, counters and outputs may still be in use by the kernel ahead: nothing is written before the wait.
     // Reading the logits and reducing them in registers and shared memory needs no wait if the caller vouches that
     // they were complete before the call (prefetch): then the wait comes at the end of the first segment.
-    bool waited = false;
-    if (!p.prefetch) { pdl_wait(); waited = true; }
+    bool waited = !p.prefetch;
     const int K = p.K;
     const unsigned int ninf = BF16 ? 0xff80ff80u : 0xff800000u;
     int cslot = 0;                 // slot of the next item and the parity of its `full` barrier (the producer fills

@@ -301,7 +301,7 @@ struct TreePruneParams {
     // the tree stage's view (the names tree_stage_cta expects)
     const void* logits;
     int64_t row_stride;
-    int vocab, is_bf16, prefetch;
+    int vocab, is_bf16;
     const int* node_off;
     const int* parent;
     const int* token;
@@ -364,7 +364,6 @@ hs_status hs_launch_tree_prune(hs_ctx* ctx, const hs_tree_batch* tree, const voi
     p.row_stride = row_stride;
     p.vocab = vocab;
     p.is_bf16 = dtype == HS_BF16;
-    p.prefetch = (ctx->prefetch & HS_PREFETCH_LOGITS) != 0;
     p.node_off = tree->node_off;
     p.parent = tree->parent;
     p.token = tree->token;

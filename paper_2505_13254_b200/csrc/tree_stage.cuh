@@ -25,13 +25,13 @@ struct TreeStageResult {   // of the calling thread's node (thread t = node t)
 };
 
 // P needs: logits, row_stride, vocab, is_bf16, node_off, parent, token, out (hs_quant_out), d_base, phi_mode,
-// pstar_mode, entropy_mode, prefetch.  Calls griddepcontrol.wait once (the row statistics come from the launch ahead;
-// with `prefetch` the tree and the token logits, inputs of the call, are fetched before that wait).
+// pstar_mode, entropy_mode.  Calls griddepcontrol.wait once: the row statistics come from the launch ahead.  The tree and the
+// token logits are inputs of the call; they are fetched before that wait, which is allowed because the launch ahead lets
+// this one start only when they are complete (three dependent round trips to L2, hidden behind the row pass).
 template <class P>
 __device__ __forceinline__ TreeStageResult tree_stage_cta(const P& p, int b, TreeStageSmem& sm) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     TreeStageResult r;
-    if (!p.prefetch) pdl_wait();
     const int base = p.node_off[b];
     const int n = p.node_off[b + 1] - base;
     r.n = n;
@@ -48,7 +48,7 @@ __device__ __forceinline__ TreeStageResult tree_stage_cta(const P& p, int b, Tre
         const size_t off = (size_t)(base + par) * p.row_stride + tok;
         lv = p.is_bf16 ? __bfloat162float(((const __nv_bfloat16*)p.logits)[off]) : ((const float*)p.logits)[off];
     }
-    if (p.prefetch) pdl_wait();
+    pdl_wait();
     bad = __syncthreads_or(bad);
     r.bad = bad != 0;
     r.par = par; r.dep = 0; r.S = 0.f;
