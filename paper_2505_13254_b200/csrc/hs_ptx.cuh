@@ -59,6 +59,25 @@ __device__ __forceinline__ bool mbar_wait(unsigned int bar, unsigned int parity,
     return mbar_wait_limit(bar, parity, err, HS_WAIT_LIMIT_NS);
 }
 
+// The same for data that other CTAs of the cluster stored (acquire at cluster scope).
+__device__ __forceinline__ bool mbar_wait_cluster(unsigned int bar, unsigned int parity, int* err) {
+    const unsigned long long t0 = global_timer_ns();
+    for (;;) {
+#pragma unroll 1
+        for (int i = 0; i < 128; ++i) {
+            unsigned int ok;
+            asm volatile(
+                "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+                : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+            if (ok) return true;
+        }
+        if (global_timer_ns() - t0 > HS_WAIT_LIMIT_NS) {
+            atomicExch(err, (int)HS_ERR_TIMEOUT);
+            return false;
+        }
+    }
+}
+
 // Untiled bulk copy global -> shared (both 16-byte aligned, size a multiple of 16), completion
 // signalled on an mbarrier as transferred bytes.
 __device__ __forceinline__ void bulk_load(unsigned int dst, const void* src, unsigned int bytes, unsigned int bar) {
@@ -231,12 +250,17 @@ __device__ __forceinline__ unsigned int cluster_map_addr(unsigned int local_addr
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_addr), "r"(rank));
     return r;
 }
-// Bulk copy from this CTA's shared memory into another CTA's (addresses 16-byte aligned, size a multiple
-// of 16); the transferred bytes are signalled on an mbarrier of the destination CTA.
-__device__ __forceinline__ void bulk_push(unsigned int dst_cluster_addr, unsigned int src_addr, unsigned int bytes,
-                                          unsigned int bar_cluster_addr) {
-    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(dst_cluster_addr), "r"(src_addr), "r"(bytes), "r"(bar_cluster_addr) : "memory");
+// Asynchronous stores from registers into another CTA's shared memory (addresses aligned to the size); the bytes are
+// signalled on an mbarrier of the same CTA as the destination.
+__device__ __forceinline__ void st_async_v4(unsigned int dst_cluster_addr, unsigned int a, unsigned int b, unsigned int c,
+                                            unsigned int d, unsigned int bar_cluster_addr) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(dst_cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d), "r"(bar_cluster_addr) : "memory");
+}
+__device__ __forceinline__ void st_async_v2(unsigned int dst_cluster_addr, unsigned int a, unsigned int b,
+                                            unsigned int bar_cluster_addr) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
+                 ::"r"(dst_cluster_addr), "r"(a), "r"(b), "r"(bar_cluster_addr) : "memory");
 }
 // split cluster barrier (every thread of every CTA of the cluster executes both halves once)
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }

@@ -44,6 +44,7 @@ struct AttnParams {
     const int* node_off;
     const int* kv_off;
     int batch, hq, hkv, G, layout, nsplit, head_first, prefetch;
+    unsigned int inv_g;       // ceil(2^16 / G): r / G = r * inv_g >> 16 for the row numbers r < 2^11
     float scale_log2;
     int* err;
 };
@@ -90,8 +91,9 @@ __device__ __forceinline__ void prefix_range(int L, int nsplit, int split, int& 
 #define UM_MAP_BYTES 1024                            // output-row map of the rows a CTA merges (<= 65 rows x 8 bytes)
 #define UM_TMEM_COLS 512                             // S of stream g: columns 64 g ..; O: 128 + 128 g ..; P (bf16 pairs): 384 + 32 g ..
 #define UM_STAGES 4
-#define UM_RECV_BYTES (40 * 1024)                    // after the tile loop: partials pushed by the splits of the cluster
-#define UM_SMEM_BYTES (UM_STAGES * ATT_STAGE_BYTES + ATT_Q_BYTES + UM_MAP_BYTES + 4096 + 1024)
+#define UM_WT_BYTES (66 * ATT_MAX_SPLIT * 4 + 64)    // split weights of the rows a CTA merges
+#define UM_RECV_BYTES (ATT_PB_STRIDE * (ATT_BM + 2 * ATT_MAX_SPLIT))     // partials pushed by the splits of the cluster
+#define UM_SMEM_BYTES (UM_STAGES * ATT_STAGE_BYTES + ATT_Q_BYTES + UM_MAP_BYTES + 1024 + 2048 + UM_WT_BYTES + UM_RECV_BYTES + 1024)
 
 __global__ void __launch_bounds__(UM_THREADS, 1)
 tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV) {
@@ -134,6 +136,7 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
                        bar_p = bar_done + 8, bar_sr = bar_p + 16, tslot = bar_sr + 16;
     unsigned char* gQ = smem_gen + UM_STAGES * ATT_STAGE_BYTES;
     unsigned char* gM = gQ + ATT_Q_BYTES;
+    unsigned char* gR = gM + UM_MAP_BYTES + 1024 + 2048 + UM_WT_BYTES;      // partials received from the cluster
     volatile unsigned int* tslot_gen = reinterpret_cast<volatile unsigned int*>(gM + UM_MAP_BYTES + (4 * UM_STAGES + 8) * 8);
     float* s_mx = reinterpret_cast<float*>(gM + UM_MAP_BYTES + 1024);      // [2][128]: the streams' row maxima at the end
     float* s_lx = s_mx + 2 * ATT_BM;                                     // [2][128]: the streams' row sums
@@ -168,6 +171,9 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
         mbar_init(bar_p + 8, UM_ROWS_THREADS);
         mbar_init(bar_sr, UM_ROWS_THREADS);              // S of a tile is in registers: its buffer may take the next S
         mbar_init(bar_sr + 8, UM_ROWS_THREADS);
+        if (p.nsplit > 1)                                // the partials of the rows this CTA will own: 128 bf16 and {max, sum} each
+            mbar_expect_tx(bar_r, (unsigned int)(p.nsplit * (((split + 1) * ATT_BM + p.nsplit - 1) / p.nsplit - (split * ATT_BM + p.nsplit - 1) / p.nsplit) *
+                                                 (HS_HEAD_DIM * 2 + 8)));
         mbar_init_fence();
         if (p.prefetch)                                  // the caller vouches for the cache: tiles requested ahead of the wait
             for (int i = 0; i < pre; ++i) { issue_kv(i, false); issue_kv(i, true); }
@@ -177,7 +183,13 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
         tmem_relinquish();
     }
     pdl_launch_dependents();
+    // First half of a cluster barrier: when it completes every CTA of the cluster runs with its barriers initialised, and its
+    // shared memory may be written from outside.
+    if (p.nsplit > 1) cluster_arrive();
     pdl_wait();                                      // the pruned tree, q, k_tree, v_tree come from upstream
+    // the sequence's entries of the pruned tree in one round trip
+    const int nk_b = p.n_keep[b], st_b = p.status[b], koff = p.keep_off[b];
+    const int nbase = p.layout == HS_ROWS_ORIGINAL ? p.node_off[b] : 0;
     if (tid == 0 && !p.prefetch)
         for (int i = 0; i < pre; ++i) { issue_kv(i, false); issue_kv(i, true); }
     tc_fence_before_sync();
@@ -188,7 +200,7 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
     const int row = tid & (ATT_BM - 1), half = (tid >> 7) & 1;               // the thread's query row and stream
     const unsigned int tS = tmem_base, tO = tmem_base + 128, tP = tmem_base + 384;   // (+ 64 / + 128 / + 32 columns for stream 1)
 
-    const int nk = (p.status[b] == 0) ? p.n_keep[b] : 0;
+    const int nk = st_b == 0 ? nk_b : 0;
     const int M = nk * p.G;
     if (m0 >= M) {                                   // nothing to do (the same for every CTA of the cluster)
         if (tid == 0)
@@ -198,9 +210,11 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
             }
         __syncthreads();
         if (warp == 0) tmem_dealloc(tmem_base, UM_TMEM_COLS);
+        if (p.nsplit > 1) cluster_wait();
         return;
     }
-    const int koff = p.keep_off[b];
+    // row of q / k_tree / v_tree of kept node `node` (times heads)
+    auto kept_row_of = [&](int node) { return p.layout == HS_ROWS_ORIGINAL ? nbase + p.keep_idx[koff + node] : koff + node; };
     const int nt_tree = (split == p.nsplit - 1) ? (nk + ATT_BN - 1) / ATT_BN : 0;
     const int ntiles = np + nt_tree;
 
@@ -216,7 +230,7 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
         for (int it = 0; it < 4; ++it) {
             const int j = j0 + ((t + (it0 + it) * nthr) >> 4);
             trow[it] = -1;
-            if (j < nk) trow[it] = (p.layout == HS_ROWS_ORIGINAL) ? p.node_off[b] + p.keep_idx[koff + j] : koff + j;
+            if (j < nk) trow[it] = kept_row_of(j);
         }
 #pragma unroll
         for (int it = 0; it < 4; ++it) {
@@ -236,28 +250,32 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
         }
     };
 
-    // ---- this thread's query row -> shared memory, its ancestor mask and output row ---------------------------
+    // ---- query rows -> shared memory: 16 lanes per row (a thread fetching a row of its own touched 32 cache lines with
+    // every load: 1 us of 2.3 us ahead of the first product) ------------------------------------------------------------
+    if (warp < 8) {
+        int qrow[8];
+        uint4 qv[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int r = m0 + (tid >> 4) + 16 * i, node = (int)((unsigned int)r * p.inv_g >> 16);
+            qrow[i] = r < M ? kept_row_of(node) * p.hq + h * p.G + (r - node * p.G) : -1;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            qv[i] = qrow[i] >= 0 ? __ldg(reinterpret_cast<const uint4*>(p.q + (size_t)qrow[i] * HS_HEAD_DIM) + (tid & 15))
+                                 : make_uint4(0, 0, 0, 0);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) *reinterpret_cast<uint4*>(gQ + q_off((tid >> 4) + 16 * i, tid & 15)) = qv[i];
+    }
+    // this thread's own row: its ancestor mask and output row
     const int r = m0 + row;
     long long orow = -1;
     unsigned long long mk0 = 0ull, mk1 = 0ull;
-    {
-        uint4 qv[8];                                     // this thread's half of the row
-#pragma unroll
-        for (int c = 0; c < 8; ++c) qv[c] = make_uint4(0, 0, 0, 0);
-        if (r < M && warp < 8) {
-            const int node = r / p.G, g = r - node * p.G;
-            const int trow = (p.layout == HS_ROWS_ORIGINAL) ? p.node_off[b] + p.keep_idx[koff + node] : koff + node;
-            orow = (long long)trow * p.hq + h * p.G + g;
-            mk0 = p.anc_mask[2 * (size_t)(koff + node)];
-            mk1 = p.anc_mask[2 * (size_t)(koff + node) + 1];
-            const uint4* src = reinterpret_cast<const uint4*>(p.q + (size_t)orow * HS_HEAD_DIM) + half * 8;
-#pragma unroll
-            for (int c = 0; c < 8; ++c) qv[c] = __ldg(src + c);
-        }
-        if (warp < 8) {
-#pragma unroll
-            for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(gQ + q_off(row, half * 8 + c)) = qv[c];
-        }
+    if (r < M && warp < 8) {
+        const int node = (int)((unsigned int)r * p.inv_g >> 16);
+        orow = (long long)kept_row_of(node) * p.hq + h * p.G + (r - node * p.G);
+        mk0 = p.anc_mask[2 * (size_t)(koff + node)];
+        mk1 = p.anc_mask[2 * (size_t)(koff + node) + 1];
     }
     if (warp < 8)
         for (int i = np; i < min(ntiles, UM_STAGES); ++i) gather_tree(i, tid, UM_SM_THREADS, 0, true, true);  // tree tiles that open the pipeline
@@ -497,81 +515,77 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
         for (int ch = 0; ch < 2 && warp < 8; ++ch) {
             unsigned int ov[32];
             load_o(ch, ov);
-            if (orow >= 0) {
-                uint4* dst = reinterpret_cast<uint4*>(p.out + (size_t)orow * HS_HEAD_DIM + half * 64 + ch * 32);
+            uint4 o[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    uint4 pk;
-                    pk.x = pack_bf16(__uint_as_float(ov[q * 8 + 0]) * inv, __uint_as_float(ov[q * 8 + 1]) * inv);
-                    pk.y = pack_bf16(__uint_as_float(ov[q * 8 + 2]) * inv, __uint_as_float(ov[q * 8 + 3]) * inv);
-                    pk.z = pack_bf16(__uint_as_float(ov[q * 8 + 4]) * inv, __uint_as_float(ov[q * 8 + 5]) * inv);
-                    pk.w = pack_bf16(__uint_as_float(ov[q * 8 + 6]) * inv, __uint_as_float(ov[q * 8 + 7]) * inv);
-                    dst[q] = pk;
-                }
+            for (int q = 0; q < 4; ++q) {
+                o[q].x = pack_bf16(__uint_as_float(ov[q * 8 + 0]) * inv, __uint_as_float(ov[q * 8 + 1]) * inv);
+                o[q].y = pack_bf16(__uint_as_float(ov[q * 8 + 2]) * inv, __uint_as_float(ov[q * 8 + 3]) * inv);
+                o[q].z = pack_bf16(__uint_as_float(ov[q * 8 + 4]) * inv, __uint_as_float(ov[q * 8 + 5]) * inv);
+                o[q].w = pack_bf16(__uint_as_float(ov[q * 8 + 6]) * inv, __uint_as_float(ov[q * 8 + 7]) * inv);
+            }
+            // 4 x 4 transpose over four lanes: lane q then holds chunk q of the four rows, and 64 bytes of a row leave in one
+            // instruction (a lane storing its own row touched 32 cache lines with every instruction)
+            const int lane = tid & 31;
+            auto swap = [&](uint4& a, uint4& b, int m) {                  // a of the upper lane <-> b of the lower one
+                const bool up = (lane & m) != 0;
+                uint4 x = up ? a : b;
+                x.x = __shfl_xor_sync(HS_FULL_MASK, x.x, m); x.y = __shfl_xor_sync(HS_FULL_MASK, x.y, m);
+                x.z = __shfl_xor_sync(HS_FULL_MASK, x.z, m); x.w = __shfl_xor_sync(HS_FULL_MASK, x.w, m);
+                if (up) a = x; else b = x;
+            };
+            swap(o[0], o[1], 1); swap(o[2], o[3], 1);
+            swap(o[0], o[2], 2); swap(o[1], o[3], 2);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int dst = __shfl_sync(HS_FULL_MASK, (int)orow, (lane & ~3) + i);
+                if (dst >= 0)
+                    *(reinterpret_cast<uint4*>(p.out + (size_t)dst * HS_HEAD_DIM + half * 64 + ch * 32) + (lane & 3)) = o[i];
             }
         }
         if (orow >= 0 && p.lse_out && half == 0) p.lse_out[orow] = (mrun + log2f(lrun)) * LN2;
     } else {
         // ---- merge across the splits of the cluster through distributed shared memory ----------------------------
-        // Row rl of the block is merged by CTA owner(rl) = rl * ns / 128.  Every CTA stages its partial of every row,
-        // {O / l as bf16, max, sum}, in its own shared memory and one thread PUSHES each owner's rows with a bulk
-        // copy that signals the owner's mbarrier; an owner merges once all ns pieces have landed: per row the
+        // Row rl of the block is merged by CTA owner(rl) = rl * ns / 128.  Every thread sends its part of its row, {O / l as
+        // bf16, max, sum}, straight from registers into the owner's receive area (which no tile ever uses) by asynchronous
+        // remote stores that signal the owner's mbarrier; an owner merges once all ns pieces have landed: per row the
         // splits' weights 2^(max_s - max) l_s / sum once, then out = sum_s weight_s (O_s / l_s).  (A normalised
         // partial is a convex combination of V rows, so bf16 keeps it to 2^-9 of the values' magnitude: the output
-        // is bf16 anyway.)
+        // is bf16 anyway.)  A sender may leave at once: nothing reads its shared memory.  (Staging the rows, a cluster
+        // barrier and bulk copies cost 1.5 us more.)
         const int ns = p.nsplit;
-        // shared memory after the tile loop: [0, UM_RECV_BYTES) partials received from the cluster (others write
-        // here, so only after every CTA of the cluster has left its loop), then this CTA's own staged partial
-        unsigned char* po = smem_gen;                                                // [ns][rows_max] rows of ATT_PB_STRIDE bytes
-        unsigned char* stage_po = smem_gen + UM_RECV_BYTES;                          // [128] rows: own partial
-        const unsigned int s_recv = smem_base, s_stage = smem_base + UM_RECV_BYTES;
+        unsigned char* po = gR;                                                      // [ns][rows_max] rows of ATT_PB_STRIDE bytes
+        const unsigned int s_recv = smem_u32(gR);
         const int rows_max = (ATT_BM + ns - 1) / ns + 1;
         const int r_lo = (split * ATT_BM + ns - 1) / ns, r_hi = ((split + 1) * ATT_BM + ns - 1) / ns;   // rows this CTA owns
         long long* s_og = reinterpret_cast<long long*>(gM);               // output row of each owned row (or -1)
-        float* s_wt = reinterpret_cast<float*>(gM + UM_MAP_BYTES + 1024);  // [rows owned][ATT_MAX_SPLIT] weights (s_mx / s_lx are done)
-        if (tid == 0) mbar_expect_tx(bar_r, (unsigned int)(ns * (r_hi - r_lo) * ATT_PB_STRIDE));
-        if (tid < r_hi - r_lo) {
-            const int rg = m0 + r_lo + tid;
-            long long og = -1;
-            if (rg < M) {
-                const int node = rg / p.G, g = rg - node * p.G;
-                const int trow = (p.layout == HS_ROWS_ORIGINAL) ? p.node_off[b] + p.keep_idx[koff + node] : koff + node;
-                og = (long long)trow * p.hq + h * p.G + g;
-            }
-            s_og[tid] = og;
-        }
-        {
+        float* s_wt = reinterpret_cast<float*>(gM + UM_MAP_BYTES + 1024 + 2048);  // [rows owned][ATT_MAX_SPLIT] weights
+        cluster_wait();                                      // (the arrival at the start, long complete)
+        if (warp < 8) {
+            const int owner = row * ns / ATT_BM, o_lo = (owner * ATT_BM + ns - 1) / ns;
+            const unsigned int dst = cluster_map_addr(s_recv + (unsigned int)(split * rows_max + row - o_lo) * ATT_PB_STRIDE, owner);
+            const unsigned int rbar = cluster_map_addr(bar_r, owner);
+            if (half == 0) st_async_v2(dst + HS_HEAD_DIM * 2, __float_as_uint(mrun), __float_as_uint(lrun), rbar);
             const float inv = lrun > 0.f ? 1.f / lrun : 0.f;
 #pragma unroll 1
-            for (int ch = 0; ch < 2 && warp < 8; ++ch) {
+            for (int ch = 0; ch < 2; ++ch) {
                 unsigned int ov[32];
                 load_o(ch, ov);
-                uint4* dst = reinterpret_cast<uint4*>(stage_po + row * ATT_PB_STRIDE + (half * 64 + ch * 32) * 2);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    uint4 pk;
-                    pk.x = pack_bf16(__uint_as_float(ov[q * 8 + 0]) * inv, __uint_as_float(ov[q * 8 + 1]) * inv);
-                    pk.y = pack_bf16(__uint_as_float(ov[q * 8 + 2]) * inv, __uint_as_float(ov[q * 8 + 3]) * inv);
-                    pk.z = pack_bf16(__uint_as_float(ov[q * 8 + 4]) * inv, __uint_as_float(ov[q * 8 + 5]) * inv);
-                    pk.w = pack_bf16(__uint_as_float(ov[q * 8 + 6]) * inv, __uint_as_float(ov[q * 8 + 7]) * inv);
-                    dst[q] = pk;
-                }
+                for (int q = 0; q < 4; ++q)
+                    st_async_v4(dst + (half * 64 + ch * 32 + q * 8) * 2,
+                                pack_bf16(__uint_as_float(ov[q * 8 + 0]) * inv, __uint_as_float(ov[q * 8 + 1]) * inv),
+                                pack_bf16(__uint_as_float(ov[q * 8 + 2]) * inv, __uint_as_float(ov[q * 8 + 3]) * inv),
+                                pack_bf16(__uint_as_float(ov[q * 8 + 4]) * inv, __uint_as_float(ov[q * 8 + 5]) * inv),
+                                pack_bf16(__uint_as_float(ov[q * 8 + 6]) * inv, __uint_as_float(ov[q * 8 + 7]) * inv), rbar);
             }
-            if (warp < 4) *reinterpret_cast<float2*>(stage_po + row * ATT_PB_STRIDE + HS_HEAD_DIM * 2) = make_float2(mrun, lrun);
         }
-        fence_proxy_async_smem();                            // staged rows -> visible to the copy engine
-        cluster_arrive();                                    // every CTA of the cluster is done with its tiles:
-        cluster_wait();                                      // its stage buffers may now receive partials
-        if (tid < ns) {                                      // thread o: the rows of owner o
-            const int o = tid;
-            const int o_lo = (o * ATT_BM + ns - 1) / ns, o_hi = ((o + 1) * ATT_BM + ns - 1) / ns;
-            if (o_hi > o_lo)
-                bulk_push(cluster_map_addr(s_recv + (unsigned int)(split * rows_max) * ATT_PB_STRIDE, o),
-                          s_stage + (unsigned int)o_lo * ATT_PB_STRIDE, (unsigned int)(o_hi - o_lo) * ATT_PB_STRIDE,
-                          cluster_map_addr(bar_r, o));
+        int og_mine = -1;
+        if (tid < r_hi - r_lo) {
+            const int rg = m0 + r_lo + tid, node = (int)((unsigned int)rg * p.inv_g >> 16);
+            if (rg < M) og_mine = kept_row_of(node) * p.hq + h * p.G + (rg - node * p.G);
+            s_og[tid] = og_mine;
         }
-        mbar_wait(bar_r, 0u, p.err);                         // all ns pieces of this CTA's rows have landed
-        cluster_arrive();                                    // (a CTA may leave only when every copy has landed everywhere)
+        mbar_wait_cluster(bar_r, 0u, p.err);                         // all ns pieces of this CTA's rows have landed
         // the splits' weights of every owned row, once
         if (tid < r_hi - r_lo) {
             float2 ml[ATT_MAX_SPLIT];
@@ -591,9 +605,9 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
             const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
 #pragma unroll
             for (int s2 = 0; s2 < ATT_MAX_SPLIT; ++s2) s_wt[tid * ATT_MAX_SPLIT + s2] = w[s2] * inv;
-            const long long og = s_og[tid];
-            if (og >= 0 && p.lse_out) p.lse_out[og] = (Mx + log2f(lsum)) * LN2;
+            if (og_mine >= 0 && p.lse_out) p.lse_out[og_mine] = (Mx + log2f(lsum)) * LN2;
         }
+        __syncwarp();
         if (tid < UM_SM_THREADS)                             // the softmax threads: the weights are written
             asm volatile("bar.sync 2, %0;" ::"r"(UM_SM_THREADS) : "memory");
         // items = (row, 16-byte column group of 8); every item combines one group of each split, all from local shared memory
@@ -621,7 +635,6 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
                 *reinterpret_cast<uint4*>(p.out + (size_t)og * HS_HEAD_DIM + c8 * 8) = packed;
             }
         }
-        cluster_wait();
     }
     tc_fence_before_sync();
     __syncthreads();
@@ -715,6 +728,7 @@ hs_status hs_launch_attention(hs_ctx* ctx, const hs_pruned_tree* pruned, const h
     p.hq = d->hq;
     p.hkv = d->hkv;
     p.G = d->hq / d->hkv;
+    p.inv_g = (65536u + p.G - 1) / p.G;
     p.layout = d->layout;
     p.head_first = d->kv_head_stride > d->kv_token_stride;
     p.scale_log2 = d->sm_scale * LOG2E;
