@@ -25,8 +25,8 @@ extern "C" const char* hs_status_string(hs_status s) {
 extern "C" size_t hs_workspace_bytes(int32_t max_batch, int32_t max_rows, int32_t vocab, int32_t hq, int32_t hkv) {
     if (max_batch < 1 || max_rows < 1 || vocab < 1 || hq < 1 || hkv < 1) return 0;
     size_t chunks = hs_row_chunks(vocab, HS_F32);
-    // entropy pass: two partials per CTA, at most one CTA per SM (room for 1024)
-    size_t quant = (size_t)2 * 1024 * HS_ROW_PARTIAL_BYTES + 256;
+    // entropy pass: two partials per warp, sixteen warps per SM (room for 152 SMs; with less the shares get longer)
+    size_t quant = (size_t)2 * 152 * 16 * HS_ROW_PARTIAL_BYTES + 512;
     // acceptance: three per-row result arrays (256-byte aligned each) + chunk partials of target and draft rows
     size_t accept = 3 * hs_align_up((size_t)max_rows * 8, 256) +
                     (size_t)2 * max_rows * chunks * HS_ACC_PARTIAL_BYTES;
@@ -74,6 +74,7 @@ extern "C" hs_status hs_create(hs_ctx** out, int32_t device, size_t workspace_by
     c->attn_ready = false;
     c->walk_ready = false;
     c->quant_ready = false;
+    c->warps_ready = false;
     c->cart_ready = false;
     c->rows_ready = false;
     if (cudaDeviceSynchronize() != cudaSuccess) { cudaFree(p); delete c; return HS_ERR_CUDA; }

@@ -33,6 +33,7 @@ struct hs_ctx {
     bool walk_ready;    // acceptance walk kernel attributes set on this device
     bool rows_ready;    // streaming acceptance row pass: shared-memory attribute set on this device
     bool cart_ready;    // single-CTA stratifier training: shared-memory attribute set on this device
+    bool warps_ready;   // warp kernel of the entropy pass: shared-memory attribute set on this device
     bool quant_ready;   // streaming entropy kernel: shared-memory attribute set on this device
 };
 
@@ -122,6 +123,13 @@ __device__ __forceinline__ int key_index(unsigned long long k) { return (int)(~(
 // bf16 pair (packed in 32 bits) -> two floats, exact
 __device__ __forceinline__ float bf16_lo(unsigned int p) { return __uint_as_float(p << 16); }
 __device__ __forceinline__ float bf16_hi(unsigned int p) { return __uint_as_float(p & 0xffff0000u); }
+
+// 16 bytes that are read once: past L1
+__device__ __forceinline__ uint4 ld_stream(const uint4* p) {
+    uint4 v;
+    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
 
 // loads that bypass L1 (values written by other CTAs of the same launch)
 __device__ __forceinline__ float ld_cg_f(const float* p) { return __ldcg(p); }

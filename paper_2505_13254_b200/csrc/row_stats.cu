@@ -1,19 +1,13 @@
 // hs_entropy_quantify: two launches.
 //
-// quantify_stream_kernel   The logits matrix is one long stream of 16-byte vectors (row after row) that is cut
-//     into equal contiguous shares, one per CTA, one CTA per SM.  A producer warp brings the share on chip in
-//     items of up to 32 KiB (bulk copies into a ring of shared-memory slots, completion on mbarriers); sixteen
-//     consumer warps reduce each item in ONE pass: running maximum per thread (packed bf16 maxima), then
-//     sum e^(x-m) and sum x e^(x-m) with the exponent's multiply-add and the two sums as packed fp32 pairs.
-//     Top-K without sorting: after the first items of a row share a warp takes a lower bound of the K-th
-//     largest logit of the row share from maxima of disjoint element sets (the 32 half-warp maxima of the
-//     CTA, or its own 32 lane maxima on a short share), and only lanes whose window maximum reaches the bound
-//     re-scan their vectors in shared memory and push candidates; the few candidates are ranked by counting.
-//     A share that ends inside a row leaves a partial {max, sum, sum x e, K keys}; the last CTA of a row to
-//     arrive merges the partials into max, log-sum-exp, Shannon entropy, Top-K and the two Top-K entropies
-//     (Eq. 1 inner sum).  Rows that lie inside one share need no partial and no atomic.  With few rows every row
-//     is cut into the same number of shares, which form a thread-block cluster: the partials then go into the
-//     shared memory of the cluster's first CTA instead of through global memory.
+// quantify_cluster_kernel  Few rows (at most half as many as SMs): a row is cut into parts, one CTA each, that merge as a
+//     thread-block cluster.
+// quantify_warp_kernel     Many rows (row_warps.cuh): every warp of the device takes an equal share of the matrix on its own.
+//     Both fold four 16-byte vectors per lane at a time: packed maximum, then sum e^(x-ref) and sum x e^(x-ref) with the
+//     exponent's multiply-add and the two sums as packed fp32 pairs.  Top-K without sorting: maxima of disjoint sets (lanes,
+//     half-warps) are distinct logits, so the K-th largest of 32 of them bounds the K-th largest logit of a part; the few
+//     cells that reach the bound are read again and their logits ranked.  The parts of a row merge into max, log-sum-exp,
+//     Shannon entropy, Top-K and the two Top-K entropies (Eq. 1 inner sum).
 // tree_scores_kernel       One CTA per sequence: path confidence ln V_i (Sec. 2.2), cumulative meta-path
 //     Top-K entropy Phi (Eq. 1) and the operational path P* (Sec. 4.1).  (The fused call launches the kernel
 //     of stratify_prune.cu that runs the same tree stage and then prunes, in its place.)
@@ -21,7 +15,11 @@
 // quantify_chunk_kernel (a CTA owns one chunk of one row, registers only) serves the allocation-free entry.
 #include <math_constants.h>
 
+#include <algorithm>
 #include <mutex>
+
+using std::max;
+using std::min;
 
 #include "hs_common.cuh"
 #include "hs_layout.h"
@@ -31,13 +29,9 @@
 #define CAND_CAP 512
 #define LOG2E 1.4426950408889634f
 
-#define QS_CONSUMERS 512                      // sixteen consumer warps
-#define QS_THREADS (QS_CONSUMERS + 32)        // + the producer warp
-#define QS_ITEM_VECS 2048                     // vectors per item: 32 KiB, four per consumer thread
-#define QS_VPT (QS_ITEM_VECS / QS_CONSUMERS)
-#define QS_SLOTS 6                            // ring of item slots
-#define QS_WINDOW 4                           // items a consumer holds before it hands their slots back
-#define QS_MAX_SEGS 32                        // shares a row may be split over
+#define QS_THREADS 512                        // cluster kernel: sixteen warps
+#define QS_ITEM_VECS 2048                     // vectors per item: 32 KiB, four per thread
+#define QS_SLOTS 6                            // items a CTA has room for
 #define QS_SMEM_BYTES (QS_SLOTS * QS_ITEM_VECS * 16 + 128)
 
 struct QuantParams {
@@ -47,11 +41,9 @@ struct QuantParams {
     int nvec;        // 16-byte vectors per row, the last one may be partial
     int chunks;      // chunk kernel: CTAs per row
     int chunk_vecs;  // chunk kernel: vectors per chunk
-    int per;         // stream kernel: vectors per share
-    int split;       // stream kernel: shares per row (row-split geometry), 0 = byte-balanced stream
-    int extra;       // stream kernel, row split: the first `extra` rows have one share more
-    int nslots;      // stream kernel: item slots in shared memory
-    int clustered;   // stream kernel, row split: the shares of a row are one thread-block cluster and merge in shared memory
+    int per;         // cluster kernel: vectors per part; warp kernel: places of the stream per share
+    int split;       // cluster kernel: parts per row = cluster size
+    int extra;       // warp kernel: places ahead of every row
     int rows;
     int batch;
     const int* node_off;
@@ -151,15 +143,15 @@ __device__ __noinline__ void topk_by_rounds(const char* rowp, int v0, int v1, in
     }
 }
 
-// One warp: the statistics of a whole row from its {max, sum e^(x-max), sum x e^(x-max)} and its K best keys
-// (s_top, 0 = none): log-sum-exp, Shannon entropy, Top-K values and token ids, the entropy of the renormalised
+// One warp: the statistics of a whole row from its maximum M, {sum e^(x-R), sum x e^(x-R)} and its K best keys (`key`:
+// lane i has the i-th, 0 = none): log-sum-exp, Shannon entropy, Top-K values and token ids, the entropy of the renormalised
 // Top-K probabilities (Eq. 1 inner sum) and the truncated variant.
-__device__ __forceinline__ void finalize_row(const QuantParams& p, int row, float M, float S, float U,
-                                             const unsigned long long* s_top, int lane) {
+__device__ __forceinline__ void finalize_row(const QuantParams& p, int row, float M, float R, float S, float U,
+                                             unsigned long long key, int lane) {
     const int K = p.K;
-    const float lse = M + logf(S);
+    const float lse = R + logf(S);
     const float H = lse - U / S;
-    const unsigned long long key = (lane < K) ? s_top[lane] : 0ull;
+    if (lane >= K) key = 0ull;
     const bool valid = key != 0ull;
     const float tv = valid ? key_value(key) : 0.f;
     const float t0 = __shfl_sync(HS_FULL_MASK, tv, 0);
@@ -194,448 +186,197 @@ __device__ __forceinline__ float warp_kth_largest(float v, int K, int lane) {
     return mx ? order_bits_float(mx) : -CUDART_INF_F;
 }
 
-// ================================================================================================================
-// The streaming kernel
-// ================================================================================================================
-// Geometry of the shares.  split == 0 ("stream"): the rows form one stream of rows * nvec vectors, share c is
-// [c * per, (c + 1) * per), a share may hold several rows and a row may lie in several shares.  split == S > 0 ("row
-// split", for launches with at most one row per SM): the first `extra` rows are cut into S + 1 equal parts, the
-// others into S, one share per part, so that every share is a single row segment.  split < 0 ("whole rows", for
-// launches with many rows per SM): share c of `extra` shares holds the rows [c * rows / extra, (c + 1) * rows / extra).
-struct Share {
-    long long g0, g1;
-};
-__device__ __forceinline__ void shares_of_row(const QuantParams& p, int row, int& c_first, int& nseg) {
-    if (p.split < 0) {
-        c_first = 0; nseg = 1;
-    } else if (p.split) {
-        if (row < p.extra) { c_first = row * (p.split + 1); nseg = p.split + 1; }
-        else { c_first = p.extra * (p.split + 1) + (row - p.extra) * p.split; nseg = p.split; }
-    } else {
-        const long long r0 = (long long)row * p.nvec;
-        c_first = (int)(r0 / p.per);
-        nseg = (int)((r0 + p.nvec - 1) / p.per) - c_first + 1;
-    }
-}
-__device__ __forceinline__ Share share_of(const QuantParams& p, int c) {
-    Share sh;
-    if (p.split < 0) {
-        sh.g0 = ((long long)c * p.rows / p.extra) * p.nvec;
-        sh.g1 = ((long long)(c + 1) * p.rows / p.extra) * p.nvec;
-    } else if (p.split) {
-        const int wide = p.extra * (p.split + 1);           // shares of the rows with S + 1 parts
-        const int parts = c < wide ? p.split + 1 : p.split;
-        const int row = c < wide ? c / parts : p.extra + (c - wide) / parts;
-        const int part = c < wide ? c - row * parts : (c - wide) - (row - p.extra) * parts;
-        const int pv = (p.nvec + parts - 1) / parts;
-        sh.g0 = (long long)row * p.nvec + min(part * pv, p.nvec);
-        sh.g1 = (long long)row * p.nvec + min((part + 1) * pv, p.nvec);
-    } else {
-        sh.g0 = (long long)c * p.per;
-        sh.g1 = min(sh.g0 + (long long)p.per, (long long)p.rows * p.nvec);
-    }
-    return sh;
-}
-// partial slot of share c for `row`: stream mode has two per share (the leading one for a row that began in an
-// earlier share), row-split mode one
-__device__ __forceinline__ int partial_slot(const QuantParams& p, int row, int c) {
-    if (p.split) return c;
-    return 2 * c + ((long long)row * p.nvec < (long long)c * p.per ? 0 : 1);
-}
+#include "row_warps.cuh"
 
-// 72 registers per thread (no spills): the 17 warps then leave room in the register file for a CTA of the kernel
-// ahead that is still at work on the same SM (in a decode loop: the CTA that walks the accepted path of the step
-// before), so this kernel's CTA is resident, and its share on chip, before that kernel has ended.
+// ================================================================================================================
+// The cluster kernel: few rows (at most half as many as SMs)
+// ================================================================================================================
+// Every row is cut into the same number of parts (at most eight, the portable cluster size), one CTA of 16 warps per part;
+// the CTAs of a row are one thread-block cluster.  A part is at most QS_SLOTS items of 32 KiB, all of which are requested
+// at once by bulk copies into shared memory of their own (with prefetch ahead of the dependency wait), so the pass is a chain
+// of latencies, not a stream: items as they land, one bound for the Top-K of the part from the CTA's 32 half-warp maxima, the
+// few cells that reach it read again from shared memory, ranked by counting, and the parts merged in the shared memory of
+// the row's first CTA (asynchronous remote stores; the other CTAs leave at once).
+// 72 registers per thread: the CTA then fits into the register file beside a CTA of the kernel ahead that is still at work on
+// the same SM (in a decode loop: the CTA that walks the accepted path of the step before).
 template <bool BF16>
-__global__ void __maxnreg__(72) quantify_stream_kernel(const QuantParams p) {
+__global__ void __maxnreg__(72) quantify_cluster_kernel(const __grid_constant__ QuantParams p) {
     constexpr int VE = BF16 ? 8 : 4;
-    constexpr int NW = QS_CONSUMERS / 32;
+    constexpr int NW = QS_THREADS / 32;
     extern __shared__ __align__(128) unsigned char s_dyn[];
-    __shared__ unsigned long long s_full[QS_SLOTS], s_empty[QS_SLOTS];
+    __shared__ unsigned long long s_full[QS_SLOTS], s_merge;
     __shared__ unsigned long long s_list[CAND_CAP];
-    __shared__ unsigned long long s_top[2][HS_MAX_TOPK];   // (two copies: a finished row is written out by warp 0
-    __shared__ unsigned long long s_red[NW];               //  while the other warps read the next one)
+    __shared__ unsigned long long s_top[HS_MAX_TOPK], s_red[NW];
     __shared__ __align__(16) float s_gm[32];
-    __shared__ __align__(16) float s_lm[NW][32];
-    __shared__ float s_wstat[2][NW][3];
+    __shared__ float4 s_wstat[NW];                               // {ref, sum e, sum x e, max} per warp
     __shared__ int s_cnt;
-    __shared__ int s_flag;
-    __shared__ unsigned long long s_ck[8][HS_MAX_TOPK];   // clustered launch, first CTA of a row: the shares' Top-K keys
-    __shared__ __align__(16) float4 s_cs[8];               //   and their {max, sum e, sum x e}
+    __shared__ __align__(16) unsigned long long s_ck[8][HS_MAX_TOPK];   // first CTA of a row: the parts' Top-K keys
+    __shared__ __align__(16) float4 s_cs[8];                            //   and their {ref, sum e, sum x e, max}
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int parts = p.split, row = blockIdx.x / parts, part = blockIdx.x - row * parts;
+    const int sv0 = min(part * p.per, p.nvec), sv1 = min(sv0 + p.per, p.nvec);
+    const int nit = (sv1 - sv0 + QS_ITEM_VECS - 1) / QS_ITEM_VECS;
+    const char* rowp = (const char*)p.logits + (size_t)row * p.row_stride * (BF16 ? 2 : 4);
     const unsigned int slots0 = (smem_u32(s_dyn) + 127u) & ~127u;
-    const unsigned char* slots_gen = s_dyn + (slots0 - smem_u32(s_dyn));
-    const Share sh = share_of(p, blockIdx.x);
-    const long long g0 = sh.g0, g1 = sh.g1;
-    const size_t esz = BF16 ? 2 : 4;
-    const int nslots = p.nslots;
+    const uint4* slots = reinterpret_cast<const uint4*>(s_dyn + (slots0 - smem_u32(s_dyn)));
+    const int K = p.K;
 
     if (tid == 0) {
-        for (int s = 0; s < nslots; ++s) {
-            mbar_init(smem_u32(&s_full[s]), 1);
-            mbar_init(smem_u32(&s_empty[s]), NW);
-        }
+        for (int s = 0; s < nit; ++s) mbar_init(smem_u32(&s_full[s]), 1);
+        mbar_init(smem_u32(&s_merge), 1);
+        if (part == 0 && parts > 1) mbar_expect_tx(smem_u32(&s_merge), (unsigned int)(parts - 1) * (16u + HS_MAX_TOPK * 8u));
         mbar_init_fence();
         s_cnt = 0;
     }
-    __syncthreads();
     // The tree stage behind this kernel may start once every CTA has passed this point.  Without prefetch that is behind
     // the dependency wait, so whatever was written ahead of the call is complete by then and the tree stage may read its
     // inputs (not this kernel's results) without waiting.
     if (!p.prefetch) pdl_wait();
     pdl_launch_dependents();
-    // Clustered launch: first half of a cluster barrier - when it completes every CTA of the row's cluster runs and
-    // its shared memory may be written from outside.  Every thread of the CTA, the producer warp included, takes part
-    // in the two barrier phases of the launch.
-    if (p.clustered) cluster_arrive();
-
-    if (warp == NW) {
-        // ---- producer: one lane walks the share item by item ----------------------------------------------------
-        if (lane == 0) {
-            long long g = g0;
-            int it = 0, slot = 0;
-            unsigned int epar = 1u;          // parity of the slot's `empty` barrier before its first completion
-            bool waited = !p.prefetch;
-            while (g < g1) {
-                const int row = (int)(g / p.nvec);
-                const int v = (int)(g - (long long)row * p.nvec);
-                const int len = (int)min((long long)min(QS_ITEM_VECS, p.nvec - v), g1 - g);
-                if (it >= nslots) {
-                    if (!waited) { pdl_wait(); waited = true; }     // (nothing of this kernel is written by the producer)
-                    mbar_wait(smem_u32(&s_empty[slot]), epar, p.err);
-                }
-                const unsigned int bar = smem_u32(&s_full[slot]);
-                mbar_expect_tx(bar, (unsigned int)len * 16u);
-                bulk_load(slots0 + (unsigned int)slot * (QS_ITEM_VECS * 16),
-                          (const char*)p.logits + (size_t)row * p.row_stride * esz + (size_t)v * 16, (unsigned int)len * 16u, bar);
-                g += len;
-                ++it;
-                if (++slot == nslots) { slot = 0; epar ^= 1u; }
-            }
+    if (tid == 0)
+        for (int s = 0; s < nit; ++s) {
+            const int len = min(QS_ITEM_VECS, sv1 - sv0 - s * QS_ITEM_VECS);
+            mbar_expect_tx(smem_u32(&s_full[s]), (unsigned int)len * 16u);
+            bulk_load(slots0 + (unsigned int)s * (QS_ITEM_VECS * 16), rowp + (size_t)(sv0 + s * QS_ITEM_VECS) * 16,
+                      (unsigned int)len * 16u, smem_u32(&s_full[s]));
         }
-        if (p.clustered) {
-            __syncwarp();
-            cluster_wait();
-            cluster_arrive();
-            cluster_wait();
-        }
-        return;
-    }
+    if (tid < HS_MAX_TOPK) s_top[tid] = 0ull;
+    __syncthreads();
+    // First half of a cluster barrier: when it completes every CTA of the cluster runs with its barrier initialised, and its
+    // shared memory may be written from outside.
+    if (parts > 1) cluster_arrive();
 
-    // ---- consumers -------------------------------------------------------------------------------------------------
-    // Partials, counters and outputs may still be in use by the kernel ahead: nothing is written before the wait.
-    // Reading the logits and reducing them in registers and shared memory needs no wait if the caller vouches that
-    // they were complete before the call (prefetch): then the wait comes at the end of the first segment.
-    bool waited = !p.prefetch;
-    const int K = p.K;
+    // ---- the part's items -------------------------------------------------------------------------------------------
     const unsigned int ninf = BF16 ? 0xff80ff80u : 0xff800000u;
-    int cslot = 0;                 // slot of the next item and the parity of its `full` barrier (the producer fills
-    unsigned int cpar = 0u;        // the slots round-robin in the same order)
-    int seg = 0;                   // segments of this share finished so far (parity selects the s_top / s_wstat copy)
-    long long g = g0;
-
-    // One item: waits for its slot, keeps the maxima of the thread's QS_VPT vectors in vm[], folds the item into the
-    // thread's running (max, sum e^(x-max), sum x e^(x-max)).
-    auto consume_item = [&](int slot, int v_item, int len, float* vm, float& m_t, float2& s2, float2& u2) {
-        mbar_wait(smem_u32(&s_full[slot]), cpar, p.err);
-        if (++cslot == nslots) { cslot = 0; cpar ^= 1u; }
-        const uint4* st = reinterpret_cast<const uint4*>(slots_gen + (size_t)slot * (QS_ITEM_VECS * 16));
-        uint4 d[QS_VPT];
-        float imax = -CUDART_INF_F;
-        if (len == QS_ITEM_VECS) {                                           // (the usual case: no lane is idle)
+    float ref = -CUDART_INF_F, nref = 0.f, lm = -CUDART_INF_F;
+    float2 s2 = make_float2(0.f, 0.f), u2 = make_float2(0.f, 0.f);
+    float cm[QS_SLOTS];                                          // this lane's maximum of each item
 #pragma unroll
-            for (int j = 0; j < QS_VPT; ++j) d[j] = st[tid + j * QS_CONSUMERS];
-        } else {
+    for (int it = 0; it < QS_SLOTS; ++it) {
+        cm[it] = -CUDART_INF_F;
+        if (it < nit) {
+            const int len = min(QS_ITEM_VECS, sv1 - sv0 - it * QS_ITEM_VECS);
+            mbar_wait(smem_u32(&s_full[it]), 0u, p.err);
+            __syncwarp();
+            const uint4* st = slots + it * QS_ITEM_VECS;
+            uint4 d[4];
+            if (len == QS_ITEM_VECS) {
 #pragma unroll
-            for (int j = 0; j < QS_VPT; ++j) {
-                const int vl = tid + j * QS_CONSUMERS;
-                d[j] = (vl < len) ? st[vl] : make_uint4(ninf, ninf, ninf, ninf);
-            }
-        }
-        if (v_item + len == p.nvec && p.nvec * VE != p.vocab) {               // the row's last vector runs past vocab
-#pragma unroll
-            for (int j = 0; j < QS_VPT; ++j) {
-                if (v_item + tid + j * QS_CONSUMERS == p.nvec - 1) {
-                    unsigned int* wd = reinterpret_cast<unsigned int*>(&d[j]);
-#pragma unroll
-                    for (int e = 0; e < VE; ++e)
-                        if ((p.nvec - 1) * VE + e >= p.vocab) {
-                            if (BF16) wd[e >> 1] = (e & 1) ? ((wd[e >> 1] & 0x0000ffffu) | 0xff800000u)
-                                                           : ((wd[e >> 1] & 0xffff0000u) | 0x0000ff80u);
-                            else wd[e] = 0xff800000u;
-                        }
-                }
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < QS_VPT; ++j) {
-            if (BF16) {
-                const __nv_bfloat162 a = __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&d[j].x),
-                                                *reinterpret_cast<const __nv_bfloat162*>(&d[j].y));
-                const __nv_bfloat162 b = __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&d[j].z),
-                                                *reinterpret_cast<const __nv_bfloat162*>(&d[j].w));
-                const __nv_bfloat162 c = __hmax2(a, b);
-                const unsigned int cw = *reinterpret_cast<const unsigned int*>(&c);
-                vm[j] = fmaxf(bf16_lo(cw), bf16_hi(cw));
-            } else {
-                vm[j] = fmaxf(fmaxf(__uint_as_float(d[j].x), __uint_as_float(d[j].y)),
-                              fmaxf(__uint_as_float(d[j].z), __uint_as_float(d[j].w)));
-            }
-            imax = fmaxf(imax, vm[j]);
-        }
-        if (imax > m_t) {                         // the thread's maximum grows: rescale its sums
-            const float f = (m_t == -CUDART_INF_F) ? 0.f : ex2f((m_t - imax) * LOG2E);
-            s2.x *= f; s2.y *= f; u2.x *= f; u2.y *= f;
-            m_t = imax;
-        }
-        const float nml = (m_t == -CUDART_INF_F) ? 0.f : -m_t * LOG2E;
-        const float2 l2 = make_float2(LOG2E, LOG2E), n2 = make_float2(nml, nml);
-        const unsigned int floor2 = 0xf149f149u;  // bf16 pair of -1e30: keeps 0 * x finite for x = -inf
-#pragma unroll
-        for (int j = 0; j < QS_VPT; ++j) {
-            const unsigned int* wd = reinterpret_cast<const unsigned int*>(&d[j]);
-            if (BF16) {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const __nv_bfloat162 cl = __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&wd[q]),
-                                                     *reinterpret_cast<const __nv_bfloat162*>(&floor2));
-                    const unsigned int cw = *reinterpret_cast<const unsigned int*>(&cl);
-                    const float2 x = make_float2(bf16_lo(cw), bf16_hi(cw));
-                    const float2 t = fma2_ftz(x, l2, n2);
-                    const float2 e = make_float2(ex2f(t.x), ex2f(t.y));
-                    s2 = add2_ftz(s2, e);
-                    u2 = fma2_ftz(e, x, u2);
-                }
+                for (int j = 0; j < 4; ++j) d[j] = st[tid + j * QS_THREADS];
             } else {
 #pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const float2 x = make_float2(fmaxf(__uint_as_float(wd[2 * q]), -1e30f),
-                                                 fmaxf(__uint_as_float(wd[2 * q + 1]), -1e30f));
-                    const float2 t = fma2_ftz(x, l2, n2);
-                    const float2 e = make_float2(ex2f(t.x), ex2f(t.y));
-                    s2 = add2_ftz(s2, e);
-                    u2 = fma2_ftz(e, x, u2);
+                for (int j = 0; j < 4; ++j) {
+                    const int vl = tid + j * QS_THREADS;
+                    d[j] = vl < len ? st[vl] : make_uint4(ninf, ninf, ninf, ninf);
                 }
             }
-        }
-    };
-    // A lower bound of the segment's K-th largest logit.  Maxima of disjoint element sets are distinct elements, so
-    // the K-th largest of any such family is a bound.  With at least one full item behind the segment: the CTA's 32
-    // half-warp maxima (published in shared memory; an entry another warp has not refreshed yet is an older maximum
-    // of the same segment, still an element of it).  Shorter: this warp's own 32 lane maxima.
-    auto kth_bound = [&](float m_t, bool full_item, bool barrier) -> float {
-        const float4* fam;                                   // the family of 32 maxima, read back as eight float4
-        if (full_item) {
-            float hm = m_t;
-            hm = fmaxf(hm, __shfl_xor_sync(HS_FULL_MASK, hm, 1));
-            hm = fmaxf(hm, __shfl_xor_sync(HS_FULL_MASK, hm, 2));
-            hm = fmaxf(hm, __shfl_xor_sync(HS_FULL_MASK, hm, 4));
-            hm = fmaxf(hm, __shfl_xor_sync(HS_FULL_MASK, hm, 8));
-            if ((lane & 15) == 0) s_gm[warp * 2 + (lane >> 4)] = hm;
-            if (barrier) bar_sync(1, QS_CONSUMERS);          // every warp has published maxima of this segment
-            else __syncwarp();
-            fam = reinterpret_cast<const float4*>(s_gm);
-        } else {
-            s_lm[warp][lane] = m_t;
-            if (barrier) bar_sync(1, QS_CONSUMERS);          // (the same barrier count for every warp)
-            else __syncwarp();
-            fam = reinterpret_cast<const float4*>(s_lm[warp]);
-        }
-        const float w = reinterpret_cast<const float*>(fam)[lane];
-        int ge = 0;                                          // members >= this lane's
+            const int last = p.nvec - 1 - (sv0 + it * QS_ITEM_VECS);          // the row's last vector may run past vocab
+            if (last < len && p.nvec * VE != p.vocab) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const float4 f4 = fam[j];
+                for (int j = 0; j < 4; ++j)
+                    if (tid + j * QS_THREADS == last) mask_tail<BF16>(d[j], p.nvec - 1, p.vocab);
+            }
+            fold_round<BF16>(d, ref, nref, s2, u2, cm[it]);
+            lm = fmaxf(lm, cm[it]);
+        }
+    }
+    // ---- Top-K of the part: bound, candidates -------------------------------------------------------------------------
+    {
+        float hm = lm;
+        hm = fmaxf(hm, __shfl_xor_sync(HS_FULL_MASK, hm, 1));
+        hm = fmaxf(hm, __shfl_xor_sync(HS_FULL_MASK, hm, 2));
+        hm = fmaxf(hm, __shfl_xor_sync(HS_FULL_MASK, hm, 4));
+        hm = fmaxf(hm, __shfl_xor_sync(HS_FULL_MASK, hm, 8));
+        if ((lane & 15) == 0) s_gm[warp * 2 + (lane >> 4)] = hm;
+        const float wm = fmaxf(hm, __shfl_xor_sync(HS_FULL_MASK, hm, 16));
+        const float ws = warp_sum(s2.x + s2.y), wu = warp_sum(u2.x + u2.y);
+        if (lane == 0) s_wstat[warp] = make_float4(ref, ws, wu, wm);
+    }
+    __syncthreads();
+    float tau;
+    {
+        const float w = s_gm[lane];
+        int ge = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float4 f4 = reinterpret_cast<const float4*>(s_gm)[i];
             ge += (f4.x >= w) + (f4.y >= w) + (f4.z >= w) + (f4.w >= w);
         }
-        return warp_max(ge >= K ? w : -CUDART_INF_F);
-    };
-    // Candidates of one item: the warp works through the vectors whose maximum reaches the bound, four at a time
-    // (eight lanes per vector, one element each, read back from the item's slot in shared memory).
-    auto scan_item = [&](int slot, int v_item, const float* vm, float tau) {
-        unsigned int hits = 0u;
+        tau = warp_max(ge >= K ? w : -CUDART_INF_F);             // (maxima of disjoint sets are distinct logits)
+    }
 #pragma unroll
-        for (int j = 0; j < QS_VPT; ++j) hits |= (vm[j] >= tau && vm[j] > -CUDART_INF_F) ? (1u << j) : 0u;
-        unsigned int any = __ballot_sync(HS_FULL_MASK, hits != 0u);
-        while (any) {
-            const int src = __ffs(any) - 1;
-            unsigned int m = __shfl_sync(HS_FULL_MASK, hits, src);
-            any &= any - 1;                                   // (a lane has at most QS_VPT = 4 hit vectors: one round)
-            for (int q = (lane >> 3); q > 0; --q) m &= m - 1; // lanes 8q .. 8q+7 take the q-th hit vector
-            const int e = lane & 7;
-            if (m && e < VE) {
-                const int j = __ffs(m) - 1;
-                const int vl = (warp * 32 + src) + j * QS_CONSUMERS;
-                const unsigned char* vp = slots_gen + (size_t)slot * (QS_ITEM_VECS * 16) + (size_t)vl * 16;
+    for (int it = 0; it < QS_SLOTS; ++it) {
+        unsigned int hits = __ballot_sync(HS_FULL_MASK, cm[it] >= tau && cm[it] > -CUDART_INF_F);
+        for (; hits; hits &= hits - 1) {                         // a cell's four vectors, one element per lane (fp32: 16 lanes)
+            const int vl = warp * 32 + __ffs(hits) - 1 + (BF16 ? lane >> 3 : (lane >> 2) & 3) * QS_THREADS;
+            const int e = BF16 ? lane & 7 : lane & 3;
+            const int v = sv0 + it * QS_ITEM_VECS + vl, idx = v * VE + e;
+            if ((BF16 || lane < 16) && v < sv1 && idx < p.vocab) {
+                const unsigned char* vp = reinterpret_cast<const unsigned char*>(slots + it * QS_ITEM_VECS + vl);
                 const float x = BF16 ? __uint_as_float((unsigned int)reinterpret_cast<const unsigned short*>(vp)[e] << 16)
                                      : reinterpret_cast<const float*>(vp)[e];
-                const int idx = (v_item + vl) * VE + e;
-                if (x >= tau && x > -CUDART_INF_F && idx < p.vocab) {
+                if (x >= tau && x > -CUDART_INF_F) {
                     const int sl = atomicAdd(&s_cnt, 1);
                     if (sl < CAND_CAP) s_list[sl] = make_key(x, idx);
                 }
             }
-        }
-    };
-
-    while (g < g1) {
-        // ---- one segment: the part [g, seg_end) of this share inside row `row` ------------------------------------
-        const int row = (int)(g / p.nvec);
-        const long long row_g0 = (long long)row * p.nvec;
-        const int sv0 = (int)(g - row_g0);
-        const int sv1 = (int)(min(g1, row_g0 + p.nvec) - row_g0);
-        const char* rowp = (const char*)p.logits + (size_t)row * p.row_stride * esz;
-        unsigned long long* top = s_top[seg & 1];
-        float m_t = -CUDART_INF_F;                // running maximum of this thread's logits of the segment
-        float2 s2 = make_float2(0.f, 0.f), u2 = make_float2(0.f, 0.f);
-        float tau;                                // lower bound of the K-th largest logit of the segment
-        int v = sv0;
-        int items_done = 0;
-        {
-            // ---- first window: up to QS_WINDOW items are held, the bound is taken from all of them -----------------
-            float vmx[QS_WINDOW][QS_VPT];
-            int w_slot[QS_WINDOW], w_v0[QS_WINDOW];
-#pragma unroll
-            for (int wi = 0; wi < QS_WINDOW; ++wi) {
-                w_slot[wi] = -1; w_v0[wi] = 0;
-                if (v < sv1) {
-                    const int len = min(QS_ITEM_VECS, sv1 - v);
-                    w_slot[wi] = cslot; w_v0[wi] = v;
-                    consume_item(w_slot[wi], v, len, vmx[wi], m_t, s2, u2);
-                    v += len; ++items_done;
-                }
-            }
-            tau = kth_bound(m_t, v - sv0 >= QS_ITEM_VECS, true);
-#pragma unroll
-            for (int wi = 0; wi < QS_WINDOW; ++wi)
-                if (w_slot[wi] >= 0) scan_item(w_slot[wi], w_v0[wi], vmx[wi], tau);
             __syncwarp();
-            if (lane == 0) {
-#pragma unroll
-                for (int wi = 0; wi < QS_WINDOW; ++wi)
-                    if (w_slot[wi] >= 0) mbar_arrive(smem_u32(&s_empty[w_slot[wi]]));
-            }
         }
-        // ---- the rest of the segment item by item: scanned against the bound and handed back at once; the bound is
-        // refreshed whenever the number of items read reaches a power of two -----------------------------------------
-        while (v < sv1) {
-            float vm[QS_VPT];
-            const int len = min(QS_ITEM_VECS, sv1 - v);
-            const int slot = cslot;
-            consume_item(slot, v, len, vm, m_t, s2, u2);
-            ++items_done;
-            if ((items_done & (items_done - 1)) == 0) tau = fmaxf(tau, kth_bound(m_t, true, false));
-            scan_item(slot, v, vm, tau);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&s_empty[slot]));
-            v += len;
-        }
-        // ---- end of the segment: warp, then CTA reduction of (max, s, u); Top-K of the candidates ------------------
-        {
-            const float wm = warp_max(m_t);
-            const float f = (m_t == -CUDART_INF_F) ? 0.f : ex2f((m_t - wm) * LOG2E);
-            const float ws = warp_sum((s2.x + s2.y) * f), wu = warp_sum((u2.x + u2.y) * f);
-            if (lane == 0) { s_wstat[seg & 1][warp][0] = wm; s_wstat[seg & 1][warp][1] = ws; s_wstat[seg & 1][warp][2] = wu; }
-        }
-        if (tid < HS_MAX_TOPK) top[tid] = 0ull;       // (this copy was last read two segments ago)
-        bar_sync(1, QS_CONSUMERS);                    // all candidates are pushed, all warp sums written
-        const int ncand = s_cnt;
-        if (ncand <= CAND_CAP) rank_select_warps(s_list, ncand, K, top, warp, lane, NW);
-        else topk_by_rounds<BF16>(rowp, sv0, sv1, p.vocab, K, top, s_red, tid, QS_CONSUMERS, 1);   // heavy ties
-        bar_sync(1, QS_CONSUMERS);                    // the Top-K is complete; s_list and s_cnt are free again
-        if (!waited) { pdl_wait(); waited = true; }   // from here on the segment's results go to global memory
-        if (p.clustered) cluster_wait();              // (the arrival at the start: every CTA of the cluster runs)
-        int c_first, nseg;
-        shares_of_row(p, row, c_first, nseg);
-        if (warp == 0) {
-            if (lane == 0) s_cnt = 0;                 // (the next push comes after the next segment's first barrier)
-            // the consumer warps' (max, s, u) in a fixed order
-            const float wm = lane < NW ? s_wstat[seg & 1][lane][0] : -CUDART_INF_F;
-            const float M = warp_max(wm);
-            const float f = (lane >= NW || wm == -CUDART_INF_F) ? 0.f : ex2f((wm - M) * LOG2E);
-            const float S = lane < NW ? s_wstat[seg & 1][lane][1] * f : 0.f, U = lane < NW ? s_wstat[seg & 1][lane][2] * f : 0.f;
-            float St = 0.f, Ut = 0.f;
-#pragma unroll
-            for (int w = 0; w < NW; ++w) {
-                St += __shfl_sync(HS_FULL_MASK, S, w);
-                Ut += __shfl_sync(HS_FULL_MASK, U, w);
-            }
-            if (nseg == 1) {
-                // the whole row lay in this share: the other warps are already on their way to the next segment
-                finalize_row(p, row, M, St, Ut, top, lane);
-            } else if (p.clustered) {
-                // this share's partial goes into slot `part` of the first CTA of the row's cluster (posted stores
-                // through distributed shared memory; the cluster barrier below makes them visible there)
-                const int part = blockIdx.x - c_first;
-                if (lane < HS_MAX_TOPK) {
-                    const unsigned int dst = cluster_map_addr(smem_u32(&s_ck[part][lane]), 0);
-                    asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(dst), "l"((lane < K) ? top[lane] : 0ull) : "memory");
-                }
-                if (lane == 0) {
-                    const unsigned int dst = cluster_map_addr(smem_u32(&s_cs[part]), 0);
-                    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(__float_as_uint(M)),
-                                 "r"(__float_as_uint(St)), "r"(__float_as_uint(Ut)), "r"(0u) : "memory");
-                    s_flag = (part == 0);
-                }
-            } else {
-                const int ps = partial_slot(p, row, blockIdx.x);
-                if (lane == 0) p.part_stats[ps] = make_float4(M, St, Ut, 0.f);
-                if (lane < HS_MAX_TOPK) p.part_keys[(size_t)ps * HS_MAX_TOPK + lane] = (lane < K) ? top[lane] : 0ull;
-                __syncwarp();
-                if (lane == 0) {
-                    // one release-acquire arrival at device scope: the partial written by this warp (ordered before the
-                    // arrival by the warp barrier above) is visible to whoever arrives last, and the last one sees all
-                    int old;
-                    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(old) : "l"(&p.row_cnt[row]) : "memory");
-                    const int last = old == nseg - 1;
-                    if (last) p.row_cnt[row] = 0;              // ready for the next launch
-                    s_flag = last;
-                }
-            }
-        }
-        if (nseg > 1) {
-            if (p.clustered) {
-                cluster_arrive();                     // (second phase: the stores above are released, and acquired below)
-                cluster_wait();
-            } else {
-                bar_sync(1, QS_CONSUMERS);            // s_flag
-            }
-            if (s_flag) {
-                // ---- the last share of a split row (clustered: the first CTA of its cluster) merges the partials ----
-                if (tid < HS_MAX_TOPK) top[tid] = 0ull;
-                float4 stv = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);       // (warp 0: requested with the keys)
-                if (warp == 0 && lane < nseg)
-                    stv = p.clustered ? s_cs[lane] : __ldcg(&p.part_stats[partial_slot(p, row, c_first + lane)]);
-                for (int t = tid; t < nseg * HS_MAX_TOPK; t += QS_CONSUMERS) {
-                    if (p.clustered) {
-                        s_list[t] = s_ck[t / HS_MAX_TOPK][t % HS_MAX_TOPK];
-                        continue;
-                    }
-                    const int ps = partial_slot(p, row, c_first + t / HS_MAX_TOPK);
-                    s_list[t] = __ldcg(&p.part_keys[(size_t)ps * HS_MAX_TOPK + (t % HS_MAX_TOPK)]);
-                }
-                bar_sync(1, QS_CONSUMERS);
-                rank_select_warps(s_list, nseg * HS_MAX_TOPK, K, top, warp, lane, NW);
-                bar_sync(1, QS_CONSUMERS);
-                if (warp == 0) {
-                    const float m = stv.x, cs = stv.y, cu = stv.z;
-                    const float M = warp_max(m);
-                    const float f = (m == -CUDART_INF_F) ? 0.f : ex2f((m - M) * LOG2E);
-                    const float S = warp_sum(cs * f), U = warp_sum(cu * f);
-                    finalize_row(p, row, M, S, U, top, lane);
-                }
-            }
-        }
-        ++seg;
-        g = row_g0 + sv1;
     }
-    if (p.clustered && seg == 0) {                    // (a CTA without a segment still owes the cluster its two phases)
-        cluster_wait();
-        cluster_arrive();
-        cluster_wait();
+    __syncthreads();                                             // all candidates are pushed
+    const int ncand = s_cnt;
+    if (ncand <= CAND_CAP) rank_select_warps(s_list, ncand, K, s_top, warp, lane, NW);
+    else topk_by_rounds<BF16>(rowp, sv0, sv1, p.vocab, K, s_top, s_red, tid, QS_THREADS, 1);   // heavy ties
+    __syncthreads();                                             // the Top-K is complete
+    if (warp != 0 && (parts == 1 || part != 0)) {
+        if (parts > 1) cluster_wait();
+        return;
+    }
+    if (p.prefetch) pdl_wait();                                  // from here on results go to global memory
+    float R = 0.f, M = 0.f, S = 0.f, U = 0.f;
+    if (warp == 0) {                                             // the warps' (ref, s, u, max) in a fixed order
+        const float4 w = lane < NW ? s_wstat[lane] : make_float4(-CUDART_INF_F, 0.f, 0.f, -CUDART_INF_F);
+        R = warp_max(w.x); M = warp_max(w.w);
+        const float f = w.x == -CUDART_INF_F ? 0.f : ex2f((w.x - R) * LOG2E);
+        S = warp_sum(w.y * f); U = warp_sum(w.z * f);
+    }
+    if (parts == 1) {
+        finalize_row(p, row, M, R, S, U, lane < K ? s_top[lane] : 0ull, lane);
+        return;
+    }
+    cluster_wait();                                              // (the arrival above: every CTA of the cluster runs)
+    if (part != 0) {
+        // this part goes into slot `part` of the first CTA of the row's cluster
+        const unsigned int bar = cluster_map_addr(smem_u32(&s_merge), 0);
+        if (lane < HS_MAX_TOPK / 2) {
+            const unsigned long long a = s_top[2 * lane], b = s_top[2 * lane + 1];
+            st_async_v4(cluster_map_addr(smem_u32(&s_ck[part][2 * lane]), 0), (unsigned int)a, (unsigned int)(a >> 32),
+                        (unsigned int)b, (unsigned int)(b >> 32), bar);
+        } else if (lane == HS_MAX_TOPK / 2) {
+            st_async_v4(cluster_map_addr(smem_u32(&s_cs[part]), 0), __float_as_uint(R), __float_as_uint(S), __float_as_uint(U),
+                        __float_as_uint(M), bar);
+        }
+        return;
+    }
+    if (warp == 0) {
+        if (lane < HS_MAX_TOPK) s_ck[0][lane] = s_top[lane];
+        if (lane == 0) s_cs[0] = make_float4(R, S, U, M);
+    }
+    mbar_wait_cluster(smem_u32(&s_merge), 0u, p.err);
+    __syncthreads();                                             // (s_top has been read)
+    if (tid < HS_MAX_TOPK) s_top[tid] = 0ull;
+    __syncthreads();
+    rank_select_warps(&s_ck[0][0], parts * HS_MAX_TOPK, K, s_top, warp, lane, NW);
+    __syncthreads();
+    if (warp == 0) {
+        const float4 st = lane < parts ? s_cs[lane] : make_float4(-CUDART_INF_F, 0.f, 0.f, -CUDART_INF_F);
+        R = warp_max(st.x);
+        const float f = st.x == -CUDART_INF_F ? 0.f : ex2f((st.x - R) * LOG2E);
+        finalize_row(p, row, warp_max(st.w), R, warp_sum(st.y * f), warp_sum(st.z * f), lane < K ? s_top[lane] : 0ull, lane);
     }
 }
+
 
 // ================================================================================================================
 // Tree stage: one CTA of 128 threads per sequence, one thread per node
@@ -658,8 +399,6 @@ static void fill_common(QuantParams& p, const hs_tree_batch* tree, const void* l
     p.per = 0;
     p.split = 0;
     p.extra = 0;
-    p.nslots = QS_SLOTS;
-    p.clustered = 0;
     p.rows = tree->n_nodes_total;
     p.batch = tree->batch;
     p.node_off = tree->node_off;
@@ -676,56 +415,30 @@ static void fill_common(QuantParams& p, const hs_tree_batch* tree, const void* l
     p.err = nullptr;
 }
 
-// Geometry of a launch, one CTA per SM.  With at most one row per SM and rows short enough for the item slots,
-// every SM gets one part of one row (the first rows are cut into one part more than the others so that every SM
-// has work): a CTA then has a single row segment.  With two or more rows per SM every CTA takes whole rows (no row
-// needs a merge).  In between every CTA takes an equal share of the stream, at least one item long and so large
-// that no row is split over more than QS_MAX_SEGS shares.
-static void quantify_geometry(int rows, int nvec, int sm_count, QuantParams& p, int& nctas, size_t& smem) {
-    int S = rows <= sm_count ? sm_count / rows : 0;
-    while (S > 1 && (S + 1 > QS_MAX_SEGS || nvec / (S + 1) < 256)) --S;      // parts of at least 4 KiB
-    const int extra = (S >= 1 && S + 1 <= QS_MAX_SEGS && nvec / (S + 1) >= 256) ? min(rows, sm_count - rows * S) : 0;
-    const int pv_max = S >= 1 ? (nvec + S - 1) / S : 0;
-    // With at most half as many rows as SMs every row is cut into the same number of parts (at most eight, the portable
-    // cluster size): the CTAs of a row are one thread-block cluster and merge the row in the shared memory of its first
-    // CTA.  (The critical path is the same as with one part more for some rows - the rows with fewer parts - but the
-    // merge costs a cluster barrier instead of partials, an atomic and their read-back through global memory.)
-    int Sc = rows <= sm_count / 2 ? (sm_count / rows < 8 ? sm_count / rows : 8) : 0;
-    while (Sc > 1 && nvec / Sc < 256) --Sc;
-    const int pv_c = Sc >= 2 ? (nvec + Sc - 1) / Sc : 0;
-    p.clustered = 0;
-    if (rows >= 2 * sm_count) {
-        p.split = -1;
-        p.extra = sm_count;
-        p.per = 0;
-        p.nslots = QS_SLOTS;
-        nctas = sm_count;
-    } else if (Sc >= 2 && pv_c <= QS_SLOTS * QS_ITEM_VECS) {
-        p.split = Sc;
-        p.extra = 0;
-        p.per = pv_c;
-        p.nslots = (pv_c + QS_ITEM_VECS - 1) / QS_ITEM_VECS;
-        p.clustered = 1;
-        nctas = rows * Sc;
-    } else if (S >= 1 && pv_max <= QS_SLOTS * QS_ITEM_VECS) {
-        p.split = S;
-        p.extra = extra;
-        p.per = pv_max;
-        p.nslots = (pv_max + QS_ITEM_VECS - 1) / QS_ITEM_VECS;
-        nctas = rows * S + extra;
-    } else {
-        const long long total = (long long)rows * nvec;
-        long long per = (total + sm_count - 1) / sm_count;
-        const long long floor_row = (nvec + (QS_MAX_SEGS - 2) - 1) / (QS_MAX_SEGS - 2);
-        if (per < floor_row) per = floor_row;
-        if (per < QS_ITEM_VECS) per = QS_ITEM_VECS;
-        p.split = 0;
-        p.extra = 0;
-        p.per = (int)per;
-        p.nslots = QS_SLOTS;
-        nctas = (int)((total + per - 1) / per);
+// Shares of the warp kernel: equal numbers of rounds, one share per warp of the device; a row in at most QW_MAX_SEGS of
+// them, and no more shares than the workspace has partials for.
+static hs_status launch_warps(hs_ctx* ctx, QuantParams& p, hs_dtype dtype, cudaStream_t stream) {
+    if (!ctx->warps_ready) {
+        if (cudaFuncSetAttribute(quantify_warp_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)QW_SMEM_BYTES) != cudaSuccess ||
+            cudaFuncSetAttribute(quantify_warp_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)QW_SMEM_BYTES) != cudaSuccess)
+            return HS_ERR_CUDA;
+        ctx->warps_ready = true;
     }
-    smem = (size_t)p.nslots * QS_ITEM_VECS * 16 + 128;
+    p.extra = QW_ROW_END;
+    const long long rr = (p.nvec + QW_ROUND - 1) / QW_ROUND, total = (rr + p.extra) * p.rows;
+    const long long room = (long long)((ctx->scratch_bytes - 256) / (2 * (sizeof(float4) + HS_MAX_TOPK * 8)));
+    const long long shares = min((long long)ctx->sm_count * QW_WARPS, room);
+    if (shares < 1) return HS_ERR_WORKSPACE;
+    const long long per = max((total + shares - 1) / shares, (rr + QW_MAX_SEGS - 3) / (QW_MAX_SEGS - 2));
+    p.per = (int)per;
+    const int used = (int)((total + per - 1) / per);
+    p.part_stats = (float4*)ctx->scratch;
+    p.part_keys = (unsigned long long*)(ctx->scratch + hs_align_up((size_t)2 * used * sizeof(float4), 256));
+    const dim3 grid((used + QW_WARPS - 1) / QW_WARPS), one(1, 1, 1);
+    cudaError_t e = dtype == HS_BF16
+        ? hs_launch(quantify_warp_kernel<true>, grid, dim3(QW_THREADS), QW_SMEM_BYTES, stream, ctx->pdl, one, p)
+        : hs_launch(quantify_warp_kernel<false>, grid, dim3(QW_THREADS), QW_SMEM_BYTES, stream, ctx->pdl, one, p);
+    return e == cudaSuccess ? HS_OK : HS_ERR_CUDA;
 }
 
 hs_status hs_launch_quantify(hs_ctx* ctx, const hs_tree_batch* tree, const void* logits, hs_dtype dtype,
@@ -734,30 +447,33 @@ hs_status hs_launch_quantify(hs_ctx* ctx, const hs_tree_batch* tree, const void*
     QuantParams p;
     fill_common(p, tree, logits, dtype, row_stride, vocab, policy, out);
     if (p.nvec > QS_ITEM_VECS * 64) return HS_ERR_SHAPE;            // vocabulary beyond 2^20 bf16 / 2^19 fp32 logits
-    int nctas = 0;
-    size_t smem = 0;
-    quantify_geometry(p.rows, p.nvec, ctx->sm_count, p, nctas, smem);
-    const int nparts = p.split ? nctas : 2 * nctas;      // (whole rows: none is used)
-    const size_t stats_bytes = hs_align_up((size_t)nparts * sizeof(float4), 256);
-    const size_t keys_bytes = (size_t)nparts * HS_MAX_TOPK * sizeof(unsigned long long);
-    if (stats_bytes + keys_bytes > ctx->scratch_bytes) return HS_ERR_WORKSPACE;
-    p.part_stats = (float4*)ctx->scratch;
-    p.part_keys = (unsigned long long*)(ctx->scratch + stats_bytes);
     p.row_cnt = ctx->counters + HS_CNT_QUANT_ROW;
     p.err = ctx->counters + HS_CNT_ERROR;
     p.prefetch = (ctx->prefetch & HS_PREFETCH_LOGITS) != 0;
-    if (!ctx->quant_ready) {
-        if (cudaFuncSetAttribute(quantify_stream_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_BYTES) != cudaSuccess ||
-            cudaFuncSetAttribute(quantify_stream_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_BYTES) != cudaSuccess)
-            return HS_ERR_CUDA;
-        ctx->quant_ready = true;
+    // With at most half as many rows as SMs the rows are cut into parts, one CTA each (74 rows of 128256 bf16: 10.3 us,
+    // the warp kernel 12.9 us); from there on a row would have an SM to itself (24 us at 75 rows).
+    int parts = p.rows <= ctx->sm_count / 2 ? min(ctx->sm_count / p.rows, 8) : 0;
+    while (parts > 1 && p.nvec / parts < 256) --parts;              // parts of at least 4 KiB
+    const int pv = parts ? (p.nvec + parts - 1) / parts : 0;
+    cudaError_t e;
+    if (parts && pv <= QS_SLOTS * QS_ITEM_VECS) {
+        if (!ctx->quant_ready) {
+            if (cudaFuncSetAttribute(quantify_cluster_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_BYTES) != cudaSuccess ||
+                cudaFuncSetAttribute(quantify_cluster_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_BYTES) != cudaSuccess)
+                return HS_ERR_CUDA;
+            ctx->quant_ready = true;
+        }
+        p.split = parts;
+        p.per = pv;
+        const size_t smem = (size_t)((pv + QS_ITEM_VECS - 1) / QS_ITEM_VECS) * QS_ITEM_VECS * 16 + 128;
+        e = dtype == HS_BF16
+            ? hs_launch(quantify_cluster_kernel<true>, dim3(p.rows * parts), dim3(QS_THREADS), smem, stream, ctx->pdl, dim3(parts, 1, 1), p)
+            : hs_launch(quantify_cluster_kernel<false>, dim3(p.rows * parts), dim3(QS_THREADS), smem, stream, ctx->pdl, dim3(parts, 1, 1), p);
+        if (e != cudaSuccess) return HS_ERR_CUDA;
+    } else {
+        const hs_status st = launch_warps(ctx, p, dtype, stream);
+        if (st != HS_OK) return st;
     }
-    cudaError_t e = dtype == HS_BF16
-        ? hs_launch(quantify_stream_kernel<true>, dim3(nctas), dim3(QS_THREADS), smem, stream, ctx->pdl,
-                    dim3(p.clustered ? p.split : 1, 1, 1), p)
-        : hs_launch(quantify_stream_kernel<false>, dim3(nctas), dim3(QS_THREADS), smem, stream, ctx->pdl,
-                    dim3(p.clustered ? p.split : 1, 1, 1), p);
-    if (e != cudaSuccess) return HS_ERR_CUDA;
     if (!with_tree_stage) return HS_OK;              // (the caller launches the kernel that also prunes)
     e = hs_launch(tree_scores_kernel, dim3(p.batch), dim3(HS_MAX_NODES), 0, stream, ctx->pdl, dim3(1, 1, 1), p);
     return e == cudaSuccess ? HS_OK : HS_ERR_CUDA;
@@ -927,7 +643,7 @@ __global__ void __launch_bounds__(HS_ROW_THREADS, 2) quantify_chunk_kernel(const
         float M = warp_max(m);
         float f = (m == -CUDART_INF_F) ? 0.f : ex2f((m - M) * LOG2E);
         float S = warp_sum(cs * f), U = warp_sum(cu * f);
-        finalize_row(p, row, M, S, U, s_top, lane);
+        finalize_row(p, row, M, M, S, U, lane < K ? s_top[lane] : 0ull, lane);
         if (lane == 0) p.row_cnt[row] = 0;                 // ready for the next launch
     }
 }
