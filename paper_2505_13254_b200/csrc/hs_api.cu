@@ -29,7 +29,8 @@ extern "C" size_t hs_workspace_bytes(int32_t max_batch, int32_t max_rows, int32_
     size_t quant = (size_t)2 * 152 * 16 * HS_ROW_PARTIAL_BYTES + 512;
     // acceptance: three per-row result arrays (256-byte aligned each) + chunk partials of target and draft rows
     size_t accept = 3 * hs_align_up((size_t)max_rows * 8, 256) +
-                    (size_t)2 * max_rows * chunks * HS_ACC_PARTIAL_BYTES;
+                    (size_t)2 * (max_rows * chunks > 152 * 16 ? max_rows * chunks : 152 * 16) * HS_ACC_PARTIAL_BYTES +
+                    (size_t)(max_batch < 256 ? max_batch : 256) * 2048 + 512;      // shared bonus draws
     // (the attention merges its KV splits on chip: no workspace)
     size_t scratch = quant > accept ? quant : accept;
     return HS_COUNTER_BYTES + hs_align_up(scratch, 256) + 256;
@@ -76,7 +77,6 @@ extern "C" hs_status hs_create(hs_ctx** out, int32_t device, size_t workspace_by
     c->quant_ready = false;
     c->warps_ready = false;
     c->cart_ready = false;
-    c->rows_ready = false;
     if (cudaDeviceSynchronize() != cudaSuccess) { cudaFree(p); delete c; return HS_ERR_CUDA; }
     *out = c;
     return HS_OK;

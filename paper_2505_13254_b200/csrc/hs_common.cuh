@@ -31,7 +31,6 @@ struct hs_ctx {
     int attn_cap[9];    // CTAs of the attention kernel that run at once in clusters of s = 1..8
     int walk_cap;       // 16-CTA clusters of the acceptance walk that run at once
     bool walk_ready;    // acceptance walk kernel attributes set on this device
-    bool rows_ready;    // streaming acceptance row pass: shared-memory attribute set on this device
     bool cart_ready;    // single-CTA stratifier training: shared-memory attribute set on this device
     bool warps_ready;   // warp kernel of the entropy pass: shared-memory attribute set on this device
     bool quant_ready;   // streaming entropy kernel: shared-memory attribute set on this device

@@ -24,10 +24,10 @@ using std::min;
 #include "hs_common.cuh"
 #include "hs_layout.h"
 #include "hs_ptx.cuh"
+#include "row_rounds.cuh"
 #include "tree_stage.cuh"
 
 #define CAND_CAP 512
-#define LOG2E 1.4426950408889634f
 
 #define QS_THREADS 512                        // cluster kernel: sixteen warps
 #define QS_ITEM_VECS 2048                     // vectors per item: 32 KiB, four per thread
@@ -57,23 +57,6 @@ struct QuantParams {
     int prefetch;    // the rows may be fetched before the dependency wait (the caller vouches that they are complete)
     int* err;        // sticky device error word (a bounded wait that expired)
 };
-
-template <bool BF16>
-__device__ __forceinline__ void unpack(const uint4& v, float* x) {
-    if (BF16) {
-        x[0] = bf16_lo(v.x); x[1] = bf16_hi(v.x); x[2] = bf16_lo(v.y); x[3] = bf16_hi(v.y);
-        x[4] = bf16_lo(v.z); x[5] = bf16_hi(v.z); x[6] = bf16_lo(v.w); x[7] = bf16_hi(v.w);
-    } else {
-        x[0] = __uint_as_float(v.x); x[1] = __uint_as_float(v.y);
-        x[2] = __uint_as_float(v.z); x[3] = __uint_as_float(v.w);
-    }
-}
-
-__device__ __forceinline__ float ex2f(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 
 // Rank candidates s_cand[0..n) by key (all distinct, 0 = empty) and write the K best to s_top (zeroed before).
 __device__ __forceinline__ void rank_select(const unsigned long long* s_cand, int n, int K,
@@ -425,7 +408,7 @@ static hs_status launch_warps(hs_ctx* ctx, QuantParams& p, hs_dtype dtype, cudaS
         ctx->warps_ready = true;
     }
     p.extra = QW_ROW_END;
-    const long long rr = (p.nvec + QW_ROUND - 1) / QW_ROUND, total = (rr + p.extra) * p.rows;
+    const long long rr = (p.nvec + ROUND_VECS - 1) / ROUND_VECS, total = (rr + p.extra) * p.rows;
     const long long room = (long long)((ctx->scratch_bytes - 256) / (2 * (sizeof(float4) + HS_MAX_TOPK * 8)));
     const long long shares = min((long long)ctx->sm_count * QW_WARPS, room);
     if (shares < 1) return HS_ERR_WORKSPACE;

@@ -18,7 +18,6 @@
 
 #define QW_WARPS 16
 #define QW_THREADS (QW_WARPS * 32)
-#define QW_ROUND 128                    // vectors per round: four per lane
 #define QW_ROW_END 4                    // what the end of a row segment costs, in rounds
 #define QW_GROUPS 32                    // cells a lane keeps maxima for: rounds, or groups of 2^k rounds on long segments
 #define QW_CAND 128                     // candidates of a segment
@@ -33,62 +32,6 @@ struct WarpSmem {
 };
 #define QW_SMEM_BYTES (QW_WARPS * sizeof(WarpSmem))
 
-// The largest key of the warp (0 = none) and the lane that holds it; keys are distinct.
-__device__ __forceinline__ unsigned long long warp_best_key(unsigned long long k, int& src) {
-    const unsigned int hi = (unsigned int)(k >> 32), mh = __reduce_max_sync(HS_FULL_MASK, hi);
-    const unsigned int lo = hi == mh ? (unsigned int)k : 0u, ml = __reduce_max_sync(HS_FULL_MASK, lo);
-    src = __ffs(__ballot_sync(HS_FULL_MASK, hi == mh && lo == ml)) - 1;
-    return ((unsigned long long)mh << 32) | ml;
-}
-
-// -inf in place of what vector v of a row holds past the vocabulary
-template <bool BF16>
-__device__ __forceinline__ void mask_tail(uint4& d, int v, int vocab) {
-    constexpr int VE = BF16 ? 8 : 4;
-    unsigned int* wd = reinterpret_cast<unsigned int*>(&d);
-#pragma unroll
-    for (int e = 0; e < VE; ++e)
-        if (v * VE + e >= vocab) {
-            if (BF16) wd[e >> 1] = (e & 1) ? ((wd[e >> 1] & 0x0000ffffu) | 0xff800000u) : ((wd[e >> 1] & 0xffff0000u) | 0x0000ff80u);
-            else wd[e] = 0xff800000u;
-        }
-}
-
-// One round of a segment: vectors [128 r, 128 r + 128) of the row, -inf where they lie past its end.
-template <bool BF16>
-__device__ __forceinline__ void load_round(const QuantParams& p, const uint4* rowv, int r, int lane, uint4 (&d)[4]) {
-    const uint4* src = rowv + (size_t)r * QW_ROUND + lane;
-    if ((r + 1) * QW_ROUND < p.nvec) {                       // (the row's last vector may be partial: it takes the other way)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) d[j] = ld_stream(src + j * 32);
-        return;
-    }
-    const unsigned int ninf = BF16 ? 0xff80ff80u : 0xff800000u;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int v = r * QW_ROUND + j * 32 + lane;
-        d[j] = v < p.nvec ? ld_stream(src + j * 32) : make_uint4(ninf, ninf, ninf, ninf);
-        if (v == p.nvec - 1) mask_tail<BF16>(d[j], v, p.vocab);
-    }
-}
-// largest of a lane's logits of a round
-template <bool BF16>
-__device__ __forceinline__ float round_max(const uint4 (&d)[4]) {
-    if (BF16) {
-        const __nv_bfloat162* w = reinterpret_cast<const __nv_bfloat162*>(&d[0]);
-        __nv_bfloat162 a = __hmax2(w[0], w[1]), b = __hmax2(w[2], w[3]), c = __hmax2(w[4], w[5]), e = __hmax2(w[6], w[7]);
-        a = __hmax2(a, w[8]); b = __hmax2(b, w[9]); c = __hmax2(c, w[10]); e = __hmax2(e, w[11]);
-        a = __hmax2(a, w[12]); b = __hmax2(b, w[13]); c = __hmax2(c, w[14]); e = __hmax2(e, w[15]);
-        a = __hmax2(__hmax2(a, b), __hmax2(c, e));
-        const unsigned int u = *reinterpret_cast<const unsigned int*>(&a);
-        return fmaxf(bf16_lo(u), bf16_hi(u));
-    }
-    const float* x = reinterpret_cast<const float*>(&d[0]);
-    float a = max3(x[0], x[1], x[2]), b = max3(x[3], x[4], x[5]);
-    a = max3(a, x[6], x[7]); b = max3(b, x[8], x[9]);
-    a = max3(a, x[10], x[11]); b = max3(b, x[12], x[13]);
-    return fmaxf(max3(a, x[14], x[15]), b);
-}
 // s += e, u += e x of a lane's logits of a round, e = 2^(x log2(e) + n).  CLAMP keeps 0 * x finite for x = -inf.
 template <bool BF16, bool CLAMP>
 __device__ __forceinline__ void round_sums(const uint4 (&d)[4], float n, float2& s2, float2& u2) {
@@ -140,7 +83,7 @@ __device__ __noinline__ void topk_rounds_warp(const QuantParams& p, const uint4*
                 for (int j = 0; j < 4; ++j) {
                     float x[8];
                     unpack<BF16>(d[j], x);
-                    const int base = (r * QW_ROUND + j * 32 + lane) * VE;
+                    const int base = (r * ROUND_VECS + j * 32 + lane) * VE;
 #pragma unroll
                     for (int e = 0; e < VE; ++e)
                         if (x[e] > -CUDART_INF_F) {
@@ -162,7 +105,7 @@ __global__ void __launch_bounds__(QW_THREADS, 1) quantify_warp_kernel(const __gr
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     WarpSmem& sm = reinterpret_cast<WarpSmem*>(s_dyn)[warp];
     const int K = p.K, c = blockIdx.x * QW_WARPS + warp;
-    const int rr = (p.nvec + QW_ROUND - 1) / QW_ROUND;            // rounds per row
+    const int rr = (p.nvec + ROUND_VECS - 1) / ROUND_VECS;            // rounds per row
     const int rv = rr + p.extra;                                  // places per row in the stream: its end costs `extra` rounds
     const int total = p.rows * rv;
     int g = min(c * p.per, total);
@@ -243,7 +186,7 @@ __global__ void __launch_bounds__(QW_THREADS, 1) quantify_warp_kernel(const __gr
                     vec[i] = -1;
                     if (h < nhit) {
                         const int cell = sm.hit[h], rc = r0 + ((cell >> 5) << gsh) + q;
-                        const int v = rc * QW_ROUND + (lane & 3) * 32 + (cell & 31);
+                        const int v = rc * ROUND_VECS + (lane & 3) * 32 + (cell & 31);
                         if (rc < r1 && v < p.nvec) vec[i] = v;
                     }
                     d[i] = vec[i] >= 0 ? __ldg(rowv + vec[i]) : make_uint4(0, 0, 0, 0);
