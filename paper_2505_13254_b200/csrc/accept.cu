@@ -100,24 +100,44 @@ __device__ __forceinline__ void unpack_v(const uint4& v, float* x) {
 // of the consumer warps of the streaming kernel), which meet on a barrier of their own.
 __device__ __forceinline__ void walk_sync() { named_bar_sync(2, HS_ROW_THREADS); }
 
-__device__ void greedy_walk(const AcceptParams& p, int b) {
+// last b with off[b] <= k (skips empty sequences), by a whole warp
+__device__ __forceinline__ int sequence_of(const int* off, int batch, int k, int lane) {
+    int lo = 0, len = batch;
+    while (len > 1) {
+        const int step = (len + 31) / 32;
+        const bool le = lane * step < len && off[lo + lane * step] <= k;
+        const int n = __popc(__ballot_sync(HS_FULL_MASK, le));        // (off ascends: the lanes that agree are the first n)
+        lo += (n - 1) * step;
+        len = min(step, len - (n - 1) * step);
+    }
+    return lo;
+}
+
+struct WalkNode {         // kept node `threadIdx.x` of a sequence
+    int par, tok, orig;   // parent among the kept nodes, token, drafted node id
+};
+__device__ __forceinline__ WalkNode load_walk_node(const AcceptParams& p, int koff, int nk, int nbase) {
+    WalkNode n = {-1, -1, 0};
+    if ((int)threadIdx.x < nk) {
+        n.par = p.pr.new_parent[koff + threadIdx.x];
+        n.orig = p.pr.keep_idx[koff + threadIdx.x];
+        n.tok = p.token[nbase + n.orig];
+    }
+    return n;
+}
+
+__device__ void greedy_walk(const AcceptParams& p, int b, int koff, int nk, const WalkNode& node) {
     __shared__ int s_arg[HS_MAX_NODES], s_next[HS_MAX_NODES], s_orig[HS_MAX_NODES];
     const int tid = threadIdx.x, nthr = HS_ROW_THREADS;
-    const int koff = p.pr.keep_off[b];
-    const int nk = min(p.pr.n_keep[b], HS_MAX_NODES);
-    const int nbase = p.node_off[b];
+    nk = min(nk, HS_MAX_NODES);
     const int cap = p.out.path_cap;
-    // Every kept node's parent, token and its row's arg-max in one round trip; the walk itself then runs in shared
-    // memory: node j continues the path of its parent iff its token is the parent's arg-max, and of several such
-    // children (duplicate tokens among siblings) the one with the lowest index does.
-    int my_par = -1, my_tok = -1;
+    // The rows' arg-maxima in one round trip; the walk itself then runs in shared memory: node j continues the path of its
+    // parent iff its token is the parent's arg-max, and of several such children (duplicate tokens among siblings) the one
+    // with the lowest index does.
     if (tid < nk) {
-        my_par = p.pr.new_parent[koff + tid];
-        const int orig = p.pr.keep_idx[koff + tid];
         s_arg[tid] = __ldcg(&p.ro.tgt_arg[koff + tid]);
-        s_orig[tid] = orig;
+        s_orig[tid] = node.orig;
         s_next[tid] = 0x7fffffff;
-        my_tok = p.token[nbase + orig];
     }
     for (int j = tid; j < cap; j += nthr) {
         p.out.path_nodes[b * cap + j] = -1;
@@ -125,7 +145,7 @@ __device__ void greedy_walk(const AcceptParams& p, int b) {
         p.out.path_tokens[b * cap + j] = -1;
     }
     walk_sync();
-    if (tid > 0 && tid < nk && my_par >= 0 && my_par < tid && my_tok == s_arg[my_par]) atomicMin(&s_next[my_par], tid);
+    if (tid > 0 && tid < nk && node.par >= 0 && node.par < tid && node.tok == s_arg[node.par]) atomicMin(&s_next[node.par], tid);
     walk_sync();
     if (tid == 0) {
         int cur = 0, len = 0;
@@ -151,23 +171,45 @@ __device__ __forceinline__ float load_logit(const void* base, int is_bf16, size_
 
 #include "accept_det.cuh"
 
+// Few rows: a CTA per chunk of a row, all loads in flight at once.  Bound by its chain of latencies, so the chain is short: the
+// entries of the pruned tree come in one round trip for a single sequence (two for a batch), what a walk needs of the tree is
+// fetched beside the row, a thread takes packed maxima and only a warp that holds the chunk's maximum looks for its index, and
+// the chunks of a row that form a cluster send their results to its first CTA and leave.
 template <bool BF16>
 __global__ void __launch_bounds__(HS_ROW_THREADS, 4) accept_rows_kernel(const __grid_constant__ AcceptParams p) {
     constexpr int VE = BF16 ? 8 : 4;
     constexpr int VPT = HS_ROW_VPT;
-    __shared__ float s_w[8][2];
-    __shared__ unsigned long long s_key[8];
+    constexpr int NW = HS_ROW_THREADS / 32;
+    __shared__ float2 s_w[NW];                    // {max, sum} per warp
+    __shared__ unsigned int s_arg;                // first token of the chunk with its maximum
     __shared__ __align__(16) uint4 s_cl[8];       // clustered launch, first CTA of a row: the chunks' results
+    __shared__ unsigned long long s_bar;          //   and the barrier that counts them
     __shared__ int s_flag;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int chunk = blockIdx.x, k = blockIdx.y, which = blockIdx.z;   // which: 0 target, 1 draft
+    if (tid == 0) {
+        s_arg = 0x7fffffffu;
+        s_flag = 0;
+        if (p.clustered && chunk == 0) {
+            mbar_init(smem_u32(&s_bar), 1);
+            mbar_expect_tx(smem_u32(&s_bar), (unsigned int)(p.chunks - 1) * 16u);
+            mbar_init_fence();
+        }
+    }
+    __syncwarp();
     pdl_launch_dependents();
     // First half of a cluster barrier: when it completes every CTA of the row's cluster runs, and its shared memory may
     // be written from outside.  (The CTAs of a cluster take every early exit below together: same row, same sequence.)
     if (p.clustered) cluster_arrive();
     pdl_wait();                            // the pruned tree and the logits come from upstream
+    const int kept = p.pr.keep_off[p.batch], kidx = p.pr.keep_idx[k];
+    const bool check = chunk == 0 && which == 0 && k < p.batch;
+    const int e_keep = check ? p.pr.n_keep[k] : 1, e_status = check ? p.pr.status[k] : 0;
+    const int b = sequence_of(p.pr.keep_off, p.batch, k, lane);
+    const int koff = p.pr.keep_off[b], nk = p.pr.n_keep[b], md = p.mode[b], nbase = p.node_off[b];
+    const float temp = p.temperature[b];
     // sequences that kept nothing (flagged upstream) get their empty result from CTA (0, b, 0)
-    if (chunk == 0 && which == 0 && k < p.batch && (p.pr.n_keep[k] <= 0 || p.pr.status[k] != 0)) {
+    if (e_keep <= 0 || e_status != 0) {
         const int cap = p.out.path_cap;
         for (int j = tid; j < cap; j += HS_ROW_THREADS) {
             p.out.path_nodes[k * cap + j] = -1;
@@ -176,146 +218,146 @@ __global__ void __launch_bounds__(HS_ROW_THREADS, 4) accept_rows_kernel(const __
         }
         if (tid == 0) {
             p.out.accept_len[k] = 0; p.out.bonus_token[k] = -1; p.out.terminal_rank[k] = -1;
-            p.out.status[k] = p.pr.status[k] != 0 ? p.pr.status[k] : HS_ERR_BAD_TREE;
+            p.out.status[k] = e_status != 0 ? e_status : HS_ERR_BAD_TREE;
         }
     }
-    if (k >= p.pr.keep_off[p.batch]) return;
-    int lo = 0, hi = p.batch;                     // sequence of kept node k
-    while (hi - lo > 1) {
-        int mid = (lo + hi) >> 1;
-        if (p.pr.keep_off[mid] <= k) lo = mid; else hi = mid;
-    }
-    const int b = lo;
-    const int i = k - p.pr.keep_off[b];
-    const int nk = p.pr.n_keep[b];
-    const int md = p.mode[b];
+    if (k >= kept) return;
+    const int i = k - koff;
     const bool sampling = md != HS_ACCEPT_GREEDY;          // the row's normaliser is needed
     if (which == 1) {
         if (md != HS_ACCEPT_REJECTION) return;
         int internal = 0;                         // does kept node i have a kept child?
         for (int j = i + 1 + tid; j < nk; j += HS_ROW_THREADS)
-            internal |= (p.pr.new_parent[p.pr.keep_off[b] + j] == i);
+            internal |= (p.pr.new_parent[koff + j] == i);
         if (!__syncthreads_or(internal)) return;
     }
-    const int orig_row = p.node_off[b] + p.pr.keep_idx[k];
-    const int row = which == 1 ? orig_row : (p.target_layout == HS_ROWS_ORIGINAL ? orig_row : k);
+    const int row = which == 1 || p.target_layout == HS_ROWS_ORIGINAL ? nbase + kidx : k;
     const char* rowp = (const char*)(which == 1 ? p.draft : p.target) + (size_t)row * p.row_stride * (BF16 ? 2 : 4);
     const int v0 = chunk * p.chunk_vecs;
     const int v1 = min(v0 + p.chunk_vecs, p.nvec);
 
     uint4 d[VPT];
+    const unsigned int ninf = BF16 ? 0xff80ff80u : 0xff800000u;
 #pragma unroll
     for (int j = 0; j < VPT; ++j) {
-        int v = v0 + tid + j * HS_ROW_THREADS;
-        if (v < v1) {
-            d[j] = __ldcs((const uint4*)(rowp) + v);
-        } else {
-            unsigned int ninf = BF16 ? 0xff80ff80u : 0xff800000u;
-            d[j] = make_uint4(ninf, ninf, ninf, ninf);
-        }
+        const int v = v0 + tid + j * HS_ROW_THREADS;
+        d[j] = v < v1 ? ld_stream((const uint4*)rowp + v) : make_uint4(ninf, ninf, ninf, ninf);
     }
-    // per-thread best (value, lowest index)
-    float tmax = -CUDART_INF_F;
-    int targ = 0x7fffffff;
+    // the walk's view of node `tid` (a greedy sequence is walked by one of its CTAs), fetched while the row is on its way
+    WalkNode node;
+    if (md == HS_ACCEPT_GREEDY && which == 0 && (chunk == 0 || !p.clustered)) node = load_walk_node(p, koff, nk, nbase);
+    if (v1 == p.nvec && p.nvec * VE != p.vocab) {          // the row's last vector runs past vocab
 #pragma unroll
-    for (int j = 0; j < VPT; ++j) {
-        float x[8];
-        unpack_v<BF16>(d[j], x);
-        int base = (v0 + tid + j * HS_ROW_THREADS) * VE;
-#pragma unroll
-        for (int e = 0; e < VE; ++e) {
-            bool in = base + e < p.vocab;
-            if (in && x[e] > tmax) { tmax = x[e]; targ = base + e; }   // ascending index: strict > keeps the lowest
-        }
+        for (int j = 0; j < VPT; ++j)
+            if (v0 + tid + j * HS_ROW_THREADS == p.nvec - 1) mask_tail<BF16>(d[j], p.nvec - 1, p.vocab);
     }
-    unsigned long long key = (targ == 0x7fffffff) ? 0ull : make_key(tmax, targ);
-    key = warp_max_u64(key);
+    static_assert(VPT == 8, "two rounds of four vectors");
+    const uint4(&da)[4] = *reinterpret_cast<const uint4(*)[4]>(&d[0]);
+    const uint4(&db)[4] = *reinterpret_cast<const uint4(*)[4]>(&d[4]);
+    const float tmax = fmaxf(round_max<BF16>(da), round_max<BF16>(db));
+    const float wm = order_bits_float(__reduce_max_sync(HS_FULL_MASK, float_order_bits(tmax)));
+    const float invT = sampling ? LOG2E / temp : 0.f;
     float s = 0.f;
     if (sampling) {
-        const float invT = LOG2E / p.temperature[b];
-        const float nml = (tmax == -CUDART_INF_F) ? 0.f : -tmax * invT;
+        const float n = wm == -CUDART_INF_F ? 0.f : -wm * invT;
+        const float2 l2 = make_float2(invT, invT), n2 = make_float2(n, n);
+        float2 s2 = make_float2(0.f, 0.f);
+        const unsigned int* x = reinterpret_cast<const unsigned int*>(&d[0]);
 #pragma unroll
-        for (int j = 0; j < VPT; ++j) {
-            float x[8];
-            unpack_v<BF16>(d[j], x);
-            int base = (v0 + tid + j * HS_ROW_THREADS) * VE;
-#pragma unroll
-            for (int e = 0; e < VE; ++e)
-                if (base + e < p.vocab) s += ex2a(fmaf(fmaxf(x[e], -1e30f), invT, nml));
+        for (int q = 0; q < (BF16 ? 4 * VPT : 2 * VPT); ++q) {
+            const float2 t = fma2_ftz(BF16 ? make_float2(bf16_lo(x[q]), bf16_hi(x[q]))
+                                           : make_float2(__uint_as_float(x[2 * q]), __uint_as_float(x[2 * q + 1])), l2, n2);
+            s2 = add2_ftz(s2, make_float2(ex2a(t.x), ex2a(t.y)));
         }
-        float wm = warp_max(tmax);
-        float f = (tmax == -CUDART_INF_F) ? 0.f : ex2a((tmax - wm) * invT);
-        s = warp_sum(s * f);
-        if (lane == 0) { s_w[warp][0] = wm; s_w[warp][1] = s; }
+        s = warp_sum(s2.x + s2.y);
     }
-    if (lane == 0) s_key[warp] = key;
+    if (lane == 0) s_w[warp] = make_float2(wm, s);
     __syncthreads();
     if (p.clustered) cluster_wait();
-    if (tid == 0) {
-        unsigned long long best = s_key[0];
-        for (int w = 1; w < 8; ++w) best = s_key[w] > best ? s_key[w] : best;
-        float M = -CUDART_INF_F, S = 0.f;
-        if (sampling) {
-            const float invT = LOG2E / p.temperature[b];
-            for (int w = 0; w < 8; ++w) M = fmaxf(M, s_w[w][0]);
-            for (int w = 0; w < 8; ++w)
-                S += (s_w[w][0] == -CUDART_INF_F) ? 0.f : s_w[w][1] * ex2a((s_w[w][0] - M) * invT);
+    const float2 ws = lane < NW ? s_w[lane] : make_float2(-CUDART_INF_F, 0.f);
+    float M = warp_max(ws.x);
+    if (wm == M && M > -CUDART_INF_F) {                    // this warp holds the chunk's maximum: the lowest index it has it at
+        unsigned int at = 0x7fffffffu;
+        if (tmax == M) {
+#pragma unroll
+            for (int j = VPT - 1; j >= 0; --j) {
+                float x[8];
+                unpack<BF16>(d[j], x);
+#pragma unroll
+                for (int e = VE - 1; e >= 0; --e)
+                    if (x[e] == M) at = (unsigned int)((v0 + tid + j * HS_ROW_THREADS) * VE + e);
+            }
         }
-        if (p.clustered) {
-            // the chunk's result goes into slot `chunk` of the first CTA of the row's cluster (posted stores through
-            // distributed shared memory; the cluster barrier below makes them visible there)
-            const unsigned int dst = cluster_map_addr(smem_u32(&s_cl[chunk]), 0);
-            asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"((unsigned int)best),
-                         "r"((unsigned int)(best >> 32)), "r"(__float_as_uint(M)), "r"(__float_as_uint(S)) : "memory");
-            s_flag = (chunk == 0);
+        at = __reduce_min_sync(HS_FULL_MASK, at);
+        if (lane == 0) atomicMin(&s_arg, at);
+    }
+    __syncthreads();
+    bool merges = false;                                   // (warp 0: it holds the row's result)
+    if (warp == 0) {
+        float S = sampling ? warp_sum(ws.x == -CUDART_INF_F ? 0.f : ws.y * ex2a((ws.x - M) * invT)) : 0.f;
+        unsigned long long key = M > -CUDART_INF_F ? make_key(M, (int)s_arg) : 0ull;
+        if (p.chunks == 1) {
+            merges = true;
+        } else if (p.clustered) {
+            // the chunk's result goes into slot `chunk` of the first CTA of the row's cluster
+            if (chunk != 0) {
+                if (lane == 0)
+                    st_async_v4(cluster_map_addr(smem_u32(&s_cl[chunk]), 0), (unsigned int)key, (unsigned int)(key >> 32),
+                                __float_as_uint(M), __float_as_uint(S), cluster_map_addr(smem_u32(&s_bar), 0));
+            } else {
+                mbar_wait_cluster(smem_u32(&s_bar), 0u, p.err);
+                merges = true;
+            }
         } else {
-            p.partials[((size_t)which * p.part_rows + k) * p.chunks + chunk] =
-                make_uint4((unsigned int)best, (unsigned int)(best >> 32), __float_as_uint(M), __float_as_uint(S));
-            // one release-acquire arrival at device scope: this thread's partial is visible to whoever arrives last,
-            // and the last one (then, behind the barrier below, its whole CTA) sees all of them
-            int* cnt = &p.row_cnt[which * HS_MAX_ROWS + k];
-            int old;
-            asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(old) : "l"(cnt) : "memory");
-            s_flag = (old == p.chunks - 1);
-            if (s_flag) *cnt = 0;
+            if (lane == 0) {
+                p.partials[((size_t)which * p.part_rows + k) * p.chunks + chunk] =
+                    make_uint4((unsigned int)key, (unsigned int)(key >> 32), __float_as_uint(M), __float_as_uint(S));
+                // one release-acquire arrival at device scope: this thread's partial is visible to whoever arrives last,
+                // and the last one sees all of them
+                int* cnt = &p.row_cnt[which * HS_MAX_ROWS + k];
+                int old;
+                asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(old) : "l"(cnt) : "memory");
+                merges = old == p.chunks - 1;
+                if (merges) *cnt = 0;
+            }
+            merges = __shfl_sync(HS_FULL_MASK, merges, 0);
+        }
+        if (merges) {
+            if (p.chunks > 1) {                            // (chunks <= 32, one lane per chunk)
+                unsigned long long ck = 0ull;
+                float cm = -CUDART_INF_F, cs = 0.f;
+                if (lane < p.chunks) {
+                    const uint4 q = p.clustered ? s_cl[lane] : __ldcg(&p.partials[((size_t)which * p.part_rows + k) * p.chunks + lane]);
+                    ck = ((unsigned long long)q.y << 32) | q.x;
+                    cm = __uint_as_float(q.z);
+                    cs = __uint_as_float(q.w);
+                    if (p.clustered && lane == 0) { ck = key; cm = M; cs = S; }
+                }
+                int src;
+                key = warp_best_key(ck, src);
+                M = warp_max(cm);
+                if (sampling) S = warp_sum((cm == -CUDART_INF_F) ? 0.f : cs * ex2a((cm - M) * invT));
+            }
+            if (lane == 0) {
+                s_flag = 1;
+                if (which == 0) {
+                    p.ro.tgt_arg[k] = key_index(key);
+                    p.ro.tgt_ms[k] = make_float2(M, S);
+                    if (md != HS_ACCEPT_REJECTION) {
+                        int old;
+                        asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(old) : "l"(&p.seq_cnt[b]) : "memory");
+                        if (old == nk - 1) { s_flag = 2; p.seq_cnt[b] = 0; }   // the sequence's last target row: walk its tree
+                    }
+                } else {
+                    p.ro.drf_ms[k] = make_float2(M, S);
+                }
+            }
         }
     }
-    if (p.clustered) {
-        cluster_arrive();
-        cluster_wait();
-    } else {
-        __syncthreads();
-    }
-    const bool merges = s_flag != 0;
-    // CTAs of a deterministic-proposal sequence stay to take slices of its bonus draw (where the whole grid is resident)
-    if (!merges && !(p.jobs && md == HS_ACCEPT_DETERMINISTIC && which == 0)) return;
-    if (merges && warp == 0) {
-    // the CTA that merges the row (chunks <= 32, one lane per chunk)
-    unsigned long long ck = 0ull;
-    float cm = -CUDART_INF_F, cs = 0.f;
-    if (lane < p.chunks) {
-        const uint4 q = p.clustered ? s_cl[lane] : __ldcg(&p.partials[((size_t)which * p.part_rows + k) * p.chunks + lane]);
-        ck = ((unsigned long long)q.y << 32) | q.x;
-        cm = __uint_as_float(q.z);
-        cs = __uint_as_float(q.w);
-    }
-    unsigned long long best = warp_max_u64(ck);
-    float M = warp_max(cm), S = 0.f;
-    if (sampling) {
-        const float invT = LOG2E / p.temperature[b];
-        S = warp_sum((cm == -CUDART_INF_F) ? 0.f : cs * ex2a((cm - M) * invT));
-    }
-    if (lane == 0) {
-        if (which == 0) {
-            p.ro.tgt_arg[k] = key_index(best);
-            p.ro.tgt_ms[k] = make_float2(M, S);
-        } else {
-            p.ro.drf_ms[k] = make_float2(M, S);
-        }
-    }
-    }
-    // ---- greedy sequences finish here: the last target row of a sequence to be merged walks its tree ------
-    if (merges && md == HS_ACCEPT_REJECTION && !p.have_draft && which == 0 && i == 0) {
+    if (p.clustered && chunk != 0 && !(p.jobs && md == HS_ACCEPT_DETERMINISTIC && which == 0)) return;
+    __syncthreads();
+    const int flag = s_flag;
+    if (flag && md == HS_ACCEPT_REJECTION && !p.have_draft && which == 0 && i == 0) {
         // rejection sampling needs the draft distribution: the caller passed none
         const int cap = p.out.path_cap;
         for (int j = tid; j < cap; j += HS_ROW_THREADS) {
@@ -329,18 +371,12 @@ __global__ void __launch_bounds__(HS_ROW_THREADS, 4) accept_rows_kernel(const __
         }
     }
     if (which != 0 || md == HS_ACCEPT_REJECTION) return;
-    __syncthreads();
-    if (tid == 0 && merges) {                      // (the thread that wrote the row's merged result)
-        int old;
-        asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(old) : "l"(&p.seq_cnt[b]) : "memory");
-        s_flag = (old == nk - 1);
-        if (s_flag) p.seq_cnt[b] = 0;
-    }
-    __syncthreads();
+    // greedy sequences finish here; CTAs of a deterministic-proposal sequence stay to take slices of its bonus draw (where
+    // the whole grid is resident)
     if (md == HS_ACCEPT_DETERMINISTIC) {
-        if (s_flag || p.jobs) det_chunk_tail(p, b, nk, merges && s_flag);
-    } else if (s_flag) {
-        greedy_walk(p, b);
+        if (flag == 2 || p.jobs) det_chunk_tail(p, b, nk, flag == 2);
+    } else if (flag == 2) {
+        greedy_walk(p, b, koff, nk, node);
     }
 }
 
@@ -759,7 +795,7 @@ hs_status hs_launch_accept(hs_ctx* ctx, const hs_tree_batch* tree, const hs_prun
     const size_t room = ctx->scratch_bytes > o ? (ctx->scratch_bytes - o) / (2 * sizeof(uint4)) : 0;
     p.shares = (int)min((size_t)ctx->sm_count * AW_WARPS, room);
     o += streamed ? (size_t)2 * p.shares * sizeof(uint4) : (size_t)2 * rows * p.chunks * sizeof(uint4);
-    if (o > ctx->scratch_bytes || (streamed && p.shares < 1)) return HS_ERR_WORKSPACE;
+    if (o > ctx->scratch_bytes || (streamed && p.shares < ctx->sm_count)) return HS_ERR_WORKSPACE;
     p.row_cnt = ctx->counters + HS_CNT_ACC_ROW;
     p.seq_cnt = ctx->counters + HS_CNT_ACC_SEQ;
     p.err = ctx->counters + HS_CNT_ERROR;

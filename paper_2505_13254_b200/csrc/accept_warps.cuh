@@ -20,19 +20,6 @@
 #define AW_MAX_SEGS 32                        // shares a row may lie in: one lane each when they merge
 #define AW_ROW_END 4                          // what the end of a row segment costs, in rounds
 
-// last b with off[b] <= k (skips empty sequences), by a whole warp
-__device__ __forceinline__ int sequence_of(const int* off, int batch, int k, int lane) {
-    int lo = 0, len = batch;
-    while (len > 1) {
-        const int step = (len + 31) / 32;
-        const bool le = lane * step < len && off[lo + lane * step] <= k;
-        const int n = __popc(__ballot_sync(HS_FULL_MASK, le));        // (off ascends: the lanes that agree are the first n)
-        lo += (n - 1) * step;
-        len = min(step, len - (n - 1) * step);
-    }
-    return lo;
-}
-
 template <bool BF16>
 __global__ void __launch_bounds__(AW_THREADS, 1) accept_warp_kernel(const __grid_constant__ AcceptParams p) {
     constexpr int VE = BF16 ? 8 : 4;
@@ -239,7 +226,10 @@ __global__ void __launch_bounds__(AW_THREADS, 1) accept_warp_kernel(const __grid
         const int npend = s_npending;
         for (int i = 0; i < npend; ++i) {
             const int b = s_pending[i];
-            if (p.mode[b] == HS_ACCEPT_GREEDY) greedy_walk(p, b);
+            if (p.mode[b] == HS_ACCEPT_GREEDY) {
+                const int koff = p.pr.keep_off[b], nk = p.pr.n_keep[b];
+                greedy_walk(p, b, koff, nk, load_walk_node(p, koff, nk, p.node_off[b]));
+            }
             else deterministic_walk(p, b);
             walk_sync();                       // the walks' shared arrays are free again
         }

@@ -411,7 +411,7 @@ static hs_status launch_warps(hs_ctx* ctx, QuantParams& p, hs_dtype dtype, cudaS
     const long long rr = (p.nvec + ROUND_VECS - 1) / ROUND_VECS, total = (rr + p.extra) * p.rows;
     const long long room = (long long)((ctx->scratch_bytes - 256) / (2 * (sizeof(float4) + HS_MAX_TOPK * 8)));
     const long long shares = min((long long)ctx->sm_count * QW_WARPS, room);
-    if (shares < 1) return HS_ERR_WORKSPACE;
+    if (ctx->scratch_bytes < 512 || shares < ctx->sm_count / 2) return HS_ERR_WORKSPACE;
     const long long per = max((total + shares - 1) / shares, (rr + QW_MAX_SEGS - 3) / (QW_MAX_SEGS - 2));
     p.per = (int)per;
     const int used = (int)((total + per - 1) / per);
@@ -440,6 +440,7 @@ hs_status hs_launch_quantify(hs_ctx* ctx, const hs_tree_batch* tree, const void*
     const int pv = parts ? (p.nvec + parts - 1) / parts : 0;
     cudaError_t e;
     if (parts && pv <= QS_SLOTS * QS_ITEM_VECS) {
+        if ((size_t)p.rows * parts * HS_ROW_PARTIAL_BYTES > ctx->scratch_bytes) return HS_ERR_WORKSPACE;   // (not sized for the batch)
         if (!ctx->quant_ready) {
             if (cudaFuncSetAttribute(quantify_cluster_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_BYTES) != cudaSuccess ||
                 cudaFuncSetAttribute(quantify_cluster_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_BYTES) != cudaSuccess)

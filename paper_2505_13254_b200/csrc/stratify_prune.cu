@@ -207,9 +207,10 @@ __device__ __forceinline__ int cta_sum(int part, PruneSmem& sm) {
 // Reranking and compaction of sequence b by its CTA (thread t = node t with depth `dep`, parent `par`, ln V `S`):
 // Top-N' among the nodes of depth <= d' by (S descending, index ascending), ballot + prefix compaction, parents
 // re-indexed, ancestor-or-self masks.  `offset_of(n_keep)` returns where the sequence starts in the compacted arrays.
+// `path`, `up`: the node's ancestors as the tree stage keeps them (NULL: followed through the parents).
 template <class OffsetFn>
 __device__ __forceinline__ void prune_cta(const PruneParams& p, int b, int n, int status, float phi_star, int dep,
-                                          int par, float S, PruneSmem& sm, OffsetFn offset_of) {
+                                          int par, float S, PruneSmem& sm, const int* path, int up, OffsetFn offset_of) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int bin = 0, dp = 0, np = 0;
     policy_lookup(p, phi_star, bin, dp, np);
@@ -242,12 +243,20 @@ __device__ __forceinline__ void prune_cta(const PruneParams& p, int b, int n, in
     if (keep) {
         const int k = off + before;
         unsigned long long m0 = 0ull, m1 = 0ull;
-        int a = tid;
-        for (int step = 0; step <= HS_MAX_NODES && a >= 0; ++step) {   // walk to the root
-            int na = sm.nw[a];
+        auto add = [&](int a) {
+            const int na = sm.nw[a];
             if (na >= 0) {
                 if (na < 64) m0 |= 1ull << na; else m1 |= 1ull << (na - 64);
             }
+        };
+        int a = tid;
+        if (path) {                            // (independent loads; 0 = the root, an ancestor of every node)
+#pragma unroll
+            for (int q = 0; q < TS_PATH; ++q) add(path[q]);
+            a = up;
+        }
+        for (int step = 0; step <= HS_MAX_NODES && a >= 0; ++step) {   // walk to the root
+            add(a);
             a = sm.par[a];
         }
         p.out.keep_idx[k] = tid;
@@ -284,7 +293,7 @@ __global__ void __launch_bounds__(HS_MAX_NODES) stratify_prune_kernel(const Prun
         par = p.parent[base + tid];
         S = p.score[base + tid];
     }
-    prune_cta(p, b, n, status, p.phi_star[b], dep, par, S, sm, [&](int) {
+    prune_cta(p, b, n, status, p.phi_star[b], dep, par, S, sm, nullptr, 0, [&](int) {
         // offset of this sequence in the compacted arrays: the kept counts of the sequences ahead
         int part = 0;
         if (p.counted) {
@@ -326,10 +335,9 @@ __global__ void __launch_bounds__(HS_MAX_NODES) tree_prune_kernel(const __grid_c
     const int b = blockIdx.x;
     pdl_launch_dependents();
     const TreeStageResult t = tree_stage_cta(p, b, tsm);
-    __syncthreads();                                   // tsm.phi_star
     const int n = min(max(t.n, 0), HS_MAX_NODES);
     const int status = t.bad ? HS_ERR_BAD_TREE : HS_OK;
-    prune_cta(p.pr, b, n, status, t.bad ? 0.f : tsm.phi_star, t.dep, t.bad ? -1 : t.par, t.S, sm, [&](int n_keep) {
+    prune_cta(p.pr, b, n, status, t.phi_star, t.dep, t.bad ? -1 : t.par, t.S, sm, t.path, t.up, [&](int n_keep) {
         if (p.pr.batch == 1) return 0;
         if (tid == 0) st_release_gpu(&p.flags[b], n_keep + 1);
         int part = 0;

@@ -9,12 +9,13 @@
 #include "hs_layout.h"
 #include "hs_ptx.cuh"
 
+#define TS_PATH 12          // ancestors a thread keeps in registers; deeper trees walk on from there
+
 struct TreeStageSmem {
     float logc[HS_MAX_NODES], I[HS_MAX_NODES], phi[HS_MAX_NODES];
     int par[HS_MAX_NODES];
     unsigned long long best[4];
     int maxd[4];
-    float phi_star;
 };
 
 struct TreeStageResult {   // of the calling thread's node (thread t = node t)
@@ -22,12 +23,16 @@ struct TreeStageResult {   // of the calling thread's node (thread t = node t)
     bool bad;              // the sequence was flagged (empty, too large or malformed); its outputs are written
     int par, dep;
     float S;               // ln V of the node
+    float phi_star;        // of the sequence
+    int path[TS_PATH];     // the node and its ancestors below the root, 0 behind them
+    int up;                // where the path goes on (0: nowhere)
 };
 
 // P needs: logits, row_stride, vocab, is_bf16, node_off, parent, token, out (hs_quant_out), d_base, phi_mode,
 // pstar_mode, entropy_mode.  Calls griddepcontrol.wait once: the row statistics come from the launch ahead.  The tree and the
-// token logits are inputs of the call; they are fetched before that wait, which is allowed because the launch ahead lets
-// this one start only when they are complete (three dependent round trips to L2, hidden behind the row pass).
+// token logits are inputs of the call; they are fetched, and all that follows from the parents alone (depths, paths) is done,
+// before that wait, which is allowed because the launch ahead lets this one start only when they are complete: three
+// dependent round trips to L2 and the pointer chase hide behind the row pass, and the sums along a path are independent loads.
 template <class P>
 __device__ __forceinline__ TreeStageResult tree_stage_cta(const P& p, int b, TreeStageSmem& sm) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -48,11 +53,14 @@ __device__ __forceinline__ TreeStageResult tree_stage_cta(const P& p, int b, Tre
         const size_t off = (size_t)(base + par) * p.row_stride + tok;
         lv = p.is_bf16 ? __bfloat162float(((const __nv_bfloat16*)p.logits)[off]) : ((const float*)p.logits)[off];
     }
-    pdl_wait();
+    sm.par[tid] = par;
     bad = __syncthreads_or(bad);
     r.bad = bad != 0;
-    r.par = par; r.dep = 0; r.S = 0.f;
+    r.par = par; r.dep = 0; r.S = 0.f; r.phi_star = 0.f; r.up = 0;
+#pragma unroll
+    for (int q = 0; q < TS_PATH; ++q) r.path[q] = 0;
     if (bad) {
+        pdl_wait();
         for (int i = tid; i < n; i += blockDim.x) {
             p.out.logc[base + i] = 0.f; p.out.score[base + i] = 0.f; p.out.phi[base + i] = 0.f;
             p.out.depth[base + i] = 0;
@@ -60,22 +68,46 @@ __device__ __forceinline__ TreeStageResult tree_stage_cta(const P& p, int b, Tre
         if (tid == 0) { p.out.status[b] = HS_ERR_BAD_TREE; p.out.pstar_node[b] = 0; p.out.phi_star[b] = 0.f; }
         return r;
     }
+    int dep = 0;
+    {
+        int a = tid < n ? tid : 0;
+#pragma unroll
+        for (int q = 0; q < TS_PATH; ++q) {
+            r.path[q] = a;
+            if (a > 0) { a = sm.par[a]; ++dep; }
+        }
+        r.up = a;
+        while (a > 0) { a = sm.par[a]; ++dep; }
+    }
+    r.dep = dep;
+    const int wmax = __reduce_max_sync(HS_FULL_MASK, dep);
+    if (lane == 0) sm.maxd[warp] = wmax;
+    pdl_wait();
     if (tid < n) {
         sm.logc[tid] = tid > 0 ? lv - p.out.row_lse[base + par] : 0.f;
         sm.I[tid] = p.entropy_mode == 0 ? p.out.i_topk[base + tid] : p.out.i_trunc[base + tid];
-        sm.par[tid] = par;
     }
     __syncthreads();
     float S = 0.f, Phi = 0.f;
-    int dep = 0;
+    // deepest level, then P* among the nodes of depth min(d_base, deepest)
+    const int md = max(max(sm.maxd[0], sm.maxd[1]), max(sm.maxd[2], sm.maxd[3]));
+    const int t_eval = min(p.d_base, md);
     if (tid < n) {
-        int a = tid;
+        float lc[TS_PATH], en[TS_PATH];
+#pragma unroll
+        for (int q = 0; q < TS_PATH; ++q) {
+            lc[q] = sm.logc[r.path[q]];
+            en[q] = sm.I[q + 1 < TS_PATH ? r.path[q + 1] : r.up];
+        }
+#pragma unroll
+        for (int q = 0; q < TS_PATH; ++q)
+            if (r.path[q] > 0) { S += lc[q]; Phi += en[q]; }
+        int a = r.up;
         while (a > 0) {
             const int pa = sm.par[a];
             S += sm.logc[a];
             Phi += sm.I[pa];
             a = pa;
-            ++dep;
         }
         if (p.phi_mode == 1) Phi += sm.I[tid];
         sm.phi[tid] = Phi;
@@ -84,27 +116,21 @@ __device__ __forceinline__ TreeStageResult tree_stage_cta(const P& p, int b, Tre
         p.out.phi[base + tid] = Phi;
         p.out.depth[base + tid] = dep;
     }
-    r.dep = dep; r.S = S;
-    // deepest level, then P* among the nodes of depth min(d_base, deepest)
-    int md = dep;
+    r.S = S;
+    const bool cand = tid < n && dep == t_eval;
+    const unsigned int hi = cand ? float_order_bits(p.pstar_mode == 0 ? sm.logc[tid] : S) : 0u;
+    const unsigned int mh = __reduce_max_sync(HS_FULL_MASK, hi);
+    const unsigned int ml = __reduce_max_sync(HS_FULL_MASK, cand && hi == mh ? ~(unsigned int)tid : 0u);
+    if (lane == 0) sm.best[warp] = ((unsigned long long)mh << 32) | ml;
+    __syncthreads();
+    unsigned long long best = sm.best[0];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) md = max(md, __shfl_xor_sync(HS_FULL_MASK, md, o));
-    if (lane == 0) sm.maxd[warp] = md;
-    __syncthreads();
-    md = max(max(sm.maxd[0], sm.maxd[1]), max(sm.maxd[2], sm.maxd[3]));
-    const int t_eval = min(p.d_base, md);
-    unsigned long long key = 0ull;
-    if (tid < n && dep == t_eval) key = make_key(p.pstar_mode == 0 ? sm.logc[tid] : S, tid);
-    key = warp_max_u64(key);
-    if (lane == 0) sm.best[warp] = key;
-    __syncthreads();
+    for (int w = 1; w < 4; ++w) best = sm.best[w] > best ? sm.best[w] : best;
+    const int node = key_index(best);
+    r.phi_star = sm.phi[node];
     if (tid == 0) {
-        unsigned long long best = sm.best[0];
-        for (int w = 1; w < 4; ++w) best = sm.best[w] > best ? sm.best[w] : best;
-        const int node = key_index(best);
-        sm.phi_star = sm.phi[node];
         p.out.pstar_node[b] = node;
-        p.out.phi_star[b] = sm.phi[node];
+        p.out.phi_star[b] = r.phi_star;
         p.out.status[b] = HS_OK;
     }
     return r;
