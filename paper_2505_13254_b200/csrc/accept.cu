@@ -383,8 +383,8 @@ __global__ void __launch_bounds__(HS_ROW_THREADS, 4) accept_rows_kernel(const __
 #include "accept_warps.cuh"
 
 // Launches with fewer bytes of rows (draft rows counted like target rows) go to the chunk kernel, whose loads are all in flight
-// at once.  60 greedy rows of 128256 bf16 (15 MB): 8.6 us against 9.4; with draft rows (31 MB) 23.8 against 19.3, 120 greedy rows
-// 15.1 against 12.6, 347 rows of 32000 (22 MB) 13.8 against 11.6.
+// at once.  60 greedy rows of 128256 bf16 (15 MB): 6.4 us against 9.4; with draft rows (31 MB) 18.9 against 19.3, 120 greedy rows
+// (31 MB) 13.1 against 12.5.
 #define AW_MIN_BYTES ((size_t)20 << 20)
 
 // ---- the walk ----------------------------------------------------------------------------------

@@ -14,7 +14,10 @@
 // shared memory and pushes each owner's rows there by bulk copies through distributed shared memory;
 // an owner merges its rows once all pieces have landed.  No partial ever goes to global memory and
 // there is no second launch.
+//
+// Launches of more than one wave of such CTAs go to tree_attn_duo.cuh, where two CTAs share an SM.
 #include <math_constants.h>
+#include <algorithm>
 
 #include "hs_common.cuh"
 #include "hs_layout.h"
@@ -52,6 +55,26 @@ struct AttnParams {
 __device__ __forceinline__ unsigned int pack_bf16(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<unsigned int*>(&v);
+}
+// 4 x 4 transpose of 16-byte chunks over four lanes: lane q then holds chunk q of the four rows, and 64 bytes of a row leave in
+// one instruction (a lane storing its own row touched 32 cache lines with every instruction).
+__device__ __forceinline__ void quad_transpose(uint4 (&o)[4], int lane) {
+    auto swap = [&](uint4& a, uint4& b, int m) {                  // a of the upper lane <-> b of the lower one
+        const bool up = (lane & m) != 0;
+        uint4 x = up ? a : b;
+        x.x = __shfl_xor_sync(HS_FULL_MASK, x.x, m); x.y = __shfl_xor_sync(HS_FULL_MASK, x.y, m);
+        x.z = __shfl_xor_sync(HS_FULL_MASK, x.z, m); x.w = __shfl_xor_sync(HS_FULL_MASK, x.w, m);
+        if (up) a = x; else b = x;
+    };
+    swap(o[0], o[1], 1); swap(o[2], o[3], 1);
+    swap(o[0], o[2], 2); swap(o[1], o[3], 2);
+}
+// acc += w * (eight bf16 values)
+__device__ __forceinline__ void fma_bf16x8(float (&acc)[8], float w, uint4 v) {
+    acc[0] = fmaf(w, bf16_lo(v.x), acc[0]); acc[1] = fmaf(w, bf16_hi(v.x), acc[1]);
+    acc[2] = fmaf(w, bf16_lo(v.y), acc[2]); acc[3] = fmaf(w, bf16_hi(v.y), acc[3]);
+    acc[4] = fmaf(w, bf16_lo(v.z), acc[4]); acc[5] = fmaf(w, bf16_hi(v.z), acc[5]);
+    acc[6] = fmaf(w, bf16_lo(v.w), acc[6]); acc[7] = fmaf(w, bf16_hi(v.w), acc[7]);
 }
 // byte offset of (key row, 16-byte chunk 0..15 of the 128 d's) inside a swizzled 64x128 bf16 tile:
 // two halves of 64 d's, rows of 128 bytes, chunk index XOR-ed with the row (the TMA 128-byte swizzle)
@@ -523,18 +546,8 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
                 o[q].z = pack_bf16(__uint_as_float(ov[q * 8 + 4]) * inv, __uint_as_float(ov[q * 8 + 5]) * inv);
                 o[q].w = pack_bf16(__uint_as_float(ov[q * 8 + 6]) * inv, __uint_as_float(ov[q * 8 + 7]) * inv);
             }
-            // 4 x 4 transpose over four lanes: lane q then holds chunk q of the four rows, and 64 bytes of a row leave in one
-            // instruction (a lane storing its own row touched 32 cache lines with every instruction)
             const int lane = tid & 31;
-            auto swap = [&](uint4& a, uint4& b, int m) {                  // a of the upper lane <-> b of the lower one
-                const bool up = (lane & m) != 0;
-                uint4 x = up ? a : b;
-                x.x = __shfl_xor_sync(HS_FULL_MASK, x.x, m); x.y = __shfl_xor_sync(HS_FULL_MASK, x.y, m);
-                x.z = __shfl_xor_sync(HS_FULL_MASK, x.z, m); x.w = __shfl_xor_sync(HS_FULL_MASK, x.w, m);
-                if (up) a = x; else b = x;
-            };
-            swap(o[0], o[1], 1); swap(o[2], o[3], 1);
-            swap(o[0], o[2], 2); swap(o[1], o[3], 2);
+            quad_transpose(o, lane);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int dst = __shfl_sync(HS_FULL_MASK, (int)orow, (lane & ~3) + i);
@@ -620,11 +633,7 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
             for (int s2 = 0; s2 < ATT_MAX_SPLIT; ++s2) {
                 if (s2 < ns) {
                     const float w = s_wt[rl * ATT_MAX_SPLIT + s2];
-                    const uint4 v = *reinterpret_cast<const uint4*>(po + (size_t)(s2 * rows_max + rl) * ATT_PB_STRIDE + c8 * 16);
-                    acc[0] = fmaf(w, bf16_lo(v.x), acc[0]); acc[1] = fmaf(w, bf16_hi(v.x), acc[1]);
-                    acc[2] = fmaf(w, bf16_lo(v.y), acc[2]); acc[3] = fmaf(w, bf16_hi(v.y), acc[3]);
-                    acc[4] = fmaf(w, bf16_lo(v.z), acc[4]); acc[5] = fmaf(w, bf16_hi(v.z), acc[5]);
-                    acc[6] = fmaf(w, bf16_lo(v.w), acc[6]); acc[7] = fmaf(w, bf16_hi(v.w), acc[7]);
+                    fma_bf16x8(acc, w, *reinterpret_cast<const uint4*>(po + (size_t)(s2 * rows_max + rl) * ATT_PB_STRIDE + c8 * 16));
                 }
             }
             const long long og = s_og[rl];
@@ -640,29 +649,34 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem_base, UM_TMEM_COLS);
 }
+#include "tree_attn_duo.cuh"
+
+// ---- host side -----------------------------------------------------------------------------------------------------
 typedef CUresult (*encode_tiled_fn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                     const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                     CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+static bool encode(hs_ctx* ctx, CUtensorMap* tm, int rank, const void* base, const cuuint64_t* gdim, const cuuint64_t* gstr,
+                   const cuuint32_t* box) {
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return ((encode_tiled_fn)ctx->encode_tiled)(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), gdim, gstr,
+                                                box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 static bool make_kv_map(hs_ctx* ctx, CUtensorMap* tm, const void* base, const hs_attn_desc* d, bool head_first) {
-    cuuint64_t gdim[3], gstr[2];
-    cuuint32_t box[3], estr[3] = {1, 1, 1};
-    gdim[0] = HS_HEAD_DIM;
-    box[0] = 64;
-    if (head_first) {        // (d, token, head): token stride is the smaller one
-        gdim[1] = (cuuint64_t)d->kv_total; gdim[2] = (cuuint64_t)d->hkv;
-        gstr[0] = (cuuint64_t)d->kv_token_stride * 2; gstr[1] = (cuuint64_t)d->kv_head_stride * 2;
-        box[1] = ATT_BN; box[2] = 1;
-    } else {                 // (d, head, token)
-        gdim[1] = (cuuint64_t)d->hkv; gdim[2] = (cuuint64_t)d->kv_total;
-        gstr[0] = (cuuint64_t)d->kv_head_stride * 2; gstr[1] = (cuuint64_t)d->kv_token_stride * 2;
-        box[1] = 1; box[2] = ATT_BN;
-    }
-    CUresult r = ((encode_tiled_fn)ctx->encode_tiled)(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base),
-                                                     gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                                     CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                                                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS;
+    const cuuint64_t tok = (cuuint64_t)d->kv_total, heads = (cuuint64_t)d->hkv;
+    const cuuint64_t ts = (cuuint64_t)d->kv_token_stride * 2, hs = (cuuint64_t)d->kv_head_stride * 2;
+    // (d, token, head) if the token stride is the smaller one, else (d, head, token)
+    const cuuint64_t gdim[3] = {HS_HEAD_DIM, head_first ? tok : heads, head_first ? heads : tok};
+    const cuuint64_t gstr[2] = {head_first ? ts : hs, head_first ? hs : ts};
+    const cuuint32_t box[3] = {64, head_first ? (cuuint32_t)ATT_BN : 1u, head_first ? 1u : (cuuint32_t)ATT_BN};
+    return encode(ctx, tm, 3, base, gdim, gstr, box);
+}
+// rows of `width` elements, gathered one by one (box one row high)
+static bool make_row_map(hs_ctx* ctx, CUtensorMap* tm, const void* base, size_t rows, size_t width) {
+    const cuuint64_t gdim[2] = {(cuuint64_t)width, (cuuint64_t)rows}, gstr[1] = {(cuuint64_t)width * 2};
+    const cuuint32_t box[2] = {64, 1};
+    return encode(ctx, tm, 2, base, gdim, gstr, box);
 }
 
 // KV splits (= cluster size): the one with the fewest tile steps on the critical path, waves of CTAs (as
@@ -678,6 +692,31 @@ static int choose_splits(int base_ctas, int sm_count, int prefix_tiles, const in
         const long waves = (ctas + cap - 1) / cap;
         const long cost = waves * ((prefix_tiles + s - 1) / s + 2 + (s > 1 ? 2 : 0));   // + tree tiles, + merge
         if (s == 1 || cost < best_cost) { best_cost = cost; best = s; }
+    }
+    return best;
+}
+
+// Splits with which tree_attn_duo_kernel takes a launch, 0: it does not.  Two CTAs of it on an SM take 0.53 us per tile and about 10 us
+// at their ends, which overlap with the other CTA's tiles; one alone takes 0.9 us per tile at worst.  The other kernel takes 0.585 us per
+// tile and the same 10 us, which nothing overlaps.  With more blocks than SMs that kernel therefore pays for whole waves of CTAs
+// (less where lengths are mixed: 0.85).  Measured, other kernel against this one (192 to 512 blocks): 12 x 37..46 nodes, 32 / 8 heads,
+// 1200 tokens 50 us against 30; 6 x 42..59, 64 / 8, 1500..2160 tokens 56 against 38; 16 x 56, 64 / 8, 1700 tokens 87 against 70; 16 x 39..56,
+// 32 / 8, 1200..3160 tokens 52 against 53; 16 x 8..60, 32 / 8, 1024..8192 tokens 75 against 125 (75 with two splits).  With at most one block
+// per SM two splits are needed to share SMs at all, and what the merge costs is only won back by long prefixes: 4 x 60 nodes, 64 / 8 heads,
+// 32768 tokens 304 against 273, 6 x 31..48, 64 / 8, 8000 tokens 81 against 82, 4 x 59, 64 / 8, 2000..3400 tokens 35 against 37.  Up to 128 query
+// rows per head a launch is bound by its bytes and the other kernel has more of them in flight: 60.6 against 63.0.
+static int duo_splits(int base_ctas, int mblocks, int sm_count, int prefix_tiles, double mean_tiles) {
+    if (mblocks == 1) return 0;
+    if (base_ctas <= sm_count)
+        return 4 * base_ctas > 3 * sm_count && prefix_tiles >= 256 && mean_tiles >= 0.9 * prefix_tiles ? 2 : 0;
+    int best = 0;
+    double best_us = 0.85 * ((base_ctas + sm_count - 1) / sm_count) * (mean_tiles * 0.585 + 10.);
+    for (int s = 1; s <= ATT_MAX_SPLIT && (s == 1 || s <= prefix_tiles); ++s) {
+        const double longest = 10. + 0.9 * ((prefix_tiles + s) / s);
+        // (clusters that do not all run at once leave SMs idle at the end: half a CTA's time)
+        const double all = base_ctas * (mean_tiles * 0.53 + s * 10. / 2) / sm_count + (s > 1 && base_ctas * s > 2 * sm_count ? longest / 2 : 0.);
+        const double us = std::max(longest, all);
+        if (us < best_us) { best_us = us; best = s; }
     }
     return best;
 }
@@ -708,6 +747,8 @@ hs_status hs_launch_attention(hs_ctx* ctx, const hs_pruned_tree* pruned, const h
         if (cudaFuncSetAttribute(tree_attn_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, UM_SMEM_BYTES) !=
             cudaSuccess)
             return HS_ERR_CUDA;
+        if (cudaFuncSetAttribute(tree_attn_duo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AD_SMEM_BYTES) != cudaSuccess)
+            return HS_ERR_CUDA;
         query_cluster_caps(tree_attn_umma_kernel, UM_THREADS, UM_SMEM_BYTES, ctx->sm_count, cap_umma);
         ctx->attn_ready = true;
     }
@@ -734,19 +775,32 @@ hs_status hs_launch_attention(hs_ctx* ctx, const hs_pruned_tree* pruned, const h
     p.scale_log2 = d->sm_scale * LOG2E;
     p.err = ctx->counters + HS_CNT_ERROR;
     p.prefetch = (ctx->prefetch & HS_PREFETCH_KV) != 0;
-    const int pairs = d->batch * d->hkv;
-    const int mblocks = (p.G * d->max_nodes + ATT_BM - 1) / ATT_BM;
-    const int prefix_tiles = (d->max_kv_len + ATT_BN - 1) / ATT_BN;
-    p.nsplit = choose_splits(pairs * mblocks, ctx->sm_count, prefix_tiles, cap_umma);
+    const int pairs = d->batch * d->hkv, rows = p.G * d->max_nodes;
 
     CUtensorMap tmK, tmV;
     memset(&tmK, 0, sizeof(tmK));
     memset(&tmV, 0, sizeof(tmV));
+    const int mblocks = (rows + ATT_BM - 1) / ATT_BM;
+    const int prefix_tiles = (d->max_kv_len + ATT_BN - 1) / ATT_BN;
+    const int duo = duo_splits(pairs * mblocks, mblocks, ctx->sm_count, prefix_tiles, (double)d->kv_total / ATT_BN / d->batch + 1.5);
+    p.nsplit = duo ? duo : choose_splits(pairs * mblocks, ctx->sm_count, prefix_tiles, cap_umma);
     if (d->kv_total > 0) {
         if (!make_kv_map(ctx, &tmK, k_cache, d, p.head_first) || !make_kv_map(ctx, &tmV, v_cache, d, p.head_first))
             return HS_ERR_CUDA;
     }
     const dim3 grid(mblocks, p.nsplit, pairs), cl(1, p.nsplit, 1);
-    cudaError_t e = hs_launch(tree_attn_umma_kernel, grid, dim3(UM_THREADS), UM_SMEM_BYTES, stream, ctx->pdl, cl, p, tmK, tmV);
+    cudaError_t e;
+    if (duo) {
+        // (rows of the original trees may lie past max_rows, a bound of the kept ones, but not past HS_MAX_NODES per sequence)
+        const size_t n = std::max((size_t)d->max_rows, (size_t)d->batch * HS_MAX_NODES);
+        const size_t w = (size_t)d->hkv * HS_HEAD_DIM;
+        CUtensorMap tmQ, tmKT, tmVT;
+        if (!make_row_map(ctx, &tmQ, q, n * d->hq, HS_HEAD_DIM) || !make_row_map(ctx, &tmKT, k_tree, n, w) ||
+            !make_row_map(ctx, &tmVT, v_tree, n, w))
+            return HS_ERR_CUDA;
+        e = hs_launch(tree_attn_duo_kernel, grid, dim3(AD_THREADS), AD_SMEM_BYTES, stream, ctx->pdl, cl, p, tmK, tmV, tmQ, tmKT, tmVT);
+    } else {
+        e = hs_launch(tree_attn_umma_kernel, grid, dim3(UM_THREADS), UM_SMEM_BYTES, stream, ctx->pdl, cl, p, tmK, tmV);
+    }
     return e == cudaSuccess ? HS_OK : HS_ERR_CUDA;
 }
