@@ -5,13 +5,14 @@
 // 64 keys that are shared out evenly over the splits; a CTA requests its first tiles by TMA
 // (cp.async.bulk.tensor into 128-byte-swizzled shared memory, four stages, K and V on mbarriers of
 // their own) before it waits for the kernel ahead of it in the stream, because the cache does not
-// depend on the pruned tree.  The <= 128 tree keys are gathered with plain loads (their rows may be
-// indirect) and belong to the last split.  S = Q K^T and O += P V run on the 5th-generation tensor
+// depend on the pruned tree.  The <= 128 tree keys belong to the last split; their rows may be indirect.  Behind
+// prefix tiles the producer warp fetches them by tile::gather4 (plain loads by the softmax threads held up the
+// longest split: 4096 tokens, 64 / 8 heads 19.6 us against 18.0, a ragged batch of 16 75.5 against 71).  S = Q K^T and O += P V run on the 5th-generation tensor
 // cores (tcgen05.mma, accumulators in tensor memory) with fp32 accumulation; the softmax is the
 // online (running max / running sum) form in base 2.  Prefix columns are fully visible, tree column j
 // is visible to row r iff bit j of the ancestor mask of r's node is set.  The splits of one (query
-// block, head) form a thread-block cluster: every CTA stages its partial (max, sum, O) in its own
-// shared memory and pushes each owner's rows there by bulk copies through distributed shared memory;
+// block, head) form a thread-block cluster: every CTA sends its partial (max, sum, O) from registers
+// to the owner of each row by asynchronous stores through distributed shared memory;
 // an owner merges its rows once all pieces have landed.  No partial ever goes to global memory and
 // there is no second launch.
 //
@@ -119,7 +120,9 @@ __device__ __forceinline__ void prefix_range(int L, int nsplit, int split, int& 
 #define UM_SMEM_BYTES (UM_STAGES * ATT_STAGE_BYTES + ATT_Q_BYTES + UM_MAP_BYTES + 1024 + 2048 + UM_WT_BYTES + UM_RECV_BYTES + 1024)
 
 __global__ void __launch_bounds__(UM_THREADS, 1)
-tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV) {
+tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap tmK,
+                      const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmKT,
+                      const __grid_constant__ CUtensorMap tmVT) {
     extern __shared__ unsigned char smem_raw[];
     const int tid = threadIdx.x, warp = tid >> 5;
     // Sequences are taken longest prefix first (a ragged batch then ends on its short sequences, not on a long one
@@ -188,6 +191,7 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
         }
     };
     const int pre = min(np, UM_STAGES);
+    if (warp == 9 && (tid & 31) < 2) tma_prefetch_desc((tid & 31) ? &tmVT : &tmKT);
     if (tid == 0) {
         for (int i = 0; i < 4 * UM_STAGES + 4; ++i) mbar_init(bar0 + i * 8, 1);
         mbar_init(bar_p, UM_ROWS_THREADS);               // P of a tile is written: one arrival per thread of the stream
@@ -241,36 +245,53 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
     const int nt_tree = (split == p.nsplit - 1) ? (nk + ATT_BN - 1) / ATT_BN : 0;
     const int ntiles = np + nt_tree;
 
-    // tree keys and/or values of tile i: gathered rows, 16-byte loads (four of a thread's loads per matrix in flight
-    // together), swizzled stores; 1024 chunks per matrix by nthr threads (thread t of them), chunks t + (it0 .. it0 + 3) * nthr
-    auto gather_tree = [&](int i, int t, int nthr, int it0, bool do_k, bool do_v) {
-        unsigned char* gK = smem_gen + (i % UM_STAGES) * ATT_STAGE_BYTES;
+    // Tree tiles that open the pipeline (stages that no prefix tile uses): gathered rows by plain loads of the softmax threads, which
+    // have nothing else to do yet (0.6 us less than tile::gather4).  1024 chunks of 16 bytes per matrix, swizzled stores.
+    auto load_tree = [&](int i) {
+        unsigned char* gK = smem_gen + i * ATT_STAGE_BYTES;
         unsigned char* gV = gK + ATT_TILE_BYTES;
-        const int j0 = (i - np) * ATT_BN;
         uint4 kvv[4], vvv[4];
-        int trow[4];
+        int row4[4];
 #pragma unroll
         for (int it = 0; it < 4; ++it) {
-            const int j = j0 + ((t + (it0 + it) * nthr) >> 4);
-            trow[it] = -1;
-            if (j < nk) trow[it] = kept_row_of(j);
+            const int j = (i - np) * ATT_BN + ((tid + it * UM_SM_THREADS) >> 4);
+            row4[it] = j < nk ? kept_row_of(j) : -1;
         }
 #pragma unroll
         for (int it = 0; it < 4; ++it) {
             kvv[it] = make_uint4(0, 0, 0, 0);
             vvv[it] = make_uint4(0, 0, 0, 0);
-            if (trow[it] >= 0) {
-                const size_t off = ((size_t)trow[it] * p.hkv + h) * HS_HEAD_DIM + (t & 15) * 8;
-                if (do_k) kvv[it] = __ldg(reinterpret_cast<const uint4*>(p.k_tree + off));
-                if (do_v) vvv[it] = __ldg(reinterpret_cast<const uint4*>(p.v_tree + off));
+            if (row4[it] >= 0) {
+                const size_t off = ((size_t)row4[it] * p.hkv + h) * HS_HEAD_DIM + (tid & 15) * 8;
+                kvv[it] = __ldg(reinterpret_cast<const uint4*>(p.k_tree + off));
+                vvv[it] = __ldg(reinterpret_cast<const uint4*>(p.v_tree + off));
             }
         }
 #pragma unroll
         for (int it = 0; it < 4; ++it) {
-            const int c = t + (it0 + it) * nthr;
-            if (do_k) *reinterpret_cast<uint4*>(gK + tile_off(c >> 4, c & 15)) = kvv[it];
-            if (do_v) *reinterpret_cast<uint4*>(gV + tile_off(c >> 4, c & 15)) = vvv[it];
+            const int c = tid + it * UM_SM_THREADS;
+            *reinterpret_cast<uint4*>(gK + tile_off(c >> 4, c & 15)) = kvv[it];
+            *reinterpret_cast<uint4*>(gV + tile_off(c >> 4, c & 15)) = vvv[it];
         }
+    };
+    // The later ones by the producer warp: four tree rows per lane of half a warp, for each of the two tree tiles.  Keys past the last one repeat it
+    // (they are masked).
+    int trow[2][4];
+    if (warp == 9 && ntiles > np) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) trow[k >> 2][k & 3] = kept_row_of(min((k >> 2) * ATT_BN + (tid & 15) * 4 + (k & 3), nk - 1));
+    }
+    // K (V) of tree tile i (i >= np) into stage i % UM_STAGES; half a warp for each half of the columns
+    auto gather_tree = [&](int i, bool is_v) {
+        const int stage = i % UM_STAGES, lane = tid & 31;
+        const unsigned int dst = smem_base + stage * ATT_STAGE_BYTES + (is_v ? ATT_TILE_BYTES : 0);
+        const unsigned int bar = (is_v ? bar_v : bar0) + stage * 8;
+        if (lane == 0) mbar_expect_tx(bar, ATT_TILE_BYTES);
+        __syncwarp();
+        const bool second = i > np;
+        tma_gather4(dst + (lane >> 4) * (ATT_TILE_BYTES / 2) + (lane & 15) * 512, is_v ? &tmVT : &tmKT,
+                    h * HS_HEAD_DIM + (lane >> 4) * 64, second ? trow[1][0] : trow[0][0], second ? trow[1][1] : trow[0][1],
+                    second ? trow[1][2] : trow[0][2], second ? trow[1][3] : trow[0][3], bar);
     };
 
     // ---- query rows -> shared memory: 16 lanes per row (a thread fetching a row of its own touched 32 cache lines with
@@ -301,7 +322,7 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
         mk1 = p.anc_mask[2 * (size_t)(koff + node) + 1];
     }
     if (warp < 8)
-        for (int i = np; i < min(ntiles, UM_STAGES); ++i) gather_tree(i, tid, UM_SM_THREADS, 0, true, true);  // tree tiles that open the pipeline
+        for (int i = np; i < min(ntiles, UM_STAGES); ++i) load_tree(i);
     fence_proxy_async_smem();                        // generic stores -> visible to the tensor cores
     __syncthreads();
 
@@ -311,10 +332,10 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
     // shared-memory address reaches 2^18, so an offset is added to a descriptor built once.
     const unsigned long long dq0 = umma_desc_sw128(sQ, 16, 1024), dk0 = umma_desc_sw128(smem_base, 16, 1024);
     const unsigned long long dv0 = umma_desc_sw128(smem_base + ATT_TILE_BYTES, ATT_TILE_BYTES / 2, 1024);
-    // the issuing thread: S = Q K^T of tile i into S buffer i & 1 (waits for K if it comes by TMA), then commit
+    // the issuing thread: S = Q K^T of tile i into S buffer i & 1 (waits for K unless load_tree wrote it), then commit
     auto issue_qk = [&](int i) {
         const int stage = i % UM_STAGES;
-        if (i < np) mbar_wait(bar0 + stage * 8, (unsigned int)(i / UM_STAGES) & 1u, p.err);
+        if (i < np || i >= UM_STAGES) mbar_wait(bar0 + stage * 8, (unsigned int)(i / UM_STAGES) & 1u, p.err);
         tc_fence_after_sync();
         const unsigned long long dk = dk0 + (unsigned long long)(stage * (ATT_STAGE_BYTES >> 4));
         const unsigned int ts = tS + (i & 1) * ATT_BN;
@@ -325,12 +346,12 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
             umma_ss_bf16(ts, dq0 + (qoffb >> 4), dk + (koffb >> 4), idesc_qk, ks > 0 ? 1u : 0u);
         }
         umma_commit(bar_s + (i & 1) * 8);
-        if (i + UM_STAGES < np) umma_commit(bar_ek + stage * 8);     // (the producer waits for it only then)
+        if (i + UM_STAGES < ntiles) umma_commit(bar_ek + stage * 8);     // (the producer waits for it only then)
     };
-    // O of stream i & 1 += P V of tile i (waits for V if it comes by TMA), then commit
+    // O of stream i & 1 += P V of tile i (waits for V likewise), then commit
     auto issue_pv = [&](int i) {
         const int stage = i % UM_STAGES;
-        if (i < np) mbar_wait(bar_v + stage * 8, (unsigned int)(i / UM_STAGES) & 1u, p.err);
+        if (i < np || i >= UM_STAGES) mbar_wait(bar_v + stage * 8, (unsigned int)(i / UM_STAGES) & 1u, p.err);
         tc_fence_after_sync();
         const unsigned long long dv = dv0 + (unsigned long long)(stage * (ATT_STAGE_BYTES >> 4));
         const unsigned int tp = tP + (i & 1) * (ATT_BN / 2);
@@ -380,25 +401,26 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
         // The TMA producer, in the order in which the tensor pipe frees the stage halves: S runs four tiles ahead
         // of O += P V, so after the first K refills it is V of tile i + 4 (after P V of tile i), then K of tile i + 8
         // (after S of tile i + 4).
-#pragma unroll 1
-        for (int t = UM_STAGES; t < min(np, 2 * UM_STAGES); ++t) {
-            if (elect_one()) {
-                mbar_wait(bar_ek + (t % UM_STAGES) * 8, 0u, p.err);
-                issue_kv(t, false);
-            }
-            __syncwarp();
-        }
-#pragma unroll 1
-        for (int i = 0; i + UM_STAGES < np; ++i) {
-            if (elect_one()) {
-                mbar_wait(bar_ev + (i % UM_STAGES) * 8, (unsigned int)(i / UM_STAGES) & 1u, p.err);
-                issue_kv(i + UM_STAGES, true);
-                if (i + 2 * UM_STAGES < np) {
-                    mbar_wait(bar_ek + (i % UM_STAGES) * 8, (unsigned int)(i / UM_STAGES + 1) & 1u, p.err);
-                    issue_kv(i + 2 * UM_STAGES, false);
+        auto refill = [&](int i, bool is_v, unsigned int bar, unsigned int parity) {
+            if (i < np) {
+                if (elect_one()) {
+                    mbar_wait(bar, parity, p.err);
+                    issue_kv(i, is_v);
                 }
+            } else {
+                mbar_wait(bar, parity, p.err);
+                __syncwarp();
+                gather_tree(i, is_v);
             }
             __syncwarp();
+        };
+#pragma unroll 1
+        for (int t = UM_STAGES; t < min(ntiles, 2 * UM_STAGES); ++t) refill(t, false, bar_ek + (t % UM_STAGES) * 8, 0u);
+#pragma unroll 1
+        for (int i = 0; i + UM_STAGES < ntiles; ++i) {
+            refill(i + UM_STAGES, true, bar_ev + (i % UM_STAGES) * 8, (unsigned int)(i / UM_STAGES) & 1u);
+            if (i + 2 * UM_STAGES < ntiles)
+                refill(i + 2 * UM_STAGES, false, bar_ek + (i % UM_STAGES) * 8, (unsigned int)(i / UM_STAGES + 1) & 1u);
         }
     }
     // Stream `half`: tiles half, half + 2, ...  As soon as S of tile i is in registers its buffer is handed back.  The
@@ -466,20 +488,9 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
         }
         const float2 ls = add2_ftz(ls0, ls1);
         lrun = fmaf(lrun, corr, ls.x + ls.y);
-        // Tree tiles are gathered by the stream two and four tiles ahead of their use, where the stage half is free
-        // and this tile's P-written arrival publishes the stores before the issuing thread needs them: K of tile
-        // i + 4 (its stage's K was read by S of tile i, complete), V of tile i + 2 (after O += P V of tile i - 2).
-        if (i + UM_STAGES < ntiles && i + UM_STAGES >= np) {
-            gather_tree(i + UM_STAGES, row, UM_ROWS_THREADS, 0, true, false);
-            gather_tree(i + UM_STAGES, row, UM_ROWS_THREADS, 4, true, false);
-        }
         if (i >= 2) {
             mbar_wait(bar_ev + ((i - 2) % UM_STAGES) * 8, (unsigned int)((i - 2) / UM_STAGES) & 1u, p.err);
             tc_fence_after_sync();
-            if (i + 2 < ntiles && i + 2 >= np) {
-                gather_tree(i + 2, row, UM_ROWS_THREADS, 0, false, true);
-                gather_tree(i + 2, row, UM_ROWS_THREADS, 4, false, true);
-            }
         }
         // rescale this stream's O (the load/store are warp-wide: a warp rescales if any of its rows needs it)
         if (i >= 2 && __any_sync(HS_FULL_MASK, corr != 1.f)) {
@@ -497,7 +508,6 @@ tree_attn_umma_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm
         // P stays in tensor memory (the A operand of O += P V): this row's 64 bf16 values are 32 columns of its lane
         tmem_st32(tP + half * (ATT_BN / 2) + lane_off, reinterpret_cast<unsigned int*>(pk));
         tmem_wait_st();
-        if (i + UM_STAGES >= np) fence_proxy_async_smem();   // gathered tree tiles (generic stores) -> tensor cores
         tc_fence_before_sync();
         mbar_arrive(bar_p + half * 8);
     }
@@ -790,17 +800,16 @@ hs_status hs_launch_attention(hs_ctx* ctx, const hs_pruned_tree* pruned, const h
     }
     const dim3 grid(mblocks, p.nsplit, pairs), cl(1, p.nsplit, 1);
     cudaError_t e;
+    // (rows of the original trees may lie past max_rows, a bound of the kept ones, but not past HS_MAX_NODES per sequence)
+    const size_t n = std::max((size_t)d->max_rows, (size_t)d->batch * HS_MAX_NODES);
+    const size_t w = (size_t)d->hkv * HS_HEAD_DIM;
+    CUtensorMap tmQ, tmKT, tmVT;
+    if (!make_row_map(ctx, &tmKT, k_tree, n, w) || !make_row_map(ctx, &tmVT, v_tree, n, w)) return HS_ERR_CUDA;
     if (duo) {
-        // (rows of the original trees may lie past max_rows, a bound of the kept ones, but not past HS_MAX_NODES per sequence)
-        const size_t n = std::max((size_t)d->max_rows, (size_t)d->batch * HS_MAX_NODES);
-        const size_t w = (size_t)d->hkv * HS_HEAD_DIM;
-        CUtensorMap tmQ, tmKT, tmVT;
-        if (!make_row_map(ctx, &tmQ, q, n * d->hq, HS_HEAD_DIM) || !make_row_map(ctx, &tmKT, k_tree, n, w) ||
-            !make_row_map(ctx, &tmVT, v_tree, n, w))
-            return HS_ERR_CUDA;
+        if (!make_row_map(ctx, &tmQ, q, n * d->hq, HS_HEAD_DIM)) return HS_ERR_CUDA;
         e = hs_launch(tree_attn_duo_kernel, grid, dim3(AD_THREADS), AD_SMEM_BYTES, stream, ctx->pdl, cl, p, tmK, tmV, tmQ, tmKT, tmVT);
     } else {
-        e = hs_launch(tree_attn_umma_kernel, grid, dim3(UM_THREADS), UM_SMEM_BYTES, stream, ctx->pdl, cl, p, tmK, tmV);
+        e = hs_launch(tree_attn_umma_kernel, grid, dim3(UM_THREADS), UM_SMEM_BYTES, stream, ctx->pdl, cl, p, tmK, tmV, tmKT, tmVT);
     }
     return e == cudaSuccess ? HS_OK : HS_ERR_CUDA;
 }
