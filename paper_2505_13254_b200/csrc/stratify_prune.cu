@@ -25,7 +25,7 @@ struct PruneParams {
     const int* qstatus;
     hs_pruned_tree out;
     int counted;           // out.n_keep was filled by a launch ahead (prune_count_kernel or budget_kernel)
-    const int* n_override; // [B] node counts that replace the policy's N' (budget reallocation), or NULL
+    const int* n_override; // [B] node counts that replace the policy's N' (budget reallocation of large batches), or NULL
     int* base;             // [B] budget path: policy request min(N', eligible), 0 for a flagged sequence
     int* room;             // [B] budget path: eligible nodes
     const int* slo_class;  // [B] budget path
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(128) prune_count_kernel(const PruneParams p) {
     if (lane == 0) p.out.n_keep[b] = cnt;
 }
 
-// budget path, first launch: one warp per sequence, the policy's request and the eligible nodes
+// budget path of large batches, first launch: one warp per sequence, the policy's request and the eligible nodes
 __global__ void __launch_bounds__(128) budget_request_kernel(const PruneParams p) {
     const int lane = threadIdx.x & 31;
     const int b = blockIdx.x * 4 + (threadIdx.x >> 5);
@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(128) budget_request_kernel(const PruneParams p
     if (lane == 0) { p.base[b] = base; p.room[b] = elig; }
 }
 
-// budget path, second launch (one CTA): App. A.8 reading - if the requests fit the budget the left-over tokens go to
+// budget path of large batches, second launch (one CTA): App. A.8 reading - if the requests fit the budget the left-over tokens go to
 // the sequences in order of SLO class (stricter first, then sequence index), each up to its eligible nodes;
 // otherwise the excess is taken back in the opposite order, never below the root.  The order is found by a
 // bitonic sort of (class, index) keys in shared memory, the hand-out by a running sum along that order.
@@ -207,10 +207,11 @@ __device__ __forceinline__ int cta_sum(int part, PruneSmem& sm) {
 // Reranking and compaction of sequence b by its CTA (thread t = node t with depth `dep`, parent `par`, ln V `S`):
 // Top-N' among the nodes of depth <= d' by (S descending, index ascending), ballot + prefix compaction, parents
 // re-indexed, ancestor-or-self masks.  `offset_of(n_keep)` returns where the sequence starts in the compacted arrays.
-// `path`, `up`: the node's ancestors as the tree stage keeps them (NULL: followed through the parents).
+// `path`, `up`: the node's ancestors as the tree stage keeps them (NULL: followed through the parents).  `count`: the node count
+// that replaces N' (budget reallocation), -1: none.
 template <class OffsetFn>
 __device__ __forceinline__ void prune_cta(const PruneParams& p, int b, int n, int status, float phi_star, int dep,
-                                          int par, float S, PruneSmem& sm, const int* path, int up, OffsetFn offset_of) {
+                                          int par, float S, PruneSmem& sm, const int* path, int up, int count, OffsetFn offset_of) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int bin = 0, dp = 0, np = 0;
     policy_lookup(p, phi_star, bin, dp, np);
@@ -229,7 +230,7 @@ __device__ __forceinline__ void prune_cta(const PruneParams& p, int b, int n, in
                     (v.z > S || (v.z == S && j + 2 < tid)) + (v.w > S || (v.w == S && j + 3 < tid));
         }
     }
-    const bool keep = elig && rank < (p.n_override ? p.n_override[b] : np);
+    const bool keep = elig && rank < (count >= 0 ? count : np);
     // compaction: ballot inside the warp, prefix over the four warps
     const unsigned int bal = __ballot_sync(HS_FULL_MASK, keep);
     if (lane == 0) sm.warp[warp] = __popc(bal);
@@ -293,7 +294,8 @@ __global__ void __launch_bounds__(HS_MAX_NODES) stratify_prune_kernel(const Prun
         par = p.parent[base + tid];
         S = p.score[base + tid];
     }
-    prune_cta(p, b, n, status, p.phi_star[b], dep, par, S, sm, nullptr, 0, [&](int) {
+    const int count = p.n_override ? p.n_override[b] : -1;
+    prune_cta(p, b, n, status, p.phi_star[b], dep, par, S, sm, nullptr, 0, count, [&](int) {
         // offset of this sequence in the compacted arrays: the kept counts of the sequences ahead
         int part = 0;
         if (p.counted) {
@@ -303,6 +305,89 @@ __global__ void __launch_bounds__(HS_MAX_NODES) stratify_prune_kernel(const Prun
         }
         return cta_sum(part, sm);
     });
+}
+
+// Budget path of batches up to HS_MAX_NODES sequences, one launch: every CTA works out the requests and the reallocation of the
+// whole batch itself (thread t = sequence t; the order of service is a comparison of (class, index) keys, the hand-out a sum over the
+// sequences served before) and then prunes its own sequence.  Bound by latency: three launches, each with a round trip for
+// what the one before left in global memory, took 16 us of which about 11 us showed in a step of 32 sequences.
+#define BP_SEQS 4                                    // sequences a warp counts at a time: their depths are in flight together
+__global__ void __launch_bounds__(HS_MAX_NODES) budget_prune_kernel(const PruneParams p) {
+    __shared__ PruneSmem sm;
+    __shared__ int4 s_seq[HS_MAX_NODES];             // {first node, nodes (0: flagged), d', N'}
+    __shared__ int s_base[HS_MAX_NODES], s_room[HS_MAX_NODES], s_kept[HS_MAX_NODES];
+    __shared__ uint2 s_order[HS_MAX_NODES];          // {key, amount}
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = blockIdx.x, B = p.batch;
+    pdl_launch_dependents();
+    pdl_wait();                                      // scores and Phi(P*) come from the kernel ahead in the stream
+    const int first = p.node_off[b], n = min(p.node_off[b + 1] - first, HS_MAX_NODES), status = p.qstatus[b];
+    const float phi = p.phi_star[b];
+    unsigned int key = 0u;
+    int4 q = make_int4(0, 0, 0, 0);
+    if (tid < B) {
+        const int lo = p.node_off[tid], hi = p.node_off[tid + 1], st = p.qstatus[tid];
+        const float ph = p.phi_star[tid];
+        key = ((unsigned int)min(max(p.slo_class[tid], 0), 0xffff) << 16) | (unsigned int)tid;
+        int bin;
+        policy_lookup(p, ph, bin, q.z, q.w);
+        q.x = lo;
+        q.y = st == 0 ? min(hi - lo, HS_MAX_NODES) : 0;
+        if (st != 0) { s_base[tid] = 0; s_room[tid] = 0; }
+    }
+    s_seq[tid] = q;
+    int dep = 0, par = -1;
+    float S = 0.f;
+    if (tid < n && status == 0) {
+        dep = p.depth[first + tid];
+        par = p.parent[first + tid];
+        S = p.score[first + tid];
+    }
+    __syncthreads();
+    // requests: base = min(N', eligible nodes), at least the root
+    for (int s0 = warp * BP_SEQS; s0 < B; s0 += 4 * BP_SEQS) {
+        int d[BP_SEQS][HS_MAX_NODES / 32];
+#pragma unroll
+        for (int i = 0; i < BP_SEQS; ++i)
+#pragma unroll
+            for (int c = 0; c < HS_MAX_NODES / 32; ++c) {
+                d[i][c] = 0x7fffffff;
+                if (s0 + i < B) {
+                    const int4 t = s_seq[s0 + i];
+                    if (lane + 32 * c < t.y) d[i][c] = p.depth[t.x + lane + 32 * c];
+                }
+            }
+#pragma unroll
+        for (int i = 0; i < BP_SEQS; ++i) {
+            const int4 t = s_seq[min(s0 + i, HS_MAX_NODES - 1)];
+            int elig = 0;
+#pragma unroll
+            for (int c = 0; c < HS_MAX_NODES / 32; ++c)
+                elig += __popc(__ballot_sync(HS_FULL_MASK, lane + 32 * c < t.y && d[i][c] <= t.z));
+            if (lane == 0 && s0 + i < B && t.y > 0) {
+                s_room[s0 + i] = max(elig, 1);
+                s_base[s0 + i] = max(1, min(t.w, max(elig, 1)));
+            }
+        }
+    }
+    __syncthreads();
+    // reallocation: see budget_kernel
+    const int base = tid < B ? s_base[tid] : 0;
+    const int total = cta_sum(base, sm);
+    const bool fits = total <= p.budget;
+    const int amount = base > 0 ? (fits ? s_room[tid] - base : base - 1) : 0;
+    s_order[tid] = make_uint2(key, (unsigned int)amount);
+    __syncthreads();
+    int before = 0;
+    for (int j = 0; j < B; ++j) {
+        const uint2 o = s_order[j];
+        before += (fits ? o.x < key : o.x > key) ? (int)o.y : 0;
+    }
+    const int pool = fits ? p.budget - total : total - p.budget;
+    const int take = max(0, min(amount, pool - before));
+    s_kept[tid] = base == 0 ? 0 : (fits ? base + take : base - take);
+    __syncthreads();
+    prune_cta(p, b, n, status, phi, dep, par, S, sm, nullptr, 0, s_kept[b],
+              [&](int) { return cta_sum(tid < b ? s_kept[tid] : 0, sm); });
 }
 
 // ---- tree stage and pruning in one launch ---------------------------------------------------------------------
@@ -337,7 +422,7 @@ __global__ void __launch_bounds__(HS_MAX_NODES) tree_prune_kernel(const __grid_c
     const TreeStageResult t = tree_stage_cta(p, b, tsm);
     const int n = min(max(t.n, 0), HS_MAX_NODES);
     const int status = t.bad ? HS_ERR_BAD_TREE : HS_OK;
-    prune_cta(p.pr, b, n, status, t.phi_star, t.dep, t.bad ? -1 : t.par, t.S, sm, t.path, t.up, [&](int n_keep) {
+    prune_cta(p.pr, b, n, status, t.phi_star, t.dep, t.bad ? -1 : t.par, t.S, sm, t.path, t.up, -1, [&](int n_keep) {
         if (p.pr.batch == 1) return 0;
         if (tid == 0) st_release_gpu(&p.flags[b], n_keep + 1);
         int part = 0;
@@ -447,10 +532,15 @@ hs_status hs_launch_stratify_prune_budget(hs_ctx* ctx, const hs_tree_batch* tree
     p.n_default = policy->n_default;
     for (int i = 0; i < 3; ++i) p.gamma_pct[i] = policy->gamma_pct[i];
     if ((size_t)2 * p.batch * sizeof(int) > ctx->scratch_bytes) return HS_ERR_WORKSPACE;
-    p.base = (int*)ctx->scratch;
-    p.room = p.base + p.batch;
     p.slo_class = slo_class;
     p.budget = budget;
+    p.counted = 0;
+    p.n_override = nullptr;
+    if (p.batch <= HS_MAX_NODES)                     // (a thread per sequence)
+        return hs_launch(budget_prune_kernel, dim3(p.batch), dim3(HS_MAX_NODES), 0, stream, ctx->pdl, dim3(1, 1, 1), p) ==
+                       cudaSuccess ? HS_OK : HS_ERR_CUDA;
+    p.base = (int*)ctx->scratch;
+    p.room = p.base + p.batch;
     p.counted = 1;
     p.n_override = out->n_keep;
     if (hs_launch(budget_request_kernel, dim3((p.batch + 3) / 4), dim3(128), 0, stream, ctx->pdl, dim3(1, 1, 1), p) != cudaSuccess ||
