@@ -197,11 +197,12 @@ __global__ void __launch_bounds__(HS_ROW_THREADS, 4) accept_rows_kernel(const __
         }
     }
     __syncwarp();
-    pdl_launch_dependents();
+    if (!p.have_draft) pdl_launch_dependents();      // (else behind the wait: the walk kernel relies on it)
     // First half of a cluster barrier: when it completes every CTA of the row's cluster runs, and its shared memory may
     // be written from outside.  (The CTAs of a cluster take every early exit below together: same row, same sequence.)
     if (p.clustered) cluster_arrive();
     pdl_wait();                            // the pruned tree and the logits come from upstream
+    if (p.have_draft) pdl_launch_dependents();
     const int kept = p.pr.keep_off[p.batch], kidx = p.pr.keep_idx[k];
     const bool check = chunk == 0 && which == 0 && k < p.batch;
     const int e_keep = check ? p.pr.n_keep[k] : 1, e_status = check ? p.pr.status[k] : 0;
@@ -553,15 +554,38 @@ __global__ void __launch_bounds__(WALK_THREADS, 1) accept_walk_kernel(const __gr
     const int b = blockIdx.x / WC;
     const unsigned int rank = cluster.block_rank();
     pdl_launch_dependents();
-    pdl_wait();                            // arg-max and normalisers come from the row pass
+    // Ahead of the dependency wait: all that does not come from the row pass.  (The row pass lets this kernel start only behind its
+    // own wait, so the pruned tree and the caller's arrays are complete.)  Every candidate's logits under its parent's target and
+    // draft row and its uniform, for all kept nodes at once: a thread per node, four dependent round trips of which
+    // none is left on the path between the row pass and the walk (3 us of the 12 us of one sequence).
+    static_assert(WALK_THREADS >= HS_MAX_NODES, "a thread per node");
     const int koff = p.pr.keep_off[b];
     const int nk = p.pr.n_keep[b];
+    const int tree_status = p.pr.status[b];
     const int nbase = p.node_off[b];
     const int cap = p.out.path_cap;
     const bool sampling = p.mode[b] == HS_ACCEPT_REJECTION;
     const size_t esz = p.is_bf16 ? 2 : 4;
+    const int nkc = tree_status == 0 ? min(nk, HS_MAX_NODES) : 0;
+    const bool mine = sampling && tid < nkc;                  // this thread has node tid
+    int par = -1, orig = 0, tok = 0;
+    float lp = 0.f, lq = 0.f, u = 0.f, T = 1.f;
+    if (sampling) T = p.temperature[b];
+    if (mine) {
+        par = p.pr.new_parent[koff + tid];
+        orig = p.pr.keep_idx[koff + tid];
+        tok = p.token[nbase + orig];
+        if (par >= 0 && par < nkc) {
+            const int porig = p.pr.keep_idx[koff + par];
+            const int trow = p.target_layout == HS_ROWS_ORIGINAL ? nbase + porig : koff + par;
+            lp = load_logit((const char*)p.target + (size_t)trow * p.row_stride * esz, p.is_bf16, tok);
+            lq = load_logit((const char*)p.draft + (size_t)(nbase + porig) * p.row_stride * esz, p.is_bf16, tok);
+        }
+        u = p.uniforms ? p.uniforms[nbase + orig] : philox_uniform(p.seed, p.offset, b, orig, 0);
+    }
+    pdl_wait();                            // arg-max and normalisers come from the row pass
 
-    if (!sampling && nk > 0 && p.pr.status[b] == 0) return;      // greedy sequences were finished by the row pass
+    if (!sampling && nk > 0 && tree_status == 0) return;      // greedy sequences were finished by the row pass
     if (rank == 0) {
         for (int j = tid; j < cap; j += WALK_THREADS) {
             p.out.path_nodes[b * cap + j] = -1;
@@ -569,10 +593,10 @@ __global__ void __launch_bounds__(WALK_THREADS, 1) accept_walk_kernel(const __gr
             p.out.path_tokens[b * cap + j] = -1;
         }
     }
-    if (nk <= 0 || p.pr.status[b] != 0) {
+    if (nk <= 0 || tree_status != 0) {
         if (rank == 0 && tid == 0) {
             p.out.accept_len[b] = 0; p.out.bonus_token[b] = -1; p.out.terminal_rank[b] = -1;
-            p.out.status[b] = p.pr.status[b] != 0 ? p.pr.status[b] : HS_ERR_BAD_TREE;
+            p.out.status[b] = tree_status != 0 ? tree_status : HS_ERR_BAD_TREE;
         }
         return;
     }
@@ -614,10 +638,9 @@ __global__ void __launch_bounds__(WALK_THREADS, 1) accept_walk_kernel(const __gr
         rs.p = (const uint4*)s_rows;
         rs.q = qrow ? (const uint4*)s_rows + per : nullptr;
     };
-    // Every candidate's probability under its parent's target and draft row, its uniform and the normalisers of its
-    // own rows, for all kept nodes at once (three dependent round trips in all instead of three per visited node);
-    // the walk below then runs from shared memory until a rejection needs a vocabulary-wide residual sum.  Every CTA
-    // of the cluster fetches the same values and takes the same decisions.
+    // Every candidate's probability under its parent's target and draft row, its uniform and the normalisers of its own rows, for all
+    // kept nodes at once: one round trip for the normalisers; the walk below then runs from shared memory until a rejection needs a
+    // vocabulary-wide residual sum.  Every CTA of the cluster fetches the same values and takes the same decisions.
     __shared__ int s_par[HS_MAX_NODES], s_tok[HS_MAX_NODES], s_orig[HS_MAX_NODES];
     __shared__ float s_pt[HS_MAX_NODES], s_qt[HS_MAX_NODES], s_u[HS_MAX_NODES];
     __shared__ float2 s_pms[HS_MAX_NODES];
@@ -625,35 +648,30 @@ __global__ void __launch_bounds__(WALK_THREADS, 1) accept_walk_kernel(const __gr
     // accepted - the common step of the walk then costs two shared-memory reads.
     __shared__ int s_first[HS_MAX_NODES];
     __shared__ unsigned char s_acc0[HS_MAX_NODES];
-    const float T = p.temperature[b];
     const float invT = LOG2E / T;
-    const int nkc = min(nk, HS_MAX_NODES);
-    for (int j = tid; j < nkc; j += WALK_THREADS) s_first[j] = 0x7fffffff;
+    float2 oms = make_float2(0.f, 1.f), pms0 = oms, qms0 = oms;
+    const bool child = mine && par >= 0 && par < nkc;
+    if (mine) {
+        oms = p.ro.tgt_ms[koff + tid];
+        s_first[tid] = 0x7fffffff;
+    }
+    if (child) { pms0 = p.ro.tgt_ms[koff + par]; qms0 = p.ro.drf_ms[koff + par]; }
     __syncthreads();
-    for (int j = tid; j < nkc; j += WALK_THREADS) {
-        const int par = p.pr.new_parent[koff + j];
-        const int orig = p.pr.keep_idx[koff + j];
-        const int tok = p.token[nbase + orig];
-        s_par[j] = par; s_tok[j] = tok; s_orig[j] = orig;
-        s_pms[j] = p.ro.tgt_ms[koff + j];
+    if (mine) {
         float pt = 0.f, qt = 0.f;
-        if (par >= 0 && par < nkc) {
-            const int porig = p.pr.keep_idx[koff + par];
-            const int trow = p.target_layout == HS_ROWS_ORIGINAL ? nbase + porig : koff + par;
-            const char* prow = (const char*)p.target + (size_t)trow * p.row_stride * esz;
-            const char* qrow = (const char*)p.draft + (size_t)(nbase + porig) * p.row_stride * esz;
-            const float2 pms = p.ro.tgt_ms[koff + par], qms = p.ro.drf_ms[koff + par];
-            pt = exp2f((fmaxf(load_logit(prow, p.is_bf16, tok), -1e30f) - pms.x) * invT) * (1.f / pms.y);
-            qt = exp2f((fmaxf(load_logit(qrow, p.is_bf16, tok), -1e30f) - qms.x) * invT) * (1.f / qms.y);
+        if (child) {
+            pt = exp2f((fmaxf(lp, -1e30f) - pms0.x) * invT) * (1.f / pms0.y);
+            qt = exp2f((fmaxf(lq, -1e30f) - qms0.x) * invT) * (1.f / qms0.y);
         }
-        s_pt[j] = pt; s_qt[j] = qt;
-        const float u = p.uniforms ? p.uniforms[nbase + orig] : philox_uniform(p.seed, p.offset, b, orig, 0);
-        s_u[j] = u;
+        s_par[tid] = par; s_tok[tid] = tok; s_orig[tid] = orig;
+        s_pms[tid] = oms;
+        s_pt[tid] = pt; s_qt[tid] = qt;
+        s_u[tid] = u;
         // (the same expressions as in the sibling loop below with c = 0, W = 1: the same decision, bit for bit)
         const float r0 = fmaxf(pt - 0.f * qt, 0.f) / 1.f;
         const float a0 = qt > 0.f ? fminf(1.f, r0 / qt) : 1.f;
-        s_acc0[j] = (par >= 0 && par < j && u < a0) ? 1 : 0;
-        if (par >= 0 && par < j) atomicMin(&s_first[par], j);
+        s_acc0[tid] = (par >= 0 && par < tid && u < a0) ? 1 : 0;
+        if (par >= 0 && par < tid) atomicMin(&s_first[par], tid);
     }
     __syncthreads();
     int cur = 0, len = 0;

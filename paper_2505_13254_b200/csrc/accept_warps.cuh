@@ -30,8 +30,9 @@ __global__ void __launch_bounds__(AW_THREADS, 1) accept_warp_kernel(const __grid
     __shared__ int s_npending;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) s_npending = 0;
-    pdl_launch_dependents();
+    if (!p.have_draft) pdl_launch_dependents();      // (else behind the wait: the walk kernel relies on it)
     pdl_wait();                            // the pruned tree and the logits come from upstream
+    if (p.have_draft) pdl_launch_dependents();
 
     // ---- the rows of the stream --------------------------------------------------------------------------------
     const int T = min(p.pr.keep_off[p.batch], p.part_rows);
