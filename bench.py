@@ -374,7 +374,10 @@ def main():
         k["gbs"] = k["bytes"] / (k["us"] * 1e-6) / 1e9 if k["us"] > 0 else None
         k["frac_of_%s_hbm" % peak_kind] = k["gbs"] / peak if k["gbs"] else None
         k["frac_of_nominal_hbm"] = k["gbs"] / NOMINAL_HBM_GBS if k["gbs"] else None
-    traffic = ncu_traffic("quantify_stream_kernel", cfg.name)
+    # (the entropy pass takes few rows as clusters, more as a share of the matrix per warp)
+    few = 2 * n_rows <= torch.cuda.get_device_properties(0).multi_processor_count
+    quant_kernel = "quantify_cluster_kernel" if few else "quantify_warp_kernel"
+    traffic = ncu_traffic(quant_kernel, cfg.name)
     achieved = kern["quantify"]["gbs"]
     line = {
         "metric": METRIC, "value": whole_job_value(world, cfg.batch, args.steps, ms), "unit": UNIT, "n_gpus": world,
@@ -391,7 +394,7 @@ def main():
                 "how": "every step copies all inputs from pinned host memory and reads its results back; the copies of "
                        "step n + 1 overlap the kernels of step n (two staging buffers, two streams)"},
         "gpu_launches": (5 if db0.any_sampling else 4) * args.steps,
-        "roofline": {"kernel": "quantify_stream_kernel (hs_entropy_quantify: this kernel + the tree stage)", "bound": "hbm",
+        "roofline": {"kernel": quant_kernel + " (hs_entropy_quantify: this kernel + the tree stage)", "bound": "hbm",
                      "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                      "frac_of_nominal": achieved / NOMINAL_HBM_GBS,
                      "peak_kind": peak_kind + " (burst copy figure)", "traffic": traffic,
@@ -410,7 +413,7 @@ def main():
     a_tflops = attn_flops / (kern["attention"]["us"] * 1e-6) / 1e12
     tf_peak = tensor_peak()
     if attn_flops / (tf_peak * 1e12) > attn_bytes / (peak * 1e9):      # the tensor pipe is the longer leg
-        line["roofline_attention"] = {"kernel": "tree_attn_umma_kernel (hs_tree_verify_attention, one launch per step)",
+        line["roofline_attention"] = {"kernel": "tree_attn_umma_kernel or tree_attn_duo_kernel, by size (hs_tree_verify_attention, one launch per step)",
                                       "bound": "tensor", "achieved": a_tflops, "peak": tf_peak, "unit": "TFLOP/s",
                                       "frac": a_tflops / tf_peak, "frac_of_nominal": a_tflops / NOMINAL_BF16_TFLOPS,
                                       "peak_kind": peak_kind + " (dense bf16 burst figure)",
@@ -418,7 +421,7 @@ def main():
                                       "algorithmic_flops_per_launch": attn_flops,
                                       "algorithmic_bytes_per_launch": attn_bytes}
     else:
-        line["roofline_attention"] = {"kernel": "tree_attn_umma_kernel (hs_tree_verify_attention, one launch per step)",
+        line["roofline_attention"] = {"kernel": "tree_attn_umma_kernel or tree_attn_duo_kernel, by size (hs_tree_verify_attention, one launch per step)",
                                       "bound": "hbm", "achieved": a_gbs, "peak": peak, "unit": "GB/s",
                                       "frac": a_gbs / peak if a_gbs else None,
                                       "frac_of_nominal": a_gbs / NOMINAL_HBM_GBS if a_gbs else None,
