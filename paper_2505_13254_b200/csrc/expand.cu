@@ -10,6 +10,7 @@
 // finds the N-th largest value by binary search; compaction by warp ballots and a prefix sum over the warps.
 #include <math_constants.h>
 
+#include "expand_child.h"
 #include "hs_common.cuh"
 #include "hs_layout.h"
 #include "hs_ptx.cuh"
@@ -30,35 +31,28 @@ __global__ void expand_init_kernel(hs_expand_state st) {
     st.status[b] = HS_OK;
 }
 
-// Two round trips to global memory: everything that does not depend on another load first (the statistics of slot (j, i)
-// are addressed by the thread's number alone), then the parents' values.  The rank among the new children reads four
-// values per shared-memory access.
-// (Growing four trees of 8 levels: 164 -> 136 us a pass, with the tree stage's early loads and the reranking below.)
+// Two round trips to global memory: the sequence's numbers and the frontier, then the row statistics of the frontier's children
+// and their parents' values.  The rank among the new children reads four values per shared-memory access.
 __global__ void __launch_bounds__(EX_THREADS) expand_level_kernel(hs_expand_state st, const float* topk_val,
                                                                   const int* topk_idx, const float* row_lse, int K) {
     __shared__ __align__(16) float s_S[HS_MAX_TOPK * HS_MAX_TOPK];
     const int b = blockIdx.x, tid = threadIdx.x;
     const int k = st.top_k;
     const size_t o = (size_t)b * st.cap;
-    const int j = tid / k, i = tid - j * k, row = b * k + j;
     pdl_launch_dependents();
     pdl_wait();                                    // the row statistics come from the kernel ahead
     const int status = st.status[b], n0 = st.n_cand[b], nf = st.n_frontier[b];
-    int par = -1, tok = -1, dep = 0;
-    float lc = 0.f;
-    if (j < k) {
-        par = st.frontier[(size_t)b * k + j];      // (slots past the frontier hold older candidates: not used)
-        tok = topk_idx[(size_t)row * K + i];
-        lc = topk_val[(size_t)row * K + i] - row_lse[row];
-    }
+    const int par = tid < k * k ? st.frontier[(size_t)b * k + tid / k] : -1;      // (slots past the frontier hold older candidates: not used)
     if (status != HS_OK) return;
     const int nnew = nf * k;
     if (n0 + nnew > st.cap) {                      // the arrays cannot take another level
         if (tid == 0) st.status[b] = HS_ERR_SHAPE;
         return;
     }
+    int tok = -1, dep = 0;
+    float lc = 0.f;
     float S = __int_as_float(0x7fc00000);          // (NaN: compares false, ranks nobody)
-    if (tid < nnew) {
+    if (load_child(tid, b, k, nf, K, topk_val, topk_idx, row_lse, tok, lc)) {
         S = st.score[o + par] + lc;
         dep = st.depth[o + par] + 1;
     }
