@@ -657,6 +657,7 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     }
     tc_fence_before_sync();
     __syncthreads();
+    tc_fence_after_sync();
     if (warp == 0) tmem_dealloc(tmem_base, UM_TMEM_COLS);
 }
 #include "tree_attn_duo.cuh"

@@ -22,13 +22,16 @@
 #define AD_SMEM_BYTES (AD_MISC_BYTES + ATT_Q_BYTES + AD_SLOTS * ATT_TILE_BYTES)
 #define AD_TMEM_COLS 256                            // S / P of tile i: columns 64 (i & 1) ..; O: 128 ..
 
-// Barriers 1 .. 4: the two warps that share 32 rows.  (Constant numbers: with a number in a register the kernel would claim all
-// 16 of a CTA and only one CTA would fit on an SM.)
+// The two warps that share 32 rows meet on barriers 1 .. 4.  (Constant numbers: with a number in a register the kernel would claim all
+// 16 of a CTA and only one CTA would fit on an SM.)  What one of them has read from tensor memory ahead of the barrier the other may
+// overwrite behind it (S by P), which needs tcgen05's own fences on both sides.
 __device__ __forceinline__ void pair_sync(int quad) {
+    tc_fence_before_sync();
     if (quad == 0) named_bar_sync(1, 64);
     else if (quad == 1) named_bar_sync(2, 64);
     else if (quad == 2) named_bar_sync(3, 64);
     else named_bar_sync(4, 64);
+    tc_fence_after_sync();
 }
 
 __global__ void __launch_bounds__(AD_THREADS, 2)
@@ -456,5 +459,6 @@ tree_attn_duo_kernel(const __grid_constant__ AttnParams p, const __grid_constant
     __syncwarp();
     tc_fence_before_sync();
     __syncthreads();
+    tc_fence_after_sync();
     if (warp == AD_MMA_WARP) tmem_dealloc(tmem, AD_TMEM_COLS);
 }

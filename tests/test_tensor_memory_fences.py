@@ -1,0 +1,26 @@
+"""Tensor memory handed from one warp to another across a barrier needs tcgen05.fence::before_thread_sync ahead of it and
+tcgen05.fence::after_thread_sync behind it; no result shows a missing one reliably, so the sources are read."""
+import os
+import re
+
+import pytest
+
+from paper_2505_13254_b200 import build
+
+
+def text(name):
+    return re.sub(r"//.*", "", open(os.path.join(build.CSRC, name)).read())
+
+
+def test_the_pair_barrier_carries_both_fences():
+    body = re.search(r"void pair_sync\(int quad\) \{(.*?)\n\}", text("tree_attn_duo.cuh"), re.S).group(1)
+    first, last = body.find("named_bar_sync"), body.rfind("named_bar_sync")
+    assert 0 <= body.find("tc_fence_before_sync()") < first
+    assert body.find("tc_fence_after_sync()") > last
+
+
+@pytest.mark.parametrize("name", ["tree_attention.cu", "tree_attn_duo.cuh"])
+def test_tensor_memory_is_freed_behind_a_fenced_barrier(name):
+    last = text(name).rindex("tmem_dealloc(")
+    tail = re.sub(r"\s+", "", text(name)[:last])
+    assert re.search(r"tc_fence_before_sync\(\);__syncthreads\(\);tc_fence_after_sync\(\);if\(warp==\w+\)$", tail)
