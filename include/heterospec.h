@@ -91,7 +91,7 @@ hs_status hs_destroy(hs_ctx* ctx);
  * prefix (appended a step earlier), true for logits only if something else separates producer and
  * call.  Default 0: nothing is read early. */
 #define HS_PREFETCH_LOGITS 1   /* draft logits and tree arrays (parent, token, node_off) of hs_entropy_quantify */
-#define HS_PREFETCH_KV 2       /* k_cache / v_cache of hs_tree_verify_attention */
+#define HS_PREFETCH_KV 2       /* k_cache, v_cache and kv_off of hs_tree_verify_attention */
 hs_status hs_set_prefetch(hs_ctx* ctx, int32_t flags);
 
 /* Which kernel hs_accept_path reads the vocabulary rows with (a tuning knob; the paper has no counterpart).  Both give

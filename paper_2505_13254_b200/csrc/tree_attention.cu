@@ -4,8 +4,8 @@
 // nodes forms the dense M dimension: query row r = node * G + g.  The KV prefix is cut into tiles of
 // 64 keys that are shared out evenly over the splits; a CTA requests its first tiles by TMA
 // (cp.async.bulk.tensor into 128-byte-swizzled shared memory, four stages, K and V on mbarriers of
-// their own) before it waits for the kernel ahead of it in the stream, because the cache does not
-// depend on the pruned tree.  The <= 128 tree keys belong to the last split; their rows may be indirect.  Behind
+// their own) before it waits for the kernel ahead of it in the stream if the caller vouches for the cache (it does not
+// depend on the pruned tree).  The <= 128 tree keys belong to the last split; their rows may be indirect.  Behind
 // prefix tiles the producer warp fetches them by tile::gather4 (plain loads by the softmax threads held up the
 // longest split: 4096 tokens, 64 / 8 heads 19.6 us against 18.0, a ragged batch of 16 75.5 against 71).  S = Q K^T and O += P V run on the 5th-generation tensor
 // cores (tcgen05.mma, accumulators in tensor memory) with fp32 accumulation; the softmax is the
@@ -127,7 +127,9 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     const int tid = threadIdx.x, warp = tid >> 5;
     // Sequences are taken longest prefix first (a ragged batch then ends on its short sequences, not on a long one
     // that started late): grid slot z / hkv holds the sequence of that rank by (length descending, index ascending).
-    // kv_off is an input of the call, so the ranking runs ahead of the dependency wait.
+    // kv_off is an array of the caller like any other: the ranking runs ahead of the dependency wait only where the caller
+    // vouches for the cache and with it for its offsets.  (Both instructions come again below, without effect.)
+    if (!p.prefetch) { pdl_launch_dependents(); pdl_wait(); }
     __shared__ int s_seq;
     int b = blockIdx.z / p.hkv;
     const int h = blockIdx.z % p.hkv;
@@ -167,7 +169,7 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     float* s_mx = reinterpret_cast<float*>(gM + UM_MAP_BYTES + 1024);      // [2][128]: the streams' row maxima at the end
     float* s_lx = s_mx + 2 * ATT_BM;                                     // [2][128]: the streams' row sums
 
-    // ---- before the dependency wait: barriers, tensor memory, the first KV prefix tiles -----------------
+    // ---- with prefetch before the dependency wait: barriers, tensor memory, the first KV prefix tiles -----------------
     const int kv0 = p.kv_off[b];
     const int L = p.kv_off[b + 1] - kv0;
     int t_prefix, t0, t1;

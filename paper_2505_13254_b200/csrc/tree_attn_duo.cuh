@@ -51,6 +51,9 @@ tree_attn_duo_kernel(const __grid_constant__ AttnParams p, const __grid_constant
     const unsigned int sQ = sbase + AD_MISC_BYTES, sR = sQ + ATT_Q_BYTES;      // query tile, the ring
     unsigned char* gR = smem + AD_MISC_BYTES + ATT_Q_BYTES;
 
+    // kv_off is an array of the caller like any other: it is read ahead of the dependency wait only where the caller vouches for the
+    // cache and with it for its offsets.  (Both instructions come again below, without effect.)
+    if (!p.prefetch) { pdl_launch_dependents(); pdl_wait(); }
     // sequences are taken longest prefix first (see tree_attn_umma_kernel)
     int b = blockIdx.z / p.hkv;
     const int h = blockIdx.z % p.hkv;
