@@ -34,7 +34,8 @@ __device__ __forceinline__ void slice_mass(const AcceptParams& p, const char* pr
         if (p.is_bf16) unpack_v<true>(d[q], x); else unpack_v<false>(d[q], x);
 #pragma unroll
         for (int e = 0; e < 8; ++e)
-            m[q][e] = e < ve ? ex2a((fmaxf(x[e], -1e30f) - pm) * invT) * ips : 0.f;
+            m[q][e] = e < ve ? exp2f((fmaxf(x[e], -1e30f) - pm) * invT) * ips : 0.f;     // (as in the accept tests below: the
+                                                                     // distribution is one, masses below the normal range included)
     }
     if (inside < 4 << vsh) {                                 // (the thread that runs past the vocabulary, and those behind it)
 #pragma unroll
