@@ -21,6 +21,19 @@
 #define AD_SLOTS 4                                  // ring of K and V tiles
 #define AD_SMEM_BYTES (AD_MISC_BYTES + ATT_Q_BYTES + AD_SLOTS * ATT_TILE_BYTES)
 #define AD_TMEM_COLS 256                            // S / P of tile i: columns 64 (i & 1) ..; O: 128 ..
+// Tiles after the first over which the exponents' reference follows every new row maximum.  One stream per row has one exact P where the two
+// streams of tree_attn_umma_kernel have two, so its error against fp64 was larger (2-norm relative, 16 x 50..60 nodes, 256..512 tokens:
+// 2.296e-3 against 2.251e-3; 12 x 37..46, 1200 tokens: 2.339e-3 against 2.325e-3).  Followed over one tile 2.261e-3 and 2.330e-3, over two
+// 2.230e-3 and 2.319e-3, over three 2.202e-3 and 2.313e-3; each costs 0.5 us of 18.7 and of 29.8 (one more rescale of O).
+#define AD_FOLLOW 2
+// Merge of the splits, in the memory of the query tile and the ring: (max, sum) of the warps, weights and output rows of the rows owned,
+// then the partials received, 128 fp32 of O / l and {max, sum} per row.  (As bf16 a split launch rounded O twice: 2.876e-3 from fp64 at
+// 4 x 62 nodes, 64 / 8 heads, 32768 tokens, now 2.339e-3, for 2.5 us of 276.)
+#define AD_PART_BYTES (HS_HEAD_DIM * 4 + 8)
+#define AD_PB_STRIDE (HS_HEAD_DIM * 4 + 16)
+#define AD_END_BYTES 4608
+static_assert(AD_END_BYTES % 16 == 0 && AD_END_BYTES >= 2048 + 68 * ATT_MAX_SPLIT * 4 + 68 * 4 &&
+              AD_END_BYTES + (ATT_BM + 2 * ATT_MAX_SPLIT) * AD_PB_STRIDE <= ATT_Q_BYTES + AD_SLOTS * ATT_TILE_BYTES, "partials behind the small arrays");
 
 // The two warps that share 32 rows meet on barriers 1 .. 4.  (Constant numbers: with a number in a register the kernel would claim all
 // 16 of a CTA and only one CTA would fit on an SM.)  What one of them has read from tensor memory ahead of the barrier the other may
@@ -49,7 +62,6 @@ tree_attn_duo_kernel(const __grid_constant__ AttnParams p, const __grid_constant
     int* s_seq = reinterpret_cast<int*>(smem + 264);
     float* s_pair = reinterpret_cast<float*>(smem + 512);      // [4 quads][2 parities][2 halves][32 rows]
     const unsigned int sQ = sbase + AD_MISC_BYTES, sR = sQ + ATT_Q_BYTES;      // query tile, the ring
-    unsigned char* gR = smem + AD_MISC_BYTES + ATT_Q_BYTES;
 
     // kv_off is an array of the caller like any other: it is read ahead of the dependency wait only where the caller vouches for the
     // cache and with it for its offsets.  (Both instructions come again below, without effect.)
@@ -302,8 +314,10 @@ tree_attn_duo_kernel(const __grid_constant__ AttnParams p, const __grid_constant
             xf[half * 32 + lane] = own;
             pair_sync(quad);
             const float mx = fmaxf(own, xf[(half ^ 1) * 32 + lane]);
-            // (the reference follows the maximum only when that has grown by more than 8: see tree_attn_umma_kernel)
-            const float mnew = (mx > mrun + 8.f || mrun == -CUDART_INF_F) ? fmaxf(mrun, mx) : mrun;
+            // The reference follows the maximum only when that has grown by more than 8 (see tree_attn_umma_kernel) - but closely over
+            // the first AD_FOLLOW + 1 tiles: a score that was the maximum when its tile was taken has P = 2^0, which bf16 holds without error,
+            // and those are the weights that count most.
+            const float mnew = (mx > mrun + (i <= AD_FOLLOW ? 0.f : 8.f) || mrun == -CUDART_INF_F) ? fmaxf(mrun, mx) : mrun;
             const float muse = (mnew == -CUDART_INF_F) ? 0.f : mnew;
             const float corr = ex2_approx(mrun - muse);        // 1 when the reference stays, 0 at the first tile
             mrun = mnew;
@@ -350,35 +364,30 @@ tree_attn_duo_kernel(const __grid_constant__ AttnParams p, const __grid_constant
     int r_lo, r_hi;
     owned(split, r_lo, r_hi);
     if (ns > 1) {
-        if (tid == 0) mbar_expect_tx(bar_r, (unsigned int)(ns * (r_hi - r_lo) * (HS_HEAD_DIM * 2 + 8)));
+        if (tid == 0) mbar_expect_tx(bar_r, (unsigned int)(ns * (r_hi - r_lo) * AD_PART_BYTES));
         __syncwarp();
-        cluster_arrive();                                      // partials may now arrive in this CTA's ring
+        cluster_arrive();                                      // partials may now arrive in this CTA's tiles
     }
 
     // ---- end: the parts of a row held by several threads are combined; all of this in the query tile's memory -----------------
     float2* s_ml = reinterpret_cast<float2*>(smem + AD_MISC_BYTES);                  // [8 warps][32] (max, sum)
     float* s_wt = reinterpret_cast<float*>(smem + AD_MISC_BYTES + 2048);             // [rows owned <= 65][ATT_MAX_SPLIT] weights
     int* s_og = reinterpret_cast<int*>(smem + AD_MISC_BYTES + 2048 + 68 * ATT_MAX_SPLIT * 4);   // [rows owned] output row or -1
+    const unsigned char* gP = smem + AD_MISC_BYTES + AD_END_BYTES;                              // [ns][rows_max] partials received
     if (warp < AD_MMA_WARP) {
         s_ml[warp * 32 + lane] = make_float2(mrun, lrun);
         named_bar_sync(5, AD_SM_THREADS);
         lrun += s_ml[(warp ^ 4) * 32 + lane].y;                // (the halves of a row have one reference)
         const float inv = lrun > 0.f ? 1.f / lrun : 0.f;
-        // 32 columns at a time of this thread's 64 of the normalised O row as bf16
-        auto load_piece = [&](int ch, uint4 (&o)[4]) {
+        // 32 columns at a time of this thread's 64 of the normalised O row
+        auto load_piece = [&](int ch, float (&o)[32]) {
             unsigned int oa[32];
 #pragma unroll
             for (int c = 0; c < 32; ++c) oa[c] = 0u;           // (an accumulator without tiles holds anything)
             if (ntile > 0) tmem_ld32(tmem + lane_off + 2 * ATT_BN + half * 64 + ch * 32, oa);
             tmem_wait_ld();
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                unsigned int w[4];
-#pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    w[c] = pack_bf16(__uint_as_float(oa[q * 8 + 2 * c]) * inv, __uint_as_float(oa[q * 8 + 2 * c + 1]) * inv);
-                o[q] = make_uint4(w[0], w[1], w[2], w[3]);
-            }
+            for (int c = 0; c < 32; ++c) o[c] = __uint_as_float(oa[c]) * inv;
         };
         const int col0 = half * 64;
         const bool has_ml = half == 0;                   // this thread speaks for the row's (max, sum)
@@ -386,8 +395,13 @@ tree_attn_duo_kernel(const __grid_constant__ AttnParams p, const __grid_constant
             const int orow = m0 + row < M ? query_row(m0 + row) : -1;
 #pragma unroll 1
             for (int ch = 0; ch < 2; ++ch) {
+                float of[32];
+                load_piece(ch, of);
                 uint4 o[4];
-                load_piece(ch, o);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    o[q] = make_uint4(pack_bf16(of[q * 8], of[q * 8 + 1]), pack_bf16(of[q * 8 + 2], of[q * 8 + 3]),
+                                      pack_bf16(of[q * 8 + 4], of[q * 8 + 5]), pack_bf16(of[q * 8 + 6], of[q * 8 + 7]));
                 quad_transpose(o, lane);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -405,16 +419,18 @@ tree_attn_duo_kernel(const __grid_constant__ AttnParams p, const __grid_constant
             const int owner = row * ns / ATT_BM;
             int o_lo, o_hi;
             owned(owner, o_lo, o_hi);
-            const unsigned int dst = cluster_map_addr(sR + (unsigned int)(split * rows_max + row - o_lo) * ATT_PB_STRIDE, owner);
+            const unsigned int dst = cluster_map_addr(sbase + AD_MISC_BYTES + AD_END_BYTES + (unsigned int)(split * rows_max + row - o_lo) * AD_PB_STRIDE, owner);
             const unsigned int rbar = cluster_map_addr(bar_r, owner);
-            if (has_ml) st_async_v2(dst + HS_HEAD_DIM * 2, __float_as_uint(mrun), __float_as_uint(lrun), rbar);
+            if (has_ml) st_async_v2(dst + HS_HEAD_DIM * 4, __float_as_uint(mrun), __float_as_uint(lrun), rbar);
             __syncwarp();
 #pragma unroll 1
             for (int ch = 0; ch < 2; ++ch) {
-                uint4 o[4];
+                float o[32];
                 load_piece(ch, o);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) st_async_v4(dst + (col0 + ch * 32 + i * 8) * 2, o[i].x, o[i].y, o[i].z, o[i].w, rbar);
+                for (int i = 0; i < 32; i += 4)
+                    st_async_v4(dst + (col0 + ch * 32 + i) * 4, __float_as_uint(o[i]), __float_as_uint(o[i + 1]), __float_as_uint(o[i + 2]),
+                                __float_as_uint(o[i + 3]), rbar);
             }
             mbar_wait_cluster(bar_r, 0u, p.err);               // all ns pieces of this CTA's rows have landed
             // the ranges' weights of every owned row, once
@@ -424,7 +440,7 @@ tree_attn_duo_kernel(const __grid_constant__ AttnParams p, const __grid_constant
 #pragma unroll
                 for (int s2 = 0; s2 < ATT_MAX_SPLIT; ++s2) {
                     ml[s2] = make_float2(-CUDART_INF_F, 0.f);
-                    if (s2 < ns) ml[s2] = *reinterpret_cast<const float2*>(gR + (size_t)(s2 * rows_max + tid) * ATT_PB_STRIDE + HS_HEAD_DIM * 2);
+                    if (s2 < ns) ml[s2] = *reinterpret_cast<const float2*>(gP + (size_t)(s2 * rows_max + tid) * AD_PB_STRIDE + HS_HEAD_DIM * 4);
                     Mx = fmaxf(Mx, ml[s2].x);
                 }
                 float w[ATT_MAX_SPLIT], lsum = 0.f;
@@ -440,7 +456,7 @@ tree_attn_duo_kernel(const __grid_constant__ AttnParams p, const __grid_constant
             }
             __syncwarp();
             named_bar_sync(5, AD_SM_THREADS);                  // the weights are written
-            // items = (row, 16-byte column group of 8), each over all ranges from local shared memory
+            // items = (row, column group of 8), each over all ranges from local shared memory
             for (int it = tid; it < (r_hi - r_lo) * 16; it += AD_SM_THREADS) {
                 const int rl = it >> 4, c8 = it & 15;
                 float acc[8];
@@ -448,9 +464,13 @@ tree_attn_duo_kernel(const __grid_constant__ AttnParams p, const __grid_constant
                 for (int e = 0; e < 8; ++e) acc[e] = 0.f;
 #pragma unroll
                 for (int s2 = 0; s2 < ATT_MAX_SPLIT; ++s2)
-                    if (s2 < ns)
-                        fma_bf16x8(acc, s_wt[rl * ATT_MAX_SPLIT + s2],
-                                   *reinterpret_cast<const uint4*>(gR + (size_t)(s2 * rows_max + rl) * ATT_PB_STRIDE + c8 * 16));
+                    if (s2 < ns) {
+                        const float w = s_wt[rl * ATT_MAX_SPLIT + s2];
+                        const float4* v = reinterpret_cast<const float4*>(gP + (size_t)(s2 * rows_max + rl) * AD_PB_STRIDE + c8 * 32);
+                        const float4 a = v[0], c = v[1];
+                        acc[0] = fmaf(w, a.x, acc[0]); acc[1] = fmaf(w, a.y, acc[1]); acc[2] = fmaf(w, a.z, acc[2]); acc[3] = fmaf(w, a.w, acc[3]);
+                        acc[4] = fmaf(w, c.x, acc[4]); acc[5] = fmaf(w, c.y, acc[5]); acc[6] = fmaf(w, c.z, acc[6]); acc[7] = fmaf(w, c.w, acc[7]);
+                    }
                 if (s_og[rl] >= 0)
                     *reinterpret_cast<uint4*>(p.out + (size_t)s_og[rl] * HS_HEAD_DIM + c8 * 8) =
                         make_uint4(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]), pack_bf16(acc[6], acc[7]));

@@ -1,0 +1,71 @@
+"""How far the attention kernel with two CTAs per SM may be from fp64: no further than rounding P and the output to bf16 once each
+takes it, split prefixes included, and no further than the kernel with two streams per row on the same sequences."""
+import math
+
+import pytest
+import torch
+
+from paper_2505_13254_b200 import binding as hb
+
+pytestmark = pytest.mark.gpu
+
+# Rounding to bf16: +- 2^-8 of the leading digit at most, uniform, so 2^-7 / sqrt(12) over the mantissa m in [1, 2); the mean of 1 / m^2 under the
+# density 1 / (m ln 2) is 3 / (8 ln 2).  P and the output are rounded independently.
+ROUNDING = 2 ** -7 / math.sqrt(12) * math.sqrt(3 / (8 * math.log(2)))
+
+
+def inputs(batch, nodes, hq, hkv, kv, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    rn = lambda *s: torch.randn(*s, device="cuda", generator=g, dtype=torch.bfloat16)
+    n = batch * nodes
+    return rn(n, hq, 128), rn(n, hkv, 128), rn(n, hkv, 128), rn(batch * kv, hkv, 128), rn(batch * kv, hkv, 128)
+
+
+def attend(x, b0, b1, nodes, kv):
+    """Sequences b0 .. b1 - 1 of x (all trees are chains) in one call."""
+    i32 = lambda a: torch.tensor(a, dtype=torch.int32, device="cuda")
+    q, kt, vt, kc, vc = x
+    B = b1 - b0
+    tree = hb.TreeBatch(i32([b * nodes for b in range(B + 1)]), i32(list(range(-1, nodes - 1)) * B), i32([0] * (B * nodes)), B, B * nodes)
+    policy = dict(thresholds=[-1e9] * 7, d_base=200, alpha=4, n_default=128, top_k=10, gamma_pct=[30, 60, 100], phi_mode=0, pstar_mode=0,
+                  entropy_mode=0)
+    ctx = hb.Context(0, hb.hs_workspace_bytes(B, B * nodes, 64, q.shape[1], kt.shape[1]))
+    _, pr = hb.hs_entropy_quantify_prune(ctx, tree, torch.zeros(B * nodes, 64, device="cuda"), policy)
+    r, t = slice(b0 * nodes, b1 * nodes), slice(b0 * kv, b1 * kv)
+    out = hb.hs_tree_verify_attention(ctx, pr, q[r], kt[r], vt[r], kc[t], vc[t], i32([b * kv for b in range(B + 1)]), batch=B, max_nodes=nodes,
+                                      max_kv_len=kv)
+    assert hb.hs_device_error(ctx) == 0 and pr.n_keep.tolist() == [nodes] * B
+    ctx.close()
+    return out
+
+
+def error(out, x, batch, nodes, kv):
+    q, kt, vt, kc, vc = x
+    hkv, G, num, den = kt.shape[1], q.shape[1] // kt.shape[1], 0.0, 0.0
+    mask = torch.cat([torch.ones(nodes, kv, device="cuda"), torch.tril(torch.ones(nodes, nodes, device="cuda"))], 1).bool()
+    for b in range(batch):
+        r, t = slice(b * nodes, (b + 1) * nodes), slice(b * kv, (b + 1) * kv)
+        for h in range(hkv):
+            k, v = torch.cat([kc[t, h], kt[r, h]]).double(), torch.cat([vc[t, h], vt[r, h]]).double()
+            hs = slice(h * G, (h + 1) * G)
+            s = (torch.einsum("ngd,kd->gnk", q[r, hs].double(), k) * 128 ** -0.5).masked_fill(~mask, -math.inf)
+            ref = torch.einsum("gnk,kd->ngd", torch.softmax(s, 2), v)
+            num += float(((out[r, hs].double() - ref) ** 2).sum())
+            den += float((ref ** 2).sum())
+    return math.sqrt(num / den)
+
+
+def test_a_split_prefix_rounds_the_output_once():
+    batch, nodes, kv = 4, 62, 16384                              # four query blocks x 32 (sequence, head) pairs, two splits
+    x = inputs(batch, nodes, 64, 8, kv, 5)
+    got = error(attend(x, 0, batch, nodes, kv), x, batch, nodes, kv)
+    assert got < 1.02 * math.sqrt(2) * ROUNDING, got             # (a third rounding: sqrt(3))
+
+
+@pytest.mark.parametrize("kv", [256, 640, 1000])
+def test_one_stream_per_row_is_as_exact_as_two(kv):
+    batch, nodes = 24, 60                                        # 384 query blocks at once, 128 at a time
+    x = inputs(batch, nodes, 32, 8, kv, kv)
+    one = error(attend(x, 0, batch, nodes, kv), x, batch, nodes, kv)
+    two = error(torch.cat([attend(x, b, b + 8, nodes, kv) for b in range(0, batch, 8)]), x, batch, nodes, kv)
+    assert one < 1.002 * two, (one, two)                         # (two 2-norms over 5.9 million outputs: 0.04 % of spread)
