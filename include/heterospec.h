@@ -178,7 +178,7 @@ typedef struct {
     int32_t batch;
     int32_t max_rows;      /* upper bound of kept nodes in total (host): e.g. n_nodes_total */
     int32_t max_nodes;     /* upper bound of kept nodes per sequence (host), <= HS_MAX_NODES */
-    int32_t kv_total;      /* tokens in the KV cache arrays = kv_off[B] (host copy) */
+    int32_t kv_total;      /* tokens the KV cache arrays hold, at least kv_off[B] (host) */
     int32_t max_kv_len;    /* longest prefix (host) */
     int32_t hq, hkv;       /* query heads, key/value heads; hq % hkv == 0, hq/hkv <= 16 */
     int32_t head_dim;      /* HS_HEAD_DIM */

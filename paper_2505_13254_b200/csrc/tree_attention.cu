@@ -692,9 +692,8 @@ static bool make_row_map(hs_ctx* ctx, CUtensorMap* tm, const void* base, size_t 
     return encode(ctx, tm, 2, base, gdim, gstr, box);
 }
 
-// KV splits (= cluster size): the one with the fewest tile steps on the critical path, waves of CTAs (as
-// many clusters of that size as the device runs at once) times tiles per CTA.  `step` = 1 tries 1..8,
-// `step` = 2 only powers of two.
+// KV splits (= cluster size) of tree_attn_umma_kernel: the number with the fewest tile steps on the critical path, waves of CTAs (as
+// many clusters of that size as the device runs at once) times tiles per CTA.
 static int choose_splits(int base_ctas, int sm_count, int prefix_tiles, const int* cluster_cap) {
     int best = 1;
     long best_cost = 0;
@@ -709,34 +708,34 @@ static int choose_splits(int base_ctas, int sm_count, int prefix_tiles, const in
     return best;
 }
 
-// Splits with which tree_attn_duo_kernel takes a launch, 0: it does not.  Two CTAs of it on an SM take 0.53 us per tile and about 10 us
-// at their ends, which overlap with the other CTA's tiles; one alone takes 0.9 us per tile at worst.  The other kernel takes 0.585 us per
-// tile and the same 10 us, which nothing overlaps.  With more blocks than SMs that kernel therefore pays for whole waves of CTAs
-// (less where lengths are mixed: 0.85).  Measured, other kernel against this one (192 to 512 blocks): 12 x 37..46 nodes, 32 / 8 heads,
-// 1200 tokens 50 us against 30; 6 x 42..59, 64 / 8, 1500..2160 tokens 56 against 38; 16 x 56, 64 / 8, 1700 tokens 87 against 70; 16 x 39..56,
-// 32 / 8, 1200..3160 tokens 52 against 53; 16 x 8..60, 32 / 8, 1024..8192 tokens 75 against 125 (75 with two splits).  With at most one block
-// per SM two splits are needed to share SMs at all, and what the merge costs is only won back by long prefixes: 4 x 60 nodes, 64 / 8 heads,
-// 32768 tokens 304 against 273, 6 x 31..48, 64 / 8, 8000 tokens 81 against 82, 4 x 59, 64 / 8, 2000..3400 tokens 35 against 37.  Up to 128 query
-// rows per head a launch is bound by its bytes and the other kernel has more of them in flight: 60.6 against 63.0.
-static int duo_splits(int base_ctas, int mblocks, int sm_count, int prefix_tiles, double mean_tiles) {
+// Splits with which tree_attn_duo_kernel takes a launch, 0: tree_attn_umma_kernel takes it.  The rule knows the number of query blocks (an
+// upper bound: small trees leave blocks empty) and the longest prefix; how the other lengths lie below it the host cannot tell (the cache arrays
+// may be larger than what is in use), so each line holds for equal lengths and for lengths spread over 0.2 .. 1 of the longest.
+// Times below: us a call back to back, the other kernel against this one, equal lengths | spread; 50..60 nodes a tree unless said otherwise.
+//   One query block per head: bound by the bytes, of which the other kernel has more in flight (60.6 against 63.0).
+//   At most one block per SM: only two splits share SMs at all.  128 blocks (4 trees, 64 / 8 heads): 8192 tokens 75.5 : 81.6 | 74.9 : 80.8,
+//   16384 142.3 : 143.7 | 141.0 : 139.8, 24576 212.9 : 210.9 | 208.8 : 201.9, 32768 286.2 : 280.6 | 284.5 : 265.7.  112 blocks, 32768: 283.3 : 277.4 |
+//   276.7 : 259.1; 144: 332.4 : 318.1 | 285.4 : 263.4; 96: 220.5 : 261.2 | 155.6 : 246.7.  So from 256 tiles and from three quarters of the SMs.
+//   More blocks than SMs: the other kernel pays for whole waves of CTAs, each with about 10 us around its tiles that nothing overlaps.
+//   - Up to 16 tiles those ends decide.  160 blocks, 512 tokens 23.6 : 17.9 | 17.8 : 16.0, 1024 31.1 : 26.3 | 19.8 : 23.0; 256: 24.9 : 19.3 | 20.7 : 17.8,
+//     32.2 : 27.1 | 25.2 : 25.7; 384: 36.7 : 33.2 | 31.0 : 28.2, 47.9 : 45.5 | 38.9 : 35.1; 512: 52.3 : 38.3 | 42.6 : 31.3, 63.8 : 52.4 | 52.9 : 41.2.
+//   - Up to 64 tiles a last wave that is at least a quarter empty.  160 blocks, 2048 tokens 54.8 : 43.1 | 44.0 : 37.4, 4096 91.3 : 74.3 | 76.2 : 65.4; 192: 55.9 :
+//     43.5 | 47.9 : 38.6, 77.8 : 74.2 | 63.9 : 67.1; 320: 92.2 : 70.2 | 74.8 : 41.3, 127.7 : 119.8 | 94.3 : 70.6.  Fuller waves, 2048: 256 blocks 47.8 : 42.8 |
+//     34.9 : 40.0; 384: 70.3 : 70.3 | 52.8 : 48.3, 4096 119.1 : 123.6 | 81.0 : 78.4.  Beyond, 8192: 160 blocks 127.9 : 133.0 | 100.8 : 120.8, 192: 124.6 : 134.7 | 95.4 : 124.5.
+//   - More than three waves at any length.  448 blocks, 2048 tokens 90.8 : 82.0 | 63.8 : 55.2, 8192 316 : 290 | 244 : 159; 512: 92.5 : 84.4 | 71.4 : 60.5, 342 : 303 |
+//     240 : 194, 16384 586 : 589 | 375 : 340; 576: 94.9 : 91.7 | 78.4 : 68.9, 8192 319 : 328 | 219 : 217; 1024, 2048 tokens 168 : 164 | 135 : 119.  Trees of 8..60
+//     nodes, 512 blocks, 2048: 72.8 : 79.9 | 54.3 : 54.1, 8192 272 : 278 | 188 : 159.
+static int duo_splits(int base_ctas, int mblocks, int sm_count, int prefix_tiles, int pair_cap) {
     if (mblocks == 1) return 0;
-    if (base_ctas <= sm_count)
-        return 4 * base_ctas > 3 * sm_count && prefix_tiles >= 256 && mean_tiles >= 0.9 * prefix_tiles ? 2 : 0;
-    int best = 0;
-    double best_us = 0.85 * ((base_ctas + sm_count - 1) / sm_count) * (mean_tiles * 0.585 + 10.);
-    for (int s = 1; s <= ATT_MAX_SPLIT && (s == 1 || s <= prefix_tiles); ++s) {
-        const double longest = 10. + 0.9 * ((prefix_tiles + s) / s);
-        // (clusters that do not all run at once leave SMs idle at the end: half a CTA's time)
-        const double all = base_ctas * (mean_tiles * 0.53 + s * 10. / 2) / sm_count + (s > 1 && base_ctas * s > 2 * sm_count ? longest / 2 : 0.);
-        const double us = std::max(longest, all);
-        if (us < best_us) { best_us = us; best = s; }
-    }
-    return best;
+    if (base_ctas <= sm_count)                       // (pair_cap: CTAs in clusters of two that run at once)
+        return 4 * base_ctas > 3 * sm_count && prefix_tiles >= 256 && 2 * base_ctas <= pair_cap ? 2 : 0;
+    const int waves = (base_ctas + sm_count - 1) / sm_count;
+    return prefix_tiles <= 16 || (prefix_tiles <= 64 && 4 * base_ctas <= 3 * waves * sm_count) || waves > 3 ? 1 : 0;
 }
 
 template <typename Kernel>
-static void query_cluster_caps(Kernel kernel, int threads, size_t smem, int sm_count, int* cap) {
-    for (int sz = 1; sz <= ATT_MAX_SPLIT; ++sz) {
+static void query_cluster_caps(Kernel kernel, int threads, size_t smem, int sm_count, int first, int last, int* cap) {
+    for (int sz = first; sz <= last; ++sz) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(1, sz, sm_count);
         cfg.blockDim = dim3(threads);
@@ -762,7 +761,8 @@ hs_status hs_launch_attention(hs_ctx* ctx, const hs_pruned_tree* pruned, const h
             return HS_ERR_CUDA;
         if (cudaFuncSetAttribute(tree_attn_duo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AD_SMEM_BYTES) != cudaSuccess)
             return HS_ERR_CUDA;
-        query_cluster_caps(tree_attn_umma_kernel, UM_THREADS, UM_SMEM_BYTES, ctx->sm_count, cap_umma);
+        query_cluster_caps(tree_attn_umma_kernel, UM_THREADS, UM_SMEM_BYTES, ctx->sm_count, 1, ATT_MAX_SPLIT, cap_umma);
+        query_cluster_caps(tree_attn_duo_kernel, AD_THREADS, AD_SMEM_BYTES, ctx->sm_count, 2, 2, ctx->duo_cap);
         ctx->attn_ready = true;
     }
     AttnParams p;
@@ -795,7 +795,7 @@ hs_status hs_launch_attention(hs_ctx* ctx, const hs_pruned_tree* pruned, const h
     memset(&tmV, 0, sizeof(tmV));
     const int mblocks = (rows + ATT_BM - 1) / ATT_BM;
     const int prefix_tiles = (d->max_kv_len + ATT_BN - 1) / ATT_BN;
-    const int duo = duo_splits(pairs * mblocks, mblocks, ctx->sm_count, prefix_tiles, (double)d->kv_total / ATT_BN / d->batch + 1.5);
+    const int duo = duo_splits(pairs * mblocks, mblocks, ctx->sm_count, prefix_tiles, ctx->duo_cap[2]);
     p.nsplit = duo ? duo : choose_splits(pairs * mblocks, ctx->sm_count, prefix_tiles, cap_umma);
     if (d->kv_total > 0) {
         if (!make_kv_map(ctx, &tmK, k_cache, d, p.head_first) || !make_kv_map(ctx, &tmV, v_cache, d, p.head_first))
