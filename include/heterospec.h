@@ -98,8 +98,8 @@ hs_status hs_set_prefetch(hs_ctx* ctx, int32_t flags);
  * the same results.  HS_ROW_PASS_CHUNK: one small CTA per 32 KiB of a row, all loads in flight at once - shortest
  * latency when the rows of a step are few.  HS_ROW_PASS_STREAM: every warp of the device streams an equal share of
  * the rows - highest bandwidth when the rows of a step exceed what is in flight at once.
- * HS_ROW_PASS_AUTO (default): the stream from 20 MiB of rows (upper bound of kept rows x row bytes, twice that with
- * draft logits), else chunks. */
+ * HS_ROW_PASS_AUTO (default): the stream from 20 MiB of rows (upper bound of kept rows x row bytes, twice that for a
+ * batch of several sequences with draft logits), else chunks. */
 #define HS_ROW_PASS_AUTO 0
 #define HS_ROW_PASS_CHUNK 1
 #define HS_ROW_PASS_STREAM 2

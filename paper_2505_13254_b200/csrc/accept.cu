@@ -383,9 +383,12 @@ __global__ void __launch_bounds__(HS_ROW_THREADS, 4) accept_rows_kernel(const __
 
 #include "accept_warps.cuh"
 
-// Launches with fewer bytes of rows (draft rows counted like target rows) go to the chunk kernel, whose loads are all in flight
-// at once.  60 greedy rows of 128256 bf16 (15 MB): 6.4 us against 9.4; with draft rows (31 MB) 18.9 against 19.3, 120 greedy rows
-// (31 MB) 13.1 against 12.5.
+// Launches with fewer bytes of rows go to the chunk kernel, whose loads are all in flight at once.  us a call, chunk against warp kernel,
+// greedy: 60 rows of 128256 bf16 (15 MiB) 8.3 : 11.1, 71 rows (17 MiB) 10.1 : 11.7, 92 (22 MiB) 12.6 : 12.3, 120 (29 MiB) 13.3 : 12.9, 180 of 64000
+// (22 MiB) 12.0 : 12.4.  With draft logits, which are read for the inner nodes of rejection sequences only: one such sequence is decided by the
+// same bytes (60 rows 20.0 : 20.4, alone 25.6 : 27.6).  In a batch the draft rows are counted like target rows, although 71 rows of two rejection
+// sequences take 22.0 in either kernel: the host does not see the modes, and the bonus draw of a deterministic-proposal sequence is shared
+// by the warp kernel at any size but by the chunk kernel only while its grid is resident (two such sequences, 71 rows: 55.2 : 28.0).
 #define AW_MIN_BYTES ((size_t)20 << 20)
 
 // ---- the walk ----------------------------------------------------------------------------------
@@ -807,7 +810,7 @@ hs_status hs_launch_accept(hs_ctx* ctx, const hs_tree_batch* tree, const hs_prun
     p.partials = (uint4*)(ctx->scratch + o);
     p.part_rows = rows;
     const bool streamed = ctx->row_pass == HS_ROW_PASS_STREAM ||
-                          (ctx->row_pass == HS_ROW_PASS_AUTO && (size_t)rows * p.nvec * (p.have_draft ? 32 : 16) >= AW_MIN_BYTES);
+                          (ctx->row_pass == HS_ROW_PASS_AUTO && (size_t)rows * p.nvec * (p.have_draft && p.batch > 1 ? 32 : 16) >= AW_MIN_BYTES);
     // (chunk kernel: a partial per chunk of a row; warp kernel: two per share, one share per warp of the device - fewer
     // and longer ones in a workspace without room for that)
     const size_t room = ctx->scratch_bytes > o ? (ctx->scratch_bytes - o) / (2 * sizeof(uint4)) : 0;
