@@ -151,7 +151,9 @@ def native():
 
 
 _native = None
-_raw_stream = torch._C._cuda_getCurrentRawStream
+# Handle of a device's current stream: torch's own accessor where this torch has it (a private symbol, absent from builds without
+# CUDA), else through the public stream object.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda device: torch.cuda.current_stream(device).cuda_stream)
 
 
 def hs_device_error(ctx: "Context") -> int:
