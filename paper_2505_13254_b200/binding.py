@@ -30,6 +30,8 @@ _lib = None
 i32p, f32p, u64p, vp = C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p   # device pointers travel as integers
 
 
+# Layouts of the C structs.  _PrunedTree, _AttnDesc, _ExpandState and _AcceptOut cross no call of this module (csrc/py_native.cpp fills its
+# own); a test holds their sizes against the header's.
 class _TreeBatch(C.Structure):
     _fields_ = [("batch", C.c_int32), ("n_nodes_total", C.c_int32), ("node_off", i32p), ("parent", i32p),
                 ("token", i32p)]
@@ -91,24 +93,8 @@ def lib() -> C.CDLL:
         L.hs_set_prefetch.argtypes = [C.c_void_p, C.c_int32]
         L.hs_set_row_pass.argtypes = [C.c_void_p, C.c_int32]
         L.hs_selftest_wait_timeout.argtypes = [C.c_void_p, C.c_uint64, vp]
-        L.hs_entropy_quantify.argtypes = [C.c_void_p, C.POINTER(_TreeBatch), vp, C.c_int, C.c_int64, C.c_int32,
-                                          C.POINTER(_Policy), C.POINTER(_QuantOut), vp]
-        L.hs_entropy_quantify_prune.argtypes = [C.c_void_p, C.POINTER(_TreeBatch), vp, C.c_int, C.c_int64, C.c_int32,
-                                                C.POINTER(_Policy), C.POINTER(_QuantOut), C.POINTER(_PrunedTree), vp]
         L.hs_entropy_quantify_static.argtypes = [C.POINTER(_TreeBatch), vp, C.c_int, C.c_int64, C.c_int32,
                                                  C.POINTER(_Policy), C.POINTER(_QuantOut), vp]
-        L.hs_stratify_prune.argtypes = [C.c_void_p, C.POINTER(_TreeBatch), C.POINTER(_QuantOut),
-                                        C.POINTER(_Policy), C.POINTER(_PrunedTree), vp]
-        L.hs_stratify_prune_budget.argtypes = [C.c_void_p, C.POINTER(_TreeBatch), C.POINTER(_QuantOut),
-                                               C.POINTER(_Policy), vp, C.c_int32, C.POINTER(_PrunedTree), vp]
-        L.hs_tree_verify_attention.argtypes = [C.c_void_p, C.POINTER(_PrunedTree), C.POINTER(_AttnDesc), vp, vp, vp,
-                                               vp, vp, vp, vp, vp]
-        L.hs_accept_path.argtypes = [C.c_void_p, C.POINTER(_TreeBatch), C.POINTER(_PrunedTree), vp, C.c_int32, vp,
-                                     C.c_int, C.c_int64, C.c_int32, vp, vp, C.c_uint64, C.c_uint64, vp,
-                                     C.POINTER(_AcceptOut), vp]
-        L.hs_expand_init.argtypes = [C.c_void_p, C.POINTER(_ExpandState), vp]
-        L.hs_expand_level.argtypes = [C.c_void_p, C.POINTER(_ExpandState), vp, vp, vp, C.c_int32, vp]
-        L.hs_rerank.argtypes = [C.c_void_p, C.POINTER(_ExpandState), vp, C.c_int32, vp, vp, vp, vp, vp, vp]
         L.hs_cart_workspace_bytes.restype = C.c_size_t
         L.hs_cart_workspace_bytes.argtypes = [C.c_int32]
         L.hs_cart_fit.argtypes = [C.c_void_p, vp, vp, C.c_int32, C.c_int32, vp, vp, vp]
@@ -198,7 +184,7 @@ class Context:
             pass
 
 
-# ---- tensor bundles mirroring the C structs --------------------------------------------------------
+# ---- tensor bundles with the fields of the C structs --------------------------------------------------------
 
 
 @dataclass
@@ -224,22 +210,7 @@ def make_policy(policy: dict) -> _Policy:
     return p
 
 
-class _Bundle:
-    _i32: tuple = ()
-    _f32: tuple = ()
-    _cstruct = None
-
-    def c(self):
-        s = self._cstruct()
-        for name, _ in self._cstruct._fields_:
-            v = getattr(self, name)
-            setattr(s, name, v if isinstance(v, int) else _ptr(v).value)
-        return s
-
-
-class QuantOut(_Bundle):
-    _cstruct = _QuantOut
-
+class QuantOut:
     def __init__(self, n: int, batch: int, k: int, device):
         f = lambda *s: torch.empty(*s, dtype=torch.float32, device=device)
         i = lambda *s: torch.empty(*s, dtype=torch.int32, device=device)
@@ -248,10 +219,11 @@ class QuantOut(_Bundle):
         self.logc, self.score, self.phi, self.depth = f(n), f(n), f(n), i(n)
         self.pstar_node, self.phi_star, self.status = i(batch), f(batch), i(batch)
 
+    def c(self) -> _QuantOut:
+        return _QuantOut(*(_ptr(getattr(self, name)) for name, _ in _QuantOut._fields_))
 
-class PrunedTree(_Bundle):
-    _cstruct = _PrunedTree
 
+class PrunedTree:
     def __init__(self, n: int, batch: int, device):
         i = lambda *s: torch.zeros(*s, dtype=torch.int32, device=device)
         self.bin, self.d_prime, self.n_prime, self.n_keep = i(batch), i(batch), i(batch), i(batch)
@@ -261,9 +233,7 @@ class PrunedTree(_Bundle):
         self.status = i(batch)
 
 
-class AcceptOut(_Bundle):
-    _cstruct = _AcceptOut
-
+class AcceptOut:
     def __init__(self, batch: int, path_cap: int, device):
         i = lambda *s: torch.empty(*s, dtype=torch.int32, device=device)
         self.accept_len, self.bonus_token, self.terminal_rank, self.status = i(batch), i(batch), i(batch), i(batch)
@@ -377,9 +347,8 @@ def hs_philox_uniforms(ctx: Context, seed: int, offset: int, b: torch.Tensor, no
     return out
 
 
-class ExpandState(_Bundle):
+class ExpandState:
     """Device arrays of the candidate tree (hs_expand_state)."""
-    _cstruct = _ExpandState
 
     def __init__(self, batch: int, cap: int, top_k: int, device):
         i = lambda *s: torch.zeros(*s, dtype=torch.int32, device=device)

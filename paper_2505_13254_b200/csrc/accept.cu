@@ -76,23 +76,6 @@ struct AcceptParams {
     int* err;             // sticky device error word (a bounded wait that expired)
 };
 
-__device__ __forceinline__ float ex2a(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-template <bool BF16>
-__device__ __forceinline__ void unpack_v(const uint4& v, float* x) {
-    if (BF16) {
-        x[0] = bf16_lo(v.x); x[1] = bf16_hi(v.x); x[2] = bf16_lo(v.y); x[3] = bf16_hi(v.y);
-        x[4] = bf16_lo(v.z); x[5] = bf16_hi(v.z); x[6] = bf16_lo(v.w); x[7] = bf16_hi(v.w);
-    } else {
-        x[0] = __uint_as_float(v.x); x[1] = __uint_as_float(v.y);
-        x[2] = __uint_as_float(v.z); x[3] = __uint_as_float(v.w);
-    }
-}
-
 // Greedy acceptance of sequence b by one whole CTA (Sec. 5, temperature 0): from the root, move to the kept
 // child whose token is the arg-max of the current node's target row until no child matches; the bonus
 // token is the arg-max where the walk stops.  tgt_arg was written by other CTAs: read it past L1.
@@ -268,7 +251,7 @@ __global__ void __launch_bounds__(HS_ROW_THREADS, 4) accept_rows_kernel(const __
         for (int q = 0; q < (BF16 ? 4 * VPT : 2 * VPT); ++q) {
             const float2 t = fma2_ftz(BF16 ? make_float2(bf16_lo(x[q]), bf16_hi(x[q]))
                                            : make_float2(__uint_as_float(x[2 * q]), __uint_as_float(x[2 * q + 1])), l2, n2);
-            s2 = add2_ftz(s2, make_float2(ex2a(t.x), ex2a(t.y)));
+            s2 = add2_ftz(s2, make_float2(ex2f(t.x), ex2f(t.y)));
         }
         s = warp_sum(s2.x + s2.y);
     }
@@ -295,7 +278,7 @@ __global__ void __launch_bounds__(HS_ROW_THREADS, 4) accept_rows_kernel(const __
     __syncthreads();
     bool merges = false;                                   // (warp 0: it holds the row's result)
     if (warp == 0) {
-        float S = sampling ? warp_sum(ws.x == -CUDART_INF_F ? 0.f : ws.y * ex2a((ws.x - M) * invT)) : 0.f;
+        float S = sampling ? warp_sum(ws.x == -CUDART_INF_F ? 0.f : ws.y * ex2f((ws.x - M) * invT)) : 0.f;
         unsigned long long key = M > -CUDART_INF_F ? make_key(M, (int)s_arg) : 0ull;
         if (p.chunks == 1) {
             merges = true;
@@ -337,7 +320,7 @@ __global__ void __launch_bounds__(HS_ROW_THREADS, 4) accept_rows_kernel(const __
                 int src;
                 key = warp_best_key(ck, src);
                 M = warp_max(cm);
-                if (sampling) S = warp_sum((cm == -CUDART_INF_F) ? 0.f : cs * ex2a((cm - M) * invT));
+                if (sampling) S = warp_sum((cm == -CUDART_INF_F) ? 0.f : cs * ex2f((cm - M) * invT));
             }
             if (lane == 0) {
                 s_flag = 1;
@@ -447,8 +430,8 @@ __device__ double cluster_residual_sum(const AcceptParams& p, unsigned int rank,
     for (int v = tid; v < rs.nv; v += WALK_THREADS) {
         uint4 a = rs.p[v], bq = rs.q[v];
         float x[8], y[8];
-        if (p.is_bf16) { unpack_v<true>(a, x); unpack_v<true>(bq, y); }
-        else { unpack_v<false>(a, x); unpack_v<false>(bq, y); }
+        if (p.is_bf16) { unpack<true>(a, x); unpack<true>(bq, y); }
+        else { unpack<false>(a, x); unpack<false>(bq, y); }
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             if (e < ve && (rs.v0 + v) * ve + e < p.vocab) {
@@ -484,8 +467,8 @@ __device__ void cluster_inverse_cdf(const AcceptParams& p, unsigned int rank, co
     auto masses = [&](int v, float (&m)[8]) {                               // of vector v of the slice
         float x[8], y[8];
         const uint4 a = rs.p[v];
-        if (p.is_bf16) unpack_v<true>(a, x); else unpack_v<false>(a, x);
-        if (rs.q) { const uint4 bq = rs.q[v]; if (p.is_bf16) unpack_v<true>(bq, y); else unpack_v<false>(bq, y); }
+        if (p.is_bf16) unpack<true>(a, x); else unpack<false>(a, x);
+        if (rs.q) { const uint4 bq = rs.q[v]; if (p.is_bf16) unpack<true>(bq, y); else unpack<false>(bq, y); }
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             m[e] = 0.f;

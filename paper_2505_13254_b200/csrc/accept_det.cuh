@@ -31,7 +31,7 @@ __device__ __forceinline__ void slice_mass(const AcceptParams& p, const char* pr
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         float x[8];
-        if (p.is_bf16) unpack_v<true>(d[q], x); else unpack_v<false>(d[q], x);
+        if (p.is_bf16) unpack<true>(d[q], x); else unpack<false>(d[q], x);
 #pragma unroll
         for (int e = 0; e < 8; ++e)
             m[q][e] = e < ve ? exp2f((fmaxf(x[e], -1e30f) - pm) * invT) * ips : 0.f;     // (as in the accept tests below: the

@@ -440,7 +440,9 @@ hs_status hs_launch_quantify(hs_ctx* ctx, const hs_tree_batch* tree, const void*
     const int pv = parts ? (p.nvec + parts - 1) / parts : 0;
     cudaError_t e;
     if (parts && pv <= QS_SLOTS * QS_ITEM_VECS) {
-        if ((size_t)p.rows * parts * HS_ROW_PARTIAL_BYTES > ctx->scratch_bytes) return HS_ERR_WORKSPACE;   // (not sized for the batch)
+        // (The parts merge on chip and use none of it, but a workspace that was not sized for the batch stays refused: whether a call is
+        // accepted does not depend on which kernel takes it.)
+        if ((size_t)p.rows * parts * HS_ROW_PARTIAL_BYTES > ctx->scratch_bytes) return HS_ERR_WORKSPACE;
         if (!ctx->quant_ready) {
             if (cudaFuncSetAttribute(quantify_cluster_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_BYTES) != cudaSuccess ||
                 cudaFuncSetAttribute(quantify_cluster_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_BYTES) != cudaSuccess)
