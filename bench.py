@@ -412,12 +412,13 @@ def main():
     attn_flops = float(4 * cfg.head_dim * cfg.hq * (nk_b * (kv_len + nk_b)).sum())
     a_tflops = attn_flops / (kern["attention"]["us"] * 1e-6) / 1e12
     tf_peak = tensor_peak()
+    attn_traffic = ncu_traffic("tree_attn_umma_kernel", cfg.name) or ncu_traffic("tree_attn_duo_kernel", cfg.name)
     if attn_flops / (tf_peak * 1e12) > attn_bytes / (peak * 1e9):      # the tensor pipe is the longer leg
         line["roofline_attention"] = {"kernel": "tree_attn_umma_kernel or tree_attn_duo_kernel, by size (hs_tree_verify_attention, one launch per step)",
                                       "bound": "tensor", "achieved": a_tflops, "peak": tf_peak, "unit": "TFLOP/s",
                                       "frac": a_tflops / tf_peak, "frac_of_nominal": a_tflops / NOMINAL_BF16_TFLOPS,
                                       "peak_kind": peak_kind + " (dense bf16 burst figure)",
-                                      "traffic": ncu_traffic("tree_attn_umma_kernel", cfg.name),
+                                      "traffic": attn_traffic,
                                       "algorithmic_flops_per_launch": attn_flops,
                                       "algorithmic_bytes_per_launch": attn_bytes}
     else:
@@ -426,7 +427,7 @@ def main():
                                       "frac": a_gbs / peak if a_gbs else None,
                                       "frac_of_nominal": a_gbs / NOMINAL_HBM_GBS if a_gbs else None,
                                       "peak_kind": peak_kind + " (burst copy figure)",
-                                      "traffic": ncu_traffic("tree_attn_umma_kernel", cfg.name),
+                                      "traffic": attn_traffic,
                                       "algorithmic_bytes_per_launch": attn_bytes,
                                       "algorithmic_flops_per_launch": attn_flops}
     # ---- a graph per regime (Sec. 4.3): the same tree forced into the lowest and into the highest entropy bin ---------

@@ -79,8 +79,8 @@ struct AcceptParams {
 // Greedy acceptance of sequence b by one whole CTA (Sec. 5, temperature 0): from the root, move to the kept
 // child whose token is the arg-max of the current node's target row until no child matches; the bonus
 // token is the arg-max where the walk stops.  tgt_arg was written by other CTAs: read it past L1.
-// The two walks below are run by the first HS_ROW_THREADS threads of a CTA (the whole CTA of the chunk kernel, half
-// of the consumer warps of the streaming kernel), which meet on a barrier of their own.
+// The two walks below are run by the first HS_ROW_THREADS threads of a CTA (the whole CTA of the chunk kernel, eight of the
+// sixteen warps of the warp kernel), which meet on a barrier of their own.
 __device__ __forceinline__ void walk_sync() { named_bar_sync(2, HS_ROW_THREADS); }
 
 // last b with off[b] <= k (skips empty sequences), by a whole warp
@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(WALK_THREADS, 1) accept_walk_kernel(const __gr
     __shared__ double s_part[WALK_THREADS / 32];
     __shared__ double s_scan[WALK_THREADS / 32];
     __shared__ unsigned long long s_x[2][WALK_CLUSTER];    // all-gather buffers of the cluster exchanges
-    unsigned int xch = 0;                  // exchanges through s_cta so far
+    unsigned int xch = 0;                  // exchanges through s_x so far
     __shared__ int s_pick[2];
     const int tid = threadIdx.x;
     const int b = blockIdx.x / WC;

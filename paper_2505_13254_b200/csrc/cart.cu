@@ -6,7 +6,8 @@
 //     N L = nL SyyL - SyL^2 + nR SyyR - SyR^2           (Eq. 2 times the node's sample count)
 // - and takes, per node, the position with the smallest L (ties: the smallest), between distinct feature values
 // only.  The threshold is the midpoint of the two neighbouring feature values.  (The form without divisions orders the
-// positions of a node as L does, is exact for integer ranks, and costs ten fp64 operations instead of sixty.)
+// positions of a node as L does and costs ten fp64 operations instead of sixty.  For integer ranks it is exact while n Syy stays below
+// 2^53 - ranks up to 59: 1.6 million samples - and rounded to fp64 like any other above.)
 //
 // Sort: least-significant-digit radix sort of 64-bit keys (order bits of x : bits of y), four passes over the 8-bit digits
 // of x; stable, so equal feature values keep their order and need no more passes.  A bitonic network took 65 launches

@@ -34,7 +34,7 @@ struct hs_ctx {
     bool walk_ready;    // acceptance walk kernel attributes set on this device
     bool cart_ready;    // single-CTA stratifier training: shared-memory attribute set on this device
     bool warps_ready;   // warp kernel of the entropy pass: shared-memory attribute set on this device
-    bool quant_ready;   // streaming entropy kernel: shared-memory attribute set on this device
+    bool quant_ready;   // cluster kernel of the entropy pass: shared-memory attribute set on this device
 };
 
 // The context's device must be the calling thread's current device (launches go to the current device).

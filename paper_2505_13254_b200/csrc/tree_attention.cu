@@ -16,7 +16,7 @@
 // an owner merges its rows once all pieces have landed.  No partial ever goes to global memory and
 // there is no second launch.
 //
-// Launches of more than one wave of such CTAs go to tree_attn_duo.cuh, where two CTAs share an SM.
+// Launches of more than one wave of such CTAs, and long prefixes, may go to tree_attn_duo.cuh, where two CTAs share an SM (see duo_splits).
 #include <math_constants.h>
 #include <algorithm>
 

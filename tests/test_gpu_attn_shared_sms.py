@@ -1,4 +1,4 @@
-"""Tree attention in launches of more query blocks than SMs, where two CTAs share an SM: prefixes around the edges of a key tile and
+"""Tree attention in launches of more query blocks than SMs, and of fewer with long prefixes, where two CTAs share an SM: prefixes around the edges of a key tile and
 none at all, trees of 1 to 128 nodes (one or two tree tiles, dead query blocks), grouped heads that do not divide a block, split
 prefixes, both row layouts and both cache layouts; against fp32 attention."""
 import math
@@ -17,6 +17,7 @@ pytestmark = pytest.mark.gpu
     (40, (30, 128), 21, 3, [0, 7, 64, 200, 700], hb.HS_ROWS_ORIGINAL, True, False),
     (12, (60, 128), 64, 4, [2500, 64, 3000, 1], hb.HS_ROWS_COMPACT, True, True),
     (10, (40, 60), 32, 8, [4096, 4097, 130], hb.HS_ROWS_ORIGINAL, False, True),
+    (4, (50, 62), 64, 8, [16500, 70, 0, 12000], hb.HS_ROWS_ORIGINAL, False, False),
 ])
 def test_two_ctas_per_sm(batch, nodes, hq, hkv, kv, layout, head_first, prefetch):
     rng = random.Random(batch + hq)

@@ -1,6 +1,6 @@
 """hs_accept_path reads the vocabulary rows with one of two kernels (hs_set_row_pass): small CTAs that own one
-32 KiB chunk of a row, or one persistent CTA per SM that streams its share of all rows.  The default picks by the
-size of the launch, so the small parity cases never reach the streaming kernel by themselves: here every
+32 KiB chunk of a row, or warps that each stream an equal share of all rows.  The default picks by the
+size of the launch, so the small parity cases never reach the warp kernel by themselves: here every
 acceptance case runs with each kernel forced and is compared with the CPU oracle (bit-exact paths, bonus tokens
 and ranks), including ragged vocabularies, fp32 logits, empty and malformed sequences, compacted target rows."""
 import numpy as np
