@@ -710,7 +710,7 @@ static int choose_splits(int base_ctas, int sm_count, int prefix_tiles, const in
 
 // Splits with which tree_attn_duo_kernel takes a launch, 0: tree_attn_umma_kernel takes it.  The rule knows the number of query blocks (an
 // upper bound: small trees leave blocks empty) and the longest prefix; how the other lengths lie below it the host cannot tell (the cache arrays
-// may be larger than what is in use), so each line holds for equal lengths and for lengths spread over 0.2 .. 1 of the longest.
+// may be larger than what is in use), so each line is drawn for equal lengths and for lengths spread over 0.2 .. 1 of the longest together.
 // Times below: us a call back to back, the other kernel against this one, equal lengths | spread; 50..60 nodes a tree unless said otherwise.
 //   One query block per head: bound by the bytes, of which the other kernel has more in flight (60.6 against 63.0).
 //   At most one block per SM: only two splits share SMs at all.  128 blocks (4 trees, 64 / 8 heads): 8192 tokens 75.5 : 81.6 | 74.9 : 80.8,
@@ -722,6 +722,8 @@ static int choose_splits(int base_ctas, int sm_count, int prefix_tiles, const in
 //   - Up to 64 tiles a last wave that is at least a quarter empty.  160 blocks, 2048 tokens 54.8 : 43.1 | 44.0 : 37.4, 4096 91.3 : 74.3 | 76.2 : 65.4; 192: 55.9 :
 //     43.5 | 47.9 : 38.6, 77.8 : 74.2 | 63.9 : 67.1; 320: 92.2 : 70.2 | 74.8 : 41.3, 127.7 : 119.8 | 94.3 : 70.6.  Fuller waves, 2048: 256 blocks 47.8 : 42.8 |
 //     34.9 : 40.0; 384: 70.3 : 70.3 | 52.8 : 48.3, 4096 119.1 : 123.6 | 81.0 : 78.4.  Beyond, 8192: 160 blocks 127.9 : 133.0 | 100.8 : 120.8, 192: 124.6 : 134.7 | 95.4 : 124.5.
+//   - Up to 128 tiles a second wave of at most a sixth: two splits.  160 blocks, 6144 tokens 109.7 : 105.9 | 90.6 : 71.6, 8192 128.1 : 130.1 | 103.0 : 81.9, 10000 142.2 :
+//     154.0 | 117.7 : 100.4; 168: 103.2 : 105.5 | 79.7 : 71.5; 176: 104.3 : 106.8 | 88.6 : 80.6; 192: 124.6 : 133.1 | 95.4 : 96.2 (8192).
 //   - More than three waves at any length.  448 blocks, 2048 tokens 90.8 : 82.0 | 63.8 : 55.2, 8192 316 : 290 | 244 : 159; 512: 92.5 : 84.4 | 71.4 : 60.5, 342 : 303 |
 //     240 : 194, 16384 586 : 589 | 375 : 340; 576: 94.9 : 91.7 | 78.4 : 68.9, 8192 319 : 328 | 219 : 217; 1024, 2048 tokens 168 : 164 | 135 : 119.  Trees of 8..60
 //     nodes, 512 blocks, 2048: 72.8 : 79.9 | 54.3 : 54.1, 8192 272 : 278 | 188 : 159.
@@ -729,6 +731,7 @@ static int duo_splits(int base_ctas, int mblocks, int sm_count, int prefix_tiles
     if (mblocks == 1) return 0;
     if (base_ctas <= sm_count)                       // (pair_cap: CTAs in clusters of two that run at once)
         return 4 * base_ctas > 3 * sm_count && prefix_tiles >= 256 && 2 * base_ctas <= pair_cap ? 2 : 0;
+    if (prefix_tiles > 64 && prefix_tiles <= 128 && 6 * base_ctas <= 7 * sm_count) return 2;
     const int waves = (base_ctas + sm_count - 1) / sm_count;
     return prefix_tiles <= 16 || (prefix_tiles <= 64 && 4 * base_ctas <= 3 * waves * sm_count) || waves > 3 ? 1 : 0;
 }

@@ -16,6 +16,7 @@ pytestmark = pytest.mark.gpu
     (60, 32, 8, [2048 - 151 * b for b in range(10)]),                   # a last wave that is nearly empty
     (60, 32, 8, [1024 - 61 * b for b in range(16)]),                    # 16 tiles
     (60, 32, 8, [1025 - 61 * b for b in range(16)]),                    # 17
+    (60, 32, 8, [6000 - 601 * b for b in range(10)]),                   # the same, longer: two splits
     (62, 64, 8, [16400, 0, 64, 9000]),                                  # two splits, some of them empty
     (62, 64, 8, [16320, 16300, 1, 8000]),                               # one tile less: one split of the other kernel or more
     (62, 64, 8, [300 + 17 * b for b in range(20)]),                     # more than three waves
