@@ -29,7 +29,6 @@ struct hs_ctx {
     int prefetch;       // HS_PREFETCH_* bits: inputs a kernel may fetch before its dependency wait
     bool attn_ready;    // attention kernel attributes set and cluster capacities queried on this device
     int attn_cap[9];    // CTAs of tree_attn_umma_kernel that run at once in clusters of s = 1..8
-    int duo_cap[3];     // the same of tree_attn_duo_kernel, [2]: pairs
     int walk_cap;       // 16-CTA clusters of the acceptance walk that run at once
     bool walk_ready;    // acceptance walk kernel attributes set on this device
     bool cart_ready;    // single-CTA stratifier training: shared-memory attribute set on this device

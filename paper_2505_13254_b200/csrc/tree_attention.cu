@@ -727,18 +727,19 @@ static int choose_splits(int base_ctas, int sm_count, int prefix_tiles, const in
 //   - More than three waves at any length.  448 blocks, 2048 tokens 90.8 : 82.0 | 63.8 : 55.2, 8192 316 : 290 | 244 : 159; 512: 92.5 : 84.4 | 71.4 : 60.5, 342 : 303 |
 //     240 : 194, 16384 586 : 589 | 375 : 340; 576: 94.9 : 91.7 | 78.4 : 68.9, 8192 319 : 328 | 219 : 217; 1024, 2048 tokens 168 : 164 | 135 : 119.  Trees of 8..60
 //     nodes, 512 blocks, 2048: 72.8 : 79.9 | 54.3 : 54.1, 8192 272 : 278 | 188 : 159.
-static int duo_splits(int base_ctas, int mblocks, int sm_count, int prefix_tiles, int pair_cap) {
+// Two CTAs on an SM is what runs (128 blocks of 129 tiles take 104 us alone, 256 blocks 146), also in pairs; cudaOccupancyMaxActiveClusters
+// counts one, as it does for any kernel that allocates tensor memory (it does not know how many columns), so it is not asked.
+static int duo_splits(int base_ctas, int mblocks, int sm_count, int prefix_tiles) {
     if (mblocks == 1) return 0;
-    if (base_ctas <= sm_count)                       // (pair_cap: CTAs in clusters of two that run at once)
-        return 4 * base_ctas > 3 * sm_count && prefix_tiles >= 256 && 2 * base_ctas <= pair_cap ? 2 : 0;
+    if (base_ctas <= sm_count) return 4 * base_ctas > 3 * sm_count && prefix_tiles >= 256 ? 2 : 0;
     if (prefix_tiles > 64 && prefix_tiles <= 128 && 6 * base_ctas <= 7 * sm_count) return 2;
     const int waves = (base_ctas + sm_count - 1) / sm_count;
     return prefix_tiles <= 16 || (prefix_tiles <= 64 && 4 * base_ctas <= 3 * waves * sm_count) || waves > 3 ? 1 : 0;
 }
 
 template <typename Kernel>
-static void query_cluster_caps(Kernel kernel, int threads, size_t smem, int sm_count, int first, int last, int* cap) {
-    for (int sz = first; sz <= last; ++sz) {
+static void query_cluster_caps(Kernel kernel, int threads, size_t smem, int sm_count, int* cap) {
+    for (int sz = 1; sz <= ATT_MAX_SPLIT; ++sz) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(1, sz, sm_count);
         cfg.blockDim = dim3(threads);
@@ -764,8 +765,7 @@ hs_status hs_launch_attention(hs_ctx* ctx, const hs_pruned_tree* pruned, const h
             return HS_ERR_CUDA;
         if (cudaFuncSetAttribute(tree_attn_duo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AD_SMEM_BYTES) != cudaSuccess)
             return HS_ERR_CUDA;
-        query_cluster_caps(tree_attn_umma_kernel, UM_THREADS, UM_SMEM_BYTES, ctx->sm_count, 1, ATT_MAX_SPLIT, cap_umma);
-        query_cluster_caps(tree_attn_duo_kernel, AD_THREADS, AD_SMEM_BYTES, ctx->sm_count, 2, 2, ctx->duo_cap);
+        query_cluster_caps(tree_attn_umma_kernel, UM_THREADS, UM_SMEM_BYTES, ctx->sm_count, cap_umma);
         ctx->attn_ready = true;
     }
     AttnParams p;
@@ -798,7 +798,7 @@ hs_status hs_launch_attention(hs_ctx* ctx, const hs_pruned_tree* pruned, const h
     memset(&tmV, 0, sizeof(tmV));
     const int mblocks = (rows + ATT_BM - 1) / ATT_BM;
     const int prefix_tiles = (d->max_kv_len + ATT_BN - 1) / ATT_BN;
-    const int duo = duo_splits(pairs * mblocks, mblocks, ctx->sm_count, prefix_tiles, ctx->duo_cap[2]);
+    const int duo = duo_splits(pairs * mblocks, mblocks, ctx->sm_count, prefix_tiles);
     p.nsplit = duo ? duo : choose_splits(pairs * mblocks, ctx->sm_count, prefix_tiles, cap_umma);
     if (d->kv_total > 0) {
         if (!make_kv_map(ctx, &tmK, k_cache, d, p.head_first) || !make_kv_map(ctx, &tmV, v_cache, d, p.head_first))
