@@ -7,8 +7,8 @@
 // their own) before it waits for the kernel ahead of it in the stream if the caller vouches for the cache (it does not
 // depend on the pruned tree).  The <= 128 tree keys belong to the last split; their rows may be indirect.  Behind
 // prefix tiles the producer warp fetches them by tile::gather4 (plain loads by the softmax threads held up the
-// longest split: 4096 tokens, 64 / 8 heads 19.6 us against 18.0, a ragged batch of 16 75.5 against 71).  S = Q K^T and O += P V run on the 5th-generation tensor
-// cores (tcgen05.mma, accumulators in tensor memory) with fp32 accumulation; the softmax is the
+// longest split: 4096 tokens, 64 / 8 heads 19.6 us against 18.0, a ragged batch of 16 75.5 against 71).  S = Q K^T and
+// O += P V run on the 5th-generation tensor cores (tcgen05.mma, accumulators in tensor memory) with fp32 accumulation; the softmax is the
 // online (running max / running sum) form in base 2.  Prefix columns are fully visible, tree column j
 // is visible to row r iff bit j of the ancestor mask of r's node is set.  The splits of one (query
 // block, head) form a thread-block cluster: every CTA sends its partial (max, sum, O) from registers
@@ -708,25 +708,32 @@ static int choose_splits(int base_ctas, int sm_count, int prefix_tiles, const in
     return best;
 }
 
-// Splits with which tree_attn_duo_kernel takes a launch, 0: tree_attn_umma_kernel takes it.  The rule knows the number of query blocks (an
-// upper bound: small trees leave blocks empty) and the longest prefix; how the other lengths lie below it the host cannot tell (the cache arrays
-// may be larger than what is in use), so each line is drawn for equal lengths and for lengths spread over 0.2 .. 1 of the longest together.
-// Times below: us a call back to back, the other kernel against this one, equal lengths | spread; 50..60 nodes a tree unless said otherwise.
-//   One query block per head: bound by the bytes, of which the other kernel has more in flight (60.6 against 63.0).
-//   At most one block per SM: only two splits share SMs at all.  128 blocks (4 trees, 64 / 8 heads): 8192 tokens 75.5 : 81.6 | 74.9 : 80.8,
-//   16384 142.3 : 143.7 | 141.0 : 139.8, 24576 212.9 : 210.9 | 208.8 : 201.9, 32768 286.2 : 280.6 | 284.5 : 265.7.  112 blocks, 32768: 283.3 : 277.4 |
-//   276.7 : 259.1; 144: 332.4 : 318.1 | 285.4 : 263.4; 96: 220.5 : 261.2 | 155.6 : 246.7.  So from 256 tiles and from three quarters of the SMs.
-//   More blocks than SMs: the other kernel pays for whole waves of CTAs, each with about 10 us around its tiles that nothing overlaps.
-//   - Up to 16 tiles those ends decide.  160 blocks, 512 tokens 23.6 : 17.9 | 17.8 : 16.0, 1024 31.1 : 26.3 | 19.8 : 23.0; 256: 24.9 : 19.3 | 20.7 : 17.8,
-//     32.2 : 27.1 | 25.2 : 25.7; 384: 36.7 : 33.2 | 31.0 : 28.2, 47.9 : 45.5 | 38.9 : 35.1; 512: 52.3 : 38.3 | 42.6 : 31.3, 63.8 : 52.4 | 52.9 : 41.2.
-//   - Up to 64 tiles a last wave that is at least a quarter empty.  160 blocks, 2048 tokens 54.8 : 43.1 | 44.0 : 37.4, 4096 91.3 : 74.3 | 76.2 : 65.4; 192: 55.9 :
-//     43.5 | 47.9 : 38.6, 77.8 : 74.2 | 63.9 : 67.1; 320: 92.2 : 70.2 | 74.8 : 41.3, 127.7 : 119.8 | 94.3 : 70.6.  Fuller waves, 2048: 256 blocks 47.8 : 42.8 |
-//     34.9 : 40.0; 384: 70.3 : 70.3 | 52.8 : 48.3, 4096 119.1 : 123.6 | 81.0 : 78.4.  Beyond, 8192: 160 blocks 127.9 : 133.0 | 100.8 : 120.8, 192: 124.6 : 134.7 | 95.4 : 124.5.
-//   - Up to 128 tiles a second wave of at most a sixth: two splits.  160 blocks, 6144 tokens 109.7 : 105.9 | 90.6 : 71.6, 8192 128.1 : 130.1 | 103.0 : 81.9, 10000 142.2 :
-//     154.0 | 117.7 : 100.4; 168: 103.2 : 105.5 | 79.7 : 71.5; 176: 104.3 : 106.8 | 88.6 : 80.6; 192: 124.6 : 133.1 | 95.4 : 96.2 (8192).
-//   - More than three waves at any length.  448 blocks, 2048 tokens 90.8 : 82.0 | 63.8 : 55.2, 8192 316 : 290 | 244 : 159; 512: 92.5 : 84.4 | 71.4 : 60.5, 342 : 303 |
-//     240 : 194, 16384 586 : 589 | 375 : 340; 576: 94.9 : 91.7 | 78.4 : 68.9, 8192 319 : 328 | 219 : 217; 1024, 2048 tokens 168 : 164 | 135 : 119.  Trees of 8..60
-//     nodes, 512 blocks, 2048: 72.8 : 79.9 | 54.3 : 54.1, 8192 272 : 278 | 188 : 159.
+// Splits with which tree_attn_duo_kernel takes a launch, 0: tree_attn_umma_kernel takes it.
+// What is known is the number of query blocks (an upper bound: small trees leave blocks empty) and the longest prefix; how the other
+// lengths lie below it the host cannot tell (the cache arrays may be larger than what is in use), so every line is drawn for equal
+// lengths and for lengths spread over 0.2 .. 1 of the longest together.  Measured in us a call, back to back, 50..60 nodes a tree, as
+// "other kernel : this one", equal lengths | spread:
+//   At most one block per SM: only two splits let CTAs share SMs.  From 256 tiles (16384 tokens) and three quarters of the SMs.
+//     blocks    8192 tokens               16384                         24576                         32768
+//      96                                                                                             221 : 261 | 156 : 247
+//     112        75.3 : 82.5 | 74.3 : 80.3  141 : 144 | 140 : 139         211 : 208 | 208 : 194         283 : 277 | 277 : 259
+//     128        75.5 : 81.6 | 74.9 : 80.8  142 : 144 | 141 : 140         213 : 211 | 209 : 202         286 : 281 | 285 : 266
+//     144        82.6 : 87.5 | 75.5 : 79.3  163 : 165 | 154 : 144         247 : 235 | 216 : 200         332 : 318 | 285 : 263
+//   More: the other kernel pays for whole waves of CTAs, each with about 10 us around its tiles that nothing overlaps.
+//     blocks     512 tokens                1024                          2048                          4096                          8192
+//     160        23.6 : 17.9 | 17.8 : 16.0  31.1 : 26.3 | 19.8 : 23.0     54.8 : 43.1 | 44.0 : 37.4     91.3 : 74.3 | 76.2 : 65.4     128 : 133 | 101 : 121
+//     192        24.0 : 18.2 | 20.0 : 17.2  31.3 : 26.4 | 24.6 : 24.8     55.9 : 43.5 | 47.9 : 38.6     77.8 : 74.2 | 63.9 : 67.1     125 : 135 | 95 : 125
+//     256        24.9 : 19.3 | 20.7 : 17.8  32.2 : 27.1 | 25.2 : 25.7     47.8 : 42.8 | 34.9 : 40.0     80.4 : 77.0 | 52.7 : 69.7     152 : 149 | 92 : 129
+//     320        35.5 : 32.8 | 29.1 : 24.9  47.3 : 45.5 | 35.3 : 30.1     92.2 : 70.2 | 74.8 : 41.3     128 : 120 | 94 : 71           204 : 224 | 145 : 139
+//     384        36.7 : 33.2 | 31.0 : 28.2  47.9 : 45.5 | 38.9 : 35.1     70.3 : 70.3 | 52.8 : 48.3     119 : 124 | 81 : 78           229 : 248 | 148 : 146
+//     448        48.7 : 38.0 | 40.0 : 30.5  63.3 : 52.5 | 48.7 : 39.9     90.8 : 82.0 | 63.8 : 55.2     179 : 145 | 140 : 88          316 : 290 | 244 : 159
+//     512        52.3 : 38.3 | 42.6 : 31.3  63.8 : 52.4 | 52.9 : 41.2     92.5 : 84.4 | 71.4 : 60.5     188 : 153 | 148 : 104         342 : 303 | 240 : 194
+//     1024        103 : 79 | 80 : 63         114 : 97 | 97 : 80            168 : 164 | 135 : 119         302 : 299 | 224 : 211
+//     - up to 16 tiles at any number; above three waves at any length; up to 64 tiles where the last wave is at least a quarter empty.
+//     - 65 to 128 tiles and a second wave of at most a sixth: two splits.  160 blocks, 6144 tokens 110 : 106 | 91 : 72, 8192 128 : 130 | 103 : 82,
+//       10000 142 : 154 | 118 : 100; 176: 6144 104 : 107 | 89 : 81; 192: 8192 125 : 133 | 95 : 96.
+//   One query block per head stays with the other kernel: no line is drawn for it yet.  The same ones would hold above one block per
+//   SM (8 x 20..30 nodes, 32 / 32 heads, 256 blocks: 512 tokens 23.8 : 18.3 | 19.4 : 16.3, 2048 51.5 : 47.2 | 35.8 : 40.5).
 // Two CTAs on an SM is what runs (128 blocks of 129 tiles take 104 us alone, 256 blocks 146), also in pairs; cudaOccupancyMaxActiveClusters
 // counts one, as it does for any kernel that allocates tensor memory (it does not know how many columns), so it is not asked.
 static int duo_splits(int base_ctas, int mblocks, int sm_count, int prefix_tiles) {
