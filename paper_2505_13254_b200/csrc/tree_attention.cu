@@ -18,7 +18,6 @@
 //
 // Launches of more than one wave of such CTAs, and long prefixes, may go to tree_attn_duo.cuh, where two CTAs share an SM (see duo_splits).
 #include <math_constants.h>
-#include <algorithm>
 
 #include "hs_common.cuh"
 #include "hs_layout.h"
@@ -813,8 +812,9 @@ hs_status hs_launch_attention(hs_ctx* ctx, const hs_pruned_tree* pruned, const h
     }
     const dim3 grid(mblocks, p.nsplit, pairs), cl(1, p.nsplit, 1);
     cudaError_t e;
-    // (rows of the original trees may lie past max_rows, a bound of the kept ones, but not past HS_MAX_NODES per sequence)
-    const size_t n = std::max((size_t)d->max_rows, (size_t)d->batch * HS_MAX_NODES);
+    // Rows by drafted node id may lie anywhere in the batch's rows, behind sequences that are skipped as well: past max_rows, which bounds
+    // the kept ones, but never past what a batch may hold.  (The maps only have to cover the rows that are asked for.)
+    const size_t n = HS_MAX_ROWS;
     const size_t w = (size_t)d->hkv * HS_HEAD_DIM;
     CUtensorMap tmQ, tmKT, tmVT;
     if (!make_row_map(ctx, &tmKT, k_tree, n, w) || !make_row_map(ctx, &tmVT, v_tree, n, w)) return HS_ERR_CUDA;
