@@ -333,11 +333,13 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     // shared-memory address reaches 2^18, so an offset is added to a descriptor built once.
     const unsigned long long dq0 = umma_desc_sw128(sQ, 16, 1024), dk0 = umma_desc_sw128(smem_base, 16, 1024);
     const unsigned long long dv0 = umma_desc_sw128(smem_base + ATT_TILE_BYTES, ATT_TILE_BYTES / 2, 1024);
-    // the issuing thread: S = Q K^T of tile i into S buffer i & 1 (waits for K unless load_tree wrote it), then commit
+    // the issuing warp: S = Q K^T of tile i into S buffer i & 1 (waits for K unless load_tree wrote it), then commit
     auto issue_qk = [&](int i) {
         const int stage = i % UM_STAGES;
         if (i < np || i >= UM_STAGES) mbar_wait(bar0 + stage * 8, (unsigned int)(i / UM_STAGES) & 1u, p.err);
+        __syncwarp();
         tc_fence_after_sync();
+        if (!elect_one()) return;
         const unsigned long long dk = dk0 + (unsigned long long)(stage * (ATT_STAGE_BYTES >> 4));
         const unsigned int ts = tS + (i & 1) * ATT_BN;
 #pragma unroll
@@ -349,11 +351,14 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         umma_commit(bar_s + (i & 1) * 8);
         if (i + UM_STAGES < ntiles) umma_commit(bar_ek + stage * 8);     // (the producer waits for it only then)
     };
-    // O of stream i & 1 += P V of tile i (waits for V likewise), then commit
+    // O of stream i & 1 += P V of tile i (waits for its P, and for V likewise), then commit
     auto issue_pv = [&](int i) {
         const int stage = i % UM_STAGES;
         if (i < np || i >= UM_STAGES) mbar_wait(bar_v + stage * 8, (unsigned int)(i / UM_STAGES) & 1u, p.err);
+        mbar_wait(bar_p + (i & 1) * 8, (unsigned int)(i >> 1) & 1u, p.err);   // P of tile i is written
+        __syncwarp();
         tc_fence_after_sync();
+        if (!elect_one()) return;
         const unsigned long long dv = dv0 + (unsigned long long)(stage * (ATT_STAGE_BYTES >> 4));
         const unsigned int tp = tP + (i & 1) * (ATT_BN / 2);
         const unsigned int to = tO + (i & 1) * HS_HEAD_DIM;
@@ -361,12 +366,17 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         for (int kk = 0; kk < 4; ++kk)                       // 16 keys per instruction: two 8-key groups of V
             umma_ts_bf16(to, tp + kk * 8, dv + (kk * 2048 >> 4), idesc_pv, (i > 1 || kk > 0) ? 1u : 0u);
         umma_commit(bar_ev + stage * 8);
+        // every S was read before the last P was written: all tensor-core work of this CTA is complete
+        if (i == ntiles - 1) umma_commit(bar_done);
     };
     float mrun = -CUDART_INF_F, lrun = 0.f;
 
     // ---- KV tiles ------------------------------------------------------------------------------------------
-    // Both single-thread roles sit behind a branch on a warp-uniform value with the thread chosen by elect.sync in
-    // every round (all lanes run the loop): the compiler then keeps loop counters, addresses and descriptors uniform.
+    // The single-thread roles sit behind a branch on a warp-uniform value; all lanes run the loop and wait, and elect.sync chooses the
+    // thread only for the instructions that one thread issues: the compiler then keeps loop counters, addresses and descriptors uniform.
+    // (The issuing warps are what a tile waits for - with almost no arithmetic left in the softmax warps a tile took as long.  With the waits
+    // inside the elected branch: 4 calls of 4 trees, 64 / 8 heads, 4900 tokens 188 us, now 168; 32 calls of one tree, 32 / 8 heads, 2048
+    // tokens 382, now 368; 12 trees, 32 / 32 heads, 600 - 1200 tokens 180, now 175.)
     const int warp_u = __shfl_sync(HS_FULL_MASK, warp, 0);
     if (warp_u == 8) {
         // The P V issuer: O += P V of tile i as soon as its P is written.  It is short work on the streams' critical
@@ -374,28 +384,20 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         // never held up behind the issue of an S.
 #pragma unroll 1
         for (int i = 0; i < ntiles; ++i) {
-            if (elect_one()) {
-                mbar_wait(bar_p + (i & 1) * 8, (unsigned int)(i >> 1) & 1u, p.err);   // P of tile i is written
-                issue_pv(i);
-                // every S was read before the last P was written: all tensor-core work of this CTA is complete
-                if (i == ntiles - 1) umma_commit(bar_done);
-            }
+            issue_pv(i);
             __syncwarp();
         }
     } else if (warp_u == 10) {
         // The S issuer: S of tile i + 2 as soon as the stream has S of tile i in registers, so a stream never waits
         // for its next S.
-        if (elect_one()) {
-            if (ntiles > 0) issue_qk(0);
-            if (ntiles > 1) issue_qk(1);
-        }
+        if (ntiles > 0) issue_qk(0);
+        __syncwarp();
+        if (ntiles > 1) issue_qk(1);
         __syncwarp();
 #pragma unroll 1
         for (int i = 0; i + 2 < ntiles; ++i) {
-            if (elect_one()) {
-                mbar_wait(bar_sr + (i & 1) * 8, (unsigned int)(i >> 1) & 1u, p.err);      // S of tile i is read
-                issue_qk(i + 2);
-            }
+            mbar_wait(bar_sr + (i & 1) * 8, (unsigned int)(i >> 1) & 1u, p.err);      // S of tile i is read
+            issue_qk(i + 2);
             __syncwarp();
         }
     } else if (warp_u == 9) {
@@ -404,10 +406,9 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         // (after S of tile i + 4).
         auto refill = [&](int i, bool is_v, unsigned int bar, unsigned int parity) {
             if (i < np) {
-                if (elect_one()) {
-                    mbar_wait(bar, parity, p.err);
-                    issue_kv(i, is_v);
-                }
+                mbar_wait(bar, parity, p.err);
+                __syncwarp();
+                if (elect_one()) issue_kv(i, is_v);
             } else {
                 mbar_wait(bar, parity, p.err);
                 __syncwarp();
