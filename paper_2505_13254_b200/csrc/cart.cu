@@ -14,12 +14,11 @@
 // and 0.9 ms on 2^20 samples (every exchange distance beyond shared memory is a pass over all keys); a pass here reads and
 // writes the keys once, which stay in L2.
 //   up to CT_SMALL samples   cart_small_kernel: one CTA sorts in shared memory and fits all layers - one launch, no round
-//                            trips between layers (17 us at 600 samples, 49 us at 8192; were 68 and 90).
+//                            trips between layers (15 us at 600 samples, 38 us at 8192; the grid kernel 40 at 8193).
+//   up to 8192 per SM        cart_grid_kernel (cart_grid.cuh): the same by a resident grid, one launch.
 //   more                     cart_pack_kernel (keys, digit counts of all passes), four cart_radix_kernel, cart_sums_kernel
-//                            (sums per block and their scan), one cart_level_kernel per layer: 70 us at 8193 samples (nine
-//                            launches, latency), 121 us at 2^20 and depth 3 (was 990 us): 12 us pack, 12 - 17 us a pass
-//                            (issue of the ranking ballots, and the look-back), 17 us a layer (fp64 chains and the last
-//                            CTA's reduction over the tiles).
+//                            (sums per block and their scan), one cart_level_kernel per layer (what a grid can hold takes it 1.6 times as
+//                            long: 125 us at 2^20 samples).
 #include <math_constants.h>
 
 #include "hs_common.cuh"
@@ -87,75 +86,102 @@ __device__ __forceinline__ int scan256(int v, int* s_warp, int tid) {
 }
 
 // ---- one layer: all split positions of a block of sorted keys -----------------------------------------------------
+struct LayerEntry {                                  // a split of a node
+    unsigned long long l;                            // N L as order bits, ~0: none
+    double sa, sb;                                   // running sums of y and y^2 at its position
+    float xp, x;                                     // the feature values on both sides
+    int pos;                                         // 0x7fffffff: none
+    int node;
+};
+__device__ __forceinline__ bool better(unsigned long long l, int pos, unsigned long long l2, int pos2) { return l < l2 || (l == l2 && pos < pos2); }
+
+#define CT_ENTRIES 96           // of a block: one per warp and one per boundary in it, and one per boundary inside a thread's run
 struct LayerSmem {
     int bnd[CT_MAX_NODES + 1];                       // node boundaries (positions in the sorted order)
     double sy[CT_MAX_NODES + 1], syy[CT_MAX_NODES + 1];   // running sums at the boundaries
-    unsigned long long best[CT_MAX_NODES];           // smallest N L of a node, as order bits
-    int pos[CT_MAX_NODES];                           // its position
-    double psy[CT_MAX_NODES], psyy[CT_MAX_NODES];    // running sums there
+    LayerEntry top[CT_MAX_NODES];                    // the block's best split of every node
+    LayerEntry ent[CT_ENTRIES];
+    int nent;
 };
+static_assert(CT_SMALL_THREADS / 32 + 2 * (CT_MAX_NODES - 1) <= CT_ENTRIES, "entries of a block");
 
-// Thread's run of `cnt` consecutive keys, key(j) = sorted key at position i0 + j (j = -1: the one ahead of it); (a, b):
-// running sums of y and y^2 ahead of the run.  Calls emit(node, i, N L, sums at i) for every position that may be split.
-template <class KeyFn, class EmitFn>
-__device__ __forceinline__ void scan_run(const LayerSmem& s, int nodes, int i0, int cnt, double a, double b, KeyFn key, EmitFn emit) {
-    if (cnt <= 0) return;
-    int node = 0;
-    while (node + 1 < nodes && s.bnd[node + 1] <= i0) ++node;
-    float xp = i0 > 0 ? key_x(key(-1)) : 0.f;
-    for (int j = 0; j < cnt; ++j) {
-        const int i = i0 + j;
-        while (node + 1 < nodes && s.bnd[node + 1] <= i) ++node;
-        const unsigned long long k = key(j);
-        const float x = key_x(k);
-        if (i > s.bnd[node] && xp < x) {                              // a threshold lies between distinct values
-            const double nl = (double)(i - s.bnd[node]), nr = (double)(s.bnd[node + 1] - i);
-            const double yl = a - s.sy[node], yyl = b - s.syy[node];
-            const double yr = s.sy[node + 1] - a, yyr = s.syy[node + 1] - b;
-            // (rounding spelled out: the sweeps below have to see the same bits)
-            emit(node, i, __dadd_rn(__dsub_rn(__dmul_rn(nl, yyl), __dmul_rn(yl, yl)), __dsub_rn(__dmul_rn(nr, yyr), __dmul_rn(yr, yr))), a, b);
-        }
-        const double y = key_y(k);
-        a = __dadd_rn(a, y); b = __dadd_rn(b, __dmul_rn(y, y));
-        xp = x;
-    }
+// The lane of the warp with the best (l, pos) among those that are `in`: true there, false elsewhere (and everywhere if none is in).
+__device__ __forceinline__ bool warp_best(bool in, unsigned long long l, int pos) {
+    const unsigned int hi = __reduce_min_sync(HS_FULL_MASK, in ? (unsigned int)(l >> 32) : ~0u);
+    in = in && (unsigned int)(l >> 32) == hi;
+    const unsigned int lo = __reduce_min_sync(HS_FULL_MASK, in ? (unsigned int)l : ~0u);
+    in = in && (unsigned int)l == lo;
+    const unsigned int at = __reduce_min_sync(HS_FULL_MASK, in ? (unsigned int)pos : ~0u);
+    return in && (unsigned int)pos == at;
 }
 
-// The block's best split of every node -> s.best / s.pos / s.psy / s.psyy (pos = INT_MAX: none).  A sweep over the
-// thread's run finds the smallest N L; only the threads that hold it sweep again for the smallest position that has it.
+// The block's best split of every node -> s.top (smallest N L, then smallest position).  A thread has `cnt` consecutive keys, key(j) =
+// sorted key at position i0 + j (j = -1: the one ahead of it); (a, b): running sums of y and y^2 ahead of them.  One sweep: the thread keeps
+// its best split with the sums and the feature values there (three sweeps, for N L, its position and the sums, took 2.5 times as long).
 template <class KeyFn>
 __device__ __forceinline__ void layer_block(LayerSmem& s, int nodes, int i0, int cnt, double a, double b, KeyFn key) {
-    const int tid = threadIdx.x;
-    for (int q = tid; q < nodes; q += blockDim.x) { s.best[q] = ~0ull; s.pos[q] = 0x7fffffff; }
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) s.nent = 0;
     __syncthreads();
-    int cur = -1;
-    unsigned long long m = ~0ull;
-    bool several = false;                            // the run lies in more than one node
-    {
-        scan_run(s, nodes, i0, cnt, a, b, key, [&](int node, int, double l, double, double) {
-            if (node != cur) { if (cur >= 0) { atomicMin(&s.best[cur], m); several = true; } cur = node; m = ~0ull; }
-            const unsigned long long u = order_bits_d(l);
-            m = u < m ? u : m;
-        });
-        // lanes that end in the same node as lane 0 go through one atomic
-        const int c0 = __shfl_sync(HS_FULL_MASK, cur, 0);
-        unsigned long long w = cur == c0 ? m : ~0ull;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) { const unsigned long long u = __shfl_xor_sync(HS_FULL_MASK, w, o); w = u < w ? u : w; }
-        if ((tid & 31) == 0 && c0 >= 0) atomicMin(&s.best[c0], w);
-        if (cur >= 0 && cur != c0) atomicMin(&s.best[cur], m);
+    LayerEntry t;
+    t.l = ~0ull; t.pos = 0x7fffffff; t.node = -1; t.sa = t.sb = 0.0; t.xp = t.x = 0.f;
+    double best = 0.0;
+    auto push = [&]() { t.l = order_bits_d(best); s.ent[atomicAdd(&s.nent, 1)] = t; };
+    if (cnt > 0) {
+        int node = 0, lo, hi;
+        while (node + 1 < nodes && s.bnd[node + 1] <= i0) ++node;
+        double sy, syy, ty, tyy, nl, n;                               // sums ahead of the node, its sums, keys of it ahead of i, all its keys
+        auto enter = [&]() {
+            lo = s.bnd[node]; hi = s.bnd[node + 1];
+            sy = s.sy[node]; syy = s.syy[node];
+            ty = s.sy[node + 1] - sy; tyy = s.syy[node + 1] - syy;
+            n = (double)(hi - lo);
+        };
+        enter();
+        nl = (double)(i0 - lo);
+        float xp = i0 > 0 ? key_x(key(-1)) : 0.f;
+        for (int j = 0; j < cnt; ++j) {
+            const int i = i0 + j;
+            if (i >= hi) {
+                while (node + 1 < nodes && s.bnd[node + 1] <= i) ++node;
+                enter();
+                nl = (double)(i - lo);
+            }
+            const unsigned long long k = key(j);
+            const float x = key_x(k);
+            if (i > lo && xp < x) {                                   // a threshold lies between distinct values
+                const double yl = a - sy, yyl = b - syy, yr = ty - yl, yyr = tyy - yyl;
+                if (node != t.node) {
+                    if (t.node >= 0) push();                          // (the run lies in more than one node)
+                    t.node = node; t.pos = 0x7fffffff;
+                }
+                const double l = (nl * yyl - yl * yl) + ((n - nl) * yyr - yr * yr);
+                if (t.pos == 0x7fffffff || l < best) { best = l; t.pos = i; t.sa = a; t.sb = b; t.xp = xp; t.x = x; }
+            }
+            const double y = key_y(k);
+            a += y; b += y * y;
+            nl += 1.0;
+            xp = x;
+        }
+    }
+    // the lanes' last nodes: mostly one, else one round each
+    t.l = order_bits_d(best);
+    for (unsigned int rem = __ballot_sync(HS_FULL_MASK, t.node >= 0); rem;) {
+        const int c = __shfl_sync(HS_FULL_MASK, t.node, __ffs(rem) - 1);
+        const bool in = t.node == c;
+        if (warp_best(in, t.l, t.pos)) push();
+        rem &= ~__ballot_sync(HS_FULL_MASK, in);
     }
     __syncthreads();
-    const bool again = several || (cur >= 0 && m == s.best[cur]);
-    if (again)
-        scan_run(s, nodes, i0, cnt, a, b, key, [&](int node, int i, double l, double, double) {
-            if (order_bits_d(l) == s.best[node]) atomicMin(&s.pos[node], i);
-        });
-    __syncthreads();
-    if (again)
-        scan_run(s, nodes, i0, cnt, a, b, key, [&](int node, int i, double, double sa, double sb) {
-            if (i == s.pos[node]) { s.psy[node] = sa; s.psyy[node] = sb; }
-        });
+    const int nent = s.nent;
+    for (int q = warp; q < nodes; q += blockDim.x / 32) {
+        unsigned long long l = ~0ull;
+        int pos = 0x7fffffff, e = -1;
+        for (int i = lane; i < nent; i += 32)
+            if (s.ent[i].node == q && better(s.ent[i].l, s.ent[i].pos, l, pos)) { l = s.ent[i].l; pos = s.ent[i].pos; e = i; }
+        if (warp_best(e >= 0, l, pos)) s.top[q] = s.ent[e];
+        if (!__any_sync(HS_FULL_MASK, e >= 0) && lane == 0) { s.top[q].l = ~0ull; s.top[q].pos = 0x7fffffff; }
+    }
     __syncthreads();
 }
 
@@ -264,14 +290,12 @@ __global__ void __launch_bounds__(CT_SMALL_THREADS, 1) cart_small_kernel(const f
         const int nodes = 1 << level;
         layer_block(s, nodes, i0, cnt, a, b, key);
         if (tid < nodes) {
-            int at = s.pos[tid];
+            const LayerEntry& t = s.top[tid];
+            int at = t.pos;
             float th = CUDART_NAN_F;                  // a single feature value: the node cannot be split
             double sa = s.sy[tid + 1], sb = s.syy[tid + 1];
             if (at == 0x7fffffff) { s_bad = 1; at = s.bnd[tid + 1]; }
-            else {
-                th = (float)(0.5 * ((double)key_x(s_key[pad8(at - 1)]) + (double)key_x(s_key[pad8(at)])));
-                sa = s.psy[tid]; sb = s.psyy[tid];
-            }
+            else { th = (float)(0.5 * ((double)t.xp + (double)t.x)); sa = t.sa; sb = t.sb; }
             thresholds[threshold_slot(tid, level, depth)] = th;
             s_bnd2[2 * tid] = s.bnd[tid]; s_sy2[2 * tid] = s.sy[tid]; s_syy2[2 * tid] = s.syy[tid];
             s_bnd2[2 * tid + 1] = at; s_sy2[2 * tid + 1] = sa; s_syy2[2 * tid + 1] = sb;
@@ -284,7 +308,10 @@ __global__ void __launch_bounds__(CT_SMALL_THREADS, 1) cart_small_kernel(const f
     if (tid == 0) *status = s_bad ? HS_ERR_SHAPE : HS_OK;
 }
 
-// ---- many samples ----------------------------------------------------------------------------------------------------
+// ---- up to eight samples per thread of a resident grid: one launch ------------------------------------------------------
+#include "cart_grid.cuh"
+
+// ---- more samples ----------------------------------------------------------------------------------------------------
 struct CartParams {
     const float* x;
     const float* y;
@@ -508,8 +535,8 @@ __global__ void __launch_bounds__(CT_LV_THREADS) cart_level_kernel(const CartPar
     // the nodes this tile overlaps leave their best split in entry tile + node (no two tiles share an entry)
     if (tid < nodes && s.bnd[tid] < base + nvalid && s.bnd[tid + 1] > base) {
         const int e = blockIdx.x + tid;
-        p.part_l[e] = s.best[tid]; p.part_i[e] = s.pos[tid];
-        p.part_s[2 * e] = s.psy[tid]; p.part_s[2 * e + 1] = s.psyy[tid];
+        p.part_l[e] = s.top[tid].l; p.part_i[e] = s.top[tid].pos;
+        p.part_s[2 * e] = s.top[tid].sa; p.part_s[2 * e + 1] = s.top[tid].sb;
     }
     if (!last_cta(&p.done[1 + level], &s_last)) return;
     // the best of a node's tiles: a power of two of warps per node, one tile per lane as long as they reach
@@ -569,6 +596,36 @@ extern "C" size_t hs_cart_workspace_bytes(int32_t n) {
            2 * (2 << CT_MAX_DEPTH) * 4 + (1 << CT_MAX_DEPTH) * 64 * 12 + 4096;
 }
 
+static hs_status launch_grid(hs_ctx* ctx, const float* x, const float* y, int n, int depth, float* thresholds, int* status, cudaStream_t stream) {
+    CartGrid p;
+    p.x = x; p.y = y; p.n = n; p.depth = depth; p.thresholds = thresholds; p.status = status;
+    p.per = max(CG_THREADS, (n + ctx->cart_ctas - 1) / ctx->cart_ctas);
+    const int G = (n + p.per - 1) / p.per, parts = 2 * (G + CT_MAX_NODES);
+    size_t o = 0;
+    auto take = [&](size_t bytes) { char* q = ctx->scratch + o; o += hs_align_up(bytes, 256); return q; };
+    p.keys = (unsigned long long*)take((size_t)n * 8);
+    p.keys2 = (unsigned long long*)take((size_t)n * 8);
+    p.cnt = (unsigned int*)take((size_t)CG_MAX_DIGITS * G * 4);
+    p.tot = (unsigned int*)take(CG_MAX_DIGITS * 4);
+    p.range = (uint2*)take((size_t)G * 8);
+    p.blk = (double*)take((size_t)G * 16);
+    p.part = (LayerEntry*)take((size_t)parts * sizeof(LayerEntry));
+    if (o > ctx->scratch_bytes) return HS_ERR_WORKSPACE;
+    p.bar = (unsigned int*)(ctx->counters + HS_CNT_CART);
+    p.err = ctx->counters + HS_CNT_ERROR;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(G);
+    cfg.blockDim = dim3(CG_THREADS);
+    cfg.dynamicSmemBytes = sizeof(CartGridSmem);
+    cfg.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;       // (its CTAs wait for one another)
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, cart_grid_kernel, p) == cudaSuccess ? HS_OK : HS_ERR_CUDA;
+}
+
 extern "C" hs_status hs_cart_fit(hs_ctx* ctx, const float* x, const float* y, int32_t n, int32_t depth,
                                  float* thresholds, int32_t* status, hs_stream stream_) {
     cudaStream_t stream = (cudaStream_t)stream_;
@@ -584,6 +641,16 @@ extern "C" hs_status hs_cart_fit(hs_ctx* ctx, const float* x, const float* y, in
         return hs_launch(cart_small_kernel, one, dim3(CT_SMALL_THREADS), sizeof(SmallSmem), stream, ctx->pdl, one, x, y, (int)n,
                          (int)depth, thresholds, (int*)status) == cudaSuccess ? HS_OK : HS_ERR_CUDA;
     }
+    if (!ctx->cart_ctas) {                           // CTAs of the grid kernel that run at once on this device
+        int per_sm = 0;
+        HS_CUDA_OK(cudaFuncSetAttribute(cart_grid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CartGridSmem)));
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cart_grid_kernel, CG_THREADS, sizeof(CartGridSmem)) != cudaSuccess) {
+            per_sm = 0;
+            (void)cudaGetLastError();
+        }
+        ctx->cart_ctas = per_sm > 0 ? min(ctx->sm_count, CG_MAX_CTAS) : -1;
+    }
+    if (ctx->cart_ctas > 0 && n <= ctx->cart_ctas * CG_SHARE) return launch_grid(ctx, x, y, n, depth, thresholds, (int*)status, stream);
     CartParams p;
     p.x = x; p.y = y; p.n = n; p.depth = depth; p.thresholds = thresholds; p.status = status;
     p.tiles = (n + CT_TILE - 1) / CT_TILE;

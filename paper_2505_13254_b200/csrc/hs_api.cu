@@ -77,6 +77,7 @@ extern "C" hs_status hs_create(hs_ctx** out, int32_t device, size_t workspace_by
     c->quant_ready = false;
     c->warps_ready = false;
     c->cart_ready = false;
+    c->cart_ctas = 0;
     if (cudaDeviceSynchronize() != cudaSuccess) { cudaFree(p); delete c; return HS_ERR_CUDA; }
     *out = c;
     return HS_OK;

@@ -32,6 +32,7 @@ struct hs_ctx {
     int walk_cap;       // 16-CTA clusters of the acceptance walk that run at once
     bool walk_ready;    // acceptance walk kernel attributes set on this device
     bool cart_ready;    // single-CTA stratifier training: shared-memory attribute set on this device
+    int cart_ctas;      // CTAs of the one-launch stratifier training that run at once (0: not asked yet, -1: none)
     bool warps_ready;   // warp kernel of the entropy pass: shared-memory attribute set on this device
     bool quant_ready;   // cluster kernel of the entropy pass: shared-memory attribute set on this device
 };
