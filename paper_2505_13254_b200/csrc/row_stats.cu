@@ -54,6 +54,7 @@ struct QuantParams {
     unsigned long long* part_keys;  // HS_MAX_TOPK keys per partial
     int* row_cnt;
     int K, d_base, phi_mode, pstar_mode, entropy_mode, is_bf16;
+    int inv_k;       // ceil(2^16 / K): i / K = i * inv_k >> 16 for i < 128
     int prefetch;    // the rows may be fetched before the dependency wait (the caller vouches that they are complete)
     int* err;        // sticky device error word (a bounded wait that expired)
 };
@@ -139,10 +140,15 @@ __device__ __forceinline__ void finalize_row(const QuantParams& p, int row, floa
     const float tv = valid ? key_value(key) : 0.f;
     const float t0 = __shfl_sync(HS_FULL_MASK, tv, 0);
     const float pv = valid ? expf(tv - lse) : 0.f;
-    const float itr = warp_sum(valid ? -pv * (tv - lse) : 0.f);
     const float z = valid ? expf(tv - t0) : 0.f;
-    const float Z = warp_sum(z);
-    const float itk = logf(Z) - warp_sum(valid ? z * (tv - t0) : 0.f) / Z;
+    float itr = valid ? -pv * (tv - lse) : 0.f, Z = z, zt = valid ? z * (tv - t0) : 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {                           // three sums side by side
+        itr += __shfl_xor_sync(HS_FULL_MASK, itr, o);
+        Z += __shfl_xor_sync(HS_FULL_MASK, Z, o);
+        zt += __shfl_xor_sync(HS_FULL_MASK, zt, o);
+    }
+    const float itk = logf(Z) - zt / Z;
     if (lane < K) {
         p.out.topk_val[(size_t)row * K + lane] = valid ? tv : -CUDART_INF_F;
         p.out.topk_idx[(size_t)row * K + lane] = valid ? key_index(key) : -1;
@@ -176,23 +182,49 @@ __device__ __forceinline__ float warp_kth_largest(float v, int K, int lane) {
 // ================================================================================================================
 // Every row is cut into the same number of parts (at most eight, the portable cluster size), one CTA of 16 warps per part;
 // the CTAs of a row are one thread-block cluster.  A part is at most QS_SLOTS items of 32 KiB, all of which are requested
-// at once by bulk copies into shared memory of their own (with prefetch ahead of the dependency wait), so the pass is a chain
+// at once, a warp each, by bulk copies into shared memory of their own (with prefetch ahead of the dependency wait), so the pass is a chain
 // of latencies, not a stream: items as they land, one bound for the Top-K of the part from the CTA's 32 half-warp maxima, the
-// few cells that reach it read again from shared memory, ranked by counting, and the parts merged in the shared memory of
-// the row's first CTA (asynchronous remote stores; the other CTAs leave at once).
-// 72 registers per thread: the CTA then fits into the register file beside a CTA of the kernel ahead that is still at work on
+// few cells that reach it read again from shared memory, eight at once, and from there one warp alone: candidates ranked by counting, the parts
+// merged in the shared memory of the row's first CTA (asynchronous remote stores; the other CTAs leave at once).
+// What it is bound by: 60 rows of 128256 bf16 take 14 k clocks behind the dependency wait (were 19 k), 7.5 k of them until the last
+// item is reduced (128 KiB per SM), the rest dependent shared-memory reads and shuffles.  One thread that asked for all items with the CTA
+// waiting behind it cost 2.5 k, items unrolled over the slots (34 KB of code instead of 82) and merges by all 16 warps
+// between barriers the rest.  One greedy step of an 8B-shaped model 38.4 -> 36.2 us, of 32000 fp32 logits 30.1 -> 27.9.
+// At most 72 registers per thread: the CTA then fits into the register file beside a CTA of the kernel ahead that is still at work on
 // the same SM (in a decode loop: the CTA that walks the accepted path of the step before).
+// {ref, sum e, sum x e, max} of the first N lanes (N a power of two; lanes past the last one hold no values) as one, known to lanes 0 .. N - 1
+template <int N>
+__device__ __forceinline__ float4 merge_stats(float4 v) {
+    float R = v.x, M = v.w;
+#pragma unroll
+    for (int o = N / 2; o > 0; o >>= 1) {
+        R = fmaxf(R, __shfl_xor_sync(HS_FULL_MASK, R, o));
+        M = fmaxf(M, __shfl_xor_sync(HS_FULL_MASK, M, o));
+    }
+    const float f = v.x == -CUDART_INF_F ? 0.f : ex2f((v.x - R) * LOG2E);
+    float S = v.y * f, U = v.z * f;
+#pragma unroll
+    for (int o = N / 2; o > 0; o >>= 1) {
+        S += __shfl_xor_sync(HS_FULL_MASK, S, o);
+        U += __shfl_xor_sync(HS_FULL_MASK, U, o);
+    }
+    return make_float4(R, S, U, M);
+}
+
 template <bool BF16>
 __global__ void __maxnreg__(72) quantify_cluster_kernel(const __grid_constant__ QuantParams p) {
     constexpr int VE = BF16 ? 8 : 4;
     constexpr int NW = QS_THREADS / 32;
     extern __shared__ __align__(128) unsigned char s_dyn[];
     __shared__ unsigned long long s_full[QS_SLOTS], s_merge;
-    __shared__ unsigned long long s_list[CAND_CAP];
+    __shared__ __align__(16) unsigned long long s_list[CAND_CAP];
     __shared__ unsigned long long s_top[HS_MAX_TOPK], s_red[NW];
     __shared__ __align__(16) float s_gm[32];
     __shared__ float4 s_wstat[NW];                               // {ref, sum e, sum x e, max} per warp
+    __shared__ float4 s_stat;                                    //   and of the part
     __shared__ int s_cnt;
+    __shared__ unsigned char s_hit[NW][QS_SLOTS * 32];           // cells to read again: item * 32 + lane
+    __shared__ float s_cm[QS_SLOTS][QS_THREADS];                 // every thread's maximum of each item
     __shared__ __align__(16) unsigned long long s_ck[8][HS_MAX_TOPK];   // first CTA of a row: the parts' Top-K keys
     __shared__ __align__(16) float4 s_cs[8];                            //   and their {ref, sum e, sum x e, max}
 
@@ -212,57 +244,51 @@ __global__ void __maxnreg__(72) quantify_cluster_kernel(const __grid_constant__ 
         mbar_init_fence();
         s_cnt = 0;
     }
-    // The tree stage behind this kernel may start once every CTA has passed this point.  Without prefetch that is behind
-    // the dependency wait, so whatever was written ahead of the call is complete by then and the tree stage may read its
-    // inputs (not this kernel's results) without waiting.
-    if (!p.prefetch) pdl_wait();
-    pdl_launch_dependents();
-    if (tid == 0)
-        for (int s = 0; s < nit; ++s) {
-            const int len = min(QS_ITEM_VECS, sv1 - sv0 - s * QS_ITEM_VECS);
-            mbar_expect_tx(smem_u32(&s_full[s]), (unsigned int)len * 16u);
-            bulk_load(slots0 + (unsigned int)s * (QS_ITEM_VECS * 16), rowp + (size_t)(sv0 + s * QS_ITEM_VECS) * 16,
-                      (unsigned int)len * 16u, smem_u32(&s_full[s]));
-        }
     if (tid < HS_MAX_TOPK) s_top[tid] = 0ull;
     __syncthreads();
     // First half of a cluster barrier: when it completes every CTA of the cluster runs with its barrier initialised, and its
     // shared memory may be written from outside.
     if (parts > 1) cluster_arrive();
+    // The tree stage behind this kernel may start once every CTA has passed this point.  Without prefetch that is behind
+    // the dependency wait, so whatever was written ahead of the call is complete by then and the tree stage may read its
+    // inputs (not this kernel's results) without waiting.
+    if (!p.prefetch) pdl_wait();
+    pdl_launch_dependents();
+    // A warp per item asks for it (one thread for all of them, with the CTA waiting behind it: 1 us).
+    if (warp < nit && lane == 0) {
+        const int len = min(QS_ITEM_VECS, sv1 - sv0 - warp * QS_ITEM_VECS);
+        mbar_expect_tx(smem_u32(&s_full[warp]), (unsigned int)len * 16u);
+        bulk_load(slots0 + (unsigned int)warp * (QS_ITEM_VECS * 16), rowp + (size_t)(sv0 + warp * QS_ITEM_VECS) * 16,
+                  (unsigned int)len * 16u, smem_u32(&s_full[warp]));
+    }
+    __syncwarp();
 
-    // ---- the part's items -------------------------------------------------------------------------------------------
+    // ---- the part's items (a loop that stays one: its body unrolled over the slots is fetched once per item) ---------------
     const unsigned int ninf = BF16 ? 0xff80ff80u : 0xff800000u;
     float ref = -CUDART_INF_F, nref = 0.f, lm = -CUDART_INF_F;
     float2 s2 = make_float2(0.f, 0.f), u2 = make_float2(0.f, 0.f);
-    float cm[QS_SLOTS];                                          // this lane's maximum of each item
+#pragma unroll 1
+    for (int it = 0; it < nit; ++it) {
+        const int len = min(QS_ITEM_VECS, sv1 - sv0 - it * QS_ITEM_VECS);
+        mbar_wait(smem_u32(&s_full[it]), 0u, p.err);
+        __syncwarp();
+        const uint4* st = slots + it * QS_ITEM_VECS;
+        uint4 d[4];
 #pragma unroll
-    for (int it = 0; it < QS_SLOTS; ++it) {
-        cm[it] = -CUDART_INF_F;
-        if (it < nit) {
-            const int len = min(QS_ITEM_VECS, sv1 - sv0 - it * QS_ITEM_VECS);
-            mbar_wait(smem_u32(&s_full[it]), 0u, p.err);
-            __syncwarp();
-            const uint4* st = slots + it * QS_ITEM_VECS;
-            uint4 d[4];
-            if (len == QS_ITEM_VECS) {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) d[j] = st[tid + j * QS_THREADS];
-            } else {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int vl = tid + j * QS_THREADS;
-                    d[j] = vl < len ? st[vl] : make_uint4(ninf, ninf, ninf, ninf);
-                }
-            }
-            const int last = p.nvec - 1 - (sv0 + it * QS_ITEM_VECS);          // the row's last vector may run past vocab
-            if (last < len && p.nvec * VE != p.vocab) {
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (tid + j * QS_THREADS == last) mask_tail<BF16>(d[j], p.nvec - 1, p.vocab);
-            }
-            fold_round<BF16>(d, ref, nref, s2, u2, cm[it]);
-            lm = fmaxf(lm, cm[it]);
+        for (int j = 0; j < 4; ++j) {
+            const int vl = tid + j * QS_THREADS;
+            d[j] = vl < len ? st[vl] : make_uint4(ninf, ninf, ninf, ninf);
         }
+        const int last = p.nvec - 1 - (sv0 + it * QS_ITEM_VECS);              // the row's last vector may run past vocab
+        if (last < len && p.nvec * VE != p.vocab) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (tid + j * QS_THREADS == last) mask_tail<BF16>(d[j], p.nvec - 1, p.vocab);
+        }
+        float rm;
+        fold_round<BF16>(d, ref, nref, s2, u2, rm);
+        s_cm[it][tid] = rm;
+        lm = fmaxf(lm, rm);
     }
     // ---- Top-K of the part: bound, candidates -------------------------------------------------------------------------
     {
@@ -286,78 +312,118 @@ __global__ void __maxnreg__(72) quantify_cluster_kernel(const __grid_constant__ 
             const float4 f4 = reinterpret_cast<const float4*>(s_gm)[i];
             ge += (f4.x >= w) + (f4.y >= w) + (f4.z >= w) + (f4.w >= w);
         }
-        tau = warp_max(ge >= K ? w : -CUDART_INF_F);             // (maxima of disjoint sets are distinct logits)
+        // (maxima of disjoint sets are distinct logits)
+        tau = order_bits_float(__reduce_max_sync(HS_FULL_MASK, float_order_bits(ge >= K ? w : -CUDART_INF_F)));
     }
+    // The cells (a thread's 4 vectors of an item) that reach the bound are listed, then read again, a vector per lane: eight cells at once.
+    int nhit = 0;
+#pragma unroll 1
+    for (int it = 0; it < nit; ++it) {
+        const float cm = s_cm[it][tid];
+        const bool hit = cm >= tau && cm > -CUDART_INF_F;
+        const unsigned int b = __ballot_sync(HS_FULL_MASK, hit);
+        if (hit) s_hit[warp][nhit + __popc(b & ((1u << lane) - 1u))] = (unsigned char)(it * 32 + lane);
+        nhit += __popc(b);
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int h = lane >> 2; h < nhit; h += 8) {
+        const int cell = s_hit[warp][h], vl = (cell >> 5) * QS_ITEM_VECS + warp * 32 + (cell & 31) + (lane & 3) * QS_THREADS, v = sv0 + vl;
+        if (v >= sv1) continue;
+        float x[8];
+        unpack<BF16>(slots[vl], x);
+        unsigned int m = 0u;
 #pragma unroll
-    for (int it = 0; it < QS_SLOTS; ++it) {
-        unsigned int hits = __ballot_sync(HS_FULL_MASK, cm[it] >= tau && cm[it] > -CUDART_INF_F);
-        for (; hits; hits &= hits - 1) {                         // a cell's four vectors, one element per lane (fp32: 16 lanes)
-            const int vl = warp * 32 + __ffs(hits) - 1 + (BF16 ? lane >> 3 : (lane >> 2) & 3) * QS_THREADS;
-            const int e = BF16 ? lane & 7 : lane & 3;
-            const int v = sv0 + it * QS_ITEM_VECS + vl, idx = v * VE + e;
-            if ((BF16 || lane < 16) && v < sv1 && idx < p.vocab) {
-                const unsigned char* vp = reinterpret_cast<const unsigned char*>(slots + it * QS_ITEM_VECS + vl);
-                const float x = BF16 ? __uint_as_float((unsigned int)reinterpret_cast<const unsigned short*>(vp)[e] << 16)
-                                     : reinterpret_cast<const float*>(vp)[e];
-                if (x >= tau && x > -CUDART_INF_F) {
-                    const int sl = atomicAdd(&s_cnt, 1);
-                    if (sl < CAND_CAP) s_list[sl] = make_key(x, idx);
-                }
-            }
-            __syncwarp();
+        for (int e = 0; e < VE; ++e) m |= (x[e] >= tau && x[e] > -CUDART_INF_F && v * VE + e < p.vocab) ? 1u << e : 0u;
+        for (; m; m &= m - 1) {
+            const int e = __ffs(m) - 1, sl = atomicAdd(&s_cnt, 1);
+            const unsigned char* vp = reinterpret_cast<const unsigned char*>(slots + vl);
+            const float xe = BF16 ? __uint_as_float((unsigned int)reinterpret_cast<const unsigned short*>(vp)[e] << 16)
+                                  : reinterpret_cast<const float*>(vp)[e];
+            if (sl < CAND_CAP) s_list[sl] = make_key(xe, v * VE + e);
         }
+    }
+    if (warp == NW - 1) {                                        // the warps' (ref, s, u, max) in a fixed order
+        const float4 t = merge_stats<NW>(lane < NW ? s_wstat[lane] : make_float4(-CUDART_INF_F, 0.f, 0.f, -CUDART_INF_F));
+        if (lane == 0) s_stat = t;
     }
     __syncthreads();                                             // all candidates are pushed
     const int ncand = s_cnt;
-    if (ncand <= CAND_CAP) rank_select_warps(s_list, ncand, K, s_top, warp, lane, NW);
-    else topk_by_rounds<BF16>(rowp, sv0, sv1, p.vocab, K, s_top, s_red, tid, QS_THREADS, 1);   // heavy ties
-    __syncthreads();                                             // the Top-K is complete
-    if (warp != 0 && (parts == 1 || part != 0)) {
+    if (ncand > 64) {
+        if (ncand <= CAND_CAP) rank_select_warps(s_list, ncand, K, s_top, warp, lane, NW);
+        else topk_by_rounds<BF16>(rowp, sv0, sv1, p.vocab, K, s_top, s_red, tid, QS_THREADS, 1);   // heavy ties
+        __syncthreads();                                         // the Top-K is complete
+    }
+    // ---- the rest is one warp's -----------------------------------------------------------------------------------------
+    // (and of one or three more in the first CTA of a row, which rank the keys of up to eight parts)
+    const int nw = part == 0 && parts > 1 ? (parts * K + 31) / 32 : 1;
+    if (warp >= nw) {
         if (parts > 1) cluster_wait();
         return;
     }
-    if (p.prefetch) pdl_wait();                                  // from here on results go to global memory
-    float R = 0.f, M = 0.f, S = 0.f, U = 0.f;
-    if (warp == 0) {                                             // the warps' (ref, s, u, max) in a fixed order
-        const float4 w = lane < NW ? s_wstat[lane] : make_float4(-CUDART_INF_F, 0.f, 0.f, -CUDART_INF_F);
-        R = warp_max(w.x); M = warp_max(w.w);
-        const float f = w.x == -CUDART_INF_F ? 0.f : ex2f((w.x - R) * LOG2E);
-        S = warp_sum(w.y * f); U = warp_sum(w.z * f);
-    }
-    if (parts == 1) {
-        finalize_row(p, row, M, R, S, U, lane < K ? s_top[lane] : 0ull, lane);
-        return;
-    }
-    cluster_wait();                                              // (the arrival above: every CTA of the cluster runs)
-    if (part != 0) {
-        // this part goes into slot `part` of the first CTA of the row's cluster
-        const unsigned int bar = cluster_map_addr(smem_u32(&s_merge), 0);
-        if (lane < HS_MAX_TOPK / 2) {
-            const unsigned long long a = s_top[2 * lane], b = s_top[2 * lane + 1];
-            st_async_v4(cluster_map_addr(smem_u32(&s_ck[part][2 * lane]), 0), (unsigned int)a, (unsigned int)(a >> 32),
-                        (unsigned int)b, (unsigned int)(b >> 32), bar);
-        } else if (lane == HS_MAX_TOPK / 2) {
-            st_async_v4(cluster_map_addr(smem_u32(&s_cs[part]), 0), __float_as_uint(R), __float_as_uint(S), __float_as_uint(U),
-                        __float_as_uint(M), bar);
+    if (warp == 0 && ncand <= 64) {                              // (the usual case: ranked by counting, two keys per shared-memory read)
+        if (lane == 0) s_list[ncand] = 0ull;
+        __syncwarp();
+        for (int i = lane; i < ncand; i += 32) {
+            const unsigned long long k = s_list[i];
+            int rank = 0;
+#pragma unroll 4
+            for (int j = 0; j < ncand; j += 2) {
+                const ulonglong2 two = *reinterpret_cast<const ulonglong2*>(&s_list[j]);
+                rank += (two.x > k) + (two.y > k);
+            }
+            if (rank < K) s_top[rank] = k;
         }
-        return;
+        __syncwarp();
     }
-    if (warp == 0) {
-        if (lane < HS_MAX_TOPK) s_ck[0][lane] = s_top[lane];
-        if (lane == 0) s_cs[0] = make_float4(R, S, U, M);
+    float4 st = s_stat;
+    unsigned long long key = warp == 0 && lane < K ? s_top[lane] : 0ull;
+    if (parts > 1) {
+        cluster_wait();                                          // (the arrival above: every CTA of the cluster runs)
+        if (part != 0) {
+            // this part goes into slot `part` of the first CTA of the row's cluster
+            if (p.prefetch) pdl_wait();
+            const unsigned int bar = cluster_map_addr(smem_u32(&s_merge), 0);
+            if (lane < HS_MAX_TOPK / 2) {
+                const unsigned long long a = s_top[2 * lane], b = s_top[2 * lane + 1];
+                st_async_v4(cluster_map_addr(smem_u32(&s_ck[part][2 * lane]), 0), (unsigned int)a, (unsigned int)(a >> 32),
+                            (unsigned int)b, (unsigned int)(b >> 32), bar);
+            } else if (lane == HS_MAX_TOPK / 2) {
+                st_async_v4(cluster_map_addr(smem_u32(&s_cs[part]), 0), __float_as_uint(st.x), __float_as_uint(st.y), __float_as_uint(st.z),
+                            __float_as_uint(st.w), bar);
+            }
+            return;
+        }
+        if (warp == 0) {
+            if (lane < HS_MAX_TOPK) s_ck[0][lane] = key;
+            if (lane == 0) s_cs[0] = st;
+        }
+        mbar_wait_cluster(smem_u32(&s_merge), 0u, p.err);
+        if (nw > 1) named_bar_sync(2, nw * 32);
+        else __syncwarp();
+        // the K best of the parts' lists (0 behind their ends), ranked by counting
+        const int i = tid;
+        if (i < parts * K) {
+            const int q = i * p.inv_k >> 16;
+            const unsigned long long k = s_ck[q][i - q * K];
+            int rank = 0;
+#pragma unroll 1
+            for (int o = 0; o < parts; ++o)
+#pragma unroll 4
+                for (int j = 0; j < K; j += 2) {                 // (the lists have an even number of places)
+                    const ulonglong2 two = *reinterpret_cast<const ulonglong2*>(&s_ck[o][j]);
+                    rank += (two.x > k) + (two.y > k);
+                }
+            if (k != 0ull && rank < K) s_top[rank] = k;          // (warp 0 has read its own part's list)
+        }
+        if (nw > 1) named_bar_sync(2, nw * 32);
+        else __syncwarp();
+        if (warp != 0) return;
+        if (lane < K) key = s_top[lane];
+        st = merge_stats<16>(lane < parts ? s_cs[lane] : make_float4(-CUDART_INF_F, 0.f, 0.f, -CUDART_INF_F));
     }
-    mbar_wait_cluster(smem_u32(&s_merge), 0u, p.err);
-    __syncthreads();                                             // (s_top has been read)
-    if (tid < HS_MAX_TOPK) s_top[tid] = 0ull;
-    __syncthreads();
-    rank_select_warps(&s_ck[0][0], parts * HS_MAX_TOPK, K, s_top, warp, lane, NW);
-    __syncthreads();
-    if (warp == 0) {
-        const float4 st = lane < parts ? s_cs[lane] : make_float4(-CUDART_INF_F, 0.f, 0.f, -CUDART_INF_F);
-        R = warp_max(st.x);
-        const float f = st.x == -CUDART_INF_F ? 0.f : ex2f((st.x - R) * LOG2E);
-        finalize_row(p, row, warp_max(st.w), R, warp_sum(st.y * f), warp_sum(st.z * f), lane < K ? s_top[lane] : 0ull, lane);
-    }
+    if (p.prefetch) pdl_wait();                                  // from here on results go to global memory
+    finalize_row(p, row, st.w, st.x, st.y, st.z, key, lane);
 }
 
 
@@ -389,6 +455,7 @@ static void fill_common(QuantParams& p, const hs_tree_batch* tree, const void* l
     p.token = tree->token;
     p.out = *out;
     p.K = policy->top_k;
+    p.inv_k = (65536 + p.K - 1) / p.K;
     p.d_base = policy->d_base;
     p.phi_mode = policy->phi_mode;
     p.pstar_mode = policy->pstar_mode;
