@@ -18,7 +18,12 @@
 //                      c_(k+1) = c_k + W_k, W_k = sum_v max(p_v - c_k q_v, 0), so a rejection costs
 //                      one vocabulary-wide sum, split over the CTAs of the cluster and exchanged
 //                      through distributed shared memory.  The bonus token is drawn by inverse CDF
-//                      in token order.
+//                      in token order, from the sums of the last rejection where there was one.  A node's
+//                      probabilities are exponentiated once, into registers: a rejection after the first 2.4 k
+//                      clocks instead of 4.5 k (two thirds of it shuffles and fp64 additions of three prefixes,
+//                      the rest the exchange), a draw behind rejections 0.4 k instead of 6.8 k, the first sum of a
+//                      node 4.6 - 6.2 k.  One tree, 64 heads, sampling: step 60.2 -> 56.1 us with the entropy pass of
+//                      few rows (57.9 before this).
 #include <cooperative_groups.h>
 #include <math_constants.h>
 
@@ -406,124 +411,51 @@ __device__ __forceinline__ void cluster_allgather(unsigned long long v, unsigned
     cluster_arrive();
     cluster_wait();
 }
-// the first `n` of N values as a tree (see sum8 on why)
+static_assert(WALK_THREADS / 32 == 16, "prefixes over the warps take 16 lanes");
+
+// The probabilities of a thread's tokens at the node the walk stands on, target and draft.  A thread has a contiguous run of the vectors of its
+// CTA's slice, taken in pieces of EL tokens; a run of one piece (up to 131072 bf16 logits over 16 CTAs of 512 threads) is exponentiated once
+// per node and serves every rejection there and the final draw.
+#define WALK_EL 16            // (32 spill)
+struct Masses {
+    float p[WALK_EL], q[WALK_EL];
+    int w0, w1, pieces;       // the thread's vectors of the slice, pieces of its run
+    int held;                 // piece in p, q; -1: none
+};
+struct RowScale {             // of a node: maxima, 1 / sums, log2(e) / temperature
+    float pm, ips, qm, iqs, invT;
+};
+template <bool BF16>
+__device__ __forceinline__ void fill_masses(Masses& m, int vocab, const RowSlice& rs, int piece, const RowScale& k) {
+    constexpr int VE = BF16 ? 8 : 4;
+#pragma unroll
+    for (int i = 0; i < WALK_EL / VE; ++i) {
+        const int v = m.w0 + piece * (WALK_EL / VE) + i;
+#pragma unroll
+        for (int e = 0; e < VE; ++e) m.p[i * VE + e] = m.q[i * VE + e] = 0.f;
+        if (v >= m.w1) continue;
+        float x[8];
+        const int inside = vocab - (rs.v0 + v) * VE;             // tokens of the vocabulary in this vector (and behind it)
+        unpack<BF16>(rs.p[v], x);
+#pragma unroll
+        for (int e = 0; e < VE; ++e)
+            if (e < inside) m.p[i * VE + e] = exp2f((fmaxf(x[e], -1e30f) - k.pm) * k.invT) * k.ips;
+        if (!rs.q) continue;
+        unpack<BF16>(rs.q[v], x);
+#pragma unroll
+        for (int e = 0; e < VE; ++e)
+            if (e < inside) m.q[i * VE + e] = exp2f((fmaxf(x[e], -1e30f) - k.qm) * k.invT) * k.iqs;
+    }
+}
+// inclusive prefix over lanes 0 .. N - 1
 template <int N>
-__device__ __forceinline__ double sum_first(const double* v, int n) {
-    double a[N];
+__device__ __forceinline__ double warp_prefix_d(double v, int lane) {
 #pragma unroll
-    for (int i = 0; i < N; ++i) a[i] = i < n ? v[i] : 0.0;
-    double t = sum8(a[0], a[1], a[2], a[3], a[4], a[5], a[6], a[7]);
-    if (N > 8) t += sum8(a[N - 8], a[N - 7], a[N - 6], a[N - 5], a[N - 4], a[N - 3], a[N - 2], a[N - 1]);
-    return t;
-}
-static_assert(WALK_THREADS / 32 == 16, "sum_first<16> sums the warps");
-
-// Sum over this CTA's share of the vocabulary of max(p_v - c q_v, 0), then over the cluster.
-// Every CTA returns the same value (fixed summation order).
-template <int WC>
-__device__ double cluster_residual_sum(const AcceptParams& p, unsigned int rank, const RowSlice& rs,
-                                       float pm, float ips, float qm, float iqs, float invT,
-                                       float c, double* s_part, unsigned long long (*s_x)[WALK_CLUSTER], unsigned int& xch) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int ve = p.is_bf16 ? 8 : 4;
-    float acc = 0.f;
-    for (int v = tid; v < rs.nv; v += WALK_THREADS) {
-        uint4 a = rs.p[v], bq = rs.q[v];
-        float x[8], y[8];
-        if (p.is_bf16) { unpack<true>(a, x); unpack<true>(bq, y); }
-        else { unpack<false>(a, x); unpack<false>(bq, y); }
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            if (e < ve && (rs.v0 + v) * ve + e < p.vocab) {
-                float pv = exp2f((fmaxf(x[e], -1e30f) - pm) * invT) * ips;
-                float qv = exp2f((fmaxf(y[e], -1e30f) - qm) * invT) * iqs;
-                acc += fmaxf(pv - c * qv, 0.f);
-            }
-        }
+    for (int o = 1; o < N; o <<= 1) {
+        const double up = __shfl_up_sync(HS_FULL_MASK, v, o);
+        if (lane >= o) v += up;
     }
-    double w = warp_sum_d((double)acc);
-    if (lane == 0) s_part[warp] = w;
-    __syncthreads();
-    double t = 0.0;
-    if (warp == 0) t = sum_first<16>(s_part, 16);      // the warps' sums in a fixed order, known to every lane of warp 0
-    const double* got = reinterpret_cast<const double*>(s_x[xch & 1u]);
-    cluster_allgather<WC>((unsigned long long)__double_as_longlong(t), s_x, xch, rank);
-    return sum_first<WC>(got, WC);
-}
-
-// Inverse-CDF draw from max(p - c q, 0) in token order: smallest j whose running sum exceeds
-// u * total; if rounding leaves none, the last token with positive mass.  rs.q may be NULL (c = 0).
-// A CTA covers the tokens of its slice, a thread a contiguous run of vectors; running sums in double.  One exchange: every
-// CTA learns the masses of all slices and with them which one holds the crossing; that CTA finds the token and writes it.
-template <int WC>
-__device__ void cluster_inverse_cdf(const AcceptParams& p, unsigned int rank, const RowSlice& rs,
-                                    float pm, float ips, float qm, float iqs, float invT,
-                                    float c, float u, double* s_scan, unsigned long long (*s_x)[WALK_CLUSTER],
-                                    unsigned int& xch, int* s_pick, int* bonus) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int ve = p.is_bf16 ? 8 : 4;
-    const int run_v = (rs.nv + WALK_THREADS - 1) / WALK_THREADS;           // vectors per thread
-    const int w0 = min(tid * run_v, rs.nv), w1 = min(w0 + run_v, rs.nv);
-    auto masses = [&](int v, float (&m)[8]) {                               // of vector v of the slice
-        float x[8], y[8];
-        const uint4 a = rs.p[v];
-        if (p.is_bf16) unpack<true>(a, x); else unpack<false>(a, x);
-        if (rs.q) { const uint4 bq = rs.q[v]; if (p.is_bf16) unpack<true>(bq, y); else unpack<false>(bq, y); }
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            m[e] = 0.f;
-            if (e < ve && (rs.v0 + v) * ve + e < p.vocab) {
-                m[e] = exp2f((fmaxf(x[e], -1e30f) - pm) * invT) * ips;
-                if (rs.q) m[e] = fmaxf(m[e] - c * (exp2f((fmaxf(y[e], -1e30f) - qm) * invT) * iqs), 0.f);
-            }
-        }
-    };
-    double mine = 0.0;
-    int last_pos = -1;
-    for (int v = w0; v < w1; ++v) {
-        float m[8];
-        masses(v, m);
-        mine += sum8(m);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) if (m[e] > 0.f) last_pos = (rs.v0 + v) * ve + e;
-    }
-    if (tid == 0) { s_pick[0] = 0x7fffffff; s_pick[1] = -1; }
-    // exclusive scan over the CTA's threads: inclusive shuffle scan inside a warp, then the warps' totals in order
-    double incl = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const double up = __shfl_up_sync(HS_FULL_MASK, incl, o);
-        if (lane >= o) incl += up;
-    }
-    if (lane == 31) s_scan[warp] = incl;
-    __syncthreads();
-    const double ctot = sum_first<16>(s_scan, 16), wbefore = sum_first<16>(s_scan, warp);
-    const double* got = reinterpret_cast<const double*>(s_x[xch & 1u]);
-    cluster_allgather<WC>((unsigned long long)__double_as_longlong(ctot), s_x, xch, rank);
-    const double before = sum_first<WC>(got, (int)rank), goal = (double)u * sum_first<WC>(got, WC);
-    // the slice with the crossing: the first whose running total exceeds the goal (rounding leaves none: the last with mass).
-    // Lane r of every warp tries slice r.
-    const unsigned int over = __ballot_sync(HS_FULL_MASK, lane < WC && sum_first<WC>(got, lane + 1) > goal);
-    const unsigned int full = __ballot_sync(HS_FULL_MASK, lane < WC && got[lane & (WC - 1)] > 0.0);
-    const int owner = over ? __ffs(over) - 1 : (full ? 31 - __clz(full) : 0);
-    if ((int)rank != owner) return;
-    double run = before + (wbefore + (incl - mine));
-    if (run <= goal && run + mine > goal) {          // the crossing lies in this thread's run
-        bool found = false;
-        for (int v = w0; v < w1 && !found; ++v) {
-            float m[8];
-            masses(v, m);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                run += (double)m[e];
-                if (!found && run > goal) { found = true; atomicMin(&s_pick[0], (rs.v0 + v) * ve + e); }
-            }
-        }
-        if (!found && last_pos >= 0) atomicMin(&s_pick[0], last_pos);       // (rounding)
-    }
-    if (last_pos >= 0) atomicMax(&s_pick[1], last_pos);
-    __syncthreads();
-    if (tid == 0) *bonus = s_pick[0] != 0x7fffffff ? s_pick[0] : max(s_pick[1], 0);
+    return v;
 }
 
 template <int WC>
@@ -531,12 +463,11 @@ __global__ void __launch_bounds__(WALK_THREADS, 1) accept_walk_kernel(const __gr
     cg::cluster_group cluster = cg::this_cluster();
     extern __shared__ __align__(16) unsigned char s_rows[];    // staged: this CTA's slices of p and q, `per` vectors each
     __shared__ unsigned long long s_bar;
-    __shared__ double s_part[WALK_THREADS / 32];
     __shared__ double s_scan[WALK_THREADS / 32];
     __shared__ unsigned long long s_x[2][WALK_CLUSTER];    // all-gather buffers of the cluster exchanges
     unsigned int xch = 0;                  // exchanges through s_x so far
     __shared__ int s_pick[2];
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = blockIdx.x / WC;
     const unsigned int rank = cluster.block_rank();
     pdl_launch_dependents();
@@ -569,6 +500,7 @@ __global__ void __launch_bounds__(WALK_THREADS, 1) accept_walk_kernel(const __gr
         }
         u = p.uniforms ? p.uniforms[nbase + orig] : philox_uniform(p.seed, p.offset, b, orig, 0);
     }
+    const float ufin = !sampling ? 0.f : p.uniforms ? p.uniforms[p.n_nodes_total + b] : philox_uniform(p.seed, p.offset, b, 0, 1);
     pdl_wait();                            // arg-max and normalisers come from the row pass
 
     if (!sampling && nk > 0 && tree_status == 0) return;      // greedy sequences were finished by the row pass
@@ -594,6 +526,14 @@ __global__ void __launch_bounds__(WALK_THREADS, 1) accept_walk_kernel(const __gr
     rs.v0 = rank * per;
     rs.nv = max(min(rs.v0 + per, p.nvec) - rs.v0, 0);
     rs.p = nullptr; rs.q = nullptr;
+    Masses m;
+    const int ve = p.is_bf16 ? 8 : 4;
+    {
+        const int run = (rs.nv + WALK_THREADS - 1) / WALK_THREADS;
+        m.w0 = min(tid * run, rs.nv); m.w1 = min(m.w0 + run, rs.nv);
+        m.pieces = (run * ve + WALK_EL - 1) / WALK_EL;
+        m.held = -1;
+    }
     const unsigned int bar = smem_u32(&s_bar);
     if (tid == 0 && p.staged) { mbar_init(bar, 1); mbar_init_fence(); }
     unsigned int stage_n = 0;
@@ -601,10 +541,11 @@ __global__ void __launch_bounds__(WALK_THREADS, 1) accept_walk_kernel(const __gr
     bool staged_q = false;
     auto stage = [&](int node, const char* prow, const char* qrow) {      // qrow may be NULL: only p
         if (staged_node == node && (staged_q || qrow == nullptr)) {
-            if (qrow == nullptr) rs.q = nullptr;
+            if (qrow == nullptr && rs.q != nullptr) { rs.q = nullptr; m.held = -1; }
             return;
         }
         staged_node = node; staged_q = qrow != nullptr;
+        m.held = -1;
         if (!p.staged) {
             rs.p = (const uint4*)prow + rs.v0;
             rs.q = qrow ? (const uint4*)qrow + rs.v0 : nullptr;
@@ -681,14 +622,11 @@ __global__ void __launch_bounds__(WALK_THREADS, 1) accept_walk_kernel(const __gr
             const int drow = nbase + s_orig[cur];
             const char* prow = (const char*)p.target + (size_t)trow * p.row_stride * esz;
             const char* qrow = (const char*)p.draft + (size_t)drow * p.row_stride * esz;
-            const float2 pms = s_pms[cur];
-            const float pm = pms.x, ips = 1.f / pms.y;
-            float qm = 0.f, iqs = 0.f;
-            bool have_q = false;
-            float c = 0.f;
+            RowScale k;
+            k.pm = s_pms[cur].x; k.ips = 1.f / s_pms[cur].y; k.qm = 0.f; k.iqs = 0.f; k.invT = invT;
+            float c = 0.f, c_next = 0.f;
             double W = 1.0;
             int accepted = -1;
-            bool tested = false;
             // the kept children of cur as bit masks (every warp finds them with four ballots instead of a serial scan)
             unsigned int kids[HS_MAX_NODES / 32];
 #pragma unroll
@@ -696,30 +634,81 @@ __global__ void __launch_bounds__(WALK_THREADS, 1) accept_walk_kernel(const __gr
                 const int j = w * 32 + (tid & 31);
                 kids[w] = __ballot_sync(HS_FULL_MASK, j > cur && j < nkc && s_par[j] == cur);
             }
-            for (;;) {                                           // siblings in index order
+            // Siblings in index order; each rejection takes the residual's mass, and behind the last one the bonus token is drawn from the
+            // residual, whose masses are then known already.  (One place in the code where masses are summed: what runs once is bound by
+            // instruction fetch.)
+            double mine = 0.0, incl = 0.0, wincl = 0.0, wv = 0.0, gincl = 0.0, gv = 0.0;
+            int last_pos = -1;
+            bool known = false;                                  // the sums above are those of the residual max(p - c q, 0)
+            bool draw = false;
+            for (;;) {
                 int j = -1;
 #pragma unroll
                 for (int w = HS_MAX_NODES / 32 - 1; w >= 0; --w)
                     if (kids[w]) j = w * 32 + __ffs(kids[w]) - 1;
-                if (j < 0) break;
+                draw = j < 0;
+                if (!draw) {
 #pragma unroll
-                for (int w = 0; w < HS_MAX_NODES / 32; ++w)
-                    if (j >> 5 == w) kids[w] &= kids[w] - 1;
-                tested = true;
-                const float pt = s_pt[j], qt = s_qt[j];
-                const float r = fmaxf(pt - c * qt, 0.f) / (float)W;
-                const float a = qt > 0.f ? fminf(1.f, r / qt) : 1.f;
-                if (s_u[j] < a) { accepted = j; break; }
-                if (!have_q) {
-                    const float2 qms = p.ro.drf_ms[koff + cur];
-                    qm = qms.x; iqs = 1.f / qms.y; have_q = true;
+                    for (int w = 0; w < HS_MAX_NODES / 32; ++w)
+                        if (j >> 5 == w) kids[w] &= kids[w] - 1;
+                    const float pt = s_pt[j], qt = s_qt[j];
+                    const float r = fmaxf(pt - c * qt, 0.f) / (float)W;
+                    const float a = qt > 0.f ? fminf(1.f, r / qt) : 1.f;
+                    if (s_u[j] < a) { accepted = j; break; }
+                    if (k.iqs == 0.f) {
+                        const float2 qms = p.ro.drf_ms[koff + cur];
+                        k.qm = qms.x; k.iqs = 1.f / qms.y;
+                    }
+                    c_next = c + (float)W;
+                } else if (known) {
+                    break;
+                } else {
+                    c_next = c;
                 }
-                const float c_next = c + (float)W;
-                stage(cur, prow, qrow);
-                const double W_next = cluster_residual_sum<WC>(p, rank, rs, pm, ips, qm, iqs, invT,
-                                                           c_next, s_part, s_x, xch);
-                if (!(W_next > 0.0)) { c = 0.f; W = 1.0; tested = false; break; }   // p == q: fall back to p
-                c = c_next; W = W_next;
+                stage(cur, prow, c_next > 0.f ? qrow : nullptr);
+                // ---- masses of max(p - c_next q, 0): this thread's, ahead of it in the CTA, of the CTAs --------------------------------
+                mine = 0.0;
+                last_pos = -1;
+                for (int ch = 0; ch < m.pieces; ++ch) {
+                    if (m.held != ch) {
+                        if (p.is_bf16) fill_masses<true>(m, p.vocab, rs, ch, k);
+                        else fill_masses<false>(m, p.vocab, rs, ch, k);
+                        m.held = ch;
+                    }
+                    double t[WALK_EL];
+#pragma unroll
+                    for (int e = 0; e < WALK_EL; ++e) {
+                        const float f = fmaxf(m.p[e] - c_next * m.q[e], 0.f);
+                        if (f > 0.f) last_pos = (rs.v0 + m.w0) * ve + ch * WALK_EL + e;
+                        t[e] = (double)f;
+                    }
+#pragma unroll
+                    for (int o = WALK_EL / 2; o > 0; o >>= 1)
+#pragma unroll
+                        for (int e = 0; e < o; ++e) t[e] += t[e + o];
+                    mine += t[0];
+                }
+                if (tid == 0) { s_pick[0] = 0x7fffffff; s_pick[1] = -1; }
+                incl = warp_prefix_d<32>(mine, lane);
+                __syncthreads();                                 // (s_scan may still be read from the sum before)
+                if (lane == 31) s_scan[warp] = incl;
+                __syncthreads();
+                wv = s_scan[lane & 15];
+                wincl = warp_prefix_d<16>(wv, lane);
+                const double* got = reinterpret_cast<const double*>(s_x[xch & 1u]);
+                cluster_allgather<WC>((unsigned long long)__double_as_longlong(__shfl_sync(HS_FULL_MASK, wincl, 15)), s_x, xch, rank);
+                gv = got[lane & (WC - 1)];
+                gincl = warp_prefix_d<WC>(gv, lane);
+                if (draw) break;
+                const double W_next = __shfl_sync(HS_FULL_MASK, gincl, WC - 1);
+                known = W_next > 0.0;
+                if (known) {
+                    c = c_next; W = W_next;
+                } else {                                         // p == q: fall back to p, no more siblings
+                    c = 0.f; W = 1.0;
+#pragma unroll
+                    for (int w = 0; w < HS_MAX_NODES / 32; ++w) kids[w] = 0u;
+                }
             }
             if (accepted >= 0) {
                 if (rank == 0 && tid == 0 && len < cap) p.out.path_tokens[b * cap + len] = s_tok[accepted];
@@ -727,10 +716,47 @@ __global__ void __launch_bounds__(WALK_THREADS, 1) accept_walk_kernel(const __gr
                 ++len;
                 continue;
             }
-            const float ufin = p.uniforms ? p.uniforms[p.n_nodes_total + b] : philox_uniform(p.seed, p.offset, b, 0, 1);
-            stage(cur, prow, (tested && c > 0.f) ? qrow : nullptr);
+            // ---- inverse-CDF draw from max(p - c q, 0) in token order: smallest j whose running sum exceeds u * total; if rounding leaves
+            // none, the last token with positive mass.  The slice with the crossing is the first whose running total exceeds the goal
+            // (rounding leaves none: the last with mass); that CTA finds the token and writes it.
             drawn = true;
-            cluster_inverse_cdf<WC>(p, rank, rs, pm, ips, qm, iqs, invT, c, ufin, s_scan, s_x, xch, s_pick, &p.out.bonus_token[b]);
+            const double goal = (double)ufin * __shfl_sync(HS_FULL_MASK, gincl, WC - 1);
+            const double before = __shfl_sync(HS_FULL_MASK, gincl - gv, (int)rank), wbefore = __shfl_sync(HS_FULL_MASK, wincl - wv, warp);
+            const unsigned int over = __ballot_sync(HS_FULL_MASK, lane < WC && gincl > goal);
+            const unsigned int full = __ballot_sync(HS_FULL_MASK, lane < WC && gv > 0.0);
+            const int owner = over ? __ffs(over) - 1 : (full ? 31 - __clz(full) : 0);
+            if ((int)rank == owner) {
+                double run = before + (wbefore + (incl - mine));
+                if (run <= goal && run + mine > goal) {          // the crossing lies in this thread's run
+                    bool found = false;
+                    for (int ch = 0; ch < m.pieces && !found; ++ch) {
+                        if (m.held != ch) {
+                            if (p.is_bf16) fill_masses<true>(m, p.vocab, rs, ch, k);
+                            else fill_masses<false>(m, p.vocab, rs, ch, k);
+                            m.held = ch;
+                        }
+#pragma unroll
+                        for (int e0 = 0; e0 < WALK_EL; e0 += 4) {    // four at a time: dependent fp64 additions are 64 clocks each
+                            double t[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) t[e] = (double)fmaxf(m.p[e0 + e] - c * m.q[e0 + e], 0.f);
+                            const double next = run + ((t[0] + t[1]) + (t[2] + t[3]));
+                            if (!found && next > goal) {
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    run += t[e];
+                                    if (!found && run > goal) { found = true; atomicMin(&s_pick[0], (rs.v0 + m.w0) * ve + ch * WALK_EL + e0 + e); }
+                                }
+                            }
+                            run = next;
+                        }
+                    }
+                    if (!found && last_pos >= 0) atomicMin(&s_pick[0], last_pos);       // (rounding)
+                }
+                if (last_pos >= 0) atomicMax(&s_pick[1], last_pos);
+                __syncthreads();
+                if (tid == 0) p.out.bonus_token[b] = s_pick[0] != 0x7fffffff ? s_pick[0] : max(s_pick[1], 0);
+            }
             break;
         }
     }
