@@ -596,7 +596,8 @@ extern "C" size_t hs_cart_workspace_bytes(int32_t n) {
            2 * (2 << CT_MAX_DEPTH) * 4 + (1 << CT_MAX_DEPTH) * 64 * 12 + 4096;
 }
 
-static hs_status launch_grid(hs_ctx* ctx, const float* x, const float* y, int n, int depth, float* thresholds, int* status, cudaStream_t stream) {
+// (too_large: the stream has fewer SMs than the device, as under a partition of it; nothing was launched)
+static hs_status launch_grid(hs_ctx* ctx, const float* x, const float* y, int n, int depth, float* thresholds, int* status, cudaStream_t stream, bool& too_large) {
     CartGrid p;
     p.x = x; p.y = y; p.n = n; p.depth = depth; p.thresholds = thresholds; p.status = status;
     p.per = max(CG_THREADS, (n + ctx->cart_ctas - 1) / ctx->cart_ctas);
@@ -623,7 +624,10 @@ static hs_status launch_grid(hs_ctx* ctx, const float* x, const float* y, int n,
     at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, cart_grid_kernel, p) == cudaSuccess ? HS_OK : HS_ERR_CUDA;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, cart_grid_kernel, p);
+    too_large = e == cudaErrorCooperativeLaunchTooLarge;
+    if (too_large) (void)cudaGetLastError();
+    return e == cudaSuccess ? HS_OK : HS_ERR_CUDA;
 }
 
 extern "C" hs_status hs_cart_fit(hs_ctx* ctx, const float* x, const float* y, int32_t n, int32_t depth,
@@ -650,7 +654,11 @@ extern "C" hs_status hs_cart_fit(hs_ctx* ctx, const float* x, const float* y, in
         }
         ctx->cart_ctas = per_sm > 0 ? min(ctx->sm_count, CG_MAX_CTAS) : -1;
     }
-    if (ctx->cart_ctas > 0 && n <= ctx->cart_ctas * CG_SHARE) return launch_grid(ctx, x, y, n, depth, thresholds, (int*)status, stream);
+    if (ctx->cart_ctas > 0 && n <= ctx->cart_ctas * CG_SHARE) {
+        bool too_large = false;
+        const hs_status st = launch_grid(ctx, x, y, n, depth, thresholds, (int*)status, stream, too_large);
+        if (!too_large) return st;
+    }
     CartParams p;
     p.x = x; p.y = y; p.n = n; p.depth = depth; p.thresholds = thresholds; p.status = status;
     p.tiles = (n + CT_TILE - 1) / CT_TILE;
