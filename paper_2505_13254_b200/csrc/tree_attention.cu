@@ -692,9 +692,18 @@ static bool make_row_map(hs_ctx* ctx, CUtensorMap* tm, const void* base, size_t 
     return encode(ctx, tm, 2, base, gdim, gstr, box);
 }
 
-// KV splits (= cluster size) of tree_attn_umma_kernel: the number with the fewest tile steps on the critical path, waves of CTAs (as
-// many clusters of that size as the device runs at once) times tiles per CTA.
+// KV splits (= cluster size) of tree_attn_umma_kernel: the number with the least time on the critical path, waves of CTAs (as many
+// clusters of that size as the device runs at once) times {tiles per CTA, what lies around them, merge}, in half tiles.  A tile is
+// 0.55 us; start, tree tiles and output 6.5 us, the merge of splits 2.5 us.  (The start was counted as the tree's two tiles, as if
+// a further wave cost nothing else.)  us a call, splits then : now, equal lengths | lengths spread over 0.2 .. 1 of the longest:
+//   one tree, 32 / 8 heads, 256 tokens 8.7 : 7.7, 320 9.0 : 8.2, of 32 / 32 heads 384 10.9 : 9.2; two trees, 32 / 32, 512 12.4 : 10.4
+//   80 blocks, 2048 tokens 29.9 : 23.3 | 25.4 : 18.9;  96 blocks, 4096 51 .. 56 : 39 .. 41 | 43 : 34, 8192 71 .. 83 : 68 .. 76 | 57 .. 71 : 58 .. 75
+// More blocks than SMs: their waves fill up, and with lengths that differ short blocks run beside a long one, where splits of it
+// only add starts and merges.  No splits up to 128 tiles:
+//   160 blocks, 2048 tokens 54 : 47 | 43 .. 52 : 24, 4096 91 : 80 | 68 .. 78 : 36 .. 44, 8192 138 : 145 | 112 : 75 (16384 226 : 295 | 156 : 135)
+//   192 blocks, 2048 56 : 48 | 44 .. 49 : 25 .. 34, 4096 86 : 82 | 58 : 42; 320 blocks, 4096 142 : 126 | 103 : 78
 static int choose_splits(int base_ctas, int sm_count, int prefix_tiles, const int* cluster_cap) {
+    if (base_ctas > sm_count && prefix_tiles <= 128) return 1;
     int best = 1;
     long best_cost = 0;
     for (int s = 1; s <= ATT_MAX_SPLIT; ++s) {
@@ -702,7 +711,7 @@ static int choose_splits(int base_ctas, int sm_count, int prefix_tiles, const in
         const long ctas = (long)base_ctas * s;
         const long cap = cluster_cap[s] > 0 ? cluster_cap[s] : sm_count;
         const long waves = (ctas + cap - 1) / cap;
-        const long cost = waves * ((prefix_tiles + s - 1) / s + 2 + (s > 1 ? 2 : 0));   // + tree tiles, + merge
+        const long cost = waves * (2 * ((prefix_tiles + s - 1) / s) + 24 + (s > 1 ? 9 : 0));
         if (s == 1 || cost < best_cost) { best_cost = cost; best = s; }
     }
     return best;
@@ -711,37 +720,28 @@ static int choose_splits(int base_ctas, int sm_count, int prefix_tiles, const in
 // Splits with which tree_attn_duo_kernel takes a launch, 0: tree_attn_umma_kernel takes it.
 // What is known is the number of query blocks (an upper bound: small trees leave blocks empty) and the longest prefix; how the other
 // lengths lie below it the host cannot tell (the cache arrays may be larger than what is in use), so every line is drawn for equal
-// lengths and for lengths spread over 0.2 .. 1 of the longest together.  Measured in us a call, back to back, 50..60 nodes a tree, as
-// "other kernel : this one", equal lengths | spread:
-//   At most one block per SM: only two splits let CTAs share SMs.  From 256 tiles (16384 tokens) and three quarters of the SMs.
-//     blocks    8192 tokens               16384                         24576                         32768
-//      96                                                                                             221 : 261 | 156 : 247
-//     112        75.3 : 82.5 | 74.3 : 80.3  141 : 144 | 140 : 139         211 : 208 | 208 : 194         283 : 277 | 277 : 259
-//     128        75.5 : 81.6 | 74.9 : 80.8  142 : 144 | 141 : 140         213 : 211 | 209 : 202         286 : 281 | 285 : 266
-//     144        82.6 : 87.5 | 75.5 : 79.3  163 : 165 | 154 : 144         247 : 235 | 216 : 200         332 : 318 | 285 : 263
-//   More: the other kernel pays for whole waves of CTAs, each with about 10 us around its tiles that nothing overlaps.
-//     blocks     512 tokens                1024                          2048                          4096                          8192
-//     160        23.6 : 17.9 | 17.8 : 16.0  31.1 : 26.3 | 19.8 : 23.0     54.8 : 43.1 | 44.0 : 37.4     91.3 : 74.3 | 76.2 : 65.4     128 : 133 | 101 : 121
-//     192        24.0 : 18.2 | 20.0 : 17.2  31.3 : 26.4 | 24.6 : 24.8     55.9 : 43.5 | 47.9 : 38.6     77.8 : 74.2 | 63.9 : 67.1     125 : 135 | 95 : 125
-//     256        24.9 : 19.3 | 20.7 : 17.8  32.2 : 27.1 | 25.2 : 25.7     47.8 : 42.8 | 34.9 : 40.0     80.4 : 77.0 | 52.7 : 69.7     152 : 149 | 92 : 129
-//     320        35.5 : 32.8 | 29.1 : 24.9  47.3 : 45.5 | 35.3 : 30.1     92.2 : 70.2 | 74.8 : 41.3     128 : 120 | 94 : 71           204 : 224 | 145 : 139
-//     384        36.7 : 33.2 | 31.0 : 28.2  47.9 : 45.5 | 38.9 : 35.1     70.3 : 70.3 | 52.8 : 48.3     119 : 124 | 81 : 78           229 : 248 | 148 : 146
-//     448        48.7 : 38.0 | 40.0 : 30.5  63.3 : 52.5 | 48.7 : 39.9     90.8 : 82.0 | 63.8 : 55.2     179 : 145 | 140 : 88          316 : 290 | 244 : 159
-//     512        52.3 : 38.3 | 42.6 : 31.3  63.8 : 52.4 | 52.9 : 41.2     92.5 : 84.4 | 71.4 : 60.5     188 : 153 | 148 : 104         342 : 303 | 240 : 194
-//     1024        103 : 79 | 80 : 63         114 : 97 | 97 : 80            168 : 164 | 135 : 119         302 : 299 | 224 : 211
-//     - up to 16 tiles at any number; above three waves at any length; up to 64 tiles where the last wave is at least a quarter empty.
-//     - 65 to 128 tiles and a second wave of at most a sixth: two splits.  160 blocks, 6144 tokens 110 : 106 | 91 : 72, 8192 128 : 130 | 103 : 82,
-//       10000 142 : 154 | 118 : 100; 176: 6144 104 : 107 | 89 : 81; 192: 8192 125 : 133 | 95 : 96.
-//   One query block per head stays with the other kernel: no line is drawn for it yet.  The same ones would hold above one block per
-//   SM (8 x 20..30 nodes, 32 / 32 heads, 256 blocks: 512 tokens 23.8 : 18.3 | 19.4 : 16.3, 2048 51.5 : 47.2 | 35.8 : 40.5).
+// lengths and for lengths spread over 0.2 .. 1 of the longest together.  The other kernel pays for whole waves of CTAs, each with 6.5 us
+// around its tiles that nothing overlaps, but one CTA of it is through its tiles in half the time, which decides where the lengths
+// differ.  us a call, back to back, other kernel : this one, equal lengths | spread (30 .. 40 nodes of one block, 60 of two):
+//     blocks     512 tokens     1024                          2048                          4096
+//     160        22.5 : 16.0    29.5 : 23.5 | 18.9 : 23.6     47 : 39 | 23 : 35             80 : 70 | 36 : 56
+//     192        21.8 : 16.0    29.8 : 24.1 | 20.1 : 22.0     48 : 41 | 25 .. 34 : 37       82 : 73 | 42 : 61
+//     256        24.7 : 18.9    32.6 : 27.7 | 22.3 : 22.3     51 : 47 | 36 : 39             89 : 86 | 56 : 66
+//     320        34.6 : 31.7    46.3 : 48.1 | 34.3 : 27.9     73 : 79 | 46 : 40             126 : 143 | 78 : 79
+//     384        35.0 : 31.9    47.8 : 48.4 | 37.8 : 38.3     76 : 85 | 54 : 58             135 : 162 | 84 : 91
+//     512        48.8 : 36.2    64.4 : 55.2 | 48.3 : 40.0     101 : 94 | 75 : 70            188 : 153 | 148 : 104
+//     1024       103 : 79       114 : 97 | 97 : 80            168 : 164 | 135 : 119         302 : 299 | 224 : 211
+//   - a second wave of at most a sixth: up to 8 tiles; else up to 16 tiles; above three waves at any length; up to 32 tiles where the last of
+//     two or three waves is at least a quarter empty and more than a sixth full.
+//   At most one block per SM: only two splits let CTAs share SMs, which pays from 448 tiles and three quarters of the SMs on.
+//     128 blocks, 32768 tokens 306 : 302 | 251 : 291, 24576 234 : 232 | 106 : 129, 16384 136 : 151 | 104 : 128.
 // Two CTAs on an SM is what runs (128 blocks of 129 tiles take 104 us alone, 256 blocks 146), also in pairs; cudaOccupancyMaxActiveClusters
 // counts one, as it does for any kernel that allocates tensor memory (it does not know how many columns), so it is not asked.
-static int duo_splits(int base_ctas, int mblocks, int sm_count, int prefix_tiles) {
-    if (mblocks == 1) return 0;
-    if (base_ctas <= sm_count) return 4 * base_ctas > 3 * sm_count && prefix_tiles >= 256 ? 2 : 0;
-    if (prefix_tiles > 64 && prefix_tiles <= 128 && 6 * base_ctas <= 7 * sm_count) return 2;
+static int duo_splits(int base_ctas, int sm_count, int prefix_tiles) {
+    if (base_ctas <= sm_count) return 4 * base_ctas > 3 * sm_count && prefix_tiles >= 448 ? 2 : 0;
+    if (6 * base_ctas <= 7 * sm_count) return prefix_tiles <= 8 ? 1 : 0;
     const int waves = (base_ctas + sm_count - 1) / sm_count;
-    return prefix_tiles <= 16 || (prefix_tiles <= 64 && 4 * base_ctas <= 3 * waves * sm_count) || waves > 3 ? 1 : 0;
+    return prefix_tiles <= 16 || (prefix_tiles <= 32 && 4 * base_ctas <= 3 * waves * sm_count) || waves > 3 ? 1 : 0;
 }
 
 template <typename Kernel>
@@ -805,7 +805,7 @@ hs_status hs_launch_attention(hs_ctx* ctx, const hs_pruned_tree* pruned, const h
     memset(&tmV, 0, sizeof(tmV));
     const int mblocks = (rows + ATT_BM - 1) / ATT_BM;
     const int prefix_tiles = (d->max_kv_len + ATT_BN - 1) / ATT_BN;
-    const int duo = duo_splits(pairs * mblocks, mblocks, ctx->sm_count, prefix_tiles);
+    const int duo = duo_splits(pairs * mblocks, ctx->sm_count, prefix_tiles);
     p.nsplit = duo ? duo : choose_splits(pairs * mblocks, ctx->sm_count, prefix_tiles, cap_umma);
     if (d->kv_total > 0) {
         if (!make_kv_map(ctx, &tmK, k_cache, d, p.head_first) || !make_kv_map(ctx, &tmV, v_cache, d, p.head_first))
