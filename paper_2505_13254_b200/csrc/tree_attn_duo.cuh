@@ -1,4 +1,4 @@
-// The attention kernel for launches of more than one wave of CTAs and for long prefixes in pairs of splits.  Included by tree_attention.cu, whose header
+// The attention kernel for launches of more than one wave of CTAs and for the longest prefixes in pairs of splits.  Included by tree_attention.cu, whose header
 // describes the problem.
 //
 // TWO CTAs share an SM (half of its tensor memory, 99 KiB of shared memory each): while one starts (dependent loads of the pruned
@@ -8,9 +8,9 @@
 // S(i + 2) from one issuing thread.  Two threads share a row (32 keys of a tile each).  One producer warp: prefix tiles by tiled
 // copies, the indirectly indexed rows of Q and of the tree tokens by tile::gather4.
 // Bound by the chain of a tile (S, load, maximum, exponentials, P V): 0.68 us for one CTA, 1.06 us for two at once, against 1.17 us
-// for two tiles of tree_attn_umma_kernel.  4 x 62 nodes, 64 / 8 heads, 32768 tokens: 277 us against 286; 10 x 50..60 nodes, 32 / 8
-// heads, 2048 tokens: 44.0 against 54.9; 16 trees, 512 tokens 19.7 against 24.1 (which launches come here: see duo_splits).  With tiles of
-// 128 keys S and P leave room for one buffer only: 366 us at 32768 tokens.
+// for two tiles of tree_attn_umma_kernel.  4 x 62 nodes, 64 / 8 heads, 32768 tokens: 302 us against 306 (both under the power cap); 16 trees,
+// 32 / 8 heads, 512 tokens 19.3 against 24.9; 8 trees, 32 / 32 heads, 512 tokens 18.9 against 24.7 (which launches come here: see
+// duo_splits).  With tiles of 128 keys S and P leave room for one buffer only: 366 us at 32768 tokens.
 #pragma once
 
 #define AD_HALF_BYTES (ATT_TILE_BYTES / 2)          // columns 0..63 / 64..127 of a K or V tile (rows of 128 bytes, 128-byte swizzle)
