@@ -32,7 +32,8 @@ using std::min;
 #define QS_THREADS 512                        // cluster kernel: sixteen warps
 #define QS_ITEM_VECS 2048                     // vectors per item: 32 KiB, four per thread
 #define QS_SLOTS 6                            // items a CTA has room for
-#define QS_SMEM_BYTES (QS_SLOTS * QS_ITEM_VECS * 16 + 128)
+#define QS_ITEM_BYTES (QS_ITEM_VECS * 16 + QS_THREADS * 4 + QS_THREADS)     // an item, every thread's maximum of it, its cells to read again
+#define QS_SMEM_BYTES(items) ((items) * QS_ITEM_BYTES + 128)
 
 struct QuantParams {
     const void* logits;
@@ -190,7 +191,8 @@ __device__ __forceinline__ float warp_kth_largest(float v, int K, int lane) {
 // item is reduced (128 KiB per SM), the rest dependent shared-memory reads and shuffles.  One thread that asked for all items with the CTA
 // waiting behind it cost 2.5 k, items unrolled over the slots (34 KB of code instead of 82) and merges by all 16 warps
 // between barriers the rest.  One greedy step of an 8B-shaped model 38.4 -> 36.2 us, of 32000 fp32 logits 30.1 -> 27.9.
-// At most 72 registers per thread: the CTA then fits into the register file beside a CTA of the kernel ahead that is still at work on
+// At most 72 registers per thread (and 64 where the logits are fp32: two CTAs of up to three items then share an SM, which clusters of five need,
+// whose 28 do not find five SMs of a GPC each: ten levels of 28 rows of 85645 fp32 logits 141 us, with one CTA per SM 166): the CTA then fits into the register file beside a CTA of the kernel ahead that is still at work on
 // the same SM (in a decode loop: the CTA that walks the accepted path of the step before).
 // {ref, sum e, sum x e, max} of the first N lanes (N a power of two; lanes past the last one hold no values) as one, known to lanes 0 .. N - 1
 template <int N>
@@ -212,7 +214,7 @@ __device__ __forceinline__ float4 merge_stats(float4 v) {
 }
 
 template <bool BF16>
-__global__ void __maxnreg__(72) quantify_cluster_kernel(const __grid_constant__ QuantParams p) {
+__global__ void __maxnreg__(BF16 ? 72 : 64) quantify_cluster_kernel(const __grid_constant__ QuantParams p) {
     constexpr int VE = BF16 ? 8 : 4;
     constexpr int NW = QS_THREADS / 32;
     extern __shared__ __align__(128) unsigned char s_dyn[];
@@ -223,8 +225,6 @@ __global__ void __maxnreg__(72) quantify_cluster_kernel(const __grid_constant__ 
     __shared__ float4 s_wstat[NW];                               // {ref, sum e, sum x e, max} per warp
     __shared__ float4 s_stat;                                    //   and of the part
     __shared__ int s_cnt;
-    __shared__ unsigned char s_hit[NW][QS_SLOTS * 32];           // cells to read again: item * 32 + lane
-    __shared__ float s_cm[QS_SLOTS][QS_THREADS];                 // every thread's maximum of each item
     __shared__ __align__(16) unsigned long long s_ck[8][HS_MAX_TOPK];   // first CTA of a row: the parts' Top-K keys
     __shared__ __align__(16) float4 s_cs[8];                            //   and their {ref, sum e, sum x e, max}
 
@@ -235,6 +235,8 @@ __global__ void __maxnreg__(72) quantify_cluster_kernel(const __grid_constant__ 
     const char* rowp = (const char*)p.logits + (size_t)row * p.row_stride * (BF16 ? 2 : 4);
     const unsigned int slots0 = (smem_u32(s_dyn) + 127u) & ~127u;
     const uint4* slots = reinterpret_cast<const uint4*>(s_dyn + (slots0 - smem_u32(s_dyn)));
+    float* s_cm = reinterpret_cast<float*>(s_dyn + (slots0 - smem_u32(s_dyn)) + nit * QS_ITEM_VECS * 16);      // [nit][QS_THREADS] maxima
+    unsigned char* s_hit = reinterpret_cast<unsigned char*>(s_cm + nit * QS_THREADS) + warp * nit * 32;        // this warp's cells: item * 32 + lane
     const int K = p.K;
 
     if (tid == 0) {
@@ -287,7 +289,7 @@ __global__ void __maxnreg__(72) quantify_cluster_kernel(const __grid_constant__ 
         }
         float rm;
         fold_round<BF16>(d, ref, nref, s2, u2, rm);
-        s_cm[it][tid] = rm;
+        s_cm[it * QS_THREADS + tid] = rm;
         lm = fmaxf(lm, rm);
     }
     // ---- Top-K of the part: bound, candidates -------------------------------------------------------------------------
@@ -319,16 +321,16 @@ __global__ void __maxnreg__(72) quantify_cluster_kernel(const __grid_constant__ 
     int nhit = 0;
 #pragma unroll 1
     for (int it = 0; it < nit; ++it) {
-        const float cm = s_cm[it][tid];
+        const float cm = s_cm[it * QS_THREADS + tid];
         const bool hit = cm >= tau && cm > -CUDART_INF_F;
         const unsigned int b = __ballot_sync(HS_FULL_MASK, hit);
-        if (hit) s_hit[warp][nhit + __popc(b & ((1u << lane) - 1u))] = (unsigned char)(it * 32 + lane);
+        if (hit) s_hit[nhit + __popc(b & ((1u << lane) - 1u))] = (unsigned char)(it * 32 + lane);
         nhit += __popc(b);
     }
     __syncwarp();
 #pragma unroll 1
     for (int h = lane >> 2; h < nhit; h += 8) {
-        const int cell = s_hit[warp][h], vl = (cell >> 5) * QS_ITEM_VECS + warp * 32 + (cell & 31) + (lane & 3) * QS_THREADS, v = sv0 + vl;
+        const int cell = s_hit[h], vl = (cell >> 5) * QS_ITEM_VECS + warp * 32 + (cell & 31) + (lane & 3) * QS_THREADS, v = sv0 + vl;
         if (v >= sv1) continue;
         float x[8];
         unpack<BF16>(slots[vl], x);
@@ -511,14 +513,14 @@ hs_status hs_launch_quantify(hs_ctx* ctx, const hs_tree_batch* tree, const void*
         // accepted does not depend on which kernel takes it.)
         if ((size_t)p.rows * parts * HS_ROW_PARTIAL_BYTES > ctx->scratch_bytes) return HS_ERR_WORKSPACE;
         if (!ctx->quant_ready) {
-            if (cudaFuncSetAttribute(quantify_cluster_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_BYTES) != cudaSuccess ||
-                cudaFuncSetAttribute(quantify_cluster_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_BYTES) != cudaSuccess)
+            if (cudaFuncSetAttribute(quantify_cluster_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_BYTES(QS_SLOTS)) != cudaSuccess ||
+                cudaFuncSetAttribute(quantify_cluster_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_BYTES(QS_SLOTS)) != cudaSuccess)
                 return HS_ERR_CUDA;
             ctx->quant_ready = true;
         }
         p.split = parts;
         p.per = pv;
-        const size_t smem = (size_t)((pv + QS_ITEM_VECS - 1) / QS_ITEM_VECS) * QS_ITEM_VECS * 16 + 128;
+        const size_t smem = QS_SMEM_BYTES((pv + QS_ITEM_VECS - 1) / QS_ITEM_VECS);
         e = dtype == HS_BF16
             ? hs_launch(quantify_cluster_kernel<true>, dim3(p.rows * parts), dim3(QS_THREADS), smem, stream, ctx->pdl, dim3(parts, 1, 1), p)
             : hs_launch(quantify_cluster_kernel<false>, dim3(p.rows * parts), dim3(QS_THREADS), smem, stream, ctx->pdl, dim3(parts, 1, 1), p);
