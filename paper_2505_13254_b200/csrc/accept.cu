@@ -27,6 +27,7 @@
 #include <cooperative_groups.h>
 #include <math_constants.h>
 
+#include "draw_cross.h"
 #include "hs_common.cuh"
 #include "hs_layout.h"
 #include "hs_ptx.cuh"
@@ -736,19 +737,12 @@ __global__ void __launch_bounds__(WALK_THREADS, 1) accept_walk_kernel(const __gr
                             m.held = ch;
                         }
 #pragma unroll
-                        for (int e0 = 0; e0 < WALK_EL; e0 += 4) {    // four at a time: dependent fp64 additions are 64 clocks each
+                        for (int e0 = 0; e0 < WALK_EL; e0 += 4) {
                             double t[4];
 #pragma unroll
                             for (int e = 0; e < 4; ++e) t[e] = (double)fmaxf(m.p[e0 + e] - c * m.q[e0 + e], 0.f);
-                            const double next = run + ((t[0] + t[1]) + (t[2] + t[3]));
-                            if (!found && next > goal) {
-#pragma unroll
-                                for (int e = 0; e < 4; ++e) {
-                                    run += t[e];
-                                    if (!found && run > goal) { found = true; atomicMin(&s_pick[0], (rs.v0 + m.w0) * ve + ch * WALK_EL + e0 + e); }
-                                }
-                            }
-                            run = next;
+                            const int at = found ? -1 : crossing_of_four(t, goal, run);
+                            if (at >= 0) { found = true; atomicMin(&s_pick[0], (rs.v0 + m.w0) * ve + ch * WALK_EL + e0 + at); }
                         }
                     }
                     if (!found && last_pos >= 0) atomicMin(&s_pick[0], last_pos);       // (rounding)
