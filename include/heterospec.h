@@ -335,7 +335,8 @@ hs_status hs_rerank(hs_ctx* ctx, const hs_expand_state* st, const int32_t* n_top
  *   L(s) = sum over {left, right} of |D_j| / |D| * sum over D_j of (y - mean_j)^2
  * over the midpoints between consecutive distinct feature values (ties: the smallest s).  thresholds (device,
  * 2^depth - 1 floats) receives the thresholds in ascending order: with depth = 3 they are hs_policy.thresholds.
- * status (device, one int): 0, or HS_ERR_SHAPE if some node held a single feature value (its threshold is NaN).
+ * status (device, one int): 0, or HS_ERR_SHAPE if some node held a single feature value (its threshold is NaN),
+ * or HS_ERR_TIMEOUT if CTAs of the training waited in vain for others (no thresholds then; also in the error word).
  * 1 <= depth <= 6, 2^depth <= n <= 2^26.  Needs hs_cart_workspace_bytes(n) of context workspace. */
 size_t hs_cart_workspace_bytes(int32_t n);
 hs_status hs_cart_fit(hs_ctx* ctx, const float* x, const float* y, int32_t n, int32_t depth, float* thresholds,

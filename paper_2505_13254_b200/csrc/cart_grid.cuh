@@ -57,7 +57,14 @@ static_assert(CT_MAX_NODES <= CG_WARPS, "a warp per node");
 static_assert(CG_WARPS == 32, "a warp per digit of a block of 32, a lane per run of shares");
 static_assert(sizeof(CartGridSmem) <= 220 * 1024 && CG_MAX_DIGITS <= CG_THREADS, "one CTA per SM");
 
-// All CTAs of the grid have come this far and see what the others stored ahead of it.  Bounded; false for all threads when the wait expired.
+// A CTA leaves (one thread): the last one puts the counters back.  Every CTA leaves behind its last wait, so nobody looks at them any more.
+__device__ __forceinline__ void grid_leave(const CartGrid& p) {
+    if (atomicAdd(&p.bar[1], 1u) == gridDim.x - 1) { p.bar[0] = 0u; p.bar[1] = 0u; }
+}
+
+// All CTAs of the grid have come this far and see what the others stored ahead of it.  Bounded; false for all threads when the wait expired:
+// the CTA has left then and has to return at once.  Above all it arrives nowhere any more: no CTA passes a later barrier, so nobody reads
+// what has not been written, and CTA 0, whose last wait is for all, gives up as well and says so in the status.
 __device__ __forceinline__ bool grid_sync(const CartGrid& p, unsigned int& round, bool wait = true) {
     ++round;
     __syncthreads();
@@ -70,8 +77,13 @@ __device__ __forceinline__ bool grid_sync(const CartGrid& p, unsigned int& round
             unsigned int v;
             do {
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p.bar) : "memory");
-                if (v < round * gridDim.x && global_timer_ns() - t0 > HS_WAIT_LIMIT_NS) { atomicExch(p.err, (int)HS_ERR_TIMEOUT); bad = 1; }
+                if (v < round * gridDim.x && global_timer_ns() - t0 > HS_WAIT_LIMIT_NS) bad = 1;
             } while (v < round * gridDim.x && !bad);
+            if (bad) {
+                atomicExch(p.err, (int)HS_ERR_TIMEOUT);
+                if (blockIdx.x == 0) *p.status = HS_ERR_TIMEOUT;
+                grid_leave(p);
+            }
         }
     }
     return __syncthreads_or(bad) == 0;
@@ -98,7 +110,6 @@ __global__ void __launch_bounds__(CG_THREADS, 1) cart_grid_kernel(const __grid_c
     const int base = min(c * p.per, p.n), mine = min(base + p.per, p.n) - base;      // this CTA's share
     const int nit = (p.per + CG_THREADS - 1) / CG_THREADS;
     unsigned int round = 0;
-    bool ok = true;
 
     // ---- the keys, and the range of their order bits -------------------------------------------------------------------
     // (a warp has 32 nit consecutive samples, item-major)
@@ -119,7 +130,7 @@ __global__ void __launch_bounds__(CG_THREADS, 1) cart_grid_kernel(const __grid_c
     if (lane == 0) { atomicMin(&sm.lo, lo); atomicMax(&sm.hi, hi); }
     __syncthreads();
     if (tid == 0) p.range[c] = make_uint2(sm.lo, sm.hi);
-    ok = grid_sync(p, round);
+    if (!grid_sync(p, round)) return;
     {
         const uint2 r = tid < G ? __ldcg(&p.range[tid]) : make_uint2(~0u, 0u);
         lo = __reduce_min_sync(HS_FULL_MASK, r.x); hi = __reduce_max_sync(HS_FULL_MASK, r.y);
@@ -132,7 +143,7 @@ __global__ void __launch_bounds__(CG_THREADS, 1) cart_grid_kernel(const __grid_c
     const int ND = 1 << width;
 
     // ---- the sort ------------------------------------------------------------------------------------------------------
-    for (int pass = 0; pass < passes && ok; ++pass) {
+    for (int pass = 0; pass < passes; ++pass) {
         const unsigned long long* in = (pass & 1) ? p.keys2 : p.keys;
         unsigned long long* out = (pass & 1) ? p.keys : p.keys2;
         unsigned short* wcnt = sm.cnt + (warp << width);     // this warp's counters
@@ -189,7 +200,7 @@ __global__ void __launch_bounds__(CG_THREADS, 1) cart_grid_kernel(const __grid_c
                 sm.key[sm.off[d] + wcnt[d] + rank[i]] = k[i];
             }
         }
-        ok = grid_sync(p, round);
+        if (!grid_sync(p, round)) return;
         unsigned int oa = 0, ob = 0, ta = 0, tb = 0;         // of digits 2 t and 2 t + 1: keys of the shares ahead, keys of all shares
         if (G <= CG_DIRECT) {
             if (2 * tid < ND)
@@ -232,7 +243,7 @@ __global__ void __launch_bounds__(CG_THREADS, 1) cart_grid_kernel(const __grid_c
                 }
                 __syncthreads();
             }
-            ok = grid_sync(p, round) && ok;
+            if (!grid_sync(p, round)) return;
             if (2 * tid < ND) {
                 const uint2 t2 = __ldcg(reinterpret_cast<const uint2*>(p.tot) + tid), o2 = __ldcg(reinterpret_cast<const uint2*>(p.cnt + (size_t)c * ND) + tid);
                 ta = t2.x; tb = t2.y; oa = o2.x; ob = o2.y;
@@ -247,9 +258,9 @@ __global__ void __launch_bounds__(CG_THREADS, 1) cart_grid_kernel(const __grid_c
         for (int j = tid; j < mine; j += CG_THREADS) {
             const unsigned long long key = sm.key[j];
             const unsigned int to = sm.off[digit(key)] + j;
-            if (to < (unsigned int)p.n) out[to] = key;       // (out of range only after a wait that expired)
+            if (to < (unsigned int)p.n) out[to] = key;       // (always, unless two calls share the workspace at a time)
         }
-        ok = grid_sync(p, round) && ok;
+        if (!grid_sync(p, round)) return;
     }
     const unsigned long long* sorted = (passes & 1) ? p.keys2 : p.keys;
 
@@ -276,7 +287,7 @@ __global__ void __launch_bounds__(CG_THREADS, 1) cart_grid_kernel(const __grid_c
         scan_pair<CG_WARPS>(a, b, sm.w);
         if (tid == CG_THREADS - 1) { p.blk[2 * c] = a + ta; p.blk[2 * c + 1] = b + tb; }
     }
-    if (!grid_sync(p, round) || !ok) return;
+    if (!grid_sync(p, round)) return;
     {
         // sums ahead of every share, in one fixed order: thread t has share t
         double ba = tid < G ? __ldcg(&p.blk[2 * tid]) : 0.0, bb = tid < G ? __ldcg(&p.blk[2 * tid + 1]) : 0.0;
@@ -337,7 +348,6 @@ __global__ void __launch_bounds__(CG_THREADS, 1) cart_grid_kernel(const __grid_c
     }
     if (tid == 0) {
         if (c == 0) *p.status = sm.bad ? HS_ERR_SHAPE : HS_OK;
-        // the last CTA to leave puts the counters back (nobody waits on them any more: CTA 0 leaves behind its last wait)
-        if (atomicAdd(&p.bar[1], 1u) == (unsigned int)G - 1) { p.bar[0] = 0u; p.bar[1] = 0u; }
+        grid_leave(p);
     }
 }

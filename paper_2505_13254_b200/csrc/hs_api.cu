@@ -131,10 +131,7 @@ extern "C" hs_status hs_device_error(hs_ctx* ctx, int32_t* host_out) {
     HS_CUDA_OK(cudaDeviceSynchronize());
     int v = 0;
     HS_CUDA_OK(cudaMemcpy(&v, ctx->counters + HS_CNT_ERROR, sizeof(int), cudaMemcpyDeviceToHost));
-    if (v != 0) {                                     // (a grid that gave up a wait leaves its arrivals behind: the next one starts from zero)
-        HS_CUDA_OK(cudaMemset(ctx->counters + HS_CNT_CART, 0, (4 * 256 + 16) * sizeof(int)));
-        HS_CUDA_OK(cudaMemset(ctx->counters + HS_CNT_ERROR, 0, sizeof(int)));
-    }
+    if (v != 0) HS_CUDA_OK(cudaMemset(ctx->counters + HS_CNT_ERROR, 0, sizeof(int)));
     *host_out = v;
     return HS_OK;
 }

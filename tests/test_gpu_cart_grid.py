@@ -1,11 +1,16 @@
 """Stratifier training by one resident grid: shares of one to eight samples per thread, the last share short, the most a grid takes and one
 more; feature values that differ in a few bits, in up to thirty (three passes of the sort) and in all of them (four); a second call finds the
-counters at zero."""
+counters at zero, also behind a wait that ran out."""
+import ctypes
+import os
+import re
+
 import numpy as np
 import pytest
 import torch
 
 from paper_2505_13254_b200 import binding as hb
+from paper_2505_13254_b200 import build
 from test_gpu_cart_sizes import sums_fit
 
 pytestmark = pytest.mark.gpu
@@ -61,4 +66,44 @@ def test_the_grid_in_a_graph_and_behind_other_work():
     graph.replay()
     torch.cuda.synchronize()
     assert int(status) == 0 and np.array_equal(th.cpu().numpy(), sums_fit(x, y, 3).astype(np.float32))
+    ctx.close()
+
+
+def arrivals(ctx, workspace):
+    """Device address of the two words in which the CTAs of the training count their arrivals (the workspace pointer lies behind the device, the
+    SM count and the workspace's size in the context)."""
+    layout = open(os.path.join(build.CSRC, "hs_layout.h")).read()
+    head = ctypes.cast(ctx.handle, ctypes.POINTER(ctypes.c_uint64))
+    assert head[1] == workspace
+    return head[2] + 4 * int(re.search(r"#define HS_CNT_CART (\d+)", layout).group(1))
+
+
+def words(address, value=None):
+    rt = pytest.importorskip("cuda.bindings.runtime")
+    host = np.zeros(2, np.uint32) if value is None else np.array(value, np.uint32)
+    kinds = rt.cudaMemcpyKind
+    to, of, kind = (host.ctypes.data, address, kinds.cudaMemcpyDeviceToHost) if value is None else (address, host.ctypes.data, kinds.cudaMemcpyHostToDevice)
+    err, = rt.cudaMemcpy(to, of, 8, kind)
+    assert int(err) == 0
+    return host.tolist()
+
+
+@pytest.mark.parametrize("n", [9000, 60000])                       # the counts of all shares added up by every CTA, and 32 digits to a CTA
+def test_a_wait_that_runs_out_is_the_status_and_leaves_nothing_behind(n):
+    rng = np.random.default_rng(n)
+    x = feature("positive", n, rng)
+    y = np.clip(np.round(3.0 * x + rng.normal(0, 3, n)), 0, 59).astype(np.float32)
+    size = hb.hs_cart_workspace_bytes(n)
+    ctx = hb.Context(0, size)
+    at = arrivals(ctx, size)
+    xd, yd = torch.from_numpy(x).cuda(), torch.from_numpy(y).cuda()
+    torch.cuda.synchronize()
+    words(at, [2 ** 32 - 1, 0])                         # one arrival is missing: the first barrier's wait runs out (one second)
+    _, status = hb.hs_cart_fit(ctx, xd, yd, 3)
+    torch.cuda.synchronize()
+    assert int(status) == hb.HS_ERR_TIMEOUT and words(at) == [0, 0]
+    th, status = hb.hs_cart_fit(ctx, xd, yd, 3)                    # the error word has not been read yet
+    torch.cuda.synchronize()
+    assert int(status) == 0 and np.array_equal(th.cpu().numpy(), sums_fit(x, y, 3).astype(np.float32))
+    assert hb.hs_device_error(ctx) == hb.HS_ERR_TIMEOUT and hb.hs_device_error(ctx) == 0
     ctx.close()
