@@ -596,12 +596,25 @@ extern "C" size_t hs_cart_workspace_bytes(int32_t n) {
            2 * (2 << CT_MAX_DEPTH) * 4 + (1 << CT_MAX_DEPTH) * 64 * 12 + 4096;
 }
 
-// (too_large: the stream has fewer SMs than the device, as under a partition of it; nothing was launched)
+// SMs that a launch into the stream may use: the device's, or those of the partition that the stream belongs to.  (A capture takes a
+// cooperative launch that is too large for the partition without a word, and the graph as well.)
+static int stream_sms(const hs_ctx* ctx, cudaStream_t stream) {
+    if ((uintptr_t)stream <= 2 || !ctx->stream_part || !ctx->part_sms) return ctx->sm_count;      // (the default streams belong to none)
+    CUgreenCtx part = nullptr;
+    CUdevResource r;
+    if (((CUresult(*)(CUstream, CUgreenCtx*))ctx->stream_part)((CUstream)stream, &part) != CUDA_SUCCESS || !part) return ctx->sm_count;
+    if (((CUresult(*)(CUgreenCtx, CUdevResource*, CUdevResourceType))ctx->part_sms)(part, &r, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS) return ctx->sm_count;
+    return min((int)r.sm.smCount, ctx->sm_count);
+}
+
+// (too_large: fewer SMs than CTAs, whatever took them; nothing was launched)
 static hs_status launch_grid(hs_ctx* ctx, const float* x, const float* y, int n, int depth, float* thresholds, int* status, cudaStream_t stream, bool& too_large) {
     CartGrid p;
     p.x = x; p.y = y; p.n = n; p.depth = depth; p.thresholds = thresholds; p.status = status;
     p.per = max(CG_THREADS, (n + ctx->cart_ctas - 1) / ctx->cart_ctas);
     const int G = (n + p.per - 1) / p.per, parts = 2 * (G + CT_MAX_NODES);
+    too_large = G > stream_sms(ctx, stream);
+    if (too_large) return HS_OK;
     size_t o = 0;
     auto take = [&](size_t bytes) { char* q = ctx->scratch + o; o += hs_align_up(bytes, 256); return q; };
     p.keys = (unsigned long long*)take((size_t)n * 8);
@@ -652,6 +665,11 @@ extern "C" hs_status hs_cart_fit(hs_ctx* ctx, const float* x, const float* y, in
             per_sm = 0;
             (void)cudaGetLastError();
         }
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPoint("cuStreamGetGreenCtx", &ctx->stream_part, cudaEnableDefault, &found) != cudaSuccess || found != cudaDriverEntryPointSuccess)
+            ctx->stream_part = nullptr;
+        if (cudaGetDriverEntryPoint("cuGreenCtxGetDevResource", &ctx->part_sms, cudaEnableDefault, &found) != cudaSuccess || found != cudaDriverEntryPointSuccess)
+            ctx->part_sms = nullptr;
         ctx->cart_ctas = per_sm > 0 ? min(ctx->sm_count, CG_MAX_CTAS) : -1;
     }
     if (ctx->cart_ctas > 0 && n <= ctx->cart_ctas * CG_SHARE) {

@@ -78,6 +78,7 @@ extern "C" hs_status hs_create(hs_ctx** out, int32_t device, size_t workspace_by
     c->warps_ready = false;
     c->cart_ready = false;
     c->cart_ctas = 0;
+    c->stream_part = c->part_sms = nullptr;
     if (cudaDeviceSynchronize() != cudaSuccess) { cudaFree(p); delete c; return HS_ERR_CUDA; }
     *out = c;
     return HS_OK;

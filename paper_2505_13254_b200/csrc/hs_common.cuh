@@ -33,6 +33,8 @@ struct hs_ctx {
     bool walk_ready;    // acceptance walk kernel attributes set on this device
     bool cart_ready;    // single-CTA stratifier training: shared-memory attribute set on this device
     int cart_ctas;      // CTAs of the one-launch stratifier training that run at once (0: not asked yet, -1: none)
+    void* stream_part;  // cuStreamGetGreenCtx and cuGreenCtxGetDevResource, nullptr where the driver has none
+    void* part_sms;
     bool warps_ready;   // warp kernel of the entropy pass: shared-memory attribute set on this device
     bool quant_ready;   // cluster kernel of the entropy pass: shared-memory attribute set on this device
 };
