@@ -383,8 +383,8 @@ __global__ void __maxnreg__(BF16 ? 72 : 64) quantify_cluster_kernel(const __grid
     if (parts > 1) {
         cluster_wait();                                          // (the arrival above: every CTA of the cluster runs)
         if (part != 0) {
-            // this part goes into slot `part` of the first CTA of the row's cluster
-            if (p.prefetch) pdl_wait();
+            // this part goes into slot `part` of the first CTA of the row's cluster (shared memory alone: the kernel ahead is not waited for, or
+            // the first CTA's bounded wait would count its time too; that CTA waits for it, and the grid is not complete without)
             const unsigned int bar = cluster_map_addr(smem_u32(&s_merge), 0);
             if (lane < HS_MAX_TOPK / 2) {
                 const unsigned long long a = s_top[2 * lane], b = s_top[2 * lane + 1];
