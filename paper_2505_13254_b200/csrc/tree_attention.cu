@@ -19,13 +19,13 @@
 // Launches of more than one wave of such CTAs, and long prefixes, may go to tree_attn_duo.cuh, where two CTAs share an SM (see duo_splits).
 #include <math_constants.h>
 
+#include "attn_choice.h"
 #include "hs_common.cuh"
 #include "hs_layout.h"
 #include "hs_ptx.cuh"
 
 #define ATT_BM 128
 #define ATT_BN 64
-#define ATT_MAX_SPLIT 8
 #define ATT_TILE_BYTES (ATT_BN * HS_HEAD_DIM * 2)   // 16 KiB: one K or V tile
 #define ATT_STAGE_BYTES (2 * ATT_TILE_BYTES)
 #define ATT_Q_BYTES (ATT_BM * HS_HEAD_DIM * 2)      // 32 KiB
@@ -698,66 +698,6 @@ static bool make_row_map(hs_ctx* ctx, CUtensorMap* tm, const void* base, size_t 
     return encode(ctx, tm, 2, base, gdim, gstr, box);
 }
 
-// KV splits (= cluster size) of tree_attn_umma_kernel: the number with the least time on the critical path, waves of CTAs (as many
-// clusters of that size as the device runs at once) times {tiles per CTA, what lies around them, merge}, in half tiles.  A tile is
-// 0.55 us; start, tree tiles and output 6.5 us, the merge of splits 2.5 us.  (The start was counted as the tree's two tiles, as if
-// a further wave cost nothing else.)  us a call, splits then : now, equal lengths | lengths spread over 0.2 .. 1 of the longest:
-//   one tree, 32 / 8 heads, 256 tokens 8.7 : 7.7, 320 9.0 : 8.2, of 32 / 32 heads 384 10.9 : 9.2; two trees, 32 / 32, 512 12.4 : 10.4
-//   80 blocks, 2048 tokens 29.9 : 23.3 | 25.4 : 18.9;  96 blocks, 4096 51 .. 56 : 39 .. 41 | 43 : 34, 8192 71 .. 83 : 68 .. 76 | 57 .. 71 : 58 .. 75
-// More blocks than SMs: their waves fill up, and with lengths that differ short blocks run beside a long one, where splits of it
-// only add starts and merges.  No splits up to 128 tiles:
-//   160 blocks, 2048 tokens 54 : 47 | 43 .. 52 : 24, 4096 91 : 80 | 68 .. 78 : 36 .. 44, 8192 138 : 145 | 112 : 75 (16384 226 : 295 | 156 : 135)
-//   192 blocks, 2048 56 : 48 | 44 .. 49 : 25 .. 34, 4096 86 : 82 | 58 : 42; 320 blocks, 4096 142 : 126 | 103 : 78
-static int choose_splits(int base_ctas, int sm_count, int prefix_tiles, const int* cluster_cap) {
-    if (base_ctas > sm_count && prefix_tiles <= 128) return 1;
-    int best = 1;
-    long best_cost = 0;
-    for (int s = 1; s <= ATT_MAX_SPLIT; ++s) {
-        if (s > 1 && s > prefix_tiles) break;
-        const long ctas = (long)base_ctas * s;
-        const long cap = cluster_cap[s] > 0 ? cluster_cap[s] : sm_count;
-        const long waves = (ctas + cap - 1) / cap;
-        const long cost = waves * (2 * ((prefix_tiles + s - 1) / s) + 24 + (s > 1 ? 9 : 0));
-        if (s == 1 || cost < best_cost) { best_cost = cost; best = s; }
-    }
-    return best;
-}
-
-// Splits with which tree_attn_duo_kernel takes a launch, 0: tree_attn_umma_kernel takes it.
-// What is known is the number of query blocks (an upper bound: small trees leave blocks empty) and the longest prefix; how the other
-// lengths lie below it the host cannot tell (the cache arrays may be larger than what is in use), so every line is drawn for equal
-// lengths and for lengths spread over 0.2 .. 1 of the longest together.  The other kernel pays for whole waves of CTAs, each with 6.5 us
-// around its tiles that nothing overlaps, but one CTA of it is through its tiles in half the time, which decides where the lengths
-// differ.  us a call, back to back, other kernel : this one, equal lengths | spread (30 .. 40 nodes of one block, 60 of two):
-//     blocks     512 tokens     1024                          2048                          4096
-//     160        22.5 : 16.0    29.5 : 23.5 | 18.9 : 23.6     47 : 39 | 23 : 35             80 : 70 | 36 : 56
-//     192        21.8 : 16.0    29.8 : 24.1 | 20.1 : 22.0     48 : 41 | 25 .. 34 : 37       82 : 73 | 42 : 61
-//     256        24.7 : 18.9    32.6 : 27.7 | 22.3 : 22.3     51 : 47 | 36 : 39             89 : 86 | 56 : 66
-//     320        34.6 : 31.7    46.3 : 48.1 | 34.3 : 27.9     73 : 79 | 46 : 40             126 : 143 | 78 : 79
-//     384        35.0 : 31.9    47.8 : 48.4 | 37.8 : 38.3     76 : 85 | 54 : 58             135 : 162 | 84 : 91
-//     512        48.8 : 36.2    64.4 : 55.2 | 48.3 : 40.0     101 : 94 | 75 : 70            188 : 153 | 148 : 104
-//     1024       103 : 79       114 : 97 | 97 : 80            168 : 164 | 135 : 119         302 : 299 | 224 : 211
-//   - a second wave of at most a sixth: up to 8 tiles; else up to 16 tiles; above three waves at any length; up to 32 tiles where the last of
-//     two or three waves is at least a quarter empty and more than a sixth full.
-//   At most one block per SM: only two splits let CTAs share SMs, which pays from 448 tiles and three quarters of the SMs on.
-//     128 blocks, 32768 tokens 306 : 302 | 251 : 291, 24576 234 : 232 | 106 : 129, 16384 136 : 151 | 104 : 128.
-// Two CTAs on an SM is what runs (128 blocks of 129 tiles take 104 us alone, 256 blocks 146), also in pairs; cudaOccupancyMaxActiveClusters
-// counts one, as it does for any kernel that allocates tensor memory (it does not know how many columns), so it is not asked.
-static int duo_splits(int base_ctas, int sm_count, int prefix_tiles) {
-    if (base_ctas <= sm_count) return 4 * base_ctas > 3 * sm_count && prefix_tiles >= 448 ? 2 : 0;
-    if (6 * base_ctas <= 7 * sm_count) return prefix_tiles <= 8 ? 1 : 0;
-    const int waves = (base_ctas + sm_count - 1) / sm_count;
-    return prefix_tiles <= 16 || (prefix_tiles <= 32 && 4 * base_ctas <= 3 * waves * sm_count) || waves > 3 ? 1 : 0;
-}
-
-// Launches that tree_attn_duo_kernel takes about as long for and rounds a little less (FOLLOW makes up for it): second or third waves that are at least a
-// quarter empty, and most of one wave with long prefixes.
-static bool wants_follow(int base_ctas, int sm_count, int prefix_tiles) {
-    if (base_ctas <= sm_count) return 4 * base_ctas > 3 * sm_count && prefix_tiles >= 256;
-    const int waves = (base_ctas + sm_count - 1) / sm_count;
-    return prefix_tiles <= 64 ? 4 * base_ctas <= 3 * waves * sm_count : prefix_tiles <= 128 && 6 * base_ctas <= 7 * sm_count;
-}
-
 template <typename Kernel>
 static void query_cluster_caps(Kernel kernel, int threads, size_t smem, int sm_count, int* cap) {
     for (int sz = 1; sz <= ATT_MAX_SPLIT; ++sz) {
@@ -819,8 +759,8 @@ hs_status hs_launch_attention(hs_ctx* ctx, const hs_pruned_tree* pruned, const h
     memset(&tmV, 0, sizeof(tmV));
     const int mblocks = (rows + ATT_BM - 1) / ATT_BM;
     const int prefix_tiles = (d->max_kv_len + ATT_BN - 1) / ATT_BN;
-    const int duo = duo_splits(pairs * mblocks, ctx->sm_count, prefix_tiles);
-    p.nsplit = duo ? duo : choose_splits(pairs * mblocks, ctx->sm_count, prefix_tiles, cap_umma);
+    const AttnChoice how = attn_choice(pairs * mblocks, mblocks, ctx->sm_count, prefix_tiles, cap_umma);
+    p.nsplit = how.splits;
     if (d->kv_total > 0) {
         if (!make_kv_map(ctx, &tmK, k_cache, d, p.head_first) || !make_kv_map(ctx, &tmV, v_cache, d, p.head_first))
             return HS_ERR_CUDA;
@@ -833,11 +773,11 @@ hs_status hs_launch_attention(hs_ctx* ctx, const hs_pruned_tree* pruned, const h
     const size_t w = (size_t)d->hkv * HS_HEAD_DIM;
     CUtensorMap tmQ, tmKT, tmVT;
     if (!make_row_map(ctx, &tmKT, k_tree, n, w) || !make_row_map(ctx, &tmVT, v_tree, n, w)) return HS_ERR_CUDA;
-    if (duo) {
+    if (how.duo) {
         if (!make_row_map(ctx, &tmQ, q, n * d->hq, HS_HEAD_DIM)) return HS_ERR_CUDA;
         e = hs_launch(tree_attn_duo_kernel, grid, dim3(AD_THREADS), AD_SMEM_BYTES, stream, ctx->pdl, cl, p, tmK, tmV, tmQ, tmKT, tmVT);
     } else {
-        const auto kernel = wants_follow(pairs * mblocks, ctx->sm_count, prefix_tiles) ? tree_attn_umma_kernel<true> : tree_attn_umma_kernel<false>;
+        const auto kernel = how.follow ? tree_attn_umma_kernel<true> : tree_attn_umma_kernel<false>;
         e = hs_launch(kernel, grid, dim3(UM_THREADS), UM_SMEM_BYTES, stream, ctx->pdl, cl, p, tmK, tmV, tmKT, tmVT);
     }
     return e == cudaSuccess ? HS_OK : HS_ERR_CUDA;

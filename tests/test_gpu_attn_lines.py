@@ -15,7 +15,8 @@ pytestmark = pytest.mark.gpu
     (40, 32, 32, [512, 0, 1, 65, 300]), (40, 32, 32, [513, 0, 1, 65, 300]),          # 160 blocks of one each: two CTAs per SM, one
     (40, 32, 32, [2048, 5, 1024, 64, 1999, 640]), (40, 32, 32, [2049, 5, 1024, 64, 1999, 640]),    # 192 blocks, 32 and 33 tiles
     (16, 32, 32, [1024 - 64 * b for b in range(8)]), (16, 32, 32, [1025 - 64 * b for b in range(8)]),    # 256 blocks, 16 and 17
-    (62, 64, 8, [28608, 1, 640, 0]), (62, 64, 8, [28609, 1, 640, 0]),     # 128 blocks, 447 and 448 tiles
+    (62, 64, 8, [16320, 1, 640, 0]), (62, 64, 8, [16321, 1, 640, 0]),     # 128 blocks, 255 and 256 tiles
+    (62, 64, 8, [28609, 1, 640, 0]),                                      #   448 tiles
 ])
 def test_both_sides_of_a_line(nodes, hq, hkv, lens):
     choice.test_room_in_the_cache_does_not_matter(nodes, hq, hkv, lens)

@@ -5,6 +5,7 @@ import math
 import pytest
 import torch
 
+from attn_route import route
 from paper_2505_13254_b200 import binding as hb
 
 pytestmark = pytest.mark.gpu
@@ -57,6 +58,7 @@ def error(out, x, batch, nodes, kv):
 
 def test_a_split_prefix_rounds_the_output_once():
     batch, nodes, kv = 4, 62, 16384                              # four query blocks x 32 (sequence, head) pairs, two splits
+    assert route(batch, nodes, 64, 8, kv) == 2
     x = inputs(batch, nodes, 64, 8, kv, 5)
     got = error(attend(x, 0, batch, nodes, kv), x, batch, nodes, kv)
     assert got < 1.02 * math.sqrt(2) * ROUNDING, got             # (a third rounding: sqrt(3))
