@@ -63,10 +63,13 @@ inline int duo_splits(int base_ctas, int mblocks, int sm_count, int prefix_tiles
     return prefix_tiles <= 16 || (prefix_tiles <= 32 && 4 * base_ctas <= 3 * waves * sm_count) || waves > 3 ? 1 : 0;
 }
 
-// Launches that tree_attn_duo_kernel takes about as long for and rounds a little less (FOLLOW makes up for it): second or third waves that are at least a
-// quarter empty, and one query block per head in most of one wave with long prefixes.
-inline bool wants_follow(int base_ctas, int sm_count, int prefix_tiles) {
-    if (base_ctas <= sm_count) return 4 * base_ctas > 3 * sm_count && prefix_tiles >= 256;
+// Launches that tree_attn_duo_kernel takes as long for or longer, and rounds a little less (FOLLOW makes up for it): second or third waves that are at least
+// a quarter empty, with several query blocks per head.  FOLLOW has its price where two waves of equal lengths follow one another: 10 trees of 60
+// nodes, 32 / 8 heads, plain : FOLLOW : tree_attn_duo_kernel's better choice, equal | spread: 2048 tokens 42 : 44 : 55 | 24 : 23 : 42, 4096 71 : 77 : 76 | 43 : 44 :
+// 53, 8192 132 : 147 : 144 | 82 : 82 : 85.  One query block per head was never that kernel's: plain (5 trees of 40 nodes, 32 / 32 heads,
+// FOLLOW 4096 tokens 82.9 : 80.3 | 43.8 : 42.0, 8192 160 : 150 | 83 : 82).
+inline bool wants_follow(int base_ctas, int mblocks, int sm_count, int prefix_tiles) {
+    if (mblocks == 1 || base_ctas <= sm_count) return false;
     const int waves = (base_ctas + sm_count - 1) / sm_count;
     return prefix_tiles <= 64 ? 4 * base_ctas <= 3 * waves * sm_count : prefix_tiles <= 128 && 6 * base_ctas <= 7 * sm_count;
 }
@@ -80,5 +83,5 @@ struct AttnChoice {
 inline AttnChoice attn_choice(int blocks, int mblocks, int sm_count, int prefix_tiles, const int* cluster_cap) {
     const int duo = duo_splits(blocks, mblocks, sm_count, prefix_tiles);
     if (duo) return {true, false, duo};
-    return {false, wants_follow(blocks, sm_count, prefix_tiles), choose_splits(blocks, sm_count, prefix_tiles, cluster_cap)};
+    return {false, wants_follow(blocks, mblocks, sm_count, prefix_tiles), choose_splits(blocks, sm_count, prefix_tiles, cluster_cap)};
 }

@@ -118,10 +118,10 @@ __device__ __forceinline__ void prefix_range(int L, int nsplit, int split, int& 
 #define UM_RECV_BYTES (ATT_PB_STRIDE * (ATT_BM + 2 * ATT_MAX_SPLIT))     // partials pushed by the splits of the cluster
 #define UM_SMEM_BYTES (UM_STAGES * ATT_STAGE_BYTES + ATT_Q_BYTES + UM_MAP_BYTES + 1024 + 2048 + UM_WT_BYTES + UM_RECV_BYTES + 1024)
 
-// FOLLOW: the exponents' reference follows every new row maximum over the second tile of each stream too (over the first four on long ranges): a score that was its row's maximum
-// when its tile was taken has P = 2^0, which bf16 holds without error, and those are the weights that count most.  2-norm relative error
-// against fp64, 10 x 60 nodes, 32 / 8 heads, 4096 tokens: 2.3345e-3, FOLLOW 2.3273e-3 (tree_attn_duo_kernel 2.3329e-3), for half a microsecond
-// a call (one more rescale of O).
+// FOLLOW: the exponents' reference follows every new row maximum over the second tile of each stream too (over the first four on long ranges): a score that was its
+// row's maximum when its tile was taken has P = 2^0, which bf16 holds without error, and those are the weights that count most.  2-norm relative
+// error against fp64, 10 x 60 nodes, 32 / 8 heads, plain, FOLLOW, tree_attn_duo_kernel: 1500 tokens 2.325e-3, 2.309e-3, 2.322e-3; 4096 tokens 2.3345e-3,
+// 2.3195e-3, 2.3329e-3; 8192 tokens 2.339e-3, 2.332e-3, 2.334e-3.  Which launches take it, and what it costs: see wants_follow.
 template <bool FOLLOW>
 __global__ void __launch_bounds__(UM_THREADS, 1)
 tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap tmK,
