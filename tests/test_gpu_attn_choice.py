@@ -1,28 +1,30 @@
 """Which attention kernel takes a launch follows from what the caller states (blocks, longest prefix), not from the size of the cache
-arrays: a cache with room to spare gives the same bits.  Shapes on both sides of the lines, prefixes of very different lengths with
-two splits among them (a split may then have nothing of a short prefix)."""
+arrays: a cache with room to spare gives the same bits.  Shapes on both sides of the lines (`kernel`: which one takes the launch, see
+attn_route), prefixes of very different lengths with two splits among them (a split may then have nothing of a short prefix)."""
 import math
 
 import pytest
 import torch
 
+from attn_route import route
 from paper_2505_13254_b200 import binding as hb
 
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("nodes,hq,hkv,lens", [
-    (60, 32, 8, [2048 - 103 * b for b in range(16)]),                   # two full waves
-    (60, 32, 8, [2048 - 151 * b for b in range(10)]),                   # a last wave that is nearly empty
-    (60, 32, 8, [1024 - 61 * b for b in range(16)]),                    # 16 tiles
-    (60, 32, 8, [1025 - 61 * b for b in range(16)]),                    # 17
-    (60, 32, 8, [6000 - 601 * b for b in range(10)]),                   # the same, longer: two splits
-    (62, 64, 8, [16400, 0, 64, 9000]),                                  # two splits, some of them empty
-    (62, 64, 8, [16320, 16300, 1, 8000]),                               # one tile less: one split of the other kernel or more
-    (62, 64, 8, [300 + 17 * b for b in range(20)]),                     # more than three waves
+@pytest.mark.parametrize("nodes,hq,hkv,lens,kernel", [
+    (60, 32, 8, [2048 - 103 * b for b in range(16)], 0),                   # two full waves
+    (60, 32, 8, [2048 - 151 * b for b in range(10)], -1),                  # a last wave that is nearly empty
+    (60, 32, 8, [1024 - 61 * b for b in range(16)], 1),                    # 16 tiles
+    (60, 32, 8, [1025 - 61 * b for b in range(16)], 0),                    # 17
+    (60, 32, 8, [6000 - 601 * b for b in range(10)], -1),               # a last wave that is nearly empty, longer
+    (62, 64, 8, [16400, 0, 64, 9000], 2),                               # two splits, some of them empty
+    (62, 64, 8, [16320, 16300, 1, 8000], 0),                            # one tile less: the other kernel, one split or more
+    (62, 64, 8, [300 + 17 * b for b in range(20)], 1),                  # more than three waves
 ])
-def test_room_in_the_cache_does_not_matter(nodes, hq, hkv, lens):
+def test_room_in_the_cache_does_not_matter(nodes, hq, hkv, lens, kernel):
     B, G = len(lens), hq // hkv
+    assert route(B, nodes, hq, hkv, max(lens)) == kernel
     g = torch.Generator(device="cuda").manual_seed(sum(lens))
     i32 = lambda a: torch.tensor(a, dtype=torch.int32, device="cuda")
     tree = hb.TreeBatch(i32([b * nodes for b in range(B + 1)]), i32(list(range(-1, nodes - 1)) * B), i32([0] * (B * nodes)), B, B * nodes)

@@ -68,6 +68,7 @@ def test_a_split_prefix_rounds_the_output_once():
 @pytest.mark.parametrize("kv", [256, 640, 1000])
 def test_one_stream_per_row_is_as_exact_as_two(kv):
     batch, nodes = 24, 60                                        # 384 query blocks at once, 128 at a time
+    assert route(batch, nodes, 32, 8, kv) == 1 and route(8, nodes, 32, 8, kv) == 0
     x = inputs(batch, nodes, 32, 8, kv, kv)
     one = error(attend(x, 0, batch, nodes, kv), x, batch, nodes, kv)
     two = error(torch.cat([attend(x, b, b + 8, nodes, kv) for b in range(0, batch, 8)]), x, batch, nodes, kv)

@@ -1,25 +1,31 @@
 """Tree attention in launches of more query blocks than SMs, and of fewer with long prefixes, where two CTAs share an SM: prefixes around the edges of a key tile and
 none at all, trees of 1 to 128 nodes (one or two tree tiles, dead query blocks), grouped heads that do not divide a block, split
-prefixes, both row layouts and both cache layouts; against fp32 attention."""
+prefixes, both row layouts and both cache layouts; against fp32 attention.  (`kernel`: see attn_route; the launches of the other kernel's instance
+that stands for this one are among them.)"""
 import math
 import random
 
 import pytest
 import torch
 
+from attn_route import route
 from paper_2505_13254_b200 import binding as hb
 
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("batch,nodes,hq,hkv,kv,layout,head_first,prefetch", [
-    (40, (1, 128), 32, 8, [0, 1, 63, 64, 65, 127, 128, 129, 191, 192, 193, 320], hb.HS_ROWS_COMPACT, False, True),
-    (40, (30, 128), 21, 3, [0, 7, 64, 200, 700], hb.HS_ROWS_ORIGINAL, True, False),
-    (12, (60, 128), 64, 4, [2500, 64, 3000, 1], hb.HS_ROWS_COMPACT, True, True),
-    (10, (40, 60), 32, 8, [4096, 4097, 130], hb.HS_ROWS_ORIGINAL, False, True),
-    (4, (50, 62), 64, 8, [16500, 70, 0, 12000], hb.HS_ROWS_ORIGINAL, False, False),
+@pytest.mark.parametrize("batch,nodes,hq,hkv,kv,layout,head_first,prefetch,kernel", [
+    (40, (1, 128), 32, 8, [0, 1, 63, 64, 65, 127, 128, 129, 191, 192, 193, 320], hb.HS_ROWS_COMPACT, False, True, 1),
+    (40, (30, 128), 21, 3, [0, 7, 64, 200, 700], hb.HS_ROWS_ORIGINAL, True, False, 1),
+    (12, (60, 128), 64, 4, [2500, 64, 3000, 1], hb.HS_ROWS_COMPACT, True, True, 1),
+    (10, (40, 60), 32, 8, [4096, 4097, 130], hb.HS_ROWS_ORIGINAL, False, True, -1),
+    (10, (40, 60), 32, 8, [1500, 1, 640], hb.HS_ROWS_COMPACT, True, False, -1),
+    (10, (40, 60), 32, 8, [512, 449, 130], hb.HS_ROWS_ORIGINAL, False, True, 1),
+    (4, (50, 62), 64, 8, [16500, 70, 0, 12000], hb.HS_ROWS_ORIGINAL, False, False, 2),
+    (4, (50, 62), 64, 8, [100, 16385, 8200, 64], hb.HS_ROWS_COMPACT, True, True, 2),
+    (8, (33, 60), 32, 8, [16400, 8256, 63, 16321], hb.HS_ROWS_ORIGINAL, True, True, 2),
 ])
-def test_two_ctas_per_sm(batch, nodes, hq, hkv, kv, layout, head_first, prefetch):
+def test_two_ctas_per_sm(batch, nodes, hq, hkv, kv, layout, head_first, prefetch, kernel):
     rng = random.Random(batch + hq)
     g = torch.Generator(device="cuda").manual_seed(hq)
     i32 = lambda a: torch.tensor(a, dtype=torch.int32, device="cuda")
@@ -29,6 +35,7 @@ def test_two_ctas_per_sm(batch, nodes, hq, hkv, kv, layout, head_first, prefetch
         off.append(off[-1] + n)
         kvo.append(kvo[-1] + kv[b % len(kv)])
         parent += [-1] + [rng.randint(max(0, i - 12), i - 1) for i in range(1, n)]
+    assert route(batch, max(ns), hq, hkv, max(kv)) == kernel
     N, T, G = off[-1], kvo[-1], hq // hkv
     tree = hb.TreeBatch(i32(off), i32(parent), i32([rng.randrange(64) for _ in range(N)]), batch, N)
     policy = dict(thresholds=[-1e9] * 7, d_base=100, alpha=4, n_default=128, top_k=10, gamma_pct=[30, 60, 100], phi_mode=0, pstar_mode=0,
