@@ -107,3 +107,34 @@ def test_a_wait_that_runs_out_is_the_status_and_leaves_nothing_behind(n):
     assert int(status) == 0 and np.array_equal(th.cpu().numpy(), sums_fit(x, y, 3).astype(np.float32))
     assert hb.hs_device_error(ctx) == hb.HS_ERR_TIMEOUT and hb.hs_device_error(ctx) == 0
     ctx.close()
+
+
+def test_two_trainings_and_decode_steps_on_streams_of_their_own():
+    """Every CTA of a training holds an SM and waits for the others: what else is resident may only delay it."""
+    rng = np.random.default_rng(5)
+    jobs = []
+    for n in (60000, SMS * 2000):
+        x = feature("positive", n, rng)
+        y = np.clip(np.round(3.0 * x + rng.normal(0, 3, n)), 0, 59).astype(np.float32)
+        ctx = hb.Context(0, hb.hs_cart_workspace_bytes(n))
+        jobs.append((ctx, torch.from_numpy(x).cuda(), torch.from_numpy(y).cuda(), torch.cuda.Stream(), sums_fit(x, y, 3).astype(np.float32)))
+    i32 = lambda a: torch.tensor(a, dtype=torch.int32, device="cuda")
+    tree = hb.TreeBatch(i32([0, 60]), i32([-1] + [0] * 59), i32([0] * 60), 1, 60)
+    policy = dict(thresholds=[1.0] * 7, d_base=8, alpha=4, n_default=60, top_k=10, gamma_pct=[30, 60, 100], phi_mode=0, pstar_mode=0, entropy_mode=0)
+    logits = torch.randn(60, 128256, device="cuda", dtype=torch.bfloat16)
+    step = hb.Context(0, hb.hs_workspace_bytes(1, 60, 128256, 32, 8))
+    want, _ = hb.hs_entropy_quantify_prune(step, tree, logits, policy)
+    torch.cuda.synchronize()
+    got = []
+    for _ in range(30):
+        for ctx, x, y, stream, thresholds in jobs:
+            with torch.cuda.stream(stream):
+                got.append((hb.hs_cart_fit(ctx, x, y, 3), thresholds))
+        quant, _ = hb.hs_entropy_quantify_prune(step, tree, logits, policy)
+    torch.cuda.synchronize()
+    for (th, status), thresholds in got:
+        assert int(status) == 0 and np.array_equal(th.cpu().numpy(), thresholds)
+    assert torch.equal(quant.topk_idx, want.topk_idx) and torch.equal(quant.h_full, want.h_full)
+    for ctx in [step] + [j[0] for j in jobs]:
+        assert hb.hs_device_error(ctx) == 0
+        ctx.close()

@@ -1,5 +1,5 @@
-"""Stratifier training at the sizes where its kernels change: one CTA up to 8192 samples, tiles of 4096 keys beyond, the
-last tile full, nearly empty and short by one; features with heavy ties and with a single value per layer."""
+"""Stratifier training at the sizes where its kernels change: one CTA up to 8192 samples, a resident grid beyond (the same sizes through
+the launches of one pass each: test_gpu_cart_partition); features with heavy ties and with a single value per layer."""
 import numpy as np
 import pytest
 import torch
