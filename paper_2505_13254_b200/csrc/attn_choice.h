@@ -11,7 +11,7 @@
 //   80 blocks, 2048 tokens 29.9 : 23.3 | 25.4 : 18.9;  96 blocks, 4096 51 .. 56 : 39 .. 41 | 43 : 34, 8192 71 .. 83 : 68 .. 76 | 57 .. 71 : 58 .. 75
 // More blocks than SMs: their waves fill up, and with lengths that differ short blocks run beside a long one, where splits of it
 // only add starts and merges.  No splits up to 128 tiles:
-//   160 blocks, 2048 tokens 54 : 47 | 43 .. 52 : 24, 4096 91 : 80 | 68 .. 78 : 36 .. 44, 8192 138 : 145 | 112 : 75 (16384 226 : 295 | 156 : 135)
+//   160 blocks, 2048 tokens 55 : 44 | 44 : 23, 4096 85 : 77 | 53 : 44, 8192 144 : 147 | 85 : 82 (16384 226 : 295 | 156 : 135)
 //   192 blocks, 2048 56 : 48 | 44 .. 49 : 25 .. 34, 4096 86 : 82 | 58 : 42; 320 blocks, 4096 142 : 126 | 103 : 78
 inline int choose_splits(int base_ctas, int sm_count, int prefix_tiles, const int* cluster_cap) {
     if (base_ctas > sm_count && prefix_tiles <= 128) return 1;

@@ -14,7 +14,7 @@
 // and 0.9 ms on 2^20 samples (every exchange distance beyond shared memory is a pass over all keys); a pass here reads and
 // writes the keys once, which stay in L2.
 //   up to CT_SMALL samples   cart_small_kernel: one CTA sorts in shared memory and fits all layers - one launch, no round
-//                            trips between layers (15 us at 600 samples, 38 us at 8192; the grid kernel 40 at 8193).
+//                            trips between layers (15 us at 600 samples, 38 us at 8192; the grid kernel 41 at 8193).
 //   up to 8192 per SM        cart_grid_kernel (cart_grid.cuh): the same by a resident grid, one launch.
 //   more                     cart_pack_kernel (keys, digit counts of all passes), four cart_radix_kernel, cart_sums_kernel
 //                            (sums per block and their scan), one cart_level_kernel per layer (what a grid can hold takes it 1.6 times as
@@ -118,6 +118,8 @@ __device__ __forceinline__ bool warp_best(bool in, unsigned long long l, int pos
 // The block's best split of every node -> s.top (smallest N L, then smallest position).  A thread has `cnt` consecutive keys, key(j) =
 // sorted key at position i0 + j (j = -1: the one ahead of it); (a, b): running sums of y and y^2 ahead of them.  One sweep: the thread keeps
 // its best split with the sums and the feature values there (three sweeps, for N L, its position and the sums, took 2.5 times as long).
+// (The right side's sums are the node's less the left's.  Against rational arithmetic, of 7500 nodes of near-equal targets that are no whole
+// numbers 9 or 13 take another split, by which product is fused; 14 or 18 with the right side taken from its end, 24 so without fused products.)
 template <class KeyFn>
 __device__ __forceinline__ void layer_block(LayerSmem& s, int nodes, int i0, int cnt, double a, double b, KeyFn key) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;

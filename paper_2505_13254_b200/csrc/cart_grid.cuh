@@ -6,14 +6,14 @@
 // values differ (their order bits less the smallest: passes of up to ten bits, three for up to 30 such bits, else four of eight).  A pass
 // ranks and counts the digits of every share and brings the share into their order in shared memory, the counts of all shares become
 // offsets (up to 32 shares: every CTA adds up the others' itself; more: 32 digits to a CTA and one barrier more), and the shares write their
-// keys, equal digits together: two or three grid barriers of 1.2 us.  The share of the sorted order that a CTA then holds stays in its
+// keys, equal digits together: two grid barriers, or three, of 1.2 us.  The share of the sorted order that a CTA then holds stays in its
 // shared memory for all layers; a layer costs one barrier, behind which every CTA works out the same new boundaries from the
 // shares' best splits.
 //
 // Why: nine launches (pack, four look-back passes, sums, three layers) took 70 us at any size above one CTA's and 125 us at 2^20 samples:
-// their starts, the look-back chains and the reloads, not the work.  Now 40 us at 8193 samples, 45 at 20000, 52 at 200000, 76 at 2^20 and depth
-// 3: there 21 us ranking (ten ballots a key), 11 us fp64 sums of the layers, 17 us in 15 barriers.  Two CTAs of 512 threads per SM: 92 us
-// (twice the entries and counts to read for every CTA).
+// their starts, the look-back chains and the reloads, not the work.  Now 41 us at 8193 samples, 43 at 20000, 54 at 200000, 76 at 2^20 and depth
+// 3: there 21 us ranking (ten ballots a key), 11 us fp64 sums of the layers, 17 us in 14 barriers (one for the range, three a pass, one for
+// the sums, one a layer).  Two CTAs of 512 threads per SM: 92 us (twice the entries and counts to read for every CTA).
 #pragma once
 
 #define CG_THREADS 1024

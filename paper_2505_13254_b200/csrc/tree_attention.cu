@@ -381,8 +381,8 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     // The single-thread roles sit behind a branch on a warp-uniform value; all lanes run the loop and wait, and elect.sync chooses the
     // thread only for the instructions that one thread issues: the compiler then keeps loop counters, addresses and descriptors uniform.
     // (The issuing warps are what a tile waits for - with almost no arithmetic left in the softmax warps a tile took as long.  With the waits
-    // inside the elected branch: 4 calls of 4 trees, 64 / 8 heads, 4900 tokens 188 us, now 168; 32 calls of one tree, 32 / 8 heads, 2048
-    // tokens 382, now 368; 12 trees, 32 / 32 heads, 600 - 1200 tokens 180, now 175.)
+    // inside the elected branch, timed in turn: 4 calls of 4 trees, 64 / 8 heads, 4470 - 4975 tokens 215 us, now 203; 32 calls of one tree,
+    // 32 / 8 heads, 2048 tokens 380, now 366.)
     const int warp_u = __shfl_sync(HS_FULL_MASK, warp, 0);
     if (warp_u == 8) {
         // The P V issuer: O += P V of tile i as soon as its P is written.  It is short work on the streams' critical
