@@ -342,6 +342,7 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     auto issue_qk = [&](int i) {
         const int stage = i % UM_STAGES;
         if (i < np || i >= UM_STAGES) mbar_wait(bar0 + stage * 8, (unsigned int)(i / UM_STAGES) & 1u, p.err);
+        if (i >= 2) mbar_wait(bar_sr + (i & 1) * 8, (unsigned int)((i - 2) >> 1) & 1u, p.err);      // S of tile i - 2 is read
         __syncwarp();
         tc_fence_after_sync();
         if (!elect_one()) return;
@@ -402,7 +403,6 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         __syncwarp();
 #pragma unroll 1
         for (int i = 0; i + 2 < ntiles; ++i) {
-            mbar_wait(bar_sr + (i & 1) * 8, (unsigned int)(i >> 1) & 1u, p.err);      // S of tile i is read
             issue_qk(i + 2);
             __syncwarp();
         }
@@ -434,11 +434,19 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     // Stream `half`: tiles half, half + 2, ...  As soon as S of tile i is in registers its buffer is handed back.  The
     // stream's P buffer and O were last used by O += P V of tile i - 2, which is waited for before they are touched
     // (its barrier's next completion is tile i + 2's, which needs this stream's P of tile i + 2).
+    // What bounds a tile is the chain of a stream: 128 clocks for S, 140 for the maximum, 640 for the exponentials (530 with both streams at them), 30 for P,
+    // and 123 for each answer of a barrier that is long complete.  So both barriers are asked ahead of other work and the answer is looked at
+    // behind it, and the S issuer waits for K first: the slowest CTA of a launch, whose two streams are in step, takes 780 clocks a tile instead of
+    // 910.  Us a call, timed in turn: 4 x 16300 tokens, 60 nodes, 64 / 8 heads 140 -> 133, 4 x 4700 46.3 -> 44.2, 16 trees, 32 / 8 heads, 4096 tokens
+    // 78.2 -> 77.4, 14 trees of 30 nodes, 24576 tokens 201 -> 187; one tree of 2048 tokens 10.8 both ways.  (S of the next tile loaded ahead of P's store: 148
+    // for the first; Q as the A operand from tensor memory: 141; the streams' exponentials in turns: 142 .. 150.)
+    unsigned int sr[64];                                     // the row's 64 scores
+    bool ok_s = false;                                       // S of the stream's next tile was complete when last asked
 #pragma unroll 1
     for (int i = half; i < ntiles && warp < 8; i += 2) {
-        mbar_wait(bar_s + half * 8, (unsigned int)(i >> 1) & 1u, p.err);         // S of tile i is complete
+        if (!ok_s) mbar_wait(bar_s + half * 8, (unsigned int)(i >> 1) & 1u, p.err);      // S of tile i is complete
+        __syncwarp();
         tc_fence_after_sync();
-        unsigned int sr[64];                                 // the row's 64 scores
         tmem_ld32(tS + half * ATT_BN + lane_off, sr);
         tmem_ld32(tS + half * ATT_BN + 32 + lane_off, sr + 32);
         tmem_wait_ld();
@@ -450,7 +458,6 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         const int nvis = (is_tree ? nk : L) - col0;          // columns of this tile inside the sequence / tree
         // The scores stay unscaled in registers (the scale is positive: it commutes with the maximum and folds into
         // the exponent's multiply-add). A prefix tile inside the sequence needs no mask at all.
-        float mxa = -CUDART_INF_F, mxb = -CUDART_INF_F;
         if (is_tree || nvis < ATT_BN) {
             // a tree tile of 64 keys lies inside one 64-bit word of the ancestor mask
             unsigned long long vis64 = nvis >= 64 ? ~0ull : ((1ull << max(nvis, 0)) - 1ull);
@@ -462,12 +469,14 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
                 if (!((vhi >> c) & 1u)) sr[32 + c] = __float_as_uint(-CUDART_INF_F);
             }
         }
+        float m4[4];                                         // three-input maxima: half the instructions
 #pragma unroll
-        for (int c = 0; c < 32; c += 2) {                    // three-input maxima: half the instructions
-            mxa = max3(mxa, __uint_as_float(sr[c]), __uint_as_float(sr[c + 1]));
-            mxb = max3(mxb, __uint_as_float(sr[32 + c]), __uint_as_float(sr[33 + c]));
+        for (int q = 0; q < 4; ++q) {
+            m4[q] = fmaxf(__uint_as_float(sr[q * 16]), __uint_as_float(sr[q * 16 + 1]));
+#pragma unroll
+            for (int c = 2; c < 16; c += 2) m4[q] = max3(m4[q], __uint_as_float(sr[q * 16 + c]), __uint_as_float(sr[q * 16 + c + 1]));
         }
-        const float mx = fmaxf(mxa, mxb) * p.scale_log2;
+        const float mx = fmaxf(max3(m4[0], m4[1], m4[2]), m4[3]) * p.scale_log2;
         // The reference the exponents are taken against only follows the row's maximum when that has grown by more
         // than 8 (a factor 256): until then P <= 256 instead of <= 1, which costs no precision (fp32 sums, bf16 keeps
         // its relative error, the final O / l is the same quotient), and O is rescaled a few times per row instead of
@@ -481,39 +490,47 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         const float2 sc2 = make_float2(p.scale_log2, p.scale_log2), nm2 = make_float2(-muse, -muse);
         float2 ls0 = make_float2(0.f, 0.f), ls1 = make_float2(0.f, 0.f);
         uint4 pk[8];
+        float2 pv[2][4];                                     // packed one group behind: no instruction waits for the exponential ahead of it
+        bool ok_o = false;                                   // O += P V of tile i - 2 is complete
 #pragma unroll
-        for (int c8 = 0; c8 < 8; ++c8) {
-            float2 pv[4];
+        for (int c8 = 0; c8 <= 8; ++c8) {
+            if (c8 == 4) ok_o = mbar_test_wait(bar_ev + ((i + 2) & (UM_STAGES - 1)) * 8, (unsigned int)((i + 2) / UM_STAGES - 1) & 1u);
+            if (c8 < 8) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float2 x = fma2_ftz(make_float2(__uint_as_float(sr[c8 * 8 + 2 * e]), __uint_as_float(sr[c8 * 8 + 2 * e + 1])), sc2, nm2);
-                pv[e] = make_float2(ex2_approx(x.x), ex2_approx(x.y));
+                for (int e = 0; e < 4; ++e) {
+                    const float2 x = fma2_ftz(make_float2(__uint_as_float(sr[c8 * 8 + 2 * e]), __uint_as_float(sr[c8 * 8 + 2 * e + 1])), sc2, nm2);
+                    pv[c8 & 1][e] = make_float2(ex2_approx(x.x), ex2_approx(x.y));
+                }
             }
-            ls0 = add2_ftz(ls0, add2_ftz(pv[0], pv[1]));
-            ls1 = add2_ftz(ls1, add2_ftz(pv[2], pv[3]));
-            pk[c8].x = pack_bf16(pv[0].x, pv[0].y); pk[c8].y = pack_bf16(pv[1].x, pv[1].y);
-            pk[c8].z = pack_bf16(pv[2].x, pv[2].y); pk[c8].w = pack_bf16(pv[3].x, pv[3].y);
+            if (c8 > 0) {
+                const float2* v = pv[(c8 - 1) & 1];
+                ls0 = add2_ftz(ls0, add2_ftz(v[0], v[1]));
+                ls1 = add2_ftz(ls1, add2_ftz(v[2], v[3]));
+                pk[c8 - 1].x = pack_bf16(v[0].x, v[0].y); pk[c8 - 1].y = pack_bf16(v[1].x, v[1].y);
+                pk[c8 - 1].z = pack_bf16(v[2].x, v[2].y); pk[c8 - 1].w = pack_bf16(v[3].x, v[3].y);
+            }
         }
         const float2 ls = add2_ftz(ls0, ls1);
         lrun = fmaf(lrun, corr, ls.x + ls.y);
         if (i >= 2) {
-            mbar_wait(bar_ev + ((i - 2) % UM_STAGES) * 8, (unsigned int)((i - 2) / UM_STAGES) & 1u, p.err);
+            if (!ok_o) mbar_wait(bar_ev + ((i - 2) % UM_STAGES) * 8, (unsigned int)((i - 2) / UM_STAGES) & 1u, p.err);
+            __syncwarp();
             tc_fence_after_sync();
         }
         // rescale this stream's O (the load/store are warp-wide: a warp rescales if any of its rows needs it)
         if (i >= 2 && __any_sync(HS_FULL_MASK, corr != 1.f)) {
 #pragma unroll 1
-            for (int ch = 0; ch < 4; ++ch) {
-                unsigned int ov[32];
-                tmem_ld32(tO + half * HS_HEAD_DIM + lane_off + ch * 32, ov);
+            for (int ch = 0; ch < 8; ++ch) {
+                unsigned int ov[16];
+                tmem_ld16(tO + half * HS_HEAD_DIM + lane_off + ch * 16, ov);
                 tmem_wait_ld();
 #pragma unroll
-                for (int c = 0; c < 32; ++c) ov[c] = __float_as_uint(__uint_as_float(ov[c]) * corr);
-                tmem_st32(tO + half * HS_HEAD_DIM + lane_off + ch * 32, ov);
+                for (int c = 0; c < 16; ++c) ov[c] = __float_as_uint(__uint_as_float(ov[c]) * corr);
+                tmem_st16(tO + half * HS_HEAD_DIM + lane_off + ch * 16, ov);
             }
-            tmem_wait_st();
         }
         // P stays in tensor memory (the A operand of O += P V): this row's 64 bf16 values are 32 columns of its lane
+        ok_s = mbar_test_wait(bar_s + half * 8, (unsigned int)((i + 2) >> 1) & 1u);
         tmem_st32(tP + half * (ATT_BN / 2) + lane_off, reinterpret_cast<unsigned int*>(pk));
         tmem_wait_st();
         tc_fence_before_sync();
