@@ -51,7 +51,9 @@ inline int choose_splits(int base_ctas, int sm_count, int prefix_tiles, const in
 //     7 x 60, 32 / 8             111 : 110 | 107 : 107 145 : 142 | 142 : 139 210 : 201 | 210 : 203 239 : 227 | 245 : 232 281 : 264 | 287 : 271
 //     9 x 60, 32 / 8             116 : 116 | 113 : 113 153 : 150 | 154 : 151 225 : 216 | 232 : 224 264 : 253 | 289 : 276 296 : 280 | 306 : 286
 //     4 x 60, 64 / 8, <true>                           147 : 146 | 141 : 141 216 : 208 | 209 : 207 243 : 234 | 249 : 239
-//       <false> (2.342e-3 from fp64, this one 2.337e-3)  139       | 135       205       | 200       233       | 241
+//       <false> (2.342e-3 from fp64, this one 2.337e-3)  133       | 134       199       | 208       233       | 241
+//   (The other kernel's times but the last line's first two are from before its barriers were asked ahead, which took 3 to 7 % off them.  The lines stay: what goes
+//   to this kernel by them would come back less exact.)
 //     14 x 30, 32 / 8                                  145 : 146 | 141 : 145 213 : 210 | 223 : 216 238 : 239 | 264 : 252 276 : 278 | 296 : 286
 //     18 x 30, 32 / 8                                  154 : 163 | 153 : 165 231 : 240 | 249 : 257 265 : 274 | 289 : 292 314 : 320 | 339 : 332
 // Two CTAs on an SM is what runs (128 blocks of 129 tiles take 104 us alone, 256 blocks 146), also in pairs; cudaOccupancyMaxActiveClusters

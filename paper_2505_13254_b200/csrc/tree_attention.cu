@@ -112,8 +112,15 @@ __device__ __forceinline__ void prefix_range(int L, int nsplit, int split, int& 
 #define UM_ROWS_THREADS 128
 #define UM_SM_THREADS 256                            // softmax threads: row = tid & 127, stream = tid >> 7
 #define UM_MAP_BYTES 1024                            // output-row map of the rows a CTA merges (<= 65 rows x 8 bytes)
-#define UM_TMEM_COLS 512                             // S of stream g: columns 64 g ..; O: 128 + 128 g ..; P (bf16 pairs): 384 + 32 g ..
+#define UM_TMEM_COLS 512                             // S of stream g: columns 64 g ..; O: 128 + 128 g ..; P (bf16 pairs): 384 + 32 g ..; Q: 448 ..
 #define UM_STAGES 4
+// CTAs of more than UM_Q_TMEM tiles take Q as the A operand from tensor memory (columns 448 ..) from tile UM_Q_FIRST on.  With 64 columns of S the product reads Q
+// from shared memory for longer than it multiplies: 387 clocks a tile instead of 258, 623 instead of 515 with P V.  Us a call, always from shared memory : so,
+// timed in turn: 4 trees of 60 nodes, 64 / 8 heads, 4700 tokens 43.8 : 42.9, 16300 tokens 131 : 124; 10 trees, 32 / 8 heads, up to 4096 tokens 40.5 : 38.7.  From the
+// third tile on instead of the ninth 44.3, 140; with the operand chosen per loop and not per instruction 45.2, 138: the issue of an S that leaves
+// P V room between its instructions is part of the gain.  Shorter CTAs lose by it: 17 tiles 15.0 : 16.1, one tree, 2048 tokens 11.2 : 11.7, if it is taken from 9 tiles on.
+#define UM_Q_TMEM 24
+#define UM_Q_FIRST 8
 #define UM_WT_BYTES (66 * ATT_MAX_SPLIT * 4 + 64)    // split weights of the rows a CTA merges
 #define UM_RECV_BYTES (ATT_PB_STRIDE * (ATT_BM + 2 * ATT_MAX_SPLIT))     // partials pushed by the splits of the cluster
 #define UM_SMEM_BYTES (UM_STAGES * ATT_STAGE_BYTES + ATT_Q_BYTES + UM_MAP_BYTES + 1024 + 2048 + UM_WT_BYTES + UM_RECV_BYTES + 1024)
@@ -122,7 +129,8 @@ __device__ __forceinline__ void prefix_range(int L, int nsplit, int split, int& 
 // row's maximum when its tile was taken has P = 2^0, which bf16 holds without error, and those are the weights that count most.  2-norm relative
 // error against fp64, 10 x 60 nodes, 32 / 8 heads, plain, FOLLOW, tree_attn_duo_kernel: 1500 tokens 2.325e-3, 2.309e-3, 2.322e-3; 4096 tokens 2.3345e-3,
 // 2.3195e-3, 2.3329e-3; 8192 tokens 2.339e-3, 2.332e-3, 2.334e-3.  Which launches take it, and what it costs: see wants_follow.
-template <bool FOLLOW>
+// QT: Q from tensor memory in CTAs of many tiles (launches that have none run an instance without that code: 0.4 us less in a step of the smallest model).
+template <bool FOLLOW, bool QT>
 __global__ void __launch_bounds__(UM_THREADS, 1)
 tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap tmK,
                       const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmKT,
@@ -231,7 +239,7 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     const unsigned int tmem_base = *tslot_gen;
     const unsigned int lane_off = (unsigned int)((warp & 3) * 32) << 16;   // a warp reaches lanes 32 * (warp % 4) ...
     const int row = tid & (ATT_BM - 1), half = (tid >> 7) & 1;               // the thread's query row and stream
-    const unsigned int tS = tmem_base, tO = tmem_base + 128, tP = tmem_base + 384;   // (+ 64 / + 128 / + 32 columns for stream 1)
+    const unsigned int tS = tmem_base, tO = tmem_base + 128, tP = tmem_base + 384, tQ = tmem_base + 448;   // (+ 64 / + 128 / + 32 columns for stream 1)
 
     const int nk = st_b == 0 ? nk_b : 0;
     const int M = nk * p.G;
@@ -339,7 +347,7 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     const unsigned long long dq0 = umma_desc_sw128(sQ, 16, 1024), dk0 = umma_desc_sw128(smem_base, 16, 1024);
     const unsigned long long dv0 = umma_desc_sw128(smem_base + ATT_TILE_BYTES, ATT_TILE_BYTES / 2, 1024);
     // the issuing warp: S = Q K^T of tile i into S buffer i & 1 (waits for K unless load_tree wrote it), then commit
-    auto issue_qk = [&](int i) {
+    auto issue_qk = [&](int i, auto from_tmem) {
         const int stage = i % UM_STAGES;
         if (i < np || i >= UM_STAGES) mbar_wait(bar0 + stage * 8, (unsigned int)(i / UM_STAGES) & 1u, p.err);
         if (i >= 2) mbar_wait(bar_sr + (i & 1) * 8, (unsigned int)((i - 2) >> 1) & 1u, p.err);      // S of tile i - 2 is read
@@ -352,7 +360,8 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         for (int ks = 0; ks < 8; ++ks) {
             const unsigned int koffb = (ks >> 2) * (ATT_TILE_BYTES / 2) + (ks & 3) * 32;
             const unsigned int qoffb = (ks >> 2) * (ATT_Q_BYTES / 2) + (ks & 3) * 32;
-            umma_ss_bf16(ts, dq0 + (qoffb >> 4), dk + (koffb >> 4), idesc_qk, ks > 0 ? 1u : 0u);
+            if (from_tmem(i)) umma_ts_bf16(ts, tQ + ks * 8, dk + (koffb >> 4), idesc_qk, ks > 0 ? 1u : 0u);
+            else umma_ss_bf16(ts, dq0 + (qoffb >> 4), dk + (koffb >> 4), idesc_qk, ks > 0 ? 1u : 0u);
         }
         umma_commit(bar_s + (i & 1) * 8);
         if (i + UM_STAGES < ntiles) umma_commit(bar_ek + stage * 8);     // (the producer waits for it only then)
@@ -397,14 +406,24 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     } else if (warp_u == 10) {
         // The S issuer: S of tile i + 2 as soon as the stream has S of tile i in registers, so a stream never waits
         // for its next S.
-        if (ntiles > 0) issue_qk(0);
-        __syncwarp();
-        if (ntiles > 1) issue_qk(1);
-        __syncwarp();
-#pragma unroll 1
-        for (int i = 0; i + 2 < ntiles; ++i) {
-            issue_qk(i + 2);
+        auto ss = [](int) { return false; };                 // (from shared memory)
+        if (!QT || ntiles <= UM_Q_TMEM) {
+            if (ntiles > 0) issue_qk(0, ss);
             __syncwarp();
+            if (ntiles > 1) issue_qk(1, ss);
+            __syncwarp();
+#pragma unroll 1
+            for (int i = 2; i < ntiles; ++i) {
+                issue_qk(i, ss);
+                __syncwarp();
+            }
+        } else {
+#pragma unroll 1
+            for (int i = 0; i < ntiles; ++i) {
+                if (i == UM_Q_FIRST) { named_bar_sync(3, UM_SM_THREADS + 32); tc_fence_after_sync(); }
+                issue_qk(i, [](int t) { return t >= UM_Q_FIRST; });
+                __syncwarp();
+            }
         }
     } else if (warp_u == 9) {
         // The TMA producer, in the order in which the tensor pipe frees the stage halves: S runs four tiles ahead
@@ -437,15 +456,24 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     // What bounds a tile is the chain of a stream: 128 clocks for S, 140 for the maximum, 640 for the exponentials (530 with both streams at them), 30 for P,
     // and 123 for each answer of a barrier that is long complete.  So both barriers are asked ahead of other work and the answer is looked at
     // behind it, and the S issuer waits for K first: the slowest CTA of a launch, whose two streams are in step, takes 780 clocks a tile instead of
-    // 910.  Us a call, timed in turn: 4 x 16300 tokens, 60 nodes, 64 / 8 heads 140 -> 133, 4 x 4700 46.3 -> 44.2, 16 trees, 32 / 8 heads, 4096 tokens
-    // 78.2 -> 77.4, 14 trees of 30 nodes, 24576 tokens 201 -> 187; one tree of 2048 tokens 10.8 both ways.  (S of the next tile loaded ahead of P's store: 148
-    // for the first; Q as the A operand from tensor memory: 141; the streams' exponentials in turns: 142 .. 150.)
+    // 910.  Us a call, timed in turn: 4 x 16300 tokens, 60 nodes, 64 / 8 heads 141 -> 131, 4 x 4700 46.5 -> 43.8, 16 trees, 32 / 8 heads, 4096 tokens
+    // 79.3 -> 78.4, 14 trees of 30 nodes, 24576 tokens 198 -> 191; one tree of 2048 tokens 10.7 both ways.  (S of the next tile loaded ahead of P's store: 148
+    // for the first; the streams' exponentials in turns: 142 .. 150.  Packing a group behind the exponentials: the same here, and 0.4 us in a step of the
+    // smallest model.)
     unsigned int sr[64];                                     // the row's 64 scores
+    if (QT && warp < 8 && ntiles > UM_Q_TMEM) {                    // Q into tensor memory while the first S are computed: half a row per thread
+        uint4 qq[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) qq[c] = *reinterpret_cast<const uint4*>(gQ + q_off(row, half * 8 + c));
+        tmem_st32(tQ + half * 32 + lane_off, reinterpret_cast<unsigned int*>(qq));
+        tmem_wait_st();
+        tc_fence_before_sync();
+        asm volatile("bar.arrive 3, %0;" ::"r"(UM_SM_THREADS + 32) : "memory");
+    }
     bool ok_s = false;                                       // S of the stream's next tile was complete when last asked
 #pragma unroll 1
     for (int i = half; i < ntiles && warp < 8; i += 2) {
         if (!ok_s) mbar_wait(bar_s + half * 8, (unsigned int)(i >> 1) & 1u, p.err);      // S of tile i is complete
-        __syncwarp();
         tc_fence_after_sync();
         tmem_ld32(tS + half * ATT_BN + lane_off, sr);
         tmem_ld32(tS + half * ATT_BN + 32 + lane_off, sr + 32);
@@ -469,14 +497,13 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
                 if (!((vhi >> c) & 1u)) sr[32 + c] = __float_as_uint(-CUDART_INF_F);
             }
         }
-        float m4[4];                                         // three-input maxima: half the instructions
+        float mxa = -CUDART_INF_F, mxb = -CUDART_INF_F;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            m4[q] = fmaxf(__uint_as_float(sr[q * 16]), __uint_as_float(sr[q * 16 + 1]));
-#pragma unroll
-            for (int c = 2; c < 16; c += 2) m4[q] = max3(m4[q], __uint_as_float(sr[q * 16 + c]), __uint_as_float(sr[q * 16 + c + 1]));
+        for (int c = 0; c < 32; c += 2) {                    // three-input maxima: half the instructions
+            mxa = max3(mxa, __uint_as_float(sr[c]), __uint_as_float(sr[c + 1]));
+            mxb = max3(mxb, __uint_as_float(sr[32 + c]), __uint_as_float(sr[33 + c]));
         }
-        const float mx = fmaxf(max3(m4[0], m4[1], m4[2]), m4[3]) * p.scale_log2;
+        const float mx = fmaxf(mxa, mxb) * p.scale_log2;
         // The reference the exponents are taken against only follows the row's maximum when that has grown by more
         // than 8 (a factor 256): until then P <= 256 instead of <= 1, which costs no precision (fp32 sums, bf16 keeps
         // its relative error, the final O / l is the same quotient), and O is rescaled a few times per row instead of
@@ -490,31 +517,25 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         const float2 sc2 = make_float2(p.scale_log2, p.scale_log2), nm2 = make_float2(-muse, -muse);
         float2 ls0 = make_float2(0.f, 0.f), ls1 = make_float2(0.f, 0.f);
         uint4 pk[8];
-        float2 pv[2][4];                                     // packed one group behind: no instruction waits for the exponential ahead of it
         bool ok_o = false;                                   // O += P V of tile i - 2 is complete
 #pragma unroll
-        for (int c8 = 0; c8 <= 8; ++c8) {
+        for (int c8 = 0; c8 < 8; ++c8) {
             if (c8 == 4) ok_o = mbar_test_wait(bar_ev + ((i + 2) & (UM_STAGES - 1)) * 8, (unsigned int)((i + 2) / UM_STAGES - 1) & 1u);
-            if (c8 < 8) {
+            float2 pv[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float2 x = fma2_ftz(make_float2(__uint_as_float(sr[c8 * 8 + 2 * e]), __uint_as_float(sr[c8 * 8 + 2 * e + 1])), sc2, nm2);
-                    pv[c8 & 1][e] = make_float2(ex2_approx(x.x), ex2_approx(x.y));
-                }
+            for (int e = 0; e < 4; ++e) {
+                const float2 x = fma2_ftz(make_float2(__uint_as_float(sr[c8 * 8 + 2 * e]), __uint_as_float(sr[c8 * 8 + 2 * e + 1])), sc2, nm2);
+                pv[e] = make_float2(ex2_approx(x.x), ex2_approx(x.y));
             }
-            if (c8 > 0) {
-                const float2* v = pv[(c8 - 1) & 1];
-                ls0 = add2_ftz(ls0, add2_ftz(v[0], v[1]));
-                ls1 = add2_ftz(ls1, add2_ftz(v[2], v[3]));
-                pk[c8 - 1].x = pack_bf16(v[0].x, v[0].y); pk[c8 - 1].y = pack_bf16(v[1].x, v[1].y);
-                pk[c8 - 1].z = pack_bf16(v[2].x, v[2].y); pk[c8 - 1].w = pack_bf16(v[3].x, v[3].y);
-            }
+            ls0 = add2_ftz(ls0, add2_ftz(pv[0], pv[1]));
+            ls1 = add2_ftz(ls1, add2_ftz(pv[2], pv[3]));
+            pk[c8].x = pack_bf16(pv[0].x, pv[0].y); pk[c8].y = pack_bf16(pv[1].x, pv[1].y);
+            pk[c8].z = pack_bf16(pv[2].x, pv[2].y); pk[c8].w = pack_bf16(pv[3].x, pv[3].y);
         }
         const float2 ls = add2_ftz(ls0, ls1);
         lrun = fmaf(lrun, corr, ls.x + ls.y);
         if (i >= 2) {
             if (!ok_o) mbar_wait(bar_ev + ((i - 2) % UM_STAGES) * 8, (unsigned int)((i - 2) / UM_STAGES) & 1u, p.err);
-            __syncwarp();
             tc_fence_after_sync();
         }
         // rescale this stream's O (the load/store are warp-wide: a warp rescales if any of its rows needs it)
@@ -738,12 +759,12 @@ hs_status hs_launch_attention(hs_ctx* ctx, const hs_pruned_tree* pruned, const h
                               void* out, float* lse_out, cudaStream_t stream) {
     int* cap_umma = ctx->attn_cap;                   // CTAs that run at once in clusters of s (per device = per context)
     if (!ctx->attn_ready) {
-        if (cudaFuncSetAttribute(tree_attn_umma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, UM_SMEM_BYTES) != cudaSuccess ||
-            cudaFuncSetAttribute(tree_attn_umma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, UM_SMEM_BYTES) != cudaSuccess)
-            return HS_ERR_CUDA;
+        for (const auto kernel : {tree_attn_umma_kernel<false, false>, tree_attn_umma_kernel<false, true>, tree_attn_umma_kernel<true, false>,
+                                  tree_attn_umma_kernel<true, true>})
+            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, UM_SMEM_BYTES) != cudaSuccess) return HS_ERR_CUDA;
         if (cudaFuncSetAttribute(tree_attn_duo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AD_SMEM_BYTES) != cudaSuccess)
             return HS_ERR_CUDA;
-        query_cluster_caps(tree_attn_umma_kernel<false>, UM_THREADS, UM_SMEM_BYTES, ctx->sm_count, cap_umma);
+        query_cluster_caps(tree_attn_umma_kernel<false, false>, UM_THREADS, UM_SMEM_BYTES, ctx->sm_count, cap_umma);
         ctx->attn_ready = true;
     }
     AttnParams p;
@@ -794,7 +815,10 @@ hs_status hs_launch_attention(hs_ctx* ctx, const hs_pruned_tree* pruned, const h
         if (!make_row_map(ctx, &tmQ, q, n * d->hq, HS_HEAD_DIM)) return HS_ERR_CUDA;
         e = hs_launch(tree_attn_duo_kernel, grid, dim3(AD_THREADS), AD_SMEM_BYTES, stream, ctx->pdl, cl, p, tmK, tmV, tmQ, tmKT, tmVT);
     } else {
-        const auto kernel = how.follow ? tree_attn_umma_kernel<true> : tree_attn_umma_kernel<false>;
+        // most tiles of a CTA: its share of the longest prefix and the tree's
+        const bool qt = (prefix_tiles + p.nsplit - 1) / p.nsplit + (d->max_nodes + ATT_BN - 1) / ATT_BN > UM_Q_TMEM;
+        const auto kernel = how.follow ? (qt ? tree_attn_umma_kernel<true, true> : tree_attn_umma_kernel<true, false>)
+                                       : (qt ? tree_attn_umma_kernel<false, true> : tree_attn_umma_kernel<false, false>);
         e = hs_launch(kernel, grid, dim3(UM_THREADS), UM_SMEM_BYTES, stream, ctx->pdl, cl, p, tmK, tmV, tmKT, tmVT);
     }
     return e == cudaSuccess ? HS_OK : HS_ERR_CUDA;
