@@ -129,7 +129,7 @@ __device__ __forceinline__ void prefix_range(int L, int nsplit, int split, int& 
 // row's maximum when its tile was taken has P = 2^0, which bf16 holds without error, and those are the weights that count most.  2-norm relative
 // error against fp64, 10 x 60 nodes, 32 / 8 heads, plain, FOLLOW, tree_attn_duo_kernel: 1500 tokens 2.325e-3, 2.309e-3, 2.322e-3; 4096 tokens 2.3345e-3,
 // 2.3195e-3, 2.3329e-3; 8192 tokens 2.339e-3, 2.332e-3, 2.334e-3.  Which launches take it, and what it costs: see wants_follow.
-// QT: Q from tensor memory in CTAs of many tiles (launches that have none run an instance without that code: 0.4 us less in a step of the smallest model).
+// QT: Q from tensor memory in CTAs of many tiles; launches that have none run an instance without that code.
 template <bool FOLLOW, bool QT>
 __global__ void __launch_bounds__(UM_THREADS, 1)
 tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap tmK,
@@ -458,8 +458,7 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     // behind it, and the S issuer waits for K first: the slowest CTA of a launch, whose two streams are in step, takes 780 clocks a tile instead of
     // 910.  Us a call, timed in turn: 4 x 16300 tokens, 60 nodes, 64 / 8 heads 141 -> 131, 4 x 4700 46.5 -> 43.8, 16 trees, 32 / 8 heads, 4096 tokens
     // 79.3 -> 78.4, 14 trees of 30 nodes, 24576 tokens 198 -> 191; one tree of 2048 tokens 10.7 both ways.  (S of the next tile loaded ahead of P's store: 148
-    // for the first; the streams' exponentials in turns: 142 .. 150.  Packing a group behind the exponentials: the same here, and 0.4 us in a step of the
-    // smallest model.)
+    // for the first; the streams' exponentials in turns: 142 .. 150.)
     unsigned int sr[64];                                     // the row's 64 scores
     if (QT && warp < 8 && ntiles > UM_Q_TMEM) {                    // Q into tensor memory while the first S are computed: half a row per thread
         uint4 qq[8];
