@@ -473,6 +473,7 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
 #pragma unroll 1
     for (int i = half; i < ntiles && warp < 8; i += 2) {
         if (!ok_s) mbar_wait(bar_s + half * 8, (unsigned int)(i >> 1) & 1u, p.err);      // S of tile i is complete
+        __syncwarp();                                        // (each lane has waited by its own answer; warp-aligned loads follow)
         tc_fence_after_sync();
         tmem_ld32(tS + half * ATT_BN + lane_off, sr);
         tmem_ld32(tS + half * ATT_BN + 32 + lane_off, sr + 32);
@@ -537,7 +538,8 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
             if (!ok_o) mbar_wait(bar_ev + ((i - 2) % UM_STAGES) * 8, (unsigned int)((i - 2) / UM_STAGES) & 1u, p.err);
             tc_fence_after_sync();
         }
-        // rescale this stream's O (the load/store are warp-wide: a warp rescales if any of its rows needs it)
+        // rescale this stream's O (the load/store are warp-wide: a warp rescales if any of its rows needs it; the vote is where its lanes
+        // meet again - a __syncwarp ahead of it as well makes 4 trees of 60 nodes, 64 / 8 heads, 4700 tokens 47.8 us instead of 43.0)
         if (i >= 2 && __any_sync(HS_FULL_MASK, corr != 1.f)) {
 #pragma unroll 1
             for (int ch = 0; ch < 8; ++ch) {

@@ -24,3 +24,12 @@ def test_tensor_memory_is_freed_behind_a_fenced_barrier(name):
     last = text(name).rindex("tmem_dealloc(")
     tail = re.sub(r"\s+", "", text(name)[:last])
     assert re.search(r"tc_fence_before_sync\(\);__syncthreads\(\);tc_fence_after_sync\(\);if\(warp==\w+\)$", tail)
+
+
+def test_lanes_that_waited_alone_meet_again_ahead_of_tensor_memory():
+    # `if (!ok) mbar_wait(...)`: a lane waits by its own answer, and tcgen05.ld / st (.sync.aligned) need all lanes of the warp
+    body = text("tree_attention.cu")
+    waits = [m.end() for m in re.finditer(r"if \(!ok_\w+\) mbar_wait\(", body)]
+    assert len(waits) == 2
+    for at in waits:
+        assert re.search(r"\btmem_\w+\(|__syncwarp\(\)|__any_sync\(HS_FULL_MASK", body[at:]).group(0).startswith("__")
