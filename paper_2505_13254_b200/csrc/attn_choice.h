@@ -87,3 +87,21 @@ inline AttnChoice attn_choice(int blocks, int mblocks, int sm_count, int prefix_
     if (duo) return {true, false, duo};
     return {false, wants_follow(blocks, mblocks, sm_count, prefix_tiles), choose_splits(blocks, sm_count, prefix_tiles, cluster_cap)};
 }
+
+// Does a launch of tree_attn_umma_kernel have CTAs that take Q as the A operand from tensor memory: those of more than ATT_Q_TILES tiles?
+// With 64 columns of S the product reads Q from shared memory for longer than it multiplies (387 clocks a tile instead of 258, 623 instead of 515 with P V), but the copy
+// of Q and the slower issue are paid for first, and where the tiles are not what a launch waits for nothing comes back.  us a call, from shared memory : so,
+// equal lengths | mean of three draws of spread ones; tokens for each split, i.e. 27, 32, 36, 41, 64, 128 tiles in a CTA and the tree's:
+//     trees x nodes, heads     1700                      2000                      2300                      2600                      4096                      8192
+//     4 x 60, 64 / 8           20.1 : 20.3 | 20.2 : 20.2 22.4 : 22.3 | 22.7 : 22.0 24.4 : 23.8 | 24.5 : 23.9 27.2 : 26.1 | 26.9 : 25.4 37.1 : 35.5 | 37.8 : 34.7 66.9 : 64.1 | 63.0 : 60.3
+//     7 x 60, 32 / 8           20.1 : 20.2 | 19.4 : 19.5 22.2 : 22.3 | 22.0 : 21.6 24.4 : 24.6 | 23.9 : 23.2 25.7 : 26.3 | 26.1 : 25.3 38.7 : 36.2 | 35.3 : 35.0 69.5 : 63.9 | 65.2 : 60.2
+//     4 x 60, 32 / 8, 2 splits 22.0 : 23.1 | 22.5 : 21.9 24.1 : 24.8 | 24.6 : 23.5 27.4 : 27.2 | 26.8 : 25.5 30.2 : 29.3 | 29.7 : 27.6 41.8 : 39.1 | 41.3 : 37.6 76.1 : 70.0 | 72.5 : 62.7
+//     2 x 60, 32 / 8, 4 splits 21.2 : 22.5 | 21.4 : 21.1 23.7 : 23.9 | 24.0 : 23.0 27.2 : 26.9 | 26.7 : 25.7 29.1 : 28.6 | 28.4 : 26.5 41.1 : 38.7 | 40.8 : 36.7 76.0 : 69.9 | 73.2 : 64.0
+// Not in more than one wave (16 x 60, 32 / 8, 1700 tokens 41.5 : 44.0 | 33.3 : 33.7, 4096 77.2 : 77.4 | 50.1 : 51.9; 10 x 60 1700 37.4 : 40.8 | 23.0 : 23.0, 12000 in splits 156 :
+// 162 | 114 : 118; 8 x 60, 64 / 8, 4096 72.5 : 74.8 | 60.4 : 62.9) but for FOLLOW's above 64 tiles (10 x 60, 8192 124 : 127 | 73.5 : 69.9), and not with one query
+// block per head, where K and V come from DRAM (10 x 30, 32 / 8, 8192 66.5 : 68.7 | 49.3 : 50.4; 4 x 60, 32 / 32, 1700 23.1 : 24.2 | 21.0 : 21.2).
+#define ATT_Q_TILES 31
+inline bool q_from_tensor_memory(int blocks, int mblocks, int sm_count, int prefix_tiles, int tree_tiles, const AttnChoice& c) {
+    if (c.duo || mblocks == 1 || (prefix_tiles + c.splits - 1) / c.splits + tree_tiles <= ATT_Q_TILES) return false;
+    return c.follow ? prefix_tiles > 64 : blocks * c.splits <= sm_count;
+}

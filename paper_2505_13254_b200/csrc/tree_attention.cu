@@ -47,6 +47,7 @@ struct AttnParams {
     const int* node_off;
     const int* kv_off;
     int batch, hq, hkv, G, layout, nsplit, head_first, prefetch;
+    int follow;               // of the instance that takes Q from tensor memory: FOLLOW at run time
     unsigned int inv_g;       // ceil(2^16 / G): r / G = r * inv_g >> 16 for the row numbers r < 2^11
     float scale_log2;
     int* err;
@@ -114,13 +115,11 @@ __device__ __forceinline__ void prefix_range(int L, int nsplit, int split, int& 
 #define UM_MAP_BYTES 1024                            // output-row map of the rows a CTA merges (<= 65 rows x 8 bytes)
 #define UM_TMEM_COLS 512                             // S of stream g: columns 64 g ..; O: 128 + 128 g ..; P (bf16 pairs): 384 + 32 g ..; Q: 448 ..
 #define UM_STAGES 4
-// CTAs of more than UM_Q_TMEM tiles take Q as the A operand from tensor memory (columns 448 ..) from tile UM_Q_FIRST on.  With 64 columns of S the product reads Q
-// from shared memory for longer than it multiplies: 387 clocks a tile instead of 258, 623 instead of 515 with P V.  Us a call, always from shared memory : so,
-// timed in turn: 4 trees of 60 nodes, 64 / 8 heads, 4700 tokens 43.8 : 42.9, 16300 tokens 131 : 124; 10 trees, 32 / 8 heads, up to 4096 tokens 40.5 : 38.7.  From the
-// third tile on instead of the ninth 44.3, 140; with the operand chosen per loop and not per instruction 45.2, 138: the issue of an S that leaves
-// P V room between its instructions is part of the gain.  Shorter CTAs lose by it: 17 tiles 15.0 : 16.1, one tree, 2048 tokens 11.2 : 11.7, if it is taken from 9 tiles on.
-#define UM_Q_TMEM 24
+// CTAs of more than ATT_Q_TILES tiles may take Q as the A operand from tensor memory (columns 448 ..) from tile UM_Q_FIRST on: see q_from_tensor_memory.
+// From the third tile on instead of the ninth 4 trees of 60 nodes, 64 / 8 heads take 44.3 us for 42.9 at 4700 tokens, 140 for 124 at 16300; with the operand chosen per
+// loop and not per instruction 45.2, 138: the issue of an S that leaves P V room between its instructions is part of the gain.
 #define UM_Q_FIRST 8
+static_assert(UM_Q_FIRST <= ATT_Q_TILES, "a CTA that takes Q from tensor memory reaches the tile that waits for it");
 #define UM_WT_BYTES (66 * ATT_MAX_SPLIT * 4 + 64)    // split weights of the rows a CTA merges
 #define UM_RECV_BYTES (ATT_PB_STRIDE * (ATT_BM + 2 * ATT_MAX_SPLIT))     // partials pushed by the splits of the cluster
 #define UM_SMEM_BYTES (UM_STAGES * ATT_STAGE_BYTES + ATT_Q_BYTES + UM_MAP_BYTES + 1024 + 2048 + UM_WT_BYTES + UM_RECV_BYTES + 1024)
@@ -129,7 +128,7 @@ __device__ __forceinline__ void prefix_range(int L, int nsplit, int split, int& 
 // row's maximum when its tile was taken has P = 2^0, which bf16 holds without error, and those are the weights that count most.  2-norm relative
 // error against fp64, 10 x 60 nodes, 32 / 8 heads, plain, FOLLOW, tree_attn_duo_kernel: 1500 tokens 2.325e-3, 2.309e-3, 2.322e-3; 4096 tokens 2.3345e-3,
 // 2.3195e-3, 2.3329e-3; 8192 tokens 2.339e-3, 2.332e-3, 2.334e-3.  Which launches take it, and what it costs: see wants_follow.
-// QT: Q from tensor memory in CTAs of many tiles; launches that have none run an instance without that code.
+// QT: Q from tensor memory in CTAs of many tiles (see q_from_tensor_memory), FOLLOW at run time; other launches run an instance without that code.
 template <bool FOLLOW, bool QT>
 __global__ void __launch_bounds__(UM_THREADS, 1)
 tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap tmK,
@@ -385,7 +384,7 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         if (i == ntiles - 1) umma_commit(bar_done);
     };
     float mrun = -CUDART_INF_F, lrun = 0.f;
-    const int nfollow = ntiles > 64 ? 8 : 4;
+    const int nfollow = QT && !p.follow ? 0 : ntiles > 64 ? 8 : 4;
 
     // ---- KV tiles ------------------------------------------------------------------------------------------
     // The single-thread roles sit behind a branch on a warp-uniform value; all lanes run the loop and wait, and elect.sync chooses the
@@ -407,7 +406,7 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         // The S issuer: S of tile i + 2 as soon as the stream has S of tile i in registers, so a stream never waits
         // for its next S.
         auto ss = [](int) { return false; };                 // (from shared memory)
-        if (!QT || ntiles <= UM_Q_TMEM) {
+        if (!QT || ntiles <= ATT_Q_TILES) {
             if (ntiles > 0) issue_qk(0, ss);
             __syncwarp();
             if (ntiles > 1) issue_qk(1, ss);
@@ -460,7 +459,7 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     // 79.3 -> 78.4, 14 trees of 30 nodes, 24576 tokens 198 -> 191; one tree of 2048 tokens 10.7 both ways.  (S of the next tile loaded ahead of P's store: 148
     // for the first; the streams' exponentials in turns: 142 .. 150.)
     unsigned int sr[64];                                     // the row's 64 scores
-    if (QT && warp < 8 && ntiles > UM_Q_TMEM) {                    // Q into tensor memory while the first S are computed: half a row per thread
+    if (QT && warp < 8 && ntiles > ATT_Q_TILES) {                    // Q into tensor memory while the first S are computed: half a row per thread
         uint4 qq[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) qq[c] = *reinterpret_cast<const uint4*>(gQ + q_off(row, half * 8 + c));
@@ -760,8 +759,7 @@ hs_status hs_launch_attention(hs_ctx* ctx, const hs_pruned_tree* pruned, const h
                               void* out, float* lse_out, cudaStream_t stream) {
     int* cap_umma = ctx->attn_cap;                   // CTAs that run at once in clusters of s (per device = per context)
     if (!ctx->attn_ready) {
-        for (const auto kernel : {tree_attn_umma_kernel<false, false>, tree_attn_umma_kernel<false, true>, tree_attn_umma_kernel<true, false>,
-                                  tree_attn_umma_kernel<true, true>})
+        for (const auto kernel : {tree_attn_umma_kernel<false, false>, tree_attn_umma_kernel<true, false>, tree_attn_umma_kernel<true, true>})
             if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, UM_SMEM_BYTES) != cudaSuccess) return HS_ERR_CUDA;
         if (cudaFuncSetAttribute(tree_attn_duo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AD_SMEM_BYTES) != cudaSuccess)
             return HS_ERR_CUDA;
@@ -800,6 +798,7 @@ hs_status hs_launch_attention(hs_ctx* ctx, const hs_pruned_tree* pruned, const h
     const int prefix_tiles = (d->max_kv_len + ATT_BN - 1) / ATT_BN;
     const AttnChoice how = attn_choice(pairs * mblocks, mblocks, ctx->sm_count, prefix_tiles, cap_umma);
     p.nsplit = how.splits;
+    p.follow = how.follow;
     if (d->kv_total > 0) {
         if (!make_kv_map(ctx, &tmK, k_cache, d, p.head_first) || !make_kv_map(ctx, &tmV, v_cache, d, p.head_first))
             return HS_ERR_CUDA;
@@ -816,10 +815,9 @@ hs_status hs_launch_attention(hs_ctx* ctx, const hs_pruned_tree* pruned, const h
         if (!make_row_map(ctx, &tmQ, q, n * d->hq, HS_HEAD_DIM)) return HS_ERR_CUDA;
         e = hs_launch(tree_attn_duo_kernel, grid, dim3(AD_THREADS), AD_SMEM_BYTES, stream, ctx->pdl, cl, p, tmK, tmV, tmQ, tmKT, tmVT);
     } else {
-        // most tiles of a CTA: its share of the longest prefix and the tree's
-        const bool qt = (prefix_tiles + p.nsplit - 1) / p.nsplit + (d->max_nodes + ATT_BN - 1) / ATT_BN > UM_Q_TMEM;
-        const auto kernel = how.follow ? (qt ? tree_attn_umma_kernel<true, true> : tree_attn_umma_kernel<true, false>)
-                                       : (qt ? tree_attn_umma_kernel<false, true> : tree_attn_umma_kernel<false, false>);
+        const int tree_tiles = (d->max_nodes + ATT_BN - 1) / ATT_BN;
+        const auto kernel = q_from_tensor_memory(pairs * mblocks, mblocks, ctx->sm_count, prefix_tiles, tree_tiles, how) ? tree_attn_umma_kernel<true, true>
+                            : how.follow ? tree_attn_umma_kernel<true, false> : tree_attn_umma_kernel<false, false>;
         e = hs_launch(kernel, grid, dim3(UM_THREADS), UM_SMEM_BYTES, stream, ctx->pdl, cl, p, tmK, tmV, tmKT, tmVT);
     }
     return e == cudaSuccess ? HS_OK : HS_ERR_CUDA;

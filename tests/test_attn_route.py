@@ -1,9 +1,9 @@
-"""Which attention kernel the lines give to a launch, on the 148 SMs of the device that they are drawn for."""
+"""Which attention kernel the lines give to a launch, and where its query rows come from, on the 148 SMs of the device that they are drawn for."""
 import shutil
 
 import pytest
 
-from attn_route import route
+from attn_route import route, splits_with_q_in_tensor_memory
 
 
 @pytest.mark.skipif(not shutil.which("g++"), reason="no host compiler")
@@ -16,3 +16,18 @@ from attn_route import route
 ])
 def test_lines(batch, nodes, hq, hkv, longest, kernel):
     assert route(batch, nodes, hq, hkv, longest, 148) == kernel
+
+
+@pytest.mark.skipif(not shutil.which("g++"), reason="no host compiler")
+@pytest.mark.parametrize("batch, nodes, hq, hkv, longest, splits", [
+    (7, 60, 32, 8, 30 * 64, 0), (7, 60, 32, 8, 30 * 64 + 1, 1), (7, 60, 32, 8, 8192, 1),    # 112 blocks: from 31 prefix tiles and the tree's on
+    (4, 100, 32, 8, 29 * 64, 0), (4, 100, 32, 8, 29 * 64 + 1, 1),         # two tiles of the tree
+    (2, 60, 32, 8, 4 * 30 * 64, 0), (2, 60, 32, 8, 4 * 30 * 64 + 1, 4), (1, 60, 64, 8, 16384, 4),    # of a split's share
+    (16, 60, 32, 8, 8192, 0), (12, 60, 32, 8, 4096, 0),                   # more than one wave: not
+    (10, 60, 32, 8, 4096, 0), (10, 60, 32, 8, 4097, 1), (5, 60, 64, 8, 8192, 1), (10, 60, 32, 8, 8193, 0),    # but FOLLOW's above 64 tiles
+    (5, 60, 32, 8, 12800, 0),                                             # 80 blocks in three splits: two waves
+    (16, 30, 32, 8, 12000, 0), (2, 60, 32, 32, 8192, 0),                  # one query block per head: never
+    (4, 62, 64, 8, 16384, 0),                                             # two CTAs per SM
+])
+def test_query_operand(batch, nodes, hq, hkv, longest, splits):
+    assert splits_with_q_in_tensor_memory(batch, nodes, hq, hkv, longest, 148) == splits
