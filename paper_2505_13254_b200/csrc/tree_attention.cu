@@ -540,14 +540,18 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
         // rescale this stream's O (the load/store are warp-wide: a warp rescales if any of its rows needs it; the vote is where its lanes
         // meet again - a __syncwarp ahead of it as well makes 4 trees of 60 nodes, 64 / 8 heads, 4700 tokens 47.8 us instead of 43.0)
         if (i >= 2 && __any_sync(HS_FULL_MASK, corr != 1.f)) {
+            // in pieces of 32 columns, a round trip each, where FOLLOW may rescale often (10 trees of 60 nodes, 32 / 8 heads, spread up to 8192 tokens, pieces of 16 : so
+            // 65.7 : 62.3 us; 6000 tokens 52.8 : 50.7); the instance that serves the shortest steps rescales once or twice, and is 0.2 us shorter with 16
+            constexpr int W = QT ? 32 : 16;
 #pragma unroll 1
-            for (int ch = 0; ch < 8; ++ch) {
-                unsigned int ov[16];
-                tmem_ld16(tO + half * HS_HEAD_DIM + lane_off + ch * 16, ov);
+            for (int ch = 0; ch < HS_HEAD_DIM; ch += W) {
+                unsigned int ov[W];
+                const unsigned int at = tO + half * HS_HEAD_DIM + lane_off + ch;
+                if constexpr (QT) tmem_ld32(at, ov); else tmem_ld16(at, ov);
                 tmem_wait_ld();
 #pragma unroll
-                for (int c = 0; c < 16; ++c) ov[c] = __float_as_uint(__uint_as_float(ov[c]) * corr);
-                tmem_st16(tO + half * HS_HEAD_DIM + lane_off + ch * 16, ov);
+                for (int c = 0; c < W; ++c) ov[c] = __float_as_uint(__uint_as_float(ov[c]) * corr);
+                if constexpr (QT) tmem_st32(at, ov); else tmem_st16(at, ov);
             }
         }
         // P stays in tensor memory (the A operand of O += P V): this row's 64 bf16 values are 32 columns of its lane
