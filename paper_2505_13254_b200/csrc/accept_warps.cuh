@@ -9,8 +9,8 @@
 // such round of the warp is read once more.  Sampling sequences add sum e^((x-ref)/T) against a reference that all lanes
 // share.  Sequences that finish in the row pass (greedy, deterministic proposals) are walked at the end of the CTA that
 // merged their last target row.
-// Bound by the latencies inside a round (load, maxima, exponentials), which four warps per scheduler with one round each in
-// flight do not cover: 28 % of the issue slots, 52 % of DRAM on a batch of greedy and sampling rows.  Behind a ring of 32 KiB
+// Bound by the rounds: 36 of 40 us on a batch of greedy and sampling rows (179 MB), read at 5.0 TB/s, 1500 clocks a round with 32 KiB of loads in flight on an SM; a row end
+// takes 2 us, the last ones of all warps at the same time (stamps of every warp).  28 % of the issue slots.  Behind a ring of 32 KiB
 // items with 16 warps in lockstep the call took (now): 497 greedy rows of 128256 bf16 30.5 us (27.6), 497 rows half sampling
 // with their draft rows and the walk 75.8 (62.6), 1127 rows of 32000, three modes, 95.4 (55.4), 120 greedy rows 14.0 (12.6).
 #pragma once

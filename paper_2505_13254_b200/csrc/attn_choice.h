@@ -5,14 +5,18 @@
 
 // KV splits (= cluster size) of tree_attn_umma_kernel: the number with the least time on the critical path, waves of CTAs (as many
 // clusters of that size as the device runs at once) times {tiles per CTA, what lies around them, merge}, in half tiles.  A tile is
-// 0.55 us; start, tree tiles and output 6.5 us, the merge of splits 2.5 us.  (The start was counted as the tree's two tiles, as if
-// a further wave cost nothing else.)  us a call, splits then : now, equal lengths | lengths spread over 0.2 .. 1 of the longest:
-//   one tree, 32 / 8 heads, 256 tokens 8.7 : 7.7, 320 9.0 : 8.2, of 32 / 32 heads 384 10.9 : 9.2; two trees, 32 / 32, 512 12.4 : 10.4
-//   80 blocks, 2048 tokens 29.9 : 23.3 | 25.4 : 18.9;  96 blocks, 4096 51 .. 56 : 39 .. 41 | 43 : 34, 8192 71 .. 83 : 68 .. 76 | 57 .. 71 : 58 .. 75
+// 0.5 us (0.38 in CTAs that take Q from tensor memory), start, tree tiles and output 6 us, the merge of splits 2.2 us.  us a call in 1 .. 6 splits, * the rule's (seven and
+// eight never fit at once: another wave), trees of 60 nodes, equal lengths:
+//     one tree, 32 / 8 heads, 256 tokens     7.6* 9.1  8.4  8.5  8.6  8.7     384       8.6  9.4  9.1  8.2  8.7  9.2*    1024      12.7 11.9 10.3 9.8  9.7  9.6*
+//                             2048           20.6 15.0 13.1 11.8 11.1 11.2*   4096      32.9 23.2 18.4 15.2 14.7 13.7*   8192      57.5 36.0 28.1 23.5 22.0 19.6*
+//     one tree, 64 / 8,       512            9.7  10.1 10.3 10.3*             2048      21.3 16.1 14.2 13.7*             8192      59.3 37.1 29.6 26.0*
+//     two trees, 32 / 32,     512            9.6* 11.4                        2048      20.9 17.3*
+//     four trees, 32 / 8,     1024           13.9 13.8*                       4096      35.6 26.9*
+//   and where splits cost a wave, equal lengths | lengths spread over 0.2 .. 1 of the longest, 1 .. 3 splits:
+//     80 blocks, 4096 tokens  38.2* 46.7 39.3 | 34.6* 29.3 33.3;  96 blocks, 8192  65.7* 74.5 82.9 | 63.6* 57.5 67.0
 // More blocks than SMs: their waves fill up, and with lengths that differ short blocks run beside a long one, where splits of it
 // only add starts and merges.  No splits up to 128 tiles:
-//   160 blocks, 2048 tokens 55 : 44 | 44 : 23, 4096 85 : 77 | 53 : 44, 8192 144 : 147 | 85 : 82 (16384 226 : 295 | 156 : 135)
-//   192 blocks, 2048 56 : 48 | 44 .. 49 : 25 .. 34, 4096 86 : 82 | 58 : 42; 320 blocks, 4096 142 : 126 | 103 : 78
+//     160 blocks, 2048 tokens 41.0* 51.6 60.7 | 23.4* 39.8 49.6;  8192  121.8* 113.6 116.1 | 76.0* 86.0 98.8;  16384, four there  231 202 200 202* | 125 105 117 124*
 inline int choose_splits(int base_ctas, int sm_count, int prefix_tiles, const int* cluster_cap) {
     if (base_ctas > sm_count && prefix_tiles <= 128) return 1;
     int best = 1;
@@ -33,29 +37,29 @@ inline int choose_splits(int base_ctas, int sm_count, int prefix_tiles, const in
 // lengths lie below it the host cannot tell (the cache arrays may be larger than what is in use), so every line is drawn for equal
 // lengths and for lengths spread over 0.2 .. 1 of the longest together.  The other kernel pays for whole waves of CTAs, each with 6.5 us
 // around its tiles that nothing overlaps, but one CTA of it is through its tiles in half the time, which decides where the lengths
-// differ.  us a call, back to back, other kernel : this one, equal lengths | spread (30 .. 40 nodes of one block, 60 of two):
-//     blocks     512 tokens     1024                          2048                          4096
-//     160        22.5 : 16.0    29.5 : 23.5 | 18.9 : 23.6     47 : 39 | 23 : 35             80 : 70 | 36 : 56
-//     192        21.8 : 16.0    29.8 : 24.1 | 20.1 : 22.0     48 : 41 | 25 .. 34 : 37       82 : 73 | 42 : 61
-//     256        24.7 : 18.9    32.6 : 27.7 | 22.3 : 22.3     51 : 47 | 36 : 39             89 : 86 | 56 : 66
-//     320        34.6 : 31.7    46.3 : 48.1 | 34.3 : 27.9     73 : 79 | 46 : 40             126 : 143 | 78 : 79
-//     384        35.0 : 31.9    47.8 : 48.4 | 37.8 : 38.3     76 : 85 | 54 : 58             135 : 162 | 84 : 91
-//     512        48.8 : 36.2    64.4 : 55.2 | 48.3 : 40.0     101 : 94 | 75 : 70            188 : 153 | 148 : 104
-//     1024       103 : 79       114 : 97 | 97 : 80            168 : 164 | 135 : 119         302 : 299 | 224 : 211
+// differ.  us a call, back to back, other kernel : this one, equal lengths | mean of three draws of spread ones (trees of 60 nodes, 32 / 8 heads):
+//     blocks     512 tokens                 1024                       2048                       4096
+//     160        20.7 : 18.6 | 16.8 : 16.4  27.4 : 26.9 | 18.6 : 22.5  41.8 : 42.7 | 25.3 : 38.9  69.2 : 72.5 | 37.1 : 65.1
+//     192        21.1 : 18.6 | 16.9 : 15.9  28.0 : 26.9 | 20.9 : 23.7  43.5 : 43.9 | 28.7 : 39.7  70.8 : 75.9 | 46.0 : 70.7
+//     256        22.1 : 19.4 | 19.2 : 18.0  30.3 : 27.7 | 23.5 : 25.5  45.6 : 44.1 | 33.6 : 39.7  77.2 : 79.0 | 49.7 : 69.8
+//     320        32.0 : 31.3 | 26.4 : 24.6  45.0 : 44.6 | 34.8 : 33.5  65.5 : 70.5 | 47.0 : 42.0  107 : 123 | 72.0 : 73.1
+//     384        34.1 : 32.2 | 29.9 : 28.7  46.7 : 45.7 | 37.5 : 36.4  68.2 : 72.2 | 48.5 : 46.3  116 : 128 | 75.0 : 77.6
+//     512        48.1 : 38.2 | 39.9 : 31.0  62.1 : 53.9 | 50.8 : 41.7  89.6 : 87.4 | 68.6 : 62.7  156 : 160 | 103 : 103
+//     1024       87.7 : 70.7 | 78.3 : 60.0  114 : 98.9 | 93.2 : 76.8   168 : 169 | 127 : 119      295 : 309 | 200 : 204
 //   - a second wave of at most a sixth: up to 8 tiles; else up to 16 tiles; above three waves at any length; up to 32 tiles where the last of
 //     two or three waves is at least a quarter empty and more than a sixth full.
-//   At most one block per SM: only two splits let CTAs share SMs.  It pays in more than three quarters of the SMs from 256 tiles on, with one query
-//   block per head from 448.  Mean of equal lengths and of three draws of spread ones (the longest is the stated one), pauses of 30 ms between
-//   bursts | without pauses, under the power cap:
-//     trees x nodes, heads       12288 tokens          16384                 24576                 28000                 32768
-//     7 x 60, 32 / 8             111 : 110 | 107 : 107 145 : 142 | 142 : 139 210 : 201 | 210 : 203 239 : 227 | 245 : 232 281 : 264 | 287 : 271
-//     9 x 60, 32 / 8             116 : 116 | 113 : 113 153 : 150 | 154 : 151 225 : 216 | 232 : 224 264 : 253 | 289 : 276 296 : 280 | 306 : 286
-//     4 x 60, 64 / 8, <true>                           147 : 146 | 141 : 141 216 : 208 | 209 : 207 243 : 234 | 249 : 239
-//       <false> (2.342e-3 from fp64, this one 2.337e-3)  133       | 134       199       | 208       233       | 241
-//   (The other kernel's times but the last line's first two are from before its barriers were asked ahead, which took 3 to 7 % off them.  The lines stay: what goes
-//   to this kernel by them would come back less exact.)
-//     14 x 30, 32 / 8                                  145 : 146 | 141 : 145 213 : 210 | 223 : 216 238 : 239 | 264 : 252 276 : 278 | 296 : 286
-//     18 x 30, 32 / 8                                  154 : 163 | 153 : 165 231 : 240 | 249 : 257 265 : 274 | 289 : 292 314 : 320 | 339 : 332
+//   At most one block per SM: only two splits let CTAs share SMs.  In more than three quarters of the SMs that was the faster way from 256 tiles on, with one query
+//   block per head from 448, and as exact as the following instance.  Since the other kernel asks its barriers ahead and takes Q from tensor memory it is the slower
+//   way for several query blocks per head: the lines are from before, and would lie elsewhere today.  us a call, this kernel : <false> : <true>, equal lengths | mean of three
+//   draws of spread ones, pauses of 30 ms between bursts of 20 calls (without pauses, under the power cap, the same within 5 %):
+//     trees x nodes, heads    16384 tokens                      24576                             32768
+//     4 x 60, 64 / 8          146 : 127 : 128 | 142 : 120 : 121 213 : 189 : 190 | 203 : 175 : 176 282 : 251 : 251 | 263 : 227 : 229
+//     7 x 60, 32 / 8          147 : 127 : 128 | 136 : 118 : 118 213 : 189 : 189 | 197 : 170 : 170 281 : 251 : 252 | 257 : 223 : 224
+//     9 x 60, 32 / 8          166 : 147 : 148 | 141 : 121 : 122 245 : 221 : 221 | 205 : 179 : 179 324 : 294 : 296 | 270 : 236 : 237
+//     14 x 30, 32 / 8                                                                             320 : 311 : 315 | 263 : 241 : 247
+//     18 x 30, 32 / 8                                                                             380 : 364 : 374 | 294 : 273 : 275
+//   2-norm relative error against fp64, in 1e-3, the same order: 4 x 60 2.3423 : 2.3458 : 2.3422, 2.3416 : 2.3438 : 2.3400, 2.3436 : 2.3440 : 2.3419; 7 x 60
+//   2.3422 : 2.3450 : 2.3433, 2.3420 : 2.3467 : 2.3415, 2.3424 : 2.3438 : 2.3417.
 // Two CTAs on an SM is what runs (128 blocks of 129 tiles take 104 us alone, 256 blocks 146), also in pairs; cudaOccupancyMaxActiveClusters
 // counts one, as it does for any kernel that allocates tensor memory (it does not know how many columns), so it is not asked.
 inline int duo_splits(int base_ctas, int mblocks, int sm_count, int prefix_tiles) {
@@ -66,10 +70,9 @@ inline int duo_splits(int base_ctas, int mblocks, int sm_count, int prefix_tiles
 }
 
 // Launches that tree_attn_duo_kernel takes as long for or longer, and rounds a little less (FOLLOW makes up for it): second or third waves that are at least
-// a quarter empty, with several query blocks per head.  FOLLOW has its price where two waves of equal lengths follow one another: 10 trees of 60
-// nodes, 32 / 8 heads, plain : FOLLOW : tree_attn_duo_kernel's better choice, equal | spread: 2048 tokens 42 : 44 : 55 | 24 : 23 : 42, 4096 71 : 77 : 76 | 43 : 44 :
-// 53, 8192 132 : 147 : 144 | 82 : 82 : 85.  One query block per head was never that kernel's: plain (5 trees of 40 nodes, 32 / 32 heads,
-// FOLLOW 4096 tokens 82.9 : 80.3 | 43.8 : 42.0, 8192 160 : 150 | 83 : 82).
+// a quarter empty, with several query blocks per head.  What FOLLOW costs, 10 trees of 60 nodes, 32 / 8 heads, plain : FOLLOW : tree_attn_duo_kernel, equal | spread:
+// 2048 tokens 41.8 : 42.1 : 42.7 | 25.3 : 25.5 : 38.9, 4096 69.2 : 70.6 : 72.5 | 37.1 : 39.0 : 65.1, 8192 122 : 125 : 136 | 70.4 : 67.5 : 120 (FOLLOW's with Q from tensor memory).
+// One query block per head was never that kernel's: plain (5 trees of 40 nodes, 32 / 32 heads, 4096 tokens 78.4 : 82.3 | 47.6 : 47.7, 8192 144 : 151 | 80.5 : 80.6).
 inline bool wants_follow(int base_ctas, int mblocks, int sm_count, int prefix_tiles) {
     if (mblocks == 1 || base_ctas <= sm_count) return false;
     const int waves = (base_ctas + sm_count - 1) / sm_count;
@@ -78,7 +81,7 @@ inline bool wants_follow(int base_ctas, int mblocks, int sm_count, int prefix_ti
 
 struct AttnChoice {
     bool duo;                        // tree_attn_duo_kernel
-    bool follow;                     // tree_attn_umma_kernel<true>
+    bool follow;                     // tree_attn_umma_kernel with FOLLOW
     int splits;
 };
 // blocks: query blocks of all (sequence, head) pairs, mblocks: of one; cluster_cap[s]: CTAs of tree_attn_umma_kernel that run at once in clusters of s

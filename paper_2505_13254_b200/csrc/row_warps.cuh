@@ -11,9 +11,10 @@
 //
 // Why: the same arithmetic behind a ring of 32 KiB items and CTA-wide row ends ran at half of the issue slots with no pipe
 // above 40 % busy (16 warps in lockstep, four barriers per row, 11 instructions per logit); warps that drift apart hide one
-// another's row ends, and without the item bookkeeping a logit costs 7.2.  560 rows of 128256 bf16: 50.3 -> 36.8 us (3.9 TB/s;
-// the shares themselves are read at 6 TB/s in 24 us, the rest is the start, the row ends of the last shares and the tree stage),
-// 1088 rows: 93.8 -> 62 us, 240 rows: 37.8 -> 21.5 us, 1088 rows of 32000: 44.0 -> 24.2 us.
+// another's row ends, and without the item bookkeeping a logit costs 7.2.  560 rows of 128256 bf16: 50.3 -> 36.8 us (3.9 TB/s).
+// What bounds it, from time stamps of every warp: the rounds of 19 of 20 shares are over after 29 us, read at 5.0 TB/s (1600 clocks a round, 32 KiB of loads in
+// flight on an SM); then all warps are at the row end of their last segment at once, 4.8 us each, and for 7 us next to nothing is read.  Shorter shares pay the same
+// end: 83 MB 18 of 25 us, 74 MB in rows of 32000 18 of 25.5.  1088 rows: 93.8 -> 62 us, 240 rows: 37.8 -> 21.5 us, 1088 rows of 32000: 44.0 -> 24.2 us.
 #pragma once
 
 #define QW_WARPS 16

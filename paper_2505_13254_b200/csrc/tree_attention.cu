@@ -103,7 +103,8 @@ __device__ __forceinline__ void prefix_range(int L, int nsplit, int split, int& 
 // softmax needs no shuffles and the two streams never wait for one another: while one exponentiates (the
 // special-function unit), the other loads, masks and stores.  Three more warps give one elected thread each: the S issuer
 // (S = Q K^T of tile i + 2 as soon as S of tile i is in registers; 8 instructions of K = 16, operands
-// straight from the swizzled TMA tiles: Q and K are K-major), the P V issuer (O_g += P V as soon as a P
+// straight from the swizzled TMA tiles, Q and K are K-major; in long CTAs of some launches Q comes from tensor memory, where the
+// softmax threads copy it while the first S are computed), the P V issuer (O_g += P V as soon as a P
 // is written; V is the MN-major operand, the same swizzled tile as it arrived by TMA) and the TMA
 // producer (a stage's K is refilled as soon as the S that read it is complete, its V once its P V is).
 // A stream rescales its O in tensor memory only when a row's running maximum grows.  After the last
@@ -455,8 +456,8 @@ tree_attn_umma_kernel(const __grid_constant__ AttnParams p, const __grid_constan
     // What bounds a tile is the chain of a stream: 128 clocks for S, 140 for the maximum, 640 for the exponentials (530 with both streams at them), 30 for P,
     // and 123 for each answer of a barrier that is long complete.  So both barriers are asked ahead of other work and the answer is looked at
     // behind it, and the S issuer waits for K first: the slowest CTA of a launch, whose two streams are in step, takes 780 clocks a tile instead of
-    // 910.  Us a call, timed in turn: 4 x 16300 tokens, 60 nodes, 64 / 8 heads 141 -> 131, 4 x 4700 46.5 -> 43.8, 16 trees, 32 / 8 heads, 4096 tokens
-    // 79.3 -> 78.4, 14 trees of 30 nodes, 24576 tokens 198 -> 191; one tree of 2048 tokens 10.7 both ways.  (S of the next tile loaded ahead of P's store: 148
+    // 910.  Us a call with Q from shared memory, without : with that, timed in turn: 4 trees of 60 nodes, 64 / 8 heads, 16300 tokens 141 : 130, 4700 47.1 : 44.4; 10 trees,
+    // 32 / 8 heads, 4096 tokens 75.1 : 71.3; 16 trees 78.4 : 77.1; one tree of 2048 tokens 11.4 both ways.  (S of the next tile loaded ahead of P's store: 148
     // for the first; the streams' exponentials in turns: 142 .. 150.)
     unsigned int sr[64];                                     // the row's 64 scores
     if (QT && warp < 8 && ntiles > ATT_Q_TILES) {                    // Q into tensor memory while the first S are computed: half a row per thread

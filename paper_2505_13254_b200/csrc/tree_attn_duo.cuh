@@ -7,10 +7,10 @@
 // over tiles of 64 keys: S is double-buffered, P (bf16) overwrites the S it came from, so the tensor-core order is S(i), P V(i),
 // S(i + 2) from one issuing thread.  Two threads share a row (32 keys of a tile each).  One producer warp: prefix tiles by tiled
 // copies, the indirectly indexed rows of Q and of the tree tokens by tile::gather4.
-// Bound by the chain of a tile (S, load, maximum, exponentials, P V): 0.68 us for one CTA, 1.06 us for two at once, against 1.17 us
-// for two tiles of tree_attn_umma_kernel.  4 x 62 nodes, 64 / 8 heads, 32768 tokens: 302 us against 306 (both under the power cap); 16 trees,
-// 32 / 8 heads, 512 tokens 19.3 against 24.9; 8 trees, 32 / 32 heads, 512 tokens 18.9 against 24.7 (which launches come here: see
-// duo_splits).  With tiles of 128 keys S and P leave room for one buffer only: 366 us at 32768 tokens.
+// Bound by the chain of a tile (S, load, maximum, exponentials, P V): 0.68 us for one CTA, 1.06 us for two at once, against 0.77 to 1.0 us
+// for two tiles of tree_attn_umma_kernel, but nothing of a start or an end is left uncovered.  16 trees of 60 nodes, 32 / 8 heads, 512 tokens 19.4 us against 22.1; 32 trees 38.2
+// against 48.1 (which launches come here, and what it costs at long prefixes: see duo_splits).  With tiles of 128 keys S and P leave room for one buffer only: 4 x 62 nodes,
+// 64 / 8 heads, 32768 tokens 366 us instead of 302.
 #pragma once
 
 #define AD_HALF_BYTES (ATT_TILE_BYTES / 2)          // columns 0..63 / 64..127 of a K or V tile (rows of 128 bytes, 128-byte swizzle)

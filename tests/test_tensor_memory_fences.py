@@ -33,3 +33,13 @@ def test_lanes_that_waited_alone_meet_again_ahead_of_tensor_memory():
     assert len(waits) == 2
     for at in waits:
         assert re.search(r"\btmem_\w+\(|__syncwarp\(\)|__any_sync\(HS_FULL_MASK", body[at:]).group(0).startswith("__")
+
+
+def test_the_query_rows_are_handed_to_the_issuer_behind_both_fences():
+    body = re.sub(r"\s+", " ", text("tree_attention.cu"))
+    written = re.search(r"tmem_st32\(tQ (.*?)bar\.arrive 3, %0;\" ::\"r\"\(UM_SM_THREADS \+ 32\)", body).group(1)
+    assert 0 < written.find("tmem_wait_st()") < written.find("tc_fence_before_sync()")
+    # the issuer meets the 256 softmax threads once, ahead of the first product that reads them
+    assert re.search(r"if \(i == UM_Q_FIRST\) \{ named_bar_sync\(3, UM_SM_THREADS \+ 32\); tc_fence_after_sync\(\); \} "
+                     r"issue_qk\(i, \[\]\(int t\) \{ return t >= UM_Q_FIRST; \}\)", body)
+    assert body.count("named_bar_sync(3,") == body.count("bar.arrive 3,") == 1
