@@ -71,7 +71,7 @@ inline int duo_splits(int base_ctas, int mblocks, int sm_count, int prefix_tiles
 
 // Launches that tree_attn_duo_kernel takes as long for or longer, and rounds a little less (FOLLOW makes up for it): second or third waves that are at least
 // a quarter empty, with several query blocks per head.  What FOLLOW costs, 10 trees of 60 nodes, 32 / 8 heads, plain : FOLLOW : tree_attn_duo_kernel, equal | spread:
-// 2048 tokens 41.8 : 42.1 : 42.7 | 25.3 : 25.5 : 38.9, 4096 69.2 : 70.6 : 72.5 | 37.1 : 39.0 : 65.1, 8192 122 : 125 : 136 | 70.4 : 67.5 : 120 (FOLLOW's with Q from tensor memory).
+// 2048 tokens 41.8 : 42.1 : 42.7 | 25.3 : 25.5 : 38.9, 4096 69.2 : 72.0 : 72.5 | 37.1 : 36.5 : 65.1, 8192 122 : 125 : 136 | 70.4 : 67.5 : 120 (FOLLOW's of the last two with Q from tensor memory).
 // One query block per head was never that kernel's: plain (5 trees of 40 nodes, 32 / 32 heads, 4096 tokens 78.4 : 82.3 | 47.6 : 47.7, 8192 144 : 151 | 80.5 : 80.6).
 inline bool wants_follow(int base_ctas, int mblocks, int sm_count, int prefix_tiles) {
     if (mblocks == 1 || base_ctas <= sm_count) return false;
@@ -101,10 +101,11 @@ inline AttnChoice attn_choice(int blocks, int mblocks, int sm_count, int prefix_
 //     4 x 60, 32 / 8, 2 splits 22.0 : 23.1 | 22.5 : 21.9 24.1 : 24.8 | 24.6 : 23.5 27.4 : 27.2 | 26.8 : 25.5 30.2 : 29.3 | 29.7 : 27.6 41.8 : 39.1 | 41.3 : 37.6 76.1 : 70.0 | 72.5 : 62.7
 //     2 x 60, 32 / 8, 4 splits 21.2 : 22.5 | 21.4 : 21.1 23.7 : 23.9 | 24.0 : 23.0 27.2 : 26.9 | 26.7 : 25.7 29.1 : 28.6 | 28.4 : 26.5 41.1 : 38.7 | 40.8 : 36.7 76.0 : 69.9 | 73.2 : 64.0
 // Not in more than one wave (16 x 60, 32 / 8, 1700 tokens 41.5 : 44.0 | 33.3 : 33.7, 4096 77.2 : 77.4 | 50.1 : 51.9; 10 x 60 1700 37.4 : 40.8 | 23.0 : 23.0, 12000 in splits 156 :
-// 162 | 114 : 118; 8 x 60, 64 / 8, 4096 72.5 : 74.8 | 60.4 : 62.9) but for FOLLOW's above 64 tiles (10 x 60, 8192 124 : 127 | 73.5 : 69.9), and not with one query
+// 162 | 114 : 118; 8 x 60, 64 / 8, 4096 72.5 : 74.8 | 60.4 : 62.9; FOLLOW's 12 x 60, 32 / 8, 4096 72.8 : 74.0 | 46.8 : 47.9) but for FOLLOW's above 60 tiles with a second wave of at
+// most a sixth (10 x 60, 32 / 8, 4096 71.0 : 72.2 | 38.8 : 36.9, 8192 124 : 127 | 73.5 : 69.9; at 3500 62.0 : 65.2 | 36.9 : 36.2), and not with one query
 // block per head, where K and V come from DRAM (10 x 30, 32 / 8, 8192 66.5 : 68.7 | 49.3 : 50.4; 4 x 60, 32 / 32, 1700 23.1 : 24.2 | 21.0 : 21.2).
 #define ATT_Q_TILES 31
 inline bool q_from_tensor_memory(int blocks, int mblocks, int sm_count, int prefix_tiles, int tree_tiles, const AttnChoice& c) {
     if (c.duo || mblocks == 1 || (prefix_tiles + c.splits - 1) / c.splits + tree_tiles <= ATT_Q_TILES) return false;
-    return c.follow ? prefix_tiles > 64 : blocks * c.splits <= sm_count;
+    return c.follow ? 6 * blocks <= 7 * sm_count && prefix_tiles > 60 : blocks * c.splits <= sm_count;
 }

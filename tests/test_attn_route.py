@@ -23,8 +23,8 @@ def test_lines(batch, nodes, hq, hkv, longest, kernel):
     (7, 60, 32, 8, 30 * 64, 0), (7, 60, 32, 8, 30 * 64 + 1, 1), (7, 60, 32, 8, 8192, 1),    # 112 blocks: from 31 prefix tiles and the tree's on
     (4, 100, 32, 8, 29 * 64, 0), (4, 100, 32, 8, 29 * 64 + 1, 1),         # two tiles of the tree
     (2, 60, 32, 8, 4 * 30 * 64, 0), (2, 60, 32, 8, 4 * 30 * 64 + 1, 4), (1, 60, 64, 8, 16384, 4),    # of a split's share
-    (16, 60, 32, 8, 8192, 0), (12, 60, 32, 8, 4096, 0),                   # more than one wave: not
-    (10, 60, 32, 8, 4096, 0), (10, 60, 32, 8, 4097, 1), (5, 60, 64, 8, 8192, 1), (10, 60, 32, 8, 8193, 0),    # but FOLLOW's above 64 tiles
+    (16, 60, 32, 8, 8192, 0),                   # more than one wave: not
+    (10, 60, 32, 8, 60 * 64, 0), (10, 60, 32, 8, 60 * 64 + 1, 1), (12, 60, 32, 8, 4096, 0), (5, 60, 64, 8, 8192, 1), (10, 60, 32, 8, 8193, 0),    # but FOLLOW's above 60 tiles
     (5, 60, 32, 8, 12800, 0),                                             # 80 blocks in three splits: two waves
     (16, 30, 32, 8, 12000, 0), (2, 60, 32, 32, 8192, 0),                  # one query block per head: never
     (4, 62, 64, 8, 16384, 0),                                             # two CTAs per SM
