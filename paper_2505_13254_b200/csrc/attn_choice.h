@@ -93,19 +93,23 @@ inline AttnChoice attn_choice(int blocks, int mblocks, int sm_count, int prefix_
 
 // Does a launch of tree_attn_umma_kernel have CTAs that take Q as the A operand from tensor memory: those of more than ATT_Q_TILES tiles?
 // With 64 columns of S the product reads Q from shared memory for longer than it multiplies (387 clocks a tile instead of 258, 623 instead of 515 with P V), but the copy
-// of Q and the slower issue are paid for first, and where the tiles are not what a launch waits for nothing comes back.  us a call, from shared memory : so,
-// equal lengths | mean of three draws of spread ones; tokens for each split, i.e. 27, 32, 36, 41, 64, 128 tiles in a CTA and the tree's:
-//     trees x nodes, heads     1700                      2000                      2300                      2600                      4096                      8192
-//     4 x 60, 64 / 8           20.1 : 20.3 | 20.2 : 20.2 22.4 : 22.3 | 22.7 : 22.0 24.4 : 23.8 | 24.5 : 23.9 27.2 : 26.1 | 26.9 : 25.4 37.1 : 35.5 | 37.8 : 34.7 66.9 : 64.1 | 63.0 : 60.3
-//     7 x 60, 32 / 8           20.1 : 20.2 | 19.4 : 19.5 22.2 : 22.3 | 22.0 : 21.6 24.4 : 24.6 | 23.9 : 23.2 25.7 : 26.3 | 26.1 : 25.3 38.7 : 36.2 | 35.3 : 35.0 69.5 : 63.9 | 65.2 : 60.2
-//     4 x 60, 32 / 8, 2 splits 22.0 : 23.1 | 22.5 : 21.9 24.1 : 24.8 | 24.6 : 23.5 27.4 : 27.2 | 26.8 : 25.5 30.2 : 29.3 | 29.7 : 27.6 41.8 : 39.1 | 41.3 : 37.6 76.1 : 70.0 | 72.5 : 62.7
-//     2 x 60, 32 / 8, 4 splits 21.2 : 22.5 | 21.4 : 21.1 23.7 : 23.9 | 24.0 : 23.0 27.2 : 26.9 | 26.7 : 25.7 29.1 : 28.6 | 28.4 : 26.5 41.1 : 38.7 | 40.8 : 36.7 76.0 : 69.9 | 73.2 : 64.0
+// of Q and the slower issue are paid for first, and where the tiles are not what a launch waits for nothing comes back.  us a call, inputs rotating through more than twice
+// L2, from shared memory : so, equal lengths | mean of three draws of spread ones; tokens for each split, i.e. 30, 33, 36, 41 and 64 tiles in a CTA and the tree's:
+//     trees x nodes, heads     1900                      2100                      2300                      2600                      4096
+//     4 x 60, 64 / 8           21.9 : 22.4 | 21.8 : 21.8 23.4 : 23.7 | 23.3 : 22.9 24.8 : 25.0 | 25.2 : 24.2 27.2 : 27.1 | 27.2 : 26.5 37.9 : 37.3 | 37.1 : 35.9
+//     4 x 36, 64 / 8           20.9 : 22.1 | 20.5 : 21.4 22.4 : 23.4 | 21.7 : 22.6 23.9 : 24.7 | 22.2 : 23.6 26.0 : 26.9 | 25.5 : 26.1 37.2 : 36.9 | 34.7 : 35.2
+//     7 x 60, 32 / 8           22.2 : 22.5 | 21.2 : 21.6 23.2 : 23.9 | 22.7 : 22.9 24.8 : 25.3 | 24.1 : 24.1 27.4 : 27.6 | 26.2 : 26.4 40.6 : 37.5 | 37.2 : 36.4
+//     9 x 60, 32 / 8           22.2 : 23.5 | 21.9 : 22.2 23.9 : 25.2 | 22.8 : 22.8 25.9 : 26.5 | 24.5 : 24.3 29.0 : 28.9 | 26.6 : 26.8 42.0 : 40.2 | 39.7 : 37.4
+//     4 x 60, 32 / 8, 2 splits 25.1 : 25.9 | 24.8 : 24.1 26.6 : 26.8 | 26.4 : 25.1 28.3 : 28.3 | 28.1 : 26.6 31.1 : 30.4 | 30.6 : 28.7 43.3 : 40.2 | 42.9 : 39.0
+//     2 x 60, 32 / 8, 4 splits 24.0 : 25.2 | 23.8 : 23.4 26.0 : 26.9 | 26.0 : 25.6 27.7 : 28.3 | 27.5 : 26.8 30.1 : 30.3 | 29.2 : 27.7 42.9 : 40.6 | 42.1 : 38.2
 // Not in more than one wave (16 x 60, 32 / 8, 1700 tokens 41.5 : 44.0 | 33.3 : 33.7, 4096 77.2 : 77.4 | 50.1 : 51.9; 10 x 60 1700 37.4 : 40.8 | 23.0 : 23.0, 12000 in splits 156 :
 // 162 | 114 : 118; 8 x 60, 64 / 8, 4096 72.5 : 74.8 | 60.4 : 62.9; FOLLOW's 12 x 60, 32 / 8, 4096 72.8 : 74.0 | 46.8 : 47.9) but for FOLLOW's above 60 tiles with a second wave of at
-// most a sixth (10 x 60, 32 / 8, 4096 71.0 : 72.2 | 38.8 : 36.9, 8192 124 : 127 | 73.5 : 69.9; at 3500 62.0 : 65.2 | 36.9 : 36.2), and not with one query
-// block per head, where K and V come from DRAM (10 x 30, 32 / 8, 8192 66.5 : 68.7 | 49.3 : 50.4; 4 x 60, 32 / 32, 1700 23.1 : 24.2 | 21.0 : 21.2).
-#define ATT_Q_TILES 31
+// most a sixth (10 x 60, 32 / 8, 4096 71.0 : 72.2 | 38.8 : 36.9, 8192 124 : 127 | 73.5 : 69.9; at 3500 62.0 : 65.2 | 36.9 : 36.2).  With one query block per head, unsplit from 49 tiles on (10 x 30, 32 / 8,
+// 2500 tokens 23.4 : 22.8 | 20.0 : 21.2), up to three quarters of the SMs (one tree of 30, 32 / 8, 16384 tokens 24.7 : 24.4, 32768 41.5 : 39.1; two trees 32768 53.7 : 49.9 | 53.7 : 49.1; 10 trees 4096 42.1 : 40.1 | 35.5 : 35.1): with
+// more of them the tiles wait for DRAM (four trees, 128 CTAs, 12288 37.7 : 38.3 | 33.9 : 33.0, 24576 64.7 : 66.1 | 57.6 : 58.3; 4 x 60, 32 / 32, 1700 23.1 : 24.2 | 21.0 : 21.2).
+#define ATT_Q_TILES 34
 inline bool q_from_tensor_memory(int blocks, int mblocks, int sm_count, int prefix_tiles, int tree_tiles, const AttnChoice& c) {
-    if (c.duo || mblocks == 1 || (prefix_tiles + c.splits - 1) / c.splits + tree_tiles <= ATT_Q_TILES) return false;
-    return c.follow ? 6 * blocks <= 7 * sm_count && prefix_tiles > 60 : blocks * c.splits <= sm_count;
+    if (c.duo || (prefix_tiles + c.splits - 1) / c.splits + tree_tiles <= (mblocks > 1 || c.splits > 1 ? ATT_Q_TILES : 48)) return false;
+    if (c.follow) return 6 * blocks <= 7 * sm_count && prefix_tiles > 60;
+    return mblocks > 1 ? blocks * c.splits <= sm_count : 4 * blocks * c.splits <= 3 * sm_count;
 }

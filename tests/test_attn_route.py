@@ -20,13 +20,14 @@ def test_lines(batch, nodes, hq, hkv, longest, kernel):
 
 @pytest.mark.skipif(not shutil.which("g++"), reason="no host compiler")
 @pytest.mark.parametrize("batch, nodes, hq, hkv, longest, splits", [
-    (7, 60, 32, 8, 30 * 64, 0), (7, 60, 32, 8, 30 * 64 + 1, 1), (7, 60, 32, 8, 8192, 1),    # 112 blocks: from 31 prefix tiles and the tree's on
-    (4, 100, 32, 8, 29 * 64, 0), (4, 100, 32, 8, 29 * 64 + 1, 1),         # two tiles of the tree
-    (2, 60, 32, 8, 4 * 30 * 64, 0), (2, 60, 32, 8, 4 * 30 * 64 + 1, 4), (1, 60, 64, 8, 16384, 4),    # of a split's share
+    (7, 60, 32, 8, 33 * 64, 0), (7, 60, 32, 8, 33 * 64 + 1, 1), (7, 60, 32, 8, 8192, 1),    # 112 blocks: from 34 prefix tiles and the tree's on
+    (4, 100, 32, 8, 32 * 64, 0), (4, 100, 32, 8, 32 * 64 + 1, 1),         # two tiles of the tree
+    (2, 60, 32, 8, 4 * 33 * 64, 0), (2, 60, 32, 8, 4 * 33 * 64 + 1, 4), (1, 60, 64, 8, 16384, 4),    # of a split's share
     (16, 60, 32, 8, 8192, 0),                   # more than one wave: not
     (10, 60, 32, 8, 60 * 64, 0), (10, 60, 32, 8, 60 * 64 + 1, 1), (12, 60, 32, 8, 4096, 0), (5, 60, 64, 8, 8192, 1), (10, 60, 32, 8, 8193, 0),    # but FOLLOW's above 60 tiles
     (5, 60, 32, 8, 12800, 0),                                             # 80 blocks in three splits: two waves
-    (16, 30, 32, 8, 12000, 0), (2, 60, 32, 32, 8192, 0),                  # one query block per head: never
+    (10, 30, 32, 8, 47 * 64, 0), (10, 30, 32, 8, 47 * 64 + 1, 1), (1, 30, 32, 8, 8 * 33 * 64, 0), (1, 30, 32, 8, 8 * 33 * 64 + 1, 8), (9, 30, 32, 8, 8192, 0),    # one query block per head: 80, 64, 144 CTAs
+    (16, 30, 32, 8, 12000, 0), (2, 60, 32, 32, 8192, 0),
     (4, 62, 64, 8, 16384, 0),                                             # two CTAs per SM
 ])
 def test_query_operand(batch, nodes, hq, hkv, longest, splits):
