@@ -6,7 +6,7 @@
 // KV splits (= cluster size) of tree_attn_umma_kernel: the number with the least time on the critical path, waves of CTAs (as many
 // clusters of that size as the device runs at once) times {tiles per CTA, what lies around them, merge}, in half tiles.  A tile is
 // 0.5 us (0.38 in CTAs that take Q from tensor memory), start, tree tiles and output 6 us, the merge of splits 2.2 us.  us a call in 1 .. 6 splits, * the rule's (seven and
-// eight never fit at once: another wave), trees of 60 nodes, equal lengths:
+// eight splits of these do not fit at once: another wave), trees of 60 nodes, equal lengths:
 //     one tree, 32 / 8 heads, 256 tokens     7.6* 9.1  8.4  8.5  8.6  8.7     384       8.6  9.4  9.1  8.2  8.7  9.2*    1024      12.7 11.9 10.3 9.8  9.7  9.6*
 //                             2048           20.6 15.0 13.1 11.8 11.1 11.2*   4096      32.9 23.2 18.4 15.2 14.7 13.7*   8192      57.5 36.0 28.1 23.5 22.0 19.6*
 //     one tree, 64 / 8,       512            9.7  10.1 10.3 10.3*             2048      21.3 16.1 14.2 13.7*             8192      59.3 37.1 29.6 26.0*
